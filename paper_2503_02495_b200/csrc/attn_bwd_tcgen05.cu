@@ -49,7 +49,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 int ld_out /* elements per row of the output buffers */, const float* __restrict__ lse,
                 const float* __restrict__ delta, const int* __restrict__ pair_row, const int* __restrict__ patch_idx,
                 int c, int l_p, int Lv, int l_a, int heads, int causal, float scale_log2, float inv_sqrt_dh,
-                int* status) {
+                int* status, const __grid_constant__ Rope rope /* pair0 < 32: dq and dk are rotated back (Eq. 32) */) {
     pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -251,6 +251,20 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 for (int i = 0; i < DH / 2; ++i) acc[i] = 0.f;
             }
             if (orow < l_a) {
+                if (which == 0 && 16 * hsel + 15 >= rope.pair0) {      // gradient w.r.t. the rotated q / k -> w.r.t. the projection
+                    const int pj = patch_idx[(size_t)pair * c + orow / l_p];
+                    const float t = (float)(max(pj, 0) * l_p + orow % l_p);      // (rows of unused slots are zero)
+#pragma unroll
+                    for (int i = 0; i < DH / 4; ++i) {
+                        const int p = 16 * hsel + i;
+                        if (p < rope.pair0) continue;
+                        float cs, sn;
+                        rope_angle(rope, p, t, cs, sn);
+                        const float a0 = acc[2 * i], a1 = acc[2 * i + 1];
+                        acc[2 * i] = a0 * cs + a1 * sn;
+                        acc[2 * i + 1] = a1 * cs - a0 * sn;
+                    }
+                }
                 __nv_bfloat16* out = (which == 0 ? out0 : out1) + (size_t)(row_base + orow) * ld_out + col_h + hsel * 32;
 #pragma unroll
                 for (int ch = 0; ch < DH / 16; ++ch) {
@@ -280,7 +294,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // lse, delta: [rows_max, heads] float32 (lse as written by the forward kernel, natural logarithm).
 uoe_status launch_attention_backward(const Dims& D, const void* q, const void* k, const void* v, const void* dout,
                                      const float* lse, const float* delta, void* dq, void* dk, void* dv, int ld_out,
-                                     const int* pair_row, const int* patch_idx, bool causal, int* status,
+                                     const int* pair_row, const int* patch_idx, bool causal, const Rope& rope, int* status,
                                      cudaStream_t s) {
     if (D.d_h != DH) return UOE_ERR_UNSUPPORTED;
     static DeviceOnce once_kv, once_q;
@@ -306,14 +320,14 @@ uoe_status launch_attention_backward(const Dims& D, const void* q, const void* k
         ProfScope ps("attn_bwd_dkdv", s);
         launch_k(attn_bwd_kernel<false>, grid, dim3(kThreads), BCfg<false>::SMEM, s, tm[0], tm[1], tm[2], tm[3],
                  (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, ld_out, lse, delta, pair_row, patch_idx, D.c, D.l_p, D.Lv, D.l_a,
-                 heads, causal ? 1 : 0, scale_log2, inv_sqrt_dh, status);
+                 heads, causal ? 1 : 0, scale_log2, inv_sqrt_dh, status, rope);
     }
     UOE_LAUNCHED();
     {
         ProfScope ps("attn_bwd_dq", s);
         launch_k(attn_bwd_kernel<true>, grid, dim3(kThreads), BCfg<true>::SMEM, s, tm[0], tm[1], tm[2], tm[3],
                  (__nv_bfloat16*)dq, (__nv_bfloat16*)nullptr, ld_out, lse, delta, pair_row, patch_idx, D.c, D.l_p, D.Lv,
-                 D.l_a, heads, causal ? 1 : 0, scale_log2, inv_sqrt_dh, status);
+                 D.l_a, heads, causal ? 1 : 0, scale_log2, inv_sqrt_dh, status, rope);
     }
     UOE_LAUNCHED();
     return UOE_OK;

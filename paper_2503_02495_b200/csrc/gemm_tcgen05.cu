@@ -78,7 +78,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const float* __restrict__ blk_scale /* [rows / 128] or null: factor on the activated output (forward epilogue) */,
                  const __grid_constant__ CUtensorMap tmX, const SrcMap smap, int l_p, int Bm,
                  const __grid_constant__ CUtensorMap tmC0, const __grid_constant__ CUtensorMap tmC1,
-                 const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmPre) {
+                 const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmPre,
+                 const __grid_constant__ Rope rope /* pair0 < 32: matrices 0 and 1 hold 64-wide heads to be rotated */) {
     pdl_trigger();
     using Cf = Cfg<BN, MT, BWD, PAIR>;
     extern __shared__ uint8_t smem_raw[];
@@ -305,6 +306,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             locate(tile / n_tiles, e, row0, blocks);
             const int mat = (tile % n_tiles) / n_tiles_mat, col0 = ((tile % n_tiles) % n_tiles_mat) * BN;
             const CUtensorMap* tmC = mat == 0 ? &tmC0 : (mat == 1 ? &tmC1 : &tmC2);
+            int tok = -1;                                    // position of this thread's row in its sample
+            if (!BWD && rope.pair0 < 32 && half < blocks)    // (two dependent look-ups, under the tile's main loop)
+                tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e]);
             const bool ready = mbar_wait(&ctl->tfull[acc], acc_phase, abort_flag, status) && !*abort_flag;
             if (!__all_sync(0xffffffffu, ready)) break;      // warp-uniform: tcgen05.ld below is warp-collective
             tc_fence_after();
@@ -358,6 +362,19 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 unpack16<__nv_bfloat16>(bp[q8], bv);
 #pragma unroll
                                 for (int q = 0; q < 8; ++q) f[8 * q8 + q] += bv[q];
+                            }
+                        }
+                        if (rope.pair0 < 32 && (SIDE3 ? g : mat) < 2) {
+                            // Eq. 32 on the float32 accumulators: the head's last channels, two MUFU operations per pair
+#pragma unroll
+                            for (int p = 0; p < 32; ++p) {
+                                if (p >= rope.pair0) {
+                                    float cs, sn;
+                                    rope_angle(rope, p, (float)max(tok, 0), cs, sn);
+                                    const float a0 = f[2 * p], a1 = f[2 * p + 1];
+                                    f[2 * p] = a0 * cs - a1 * sn;
+                                    f[2 * p + 1] = a0 * sn + a1 * cs;
+                                }
                             }
                         }
                         if (pre) stage_store(f, &tmPre, col0 + g * 64, wrow0);
@@ -471,7 +488,7 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
                                              (__nv_bfloat16*)g.C2, (__nv_bfloat16*)g.pre, g.offsets, g.n, g.K, g.N,
                                              nmat, g.act, status, (const __nv_bfloat16*)g.bwd_h, g.row_gate, g.row_valid,
                                              g.dg_part, (const __nv_bfloat16*)g.bias, g.blk_scale, tmX, smap, g.l_p, g.Bm, tmC[0],
-                                             tmC[1], tmC[2], tmPre);
+                                             tmC[1], tmC[2], tmPre, g.rope ? *g.rope : Rope());
     UOE_LAUNCHED();
     return UOE_OK;
 }
@@ -501,6 +518,7 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
 uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
     if (g.K % BK != 0 || g.N % 64 != 0 || g.nmat > 3) return UOE_ERR_UNSUPPORTED;
     if ((g.bias || g.blk_scale) && (g.bwd || g.nmat > 1)) return UOE_ERR_UNSUPPORTED;      // a bias row per expert, a factor per block: plain forward GEMMs only
+    if (g.rope && g.rope->pair0 < 32 && (g.nmat != 3 || g.bwd)) return UOE_ERR_UNSUPPORTED;
     if (g.nmat > 1 && g.pre) return UOE_ERR_UNSUPPORTED;
     if (g.gather_x && ((!g.src_patch && !g.map.on()) || g.l_p < 8 || g.l_p % 8 != 0 || BM % g.l_p != 0)) return UOE_ERR_INVALID_ARG;
     if (g.rows_max % BM != 0 || g.n > 31) return UOE_ERR_UNSUPPORTED;

@@ -22,8 +22,8 @@ struct PlanPtrs {
     float* row_gate = nullptr;   // [Rmax]   backward only: combine weight of each routed row (0 on pad-token rows and unused slots)
     float* row_valid = nullptr;  // [Rmax]   backward only: 1 on rows that hold a real token, else 0
     int* src_patch = nullptr;    // [Rmax/l_p] source patch (b*m + j) of every l_p-row block of the routed buffers, -1 = zero rows
-    int* slot_pair = nullptr;    // [n,B]    plan written by the router kernel: pair (b*k + s) of the q-th sample in expert i's
-                                 //          region (it replaces src_patch, which that plan does not fill)
+    int* slot_pair = nullptr;    // [n,B]    pair (b*k + s) of the q-th sample in expert i's region (with the plan written by the
+                                 //          router kernel it also replaces src_patch, which that plan does not fill)
     bool inv_relative = false;   // inv_row holds offsets from pair_row (plan written by the router kernel)
     // plan written by the router kernel, whole samples per expert (every chosen expert takes every patch that holds a
     // real token, Eq. 21-26): slot u of a pair is patch u, so inv_row, inv_gate and patch_idx are neither written nor
@@ -107,7 +107,35 @@ inline SrcMap src_map_of(const Dims& D, const PlanPtrs& P, const int* patch_idx)
     g.B = D.B; g.k = D.k; g.c = D.c; g.m = D.m; g.l_p = D.l_p;
     return g;
 }
+// Rotary position embedding (Eq. 32) inside the q / k projection: in every head the last d_rope channels are rotated in
+// pairs (2i, 2i+1) by the angle t * 10000^(-2i/d_rope), t = the token's position in its sample (so the score of a
+// query-key pair depends on their distance in the sample, whichever patches were selected).  The frequencies are
+// turns per token, split in two floats, so that the reduction to one turn is exact to well below the result's rounding.
+// (As a kernel of its own the rotation was a second pass over q and k and two roundings, and its 128 CTAs of sine code
+// started, under programmatic launch, on the few SMs the projection left first: the wide block forward, B = 4, L = 2048,
+// d = 1024, 16 heads, took 343 us with it and takes 189 us with the rotation in the epilogue.)
+struct Rope {
+    int pair0 = 32;                    // first rotated channel pair of a 64-wide head (32: nothing is rotated)
+    SrcMap map;                        // where a routed row comes from (through slot_pair)
+    float hi[32], lo[32];              // turns per token of channel pair p: 10000^(-2 (p - pair0) / d_rope) / (2 pi)
+};
+Rope rope_of(const Dims& D, const PlanPtrs& P, const int* patch_idx);
 #ifdef __CUDACC__
+// (cos, sin) of channel pair p of the token at position t
+__device__ __forceinline__ void rope_angle(const Rope& rp, int p, float t, float& cs, float& sn) {
+    const float r = t * rp.hi[p];
+    const float frac = (r - rintf(r)) + fmaf(t, rp.lo[p], fmaf(t, rp.hi[p], -r));     // fraction of a turn, in [-1/2, 1/2]
+    __sincosf(frac * 6.283185307179586f, &sn, &cs);
+}
+// Position in its sample of the token at routed row r of expert e's region; -1 on padding rows and unused slots.
+__device__ __forceinline__ int token_of(const SrcMap& g, int r, int e, int off_e) {
+    if (r >= g.expert_end[e]) return -1;
+    const int rel = r - off_e, l_a = g.c * g.l_p;
+    const int pair = g.slot_pair[(size_t)e * g.B + rel / l_a];
+    const int u = (rel % l_a) / g.l_p;
+    const int pj = g.n_elig >= 0 ? (u < g.n_elig ? u : -1) : g.patch_idx[(size_t)pair * g.c + u];
+    return pj >= 0 && pj < g.m ? pj * g.l_p + rel % g.l_p : -1;
+}
 // Source patch (index into the [Bm patches] view of the source tensor) of the l_p-row block that starts at routed row
 // r inside the region of expert e (first row off_e); Bm (out of range: the loads return zeros) for padding rows and
 // unused slots.
@@ -184,6 +212,7 @@ struct GemmArgs {
     // bf16 path, forward epilogue: C[r,:] is multiplied, after the activation, by blk_scale[r / 128] (one combine weight
     // per 128-row block, Eq. 40 applied ahead of the second layer; `pre` keeps the unscaled pre-activation)
     const float* blk_scale = nullptr;
+    const Rope* rope = nullptr;       // nmat = 3 (q, k, v of 64-wide heads): q and k are rotated before they are stored
     bool bwd = false;
     const void* bwd_h = nullptr;
     const float* row_gate = nullptr;

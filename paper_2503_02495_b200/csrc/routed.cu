@@ -50,7 +50,8 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             int* __restrict__ pair_row, int* __restrict__ inv_row, float* __restrict__ inv_gate,
             int* __restrict__ expert_end, int* status, float* __restrict__ row_gate, float* __restrict__ row_valid,
             int Lv, int use_gate, int* __restrict__ src_patch, uint4* __restrict__ tail, long long tail_row_vecs,
-            long long rows_max, int rows_given /* pair_row already holds every pair's first row (plan_rows_kernel) */) {
+            long long rows_max, int rows_given /* pair_row already holds every pair's first row (plan_rows_kernel) */,
+            int* __restrict__ slot_pair) {
     pdl_trigger();
     pdl_wait();
     extern __shared__ int s_dyn[];
@@ -92,6 +93,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
         const int row = rows_given ? pair_row[b * k + tid] : offs[my_e[tid]] + hist[my_e[tid]] * l_a;
         prow[tid] = row;
         if (!rows_given) pair_row[b * k + tid] = row;
+        slot_pair[(size_t)my_e[tid] * B + (row - offs[my_e[tid]]) / l_a] = b * k + tid;
     }
     __syncthreads();
     for (int idx = tid; idx < m * k; idx += NT) {          // inverse map: which routed rows feed patch j
@@ -355,7 +357,7 @@ uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_id
     const int threads = (P.row_gate && (long long)D.k * D.l_a >= 4096) ? 512 : 128;      // the backward's per-row weights: k*l_a rows per sample
     launch_k(plan_kernel, dim3(D.B), dim3(threads), smem, s, expert_idx, patch_idx, gate, offsets, D.B, D.n, D.k, D.m, D.c, D.l_p,
                                     P.pair_row, P.inv_row, P.inv_gate, P.expert_end, status, P.row_gate, P.row_valid,
-                                    D.Lv, use_gate ? 1 : 0, P.src_patch, (uint4*)tail, tail_row_bytes / 16, D.Rmax, many ? 1 : 0);
+                                    D.Lv, use_gate ? 1 : 0, P.src_patch, (uint4*)tail, tail_row_bytes / 16, D.Rmax, many ? 1 : 0, P.slot_pair);
     UOE_LAUNCHED();
     return UOE_OK;
 }

@@ -1,5 +1,5 @@
 // uoe_smha_forward: SMHA forward (Eq. 27-30, 32-36) as plan -> grouped q/k/v projections in one launch,
-// gathering x inside the TMA loads (Eq. 27-30) -> optional RoPE (Eq. 32) -> attention over each pair's
+// gathering x inside the TMA loads (Eq. 27-30) and rotating q and k where they leave the accumulator (RoPE, Eq. 32) -> attention over each pair's
 // gathered tokens with the expert's output projection in the same kernel (Eq. 33-35; a separate grouped GEMM
 // when an expert has several heads or d > 512) -> weighted combine (Eq. 36).
 #include "kernels.cuh"
@@ -10,9 +10,6 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
                             const int* pair_row, const int* patch_idx, bool causal, int* status, cudaStream_t s,
                             const void* Wo = nullptr, const int* expert_idx = nullptr, void* z = nullptr);
 bool attention_can_fuse_out(const Dims& D);
-
-uoe_status launch_rope(const Dims& D, void* a, void* b, int ld, const int* pair_row, const int* patch_idx, bool inverse,
-                       cudaStream_t s);
 
 struct SmhaWs { size_t plan, xg, q, k, v, o, z, total; };
 
@@ -63,9 +60,9 @@ uoe_status uoe::smha_forward_run(const Dims& D, const uoe_problem* prob, const v
     if (fused) { gq.gather_x = x; gq.map = src_map_of(D, P, patch_idx); gq.l_p = D.l_p; gq.Bm = D.B * D.m; }
     gq.label = "qkv_proj";
     gq.nmat = 3; gq.W1 = Wk; gq.W2 = Wv; gq.C1 = k; gq.C2 = v;
+    const Rope rope = rope_of(D, P, patch_idx);      // Eq. 32 (nothing if d_rope = 0)
+    gq.rope = &rope;
     st = launch_gemm_bf16(gq, status, stream);
-    if (st != UOE_OK) return st;
-    st = launch_rope(D, q, k, D.d_g, P.pair_row, patch_idx, false, stream);      // Eq. 32 (nothing if d_rope = 0)
     if (st != UOE_OK) return st;
     const bool causal = (prob->flags & UOE_FLAG_CAUSAL) != 0;
     if (attention_can_fuse_out(D)) {          // Eq. 33-35 in one kernel: attention and the expert's output projection

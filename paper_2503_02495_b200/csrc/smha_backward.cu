@@ -20,11 +20,8 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
 bool attention_can_fuse_out(const Dims& D);
 uoe_status launch_attention_backward(const Dims& D, const void* q, const void* k, const void* v, const void* dout,
                                      const float* lse, const float* delta, void* dq, void* dk, void* dv, int ld_out,
-                                     const int* pair_row, const int* patch_idx, bool causal, int* status,
+                                     const int* pair_row, const int* patch_idx, bool causal, const Rope& rope, int* status,
                                      cudaStream_t s);
-
-uoe_status launch_rope(const Dims& D, void* a, void* b, int ld, const int* pair_row, const int* patch_idx, bool inverse,
-                       cudaStream_t s);
 
 namespace {
 
@@ -238,9 +235,9 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     if (fused) { gq.gather_x = x; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m; }
     gq.label = "qkv_proj";
     gq.nmat = 3; gq.W1 = Wk; gq.W2 = Wv; gq.C1 = k; gq.C2 = v;
+    const Rope rope = rope_of(D, P, patch_idx);      // Eq. 32 (nothing if d_rope = 0)
+    gq.rope = &rope;
     st = launch_gemm_bf16(gq, status, stream);
-    if (st != UOE_OK) return st;
-    st = launch_rope(D, q, k, D.d_g, P.pair_row, patch_idx, false, stream);      // Eq. 32 (nothing if d_rope = 0)
     if (st != UOE_OK) return st;
     st = launch_attention(D, q, k, v, o, lse, P.pair_row, patch_idx, causal, status, stream);
     if (st != UOE_OK) return st;
@@ -266,11 +263,7 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     // ---- attention backward ----
     __nv_bfloat16* dq = (__nv_bfloat16*)dqkv;
     st = launch_attention_backward(D, q, k, v, dout, lse, delta, dq, dq + D.d_g, dq + 2 * D.d_g, 3 * D.d_g, P.pair_row,
-                                   patch_idx, causal, status, stream);
-    if (st != UOE_OK) return st;
-
-    // gradients w.r.t. the rotated q, k -> w.r.t. the projections: rotate back
-    st = launch_rope(D, dq, dq + D.d_g, 3 * D.d_g, P.pair_row, patch_idx, true, stream);
+                                   patch_idx, causal, rope, status, stream);
     if (st != UOE_OK) return st;
 
     // ---- projection backward: dx_g and the q/k/v weight gradients from the concatenated [dq dk dv] ----
