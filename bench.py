@@ -82,7 +82,7 @@ def work_table(w: gen.Workload):
         t["wgrad_W1"]["bytes"] = t["wgrad_W2"]["bytes"] = (R * d + R * de) * s + n * d * de * 4
         if patch_major(w):    # dx_g and the backward combine in one kernel: reads dh, W1 and dy, writes dx
             t["bwd_dx"] = dict(flops=2 * R * d * de, bytes=(R * de + n * d * de) * s + 2 * x_bytes)
-        t["pool"] = dict(flops=0, bytes=x_bytes)
+        t["router_apply"] = dict(flops=0, bytes=x_bytes)
     if w.H:
         dg = w.d_g
         att = 4 * w.l_a * w.l_a * dg * w.B * w.k
@@ -664,7 +664,7 @@ def single_mode_of(dev, steps: int):
 
 TENSOR_KERNELS = ("gemm1_act", "gemm2", "mlp_fused", "qkv_proj", "out_proj", "attention", "bwd_da_dh", "bwd_dx", "wgrad_W1", "wgrad_W2",
                   "attn_bwd_dkdv", "attn_bwd_dq", "bwd_do", "bwd_dx_att", "wgrad_Wo", "wgrad_Wqkv")
-HBM_KERNELS = ("route", "gather", "combine", "pool")
+HBM_KERNELS = ("route", "gather", "combine", "router_apply")
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under profiles/.  Every

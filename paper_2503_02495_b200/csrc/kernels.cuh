@@ -172,10 +172,41 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
 
 // Eq. 20 / 26 / 36 / 40: y[b,t,:] = (residual ? x[b,t,:] : 0) + sum_s w_s * z[row_s(t),:], every output row
 // written once, contributions added in ascending slot order.  w_s = gate if use_gate else 1.
+// dW_r = sum over the splits of the partial sums part [nsplit, total], ascending (total = 0: nothing to add).
+struct DwrSum { const float* part = nullptr; float* dW_r = nullptr; int total = 0, nsplit = 0; };
+inline int dwr_sum_blocks(const DwrSum& s) { return (s.total + 15) / 16; }
+#ifdef __CUDACC__
+// Block `blk` of 256 threads adds 16 consecutive values: 16 threads per value take the splits in turn, their sums are
+// added in a fixed tree.
+__device__ __forceinline__ void dwr_sum(const DwrSum& s, int blk) {
+    __shared__ float red[16][17];
+    const int v = threadIdx.x & 15, g = threadIdx.x >> 4;
+    const int idx = blk * 16 + v;
+    float a = 0.f;
+    if (idx < s.total) {
+        int q = g;
+        for (; q + 48 < s.nsplit; q += 64) {
+            const float t0 = s.part[(size_t)q * s.total + idx], t1 = s.part[(size_t)(q + 16) * s.total + idx];
+            const float t2 = s.part[(size_t)(q + 32) * s.total + idx], t3 = s.part[(size_t)(q + 48) * s.total + idx];
+            a += (t0 + t1) + (t2 + t3);
+        }
+        for (; q < s.nsplit; q += 16) a += s.part[(size_t)q * s.total + idx];
+    }
+    red[g][v] = a;
+    __syncthreads();
+    if (g == 0 && idx < s.total) {
+#pragma unroll
+        for (int q = 1; q < 16; ++q) a += red[q][v];
+        s.dW_r[idx] = a;
+    }
+}
+#endif
+uoe_status launch_dwr_sum(const DwrSum& sum, cudaStream_t s);
+
 // If rvec is not null (backward through the router), every real token of patch (b,j) also receives the
-// vector rvec[b*m + j, :]  (float32 [B*m, d]).
+// vector rvec[b*m + j, :]  (float32 [B*m, d]).  `sum` is added up by extra CTAs of the same launch.
 uoe_status launch_combine(const Dims& D, const void* x, const void* z, const PlanPtrs& P, bool residual,
-                          bool use_gate, void* y, cudaStream_t s, const float* rvec = nullptr);
+                          bool use_gate, void* y, cudaStream_t s, const float* rvec = nullptr, const DwrSum& sum = DwrSum());
 
 // Grouped GEMM over the routed rows: C[r,:] = epilogue(A[r,:] @ W[e(r)]) where e(r) is the expert whose
 // region holds row r.  W is [n, K, N] (b_kmajor = false: rows of K, N contiguous) or [n, N, K] (true).
@@ -247,9 +278,7 @@ uoe_status launch_gemm_f32(const GemmArgs& g, cudaStream_t s);
 // Scratch of the router half of a backward pass (all float32).
 struct RouterBwdScratch {
     float* G;       // [B*m, n]   gradient of the router logits per (sample, patch)
-    float* pool;    // [B*m, d]   sums of the real rows of each patch
     float* rvec;    // [B*m, d]   W_r G: added to dx on every real token of the patch
-    float* dgate;   // [B,k,c]
     float* wpart;   // partial sums of dW_r
 };
 size_t router_backward_scratch_bytes(const Dims& D);
@@ -257,7 +286,8 @@ RouterBwdScratch router_backward_scratch(const Dims& D, char* base);
 // dgp: [rows, nt] float32, per-row partials of d(loss)/d(gate) (zero on rows that hold no real token).
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
-                                  const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, cudaStream_t stream);
+                                  const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
+                                  cudaStream_t stream);
 uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s);
 
 // Eq. 38-39 in one kernel for narrow experts (bf16, d_e = 256, d <= 512): z = phi(A W1[e]) W2[e] with the hidden tile

@@ -17,63 +17,68 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// dgate[b,s,u] = sum over the slab's rows and column tiles of the per-row partials; one warp per slab,
-// fixed summation order.  grid ceil(B*k*c / 4), 128 threads.
-__global__ void __launch_bounds__(128)
-dgate_kernel(const float* __restrict__ dg_part, int nt, const int* __restrict__ pair_row,
-             const int* __restrict__ patch_idx, int n_slabs, int c, int m, int l_p, float* __restrict__ dgate) {
-    pdl_trigger();
-    pdl_wait();
-    const int slab = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (slab >= n_slabs) return;
-    const int j = patch_idx[slab];
-    float a = 0.f;
-    if (j >= 0 && j < m) {
-        const float* src = dg_part + ((size_t)pair_row[slab / c] + (size_t)(slab % c) * l_p) * nt;
-        for (int q = lane; q < l_p * nt; q += 32) a += src[q];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) dgate[slab] = a;
-}
-
-// grid B, 128 threads, dynamic smem 2*n*m floats.  G[b,j,i] = dlogit_patch[b,i,j]/cnt_j + dlogit_samp[b,i]/L_valid.
-__global__ void __launch_bounds__(128)
-router_bwd_kernel(const float* __restrict__ dgate,
-                  const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
-                  const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
-                  int l_p, int Lv, float* __restrict__ G) {
+// Gradient of the router logits of one sample from the per-row gate gradients.  grid B, 512 threads, dynamic shared
+// memory (2 n m + k c) floats.  A warp per slab adds the slab's per-row, per-column-tile partials (fixed order), then the
+// softmax Jacobians of Eq. 14 and 21:  G[b,j,i] = dlogit_patch[b,i,j]/cnt_j + dlogit_samp[b,i]/L_valid.
+// Latency-bound (a sample's partials are a few KB to a few hundred KB); one launch instead of a slab-sum kernel and a
+// Jacobian kernel whose sums over a slot list were one thread's serial loop.
+constexpr int kGradThreads = 512;
+__global__ void __launch_bounds__(kGradThreads)
+router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restrict__ pair_row,
+                   const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
+                   const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
+                   int l_p, int Lv, float* __restrict__ G) {
     pdl_trigger();
     pdl_wait();
     extern __shared__ float sm[];
     float* pp = sm;                 // [n][m] patch gate
     float* dpp = sm + n * m;        // [n][m] its gradient
-    __shared__ float ps[32], dps[32], dls[32];
-    const int b = blockIdx.x, tid = threadIdx.x;
-    for (int idx = tid; idx < n * m; idx += 128) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
-    if (tid < n) { ps[tid] = p_samp[(size_t)b * n + tid]; dps[tid] = 0.f; }
-    __syncthreads();
-    // gate = P_samp * P_patch: each chosen expert's slots are handled by one thread, in slot order
-    if (tid < k) {
-        const int i = expert_idx[(size_t)b * k + tid];
-        float acc = 0.f;
-        for (int u = 0; u < c; ++u) {
-            const int j = patch_idx[((size_t)b * k + tid) * c + u];
-            if (j < 0 || j >= m) continue;
-            const float dg = dgate[((size_t)b * k + tid) * c + u];
-            acc += dg * pp[i * m + j];
-            dpp[i * m + j] = dg * ps[i];          // one (expert, patch) pair per slot: no other writer
+    float* dg = sm + 2 * n * m;     // [k][c] gradient of the combine weight of every slot
+    __shared__ float ps[32], dls[32], dps[32];
+    const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int idx = tid; idx < n * m; idx += kGradThreads) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
+    if (tid < 32) { ps[tid] = tid < n ? p_samp[(size_t)b * n + tid] : 0.f; dps[tid] = 0.f; }
+    const int len = l_p * nt;
+    for (int slab = warp; slab < k * c; slab += kGradThreads / 32) {
+        const int j = patch_idx[(size_t)b * k * c + slab];
+        float a = 0.f;
+        if (j >= 0 && j < m) {
+            const float* src = dg_part + ((size_t)pair_row[b * k + slab / c] + (size_t)(slab % c) * l_p) * nt;
+            int q = lane;
+            for (; q + 96 < len; q += 128) {
+                const float t0 = src[q], t1 = src[q + 32], t2 = src[q + 64], t3 = src[q + 96];
+                a += (t0 + t1) + (t2 + t3);
+            }
+            for (; q < len; q += 32) a += src[q];
         }
-        dps[i] = acc;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) dg[slab] = a;
     }
     __syncthreads();
-    if (tid == 0) {                                       // softmax Jacobian of the sample gate (Eq. 21)
-        float dot = 0.f;
-        for (int i = 0; i < n; ++i) dot += ps[i] * dps[i];
-        for (int i = 0; i < n; ++i) dls[i] = ps[i] * (dps[i] - dot);
+    // gate = P_samp * P_patch: a warp per chosen expert, lanes over its slots
+    for (int s = warp; s < k; s += kGradThreads / 32) {
+        const int i = expert_idx[(size_t)b * k + s];
+        float acc = 0.f;
+        for (int u = lane; u < c; u += 32) {
+            const int j = patch_idx[((size_t)b * k + s) * c + u];
+            if (j < 0 || j >= m) continue;
+            acc += dg[s * c + u] * pp[i * m + j];
+            dpp[i * m + j] = dg[s * c + u] * ps[i];      // one (expert, patch) pair per slot: no other writer
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) dps[i] = acc;
     }
     __syncthreads();
-    for (int j = tid; j < m; j += 128) {                  // softmax Jacobian of each patch gate (Eq. 14)
+    if (warp == 0) {                                      // softmax Jacobian of the sample gate (Eq. 21)
+        float dot = ps[lane] * dps[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        dls[lane] = ps[lane] * (dps[lane] - dot);
+    }
+    __syncthreads();
+    for (int j = tid; j < m; j += kGradThreads) {         // softmax Jacobian of each patch gate (Eq. 14)
         const int cnt = max(0, min(l_p, Lv - j * l_p));
         float dot = 0.f;
         for (int i = 0; i < n; ++i) dot += pp[i * m + j] * dpp[i * m + j];
@@ -84,135 +89,183 @@ router_bwd_kernel(const float* __restrict__ dgate,
     }
 }
 
-// grid B*m * column chunks (chunk fastest, so concurrent CTAs read x linearly): sum of the real rows of each
-// patch, float32 [B*m, d]
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-pool_kernel(const T* __restrict__ x, float* __restrict__ pool, int L, int Lv, int d, int m, int l_p, int CT, int nchunks) {
+// What the router's logit gradient G [B*m, n] does to W_r and x, in one pass over x:
+//   dW_r[dd, i] = sum over (b, j) of pool[bj, dd] G[bj, i],  pool = sum of the real rows of patch bj
+//   rvec[bj, dd] = sum_i W_r[dd, i] G[bj, i], which every real token of the patch receives in dx
+// Bound by reading x once.  Grid (column blocks, splits), two CTAs per SM in all; a CTA has one thread per column of its
+// block and walks batches of eight slices: slice = (unit, row thread), where a unit is a patch or a segment of at most
+// 64 rows of a longer one, 16-byte loads, about eight rows per thread and batch, so a batch is 8 / RT units whose rows
+// are dealt to RT row threads.  The next batch's loads are in flight under this batch's arithmetic.  The sums meet in shared memory, then a thread adds its column's products: the pooled tensor
+// never reaches memory.  Every split leaves its own partial dW_r (dwr_sum adds them in split order).  SPREAD: the vector
+// is written to every row of dx at once instead of to rvec (the balance loss, whose whole dx it is).
+// Against a pooling kernel, one or two product kernels, a vector kernel and a spreading kernel (us, cold caches):
+// 23 instead of 58 at B = 256, L = 224, d = 384, n = 6;  9 instead of 22 at B = 16, L = 512, d = 512, n = 8;  77 as before
+// at B = 8, L = 4096, d = 4096, n = 16 (3.9 TB/s: two CTAs per SM do not cover the batch hand-offs there);  SPREAD 39
+// instead of 84 at B = 16, L = 2048, d = 1024, n = 16.
+constexpr int kSlices = 8;
+template <int NMAX, bool SPREAD>
+__global__ void __launch_bounds__(320, NMAX > 16 ? 1 : 2)
+router_apply_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ W_r, const float* __restrict__ G,
+                    float* __restrict__ rvec, float* __restrict__ part, __nv_bfloat16* __restrict__ dx, int units, int L, int Lv,
+                    int d, int n, int m, int l_p, int nseg, int RT, int batches_per_cta) {
     pdl_trigger();
+    extern __shared__ float s_pool[];                // [kSlices][CW] column sums; SPREAD: then [kSlices / RT][CW] bfloat16
+    __shared__ float sG[kSlices * NMAX];
+    const int CW = blockDim.x, tid = threadIdx.x;    // CW: a multiple of 64
+    const int c0 = blockIdx.x * CW;
+    const int ct = tid % (CW / 8), slice = tid / (CW / 8);
+    const int PB = kSlices / RT;                     // units per batch
+    const int seg_rows = (l_p + nseg - 1) / nseg;
+    const int my_q = slice / RT, my_rt = slice % RT;
+    const int col = c0 + ct * 8, dd = c0 + tid;
     pdl_wait();
-    constexpr int V = Vec16<T>::N;
-    __shared__ float red[kThreads * V];
-    const int bj = blockIdx.x / nchunks, chunk = blockIdx.x % nchunks, b = bj / m, j = bj % m;
-    const int ct = threadIdx.x % CT, rt = threadIdx.x / CT, RT = kThreads / CT;
-    const int col = (chunk * CT + ct) * V;
-    const int rows = max(0, min(l_p, Lv - j * l_p));
-    float cs[V];
+    float acc[NMAX], w[NMAX];
 #pragma unroll
-    for (int v = 0; v < V; ++v) cs[v] = 0.f;
-    if (col < d) {
-        const T* base = x + ((size_t)b * L + (size_t)j * l_p) * d + col;
-        int r = rt;
-        for (; r + 7 * RT < rows; r += 8 * RT) {
-            uint4 q[8];
+    for (int i = 0; i < NMAX; ++i) {
+        acc[i] = 0.f;
+        w[i] = (i < n && dd < d) ? __bfloat162float(W_r[(size_t)dd * n + i]) : 0.f;
+    }
+    const int q_lo = blockIdx.y * batches_per_cta * PB, q_hi = min(units, q_lo + batches_per_cta * PB);
+    // the loads of a batch: this thread's first eight rows, and its share of the batch's G (at most four values)
+    uint4 ld[8];
+    float gv[4];
+    int rows = 0, rows_all = 0;                     // real rows of the unit, all its rows
+    const __nv_bfloat16* base = nullptr;
+    auto issue = [&](int q0) {
+        rows = rows_all = 0;
+        const int unit = q0 + my_q;
+        if (my_q < PB && unit < q_hi && col < d) {
+            const int bj = nseg == 1 ? unit : unit / nseg, b = bj / m, s0 = nseg == 1 ? 0 : (unit - bj * nseg) * seg_rows;
+            const int r0 = (bj - b * m) * l_p + s0;      // first row in the sample
+            rows_all = min(seg_rows, l_p - s0);
+            rows = max(0, min(rows_all, Lv - r0));
+            base = x + ((size_t)b * L + r0) * d + col;
+        }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) q[u] = ld_stream16(base + (size_t)(r + u * RT) * d);
+        for (int u = 0; u < 8; ++u)
+            if (my_rt + u * RT < rows) ld[u] = ld_stream16(base + (size_t)(my_rt + u * RT) * d);
+        const int ng = min(PB, q_hi - q0) * n;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                float f[V];
-                unpack16<T>(q[u], f);
+        for (int u = 0; u < 4; ++u)
+            if (tid + u * CW < ng)
+                gv[u] = nseg == 1 ? G[(size_t)q0 * n + tid + u * CW] : G[(size_t)((q0 + (tid + u * CW) / n) / nseg) * n + (tid + u * CW) % n];
+    };
+    if (q_lo < q_hi) issue(q_lo);
+    for (int q0 = q_lo; q0 < q_hi; q0 += PB) {
+        const int nb = min(PB, q_hi - q0), rows_q = rows, rows_all_q = rows_all;
+        __nv_bfloat16* dx_base = SPREAD ? dx + (base - x) : nullptr;
+        {   // ---- column sums of this thread's slice ----
+            float cs[8];
 #pragma unroll
-                for (int v = 0; v < V; ++v) cs[v] += f[v];
+            for (int v = 0; v < 8; ++v) cs[v] = 0.f;
+            auto add = [&](const uint4& t) {
+                float f[8];
+                unpack16<__nv_bfloat16>(t, f);
+#pragma unroll
+                for (int v = 0; v < 8; ++v) cs[v] += f[v];
+            };
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (my_rt + u * RT < rows) add(ld[u]);
+            int r = my_rt + 8 * RT;
+            for (; r + 3 * RT < rows; r += 4 * RT) {
+                uint4 t[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[u] = ld_stream16(base + (size_t)(r + u * RT) * d);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) add(t[u]);
             }
+            for (; r < rows; r += RT) add(ld_stream16(base + (size_t)r * d));
+#pragma unroll
+            for (int v = 0; v < 8; v += 4)
+                *(float4*)(s_pool + slice * CW + ct * 8 + v) = make_float4(cs[v], cs[v + 1], cs[v + 2], cs[v + 3]);
         }
-        for (; r < rows; r += RT) {
-            float f[V];
-            unpack16<T>(ld_stream16(base + (size_t)r * d), f);
 #pragma unroll
-            for (int v = 0; v < V; ++v) cs[v] += f[v];
+        for (int u = 0; u < 4; ++u) {
+            const int idx = tid + u * CW;
+            if (idx < nb * n) sG[(idx / n) * NMAX + idx % n] = gv[u];
         }
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) red[(rt * CT + ct) * V + v] = cs[v];
-    __syncthreads();
-    if (rt == 0 && col < d) {
-        for (int q = 1; q < RT; ++q)
-#pragma unroll
-            for (int v = 0; v < V; ++v) cs[v] += red[(q * CT + ct) * V + v];
-#pragma unroll
-        for (int v = 0; v < V; ++v) pool[(size_t)bj * d + col + v] = cs[v];
-    }
-}
-
-// rvec[bj, dd] = sum_i W_r[dd, i] * G[bj, i]: what the router path adds to dx for every real token of patch bj
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-rvec_kernel(const T* __restrict__ W_r, const float* __restrict__ G, float* __restrict__ rvec, int d, int n) {
-    pdl_trigger();
-    pdl_wait();
-    __shared__ float sG[32];
-    const int bj = blockIdx.x;
-    if (threadIdx.x < n) sG[threadIdx.x] = G[(size_t)bj * n + threadIdx.x];
-    __syncthreads();
-    constexpr int V = Vec16<T>::N;
-    const bool vec_rows = (n % V) == 0;               // a row of W_r is a whole number of 16-byte pieces
-    for (int dd = threadIdx.x; dd < d; dd += kThreads) {
-        float a = 0.f;
-        if (vec_rows) {
-            const uint4* wr = (const uint4*)(W_r + (size_t)dd * n);
-            for (int q = 0; q < n / V; ++q) {
-                float f[V];
-                unpack16<T>(wr[q], f);
-#pragma unroll
-                for (int v = 0; v < V; ++v) a = fmaf(f[v], sG[q * V + v], a);
-            }
-        } else {
-            for (int i = 0; i < n; ++i) a = fmaf(to_f32(W_r[(size_t)dd * n + i]), sG[i], a);
-        }
-        rvec[(size_t)bj * d + dd] = a;
-    }
-}
-
-// dW_r[dd, i] = sum over (b, j) of pool[bj, dd] * G[bj, i] in two fixed-order stages: grid (d/256, S) partial sums
-// over S chunks of bj, then a sum over the chunks.
-constexpr int kDwrSplit = 64;            // most splits (sizes the partial buffer)
-// splits actually used: enough (column block, split) CTAs for two per SM, no more (every split writes d*n partials)
-inline int dwr_split(int d) {
-    const int col_blocks = (d + kThreads - 1) / kThreads;
-    int s = (2 * 148 + col_blocks - 1) / col_blocks;
-    return s < 4 ? 4 : (s > kDwrSplit ? kDwrSplit : s);
-}
-__global__ void __launch_bounds__(kThreads)
-dwr_partial_kernel(const float* __restrict__ pool, const float* __restrict__ G, float* __restrict__ part, int BM, int d,
-                   int n) {
-    pdl_trigger();
-    pdl_wait();
-    __shared__ float sG[64 * 32];
-    const int dd = blockIdx.x * kThreads + threadIdx.x;
-    const int per = (BM + (int)gridDim.y - 1) / (int)gridDim.y;
-    const int lo = blockIdx.y * per, hi = min(BM, lo + per);
-    float acc[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-    for (int b0 = lo; b0 < hi; b0 += 64) {
-        const int nb = min(64, hi - b0);
         __syncthreads();
-        for (int q = threadIdx.x; q < nb * n; q += kThreads) sG[q] = G[(size_t)b0 * n + q];
-        __syncthreads();
-        if (dd < d) {
-            for (int q = 0; q < nb; ++q) {
-                const float p = pool[(size_t)(b0 + q) * d + dd];
+        if (q0 + PB < q_hi) issue(q0 + PB);
+        float rv[kSlices];
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (i < n) acc[i] = fmaf(p, sG[q * n + i], acc[i]);
+        for (int q = 0; q < kSlices; ++q) {          // (unrolled over the largest batch so that rv stays in registers)
+            rv[q] = 0.f;
+            if (q < nb) {
+                float p = 0.f;
+                for (int rt = 0; rt < RT; ++rt) p += s_pool[(q * RT + rt) * CW + tid];
+                float a = 0.f;
+#pragma unroll
+                for (int i = 0; i < NMAX; ++i) {
+                    if (i < n) {
+                        const float g = sG[q * NMAX + i];
+                        acc[i] = fmaf(p, g, acc[i]);
+                        a = fmaf(w[i], g, a);
+                    }
+                }
+                rv[q] = a;
+                if (!SPREAD && dd < d && (nseg == 1 || (q0 + q) % nseg == 0)) rvec[(size_t)(nseg == 1 ? q0 + q : (q0 + q) / nseg) * d + dd] = a;
             }
+        }
+        __syncthreads();
+        if (SPREAD) {
+            __nv_bfloat16* s_rv = (__nv_bfloat16*)s_pool;
+#pragma unroll
+            for (int q = 0; q < kSlices; ++q)
+                if (q < nb) s_rv[q * CW + tid] = __float2bfloat16(rv[q]);
+            __syncthreads();
+            if (my_q < nb && col < d) {
+                const uint4 v = *(const uint4*)(s_rv + my_q * CW + ct * 8);
+                for (int r = my_rt; r < rows_all_q; r += RT) st_stream16(dx_base + (size_t)r * d, r < rows_q ? v : make_uint4(0, 0, 0, 0));
+            }
+            __syncthreads();
         }
     }
     if (dd < d) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
+        for (int i = 0; i < NMAX; ++i)
             if (i < n) part[((size_t)blockIdx.y * d + dd) * n + i] = acc[i];
     }
 }
+
 __global__ void __launch_bounds__(kThreads)
-dwr_sum_kernel(const float* __restrict__ part, float* __restrict__ dW_r, int total, int nsplit) {
+dwr_sum_kernel(const DwrSum s) {
     pdl_trigger();
     pdl_wait();
-    const int idx = blockIdx.x * kThreads + threadIdx.x;
-    if (idx >= total) return;
-    float a = 0.f;
-    for (int s = 0; s < nsplit; ++s) a += part[(size_t)s * total + idx];
-    dW_r[idx] = a;
+    dwr_sum(s, blockIdx.x);
+}
+
+// Column block, row threads and splits of router_apply_kernel for a problem.
+struct ApplyShape { int CW, RT, nseg, col_blocks, splits, per; };
+ApplyShape apply_shape(const Dims& D) {
+    ApplyShape a;
+    a.CW = D.d < 256 ? (D.d + 63) / 64 * 64 : 256;
+    for (int cw : {256, 320, 192, 128})
+        if (D.d % cw == 0) { a.CW = cw; break; }
+    a.col_blocks = (D.d + a.CW - 1) / a.CW;
+    // rows of a patch are dealt to as many threads as leave each about eight rows, one batch of loads
+    a.nseg = (D.l_p + 63) / 64;
+    a.RT = 1;
+    while (a.RT < kSlices && (D.l_p + a.nseg - 1) / a.nseg >= 16 * a.RT) a.RT *= 2;
+    const int PB = kSlices / a.RT, batches = (D.B * D.m * a.nseg + PB - 1) / PB;
+    const int cap = 2 * 148 / a.col_blocks > 1 ? 2 * 148 / a.col_blocks : 1;        // two CTAs per SM: one full wave
+    a.splits = batches < cap ? batches : cap;
+    a.per = (batches + a.splits - 1) / a.splits;
+    a.splits = (batches + a.per - 1) / a.per;
+    return a;
+}
+template <bool SPREAD>
+void launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, const void* W_r, const float* G, float* rvec,
+                         float* part, void* dx, cudaStream_t s) {
+    auto go = [&](auto kern) {
+        launch_k(kern, dim3(a.col_blocks, a.splits), dim3(a.CW), (size_t)kSlices * a.CW * sizeof(float), s, (const __nv_bfloat16*)x,
+                 (const __nv_bfloat16*)W_r, G, rvec, part, (__nv_bfloat16*)dx, D.B * D.m * a.nseg, D.L, D.Lv, D.d, D.n, D.m, D.l_p, a.nseg,
+                 a.RT, a.per);
+    };
+    ProfScope ps("router_apply", s);
+    if (D.n <= 8) go(router_apply_kernel<8, SPREAD>);
+    else if (D.n <= 16) go(router_apply_kernel<16, SPREAD>);
+    else go(router_apply_kernel<32, SPREAD>);
 }
 
 // Gradient of the load-balancing loss (Eq. 42-44) with respect to the router logits.  grid B, 128 threads, dynamic
@@ -254,23 +307,7 @@ balance_bwd_kernel(const float* __restrict__ p_patch, const float* __restrict__ 
     }
 }
 
-// dx[b, t, :] = rvec[b, patch of t, :] on real tokens, 0 on pad tokens (bf16).  grid B*m, 256 threads.
-__global__ void __launch_bounds__(kThreads)
-spread_rvec_kernel(const float* __restrict__ rvec, __nv_bfloat16* __restrict__ dx, int L, int Lv, int d, int m, int l_p) {
-    pdl_trigger();
-    pdl_wait();
-    const int bj = blockIdx.x, b = bj / m, j = bj % m;
-    const int vpr = d / 8;
-    for (int idx = threadIdx.x; idx < l_p * vpr; idx += kThreads) {
-        const int r = idx / vpr, cv = idx % vpr, t = j * l_p + r;
-        float f[8];
-#pragma unroll
-        for (int v = 0; v < 8; ++v) f[v] = t < Lv ? rvec[(size_t)bj * d + cv * 8 + v] : 0.f;
-        st_stream16(dx + ((size_t)b * L + t) * d + (size_t)cv * 8, pack16<__nv_bfloat16>(f));
-    }
-}
-
-struct BwdWs { size_t plan, dyg, xg, dh, ag, dxg, dgp, G, pool, rvec, dgate, wpart, wgpart, total; int nt; };
+struct BwdWs { size_t plan, dyg, xg, dh, ag, dxg, dgp, G, rvec, wpart, wgpart, total; int nt; };
 
 BwdWs bwd_ws(const Dims& D) {
     WsCarver w;
@@ -287,10 +324,8 @@ BwdWs bwd_ws(const Dims& D) {
     r.dxg = w.take((size_t)D.Rmax * D.d * D.esize);
     r.dgp = w.take((size_t)D.Rmax * r.nt * sizeof(float));
     r.G = w.take((size_t)D.B * D.m * D.n * sizeof(float));
-    r.pool = w.take((size_t)D.B * D.m * D.d * sizeof(float));
     r.rvec = w.take((size_t)D.B * D.m * D.d * sizeof(float));
-    r.dgate = w.take((size_t)D.B * D.k * D.c * sizeof(float));
-    r.wpart = w.take((size_t)kDwrSplit * D.d * D.n * sizeof(float));
+    r.wpart = w.take((size_t)apply_shape(D).splits * D.d * D.n * sizeof(float));
     {   // split-K partials, sized for the larger of the two weight gradients
         const size_t s1 = wgrad_scratch_bytes(D.n, D.d, D.d_e, D.Rmax), s2 = wgrad_scratch_bytes(D.n, D.d_e, D.d, D.Rmax);
         r.wgpart = w.take((s1 > s2 ? s1 : s2) + 1024);
@@ -302,72 +337,50 @@ BwdWs bwd_ws(const Dims& D) {
 }  // namespace
 
 // Router half of a backward pass, shared by the UoME and SMHA backward: per-row partials of d(loss)/d(gate)
-// -> dgate per (sample, expert, patch) -> gradient of the router logits G (softmax Jacobians of Eq. 14 and 21)
-// -> dW_r (through the pooled token sums) and rvec, the vector every real token of a patch receives in dx.
+// -> gradient of the router logits G (softmax Jacobians of Eq. 14 and 21) -> partial dW_r (through the pooled token sums)
+// and rvec, the vector every real token of a patch receives in dx.  `sum` is the remaining addition over the partials,
+// for the caller to hand to launch_combine (which does it beside its own work) or to launch_dwr_sum.
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
-                                  const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, cudaStream_t stream) {
+                                  const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
+                                  cudaStream_t stream) {
     if (!D.bf16) return UOE_ERR_UNSUPPORTED;
+    const size_t smem = ((size_t)2 * D.n * D.m + (size_t)D.k * D.c) * sizeof(float);
     if ((size_t)2 * D.n * D.m * sizeof(float) > 40 * 1024) return UOE_ERR_UNSUPPORTED;
-    float *G = rs.G, *pool = rs.pool, *rvec = rs.rvec, *dgate = rs.dgate, *wpart = rs.wpart;
+    static DeviceOnce once;
+    const uoe_status so = smem_opt_in(once, router_grad_kernel, 80 * 1024);      // k c <= n m: at most 60 KB
+    if (so != UOE_OK) return so;
     {
-        ProfScope ps("dgate", stream);
-        const int n_slabs = D.B * D.k * D.c;
-        launch_k(dgate_kernel, dim3((n_slabs + 3) / 4), dim3(128), 0, stream, dgp, nt, P.pair_row, patch_idx, n_slabs, D.c, D.m, D.l_p,
-                                                           dgate);
+        ProfScope ps("router_grad", stream);
+        launch_k(router_grad_kernel, dim3(D.B), dim3(kGradThreads), smem, stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
+                 p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, rs.G);
     }
     UOE_LAUNCHED();
-    {
-        ProfScope ps("router_bwd", stream);
-        launch_k(router_bwd_kernel, dim3(D.B), dim3(128), (size_t)2 * D.n * D.m * sizeof(float), stream, 
-            dgate, expert_idx, patch_idx, p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, G);
-    }
+    const ApplyShape a = apply_shape(D);
+    launch_router_apply<false>(D, a, x, W_r, rs.G, rs.rvec, rs.wpart, nullptr, stream);
     UOE_LAUNCHED();
-    int CT = 64;
-    while (CT > 1 && (CT / 2) * 8 >= D.d) CT /= 2;
-    const int nchunks = (D.d + CT * 8 - 1) / (CT * 8);
-    dim3 grid((unsigned)(D.B * D.m * nchunks));
-    {
-        ProfScope ps("pool", stream);
-        launch_k(pool_kernel<__nv_bfloat16>, grid, dim3(kThreads), 0, stream, (const __nv_bfloat16*)x, pool, D.L, D.Lv, D.d,
-                                                                  D.m, D.l_p, CT, nchunks);
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("dW_r", stream);
-        dim3 g2((D.d + kThreads - 1) / kThreads, dwr_split(D.d));
-        launch_k(dwr_partial_kernel, g2, dim3(kThreads), 0, stream, pool, G, wpart, D.B * D.m, D.d, D.n);
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("dW_r_sum", stream);
-        const int total = D.d * D.n;
-        launch_k(dwr_sum_kernel, dim3((total + kThreads - 1) / kThreads), dim3(kThreads), 0, stream, wpart, dW_r, total, dwr_split(D.d));
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("router_dx_vec", stream);
-        launch_k(rvec_kernel<__nv_bfloat16>, dim3(D.B * D.m), dim3(kThreads), 0, stream, (const __nv_bfloat16*)W_r, G, rvec, D.d, D.n);
-    }
+    *sum = DwrSum{rs.wpart, dW_r, D.d * D.n, a.splits};
+    return UOE_OK;
+}
+
+uoe_status launch_dwr_sum(const DwrSum& sum, cudaStream_t s) {
+    ProfScope ps("dW_r_sum", s);
+    launch_k(dwr_sum_kernel, dim3(dwr_sum_blocks(sum)), dim3(kThreads), 0, s, sum);
     UOE_LAUNCHED();
     return UOE_OK;
 }
 
 size_t router_backward_scratch_bytes(const Dims& D) {
-    return align_up((size_t)D.B * D.m * D.n * 4, 1024) + 2 * align_up((size_t)D.B * D.m * D.d * 4, 1024) +
-           align_up((size_t)D.B * D.k * D.c * 4, 1024) + align_up((size_t)kDwrSplit * D.d * D.n * 4, 1024);
+    return align_up((size_t)D.B * D.m * D.n * 4, 1024) + align_up((size_t)D.B * D.m * D.d * 4, 1024) +
+           align_up((size_t)apply_shape(D).splits * D.d * D.n * 4, 1024);
 }
 
 RouterBwdScratch router_backward_scratch(const Dims& D, char* base) {
     RouterBwdScratch r;
     r.G = (float*)base;
     base += align_up((size_t)D.B * D.m * D.n * 4, 1024);
-    r.pool = (float*)base;
-    base += align_up((size_t)D.B * D.m * D.d * 4, 1024);
     r.rvec = (float*)base;
     base += align_up((size_t)D.B * D.m * D.d * 4, 1024);
-    r.dgate = (float*)base;
-    base += align_up((size_t)D.B * D.k * D.c * 4, 1024);
     r.wpart = (float*)base;
     return r;
 }
@@ -405,14 +418,10 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
     char* base = (char*)ws;
     int* status = (int*)base;
     const PlanPtrs P = plan_ptrs(D, base + W.plan, true);
-    // rows of the per-row weights that belong to no pair (region padding) must read as zero
-    UOE_CUDA_OK(cudaMemsetAsync(P.row_gate, 0, 2 * align_up((size_t)D.Rmax * 4, 1024), stream));
     void *dyg = base + W.dyg, *xg = base + W.xg, *dh = base + W.dh, *ag = base + W.ag, *dxg = base + W.dxg;
     float* dgp = (float*)(base + W.dgp);
     float* G = (float*)(base + W.G);
-    float* pool = (float*)(base + W.pool);
     float* rvec = (float*)(base + W.rvec);
-    float* dgate = (float*)(base + W.dgate);
     float* wpart = (float*)(base + W.wpart);
 
     st = launch_plan(D, expert_idx, patch_idx, gate, expert_offsets, P, status, stream, use_gate);
@@ -452,18 +461,22 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
                            wgrad_scratch_bytes(D.n, D.d, D.d_e, D.Rmax) ? (float*)(base + W.wgpart) : nullptr, gp);
     if (st != UOE_OK) return st;
 
+    DwrSum sum;
     if (use_gate) {
-        RouterBwdScratch rs{G, pool, rvec, dgate, wpart};
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, stream);
+        RouterBwdScratch rs{G, rvec, wpart};
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, &sum, stream);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
     }
     // dx = dy (selective residual) + the routed input gradients (the gate is already inside dh) + router term
-    if (patch_major)
+    if (patch_major) {
+        if (use_gate) st = launch_dwr_sum(sum, stream);
+        if (st != UOE_OK) return st;
         return launch_gemm2_patch(D, dh, W1, dy, dx, expert_offsets, P, residual, status, stream, true,
                                   use_gate ? rvec : nullptr, "bwd_dx");
-    return launch_combine(D, dy, dxg, P, residual, false, dx, stream, use_gate ? rvec : nullptr);
+    }
+    return launch_combine(D, dy, dxg, P, residual, false, dx, stream, use_gate ? rvec : nullptr, sum);
 }
 
 
@@ -490,38 +503,8 @@ extern "C" uoe_status uoe_route_balance_backward(const uoe_problem* prob, const 
                  D.k, D.m, D.l_p, alpha, rs.G);
     }
     UOE_LAUNCHED();
-    int CT = 64;
-    while (CT > 1 && (CT / 2) * 8 >= D.d) CT /= 2;
-    const int nchunks = (D.d + CT * 8 - 1) / (CT * 8);
-    {
-        ProfScope ps("pool", stream);
-        launch_k(pool_kernel<__nv_bfloat16>, dim3((unsigned)(D.B * D.m * nchunks)), dim3(kThreads), 0, stream,
-                 (const __nv_bfloat16*)x, rs.pool, D.L, D.Lv, D.d, D.m, D.l_p, CT, nchunks);
-    }
+    const ApplyShape a = apply_shape(D);
+    launch_router_apply<true>(D, a, x, W_r, rs.G, nullptr, rs.wpart, dx, stream);
     UOE_LAUNCHED();
-    {
-        ProfScope ps("dW_r", stream);
-        launch_k(dwr_partial_kernel, dim3((D.d + kThreads - 1) / kThreads, dwr_split(D.d)), dim3(kThreads), 0, stream, (const float*)rs.pool,
-                 (const float*)rs.G, rs.wpart, D.B * D.m, D.d, D.n);
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("dW_r_sum", stream);
-        const int total = D.d * D.n;
-        launch_k(dwr_sum_kernel, dim3((total + kThreads - 1) / kThreads), dim3(kThreads), 0, stream, (const float*)rs.wpart, dW_r, total, dwr_split(D.d));
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("router_dx_vec", stream);
-        launch_k(rvec_kernel<__nv_bfloat16>, dim3(D.B * D.m), dim3(kThreads), 0, stream, (const __nv_bfloat16*)W_r, (const float*)rs.G,
-                 rs.rvec, D.d, D.n);
-    }
-    UOE_LAUNCHED();
-    {
-        ProfScope ps("spread_rvec", stream);
-        launch_k(spread_rvec_kernel, dim3(D.B * D.m), dim3(kThreads), 0, stream, (const float*)rs.rvec, (__nv_bfloat16*)dx, D.L, D.Lv,
-                 D.d, D.m, D.l_p);
-    }
-    UOE_LAUNCHED();
-    return UOE_OK;
+    return launch_dwr_sum(DwrSum{rs.wpart, dW_r, D.d * D.n, a.splits}, stream);
 }

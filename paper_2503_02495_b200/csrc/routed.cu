@@ -128,8 +128,11 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             if (tid < n) s_end[tid] = expert_end[tid] = offs[tid] + hist[tid] * l_a;
         }
         __syncthreads();
-        for (int i = 0; i < n; ++i)
+        for (int i = 0; i < n; ++i) {
             for (int rb = s_end[i] / l_p + tid; rb < offs[i + 1] / l_p; rb += NT) src_patch[rb] = -1;
+            if (row_gate)          // padding rows weigh nothing
+                for (int r = s_end[i] + tid; r < offs[i + 1]; r += NT) { row_gate[r] = 0.f; row_valid[r] = 0.f; }
+        }
     }
     if (tail) {
         const long long r0 = offs[n];
@@ -208,9 +211,14 @@ combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __re
                int l_p, int residual, int use_gate, int rows_per_cta, const float* __restrict__ rvec,
                const int* __restrict__ pair_row /* not null: inv_row holds offsets from the pair's first row */,
                const float* __restrict__ gate_bkc /* not null: whole samples per expert (slot u is patch u): no inverse map,
-                                                     weights from the router's gate array [B,k,c] */, int c) {
+                                                     weights from the router's gate array [B,k,c] */, int c,
+               int patches, const DwrSum sum /* total > 0: the CTAs past the patches add up dW_r (backward) */) {
     pdl_trigger();
     pdl_wait();
+    if (blockIdx.x >= patches) {
+        if (blockIdx.y == 0) dwr_sum(sum, (int)blockIdx.x - patches);
+        return;
+    }
     constexpr int V = Vec16<T>::N;
     __shared__ int srow[32];
     __shared__ float sg[32];
@@ -380,7 +388,7 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
 }
 
 uoe_status launch_combine(const Dims& D, const void* x, const void* z, const PlanPtrs& P, bool residual,
-                          bool use_gate, void* y, cudaStream_t s, const float* rvec) {
+                          bool use_gate, void* y, cudaStream_t s, const float* rvec, const DwrSum& sum) {
     // 16-byte vectors per thread: two for small outputs (short dependent chains, many CTAs in flight: these launches are
     // bound by latency), four to eight once the output is tens of MB (fewer, longer CTAs: less set-up per byte; measured
     // 35 -> 31 us at 44 MB, 198 -> 183 us at 268 MB)
@@ -389,20 +397,20 @@ uoe_status launch_combine(const Dims& D, const void* x, const void* z, const Pla
     int rows_per_cta = (int)(vecs * kThreads * 16 / ((long long)D.d * D.esize));
     if (rows_per_cta < 1) rows_per_cta = 1;
     if (rows_per_cta > D.l_p) rows_per_cta = D.l_p;
-    dim3 grid(D.B * D.m, (D.l_p + rows_per_cta - 1) / rows_per_cta);
+    dim3 grid(D.B * D.m + dwr_sum_blocks(sum), (D.l_p + rows_per_cta - 1) / rows_per_cta);
     const bool ident = P.inv_relative && P.identity_patches && P.gate != nullptr;
     ProfScope ps("combine", s);
     if (D.bf16)
         launch_k(combine_kernel<__nv_bfloat16>, grid, dim3(kThreads), 0, s, 
             (const __nv_bfloat16*)x, (const __nv_bfloat16*)z, P.inv_row, P.inv_gate, (__nv_bfloat16*)y, D.L, D.Lv,
             D.d, D.m, D.k, D.l_p, residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta, rvec,
-            P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr, ident ? P.gate : (const float*)nullptr, D.c);
+            P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr, ident ? P.gate : (const float*)nullptr, D.c, D.B * D.m, sum);
     else
         launch_k(combine_kernel<float>, grid, dim3(kThreads), 0, s, (const float*)x, (const float*)z, P.inv_row, P.inv_gate,
                                                        (float*)y, D.L, D.Lv, D.d, D.m, D.k, D.l_p,
                                                        residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta, rvec,
                                                        P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr,
-                                                       ident ? P.gate : (const float*)nullptr, D.c);
+                                                       ident ? P.gate : (const float*)nullptr, D.c, D.B * D.m, sum);
     UOE_LAUNCHED();
     return UOE_OK;
 }

@@ -197,8 +197,6 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     char* base = (char*)ws;
     int* status = (int*)base;
     const PlanPtrs P = plan_ptrs(D, base + W.plan, true);
-    // rows of the per-row weights that belong to no pair (region padding) must read as zero
-    UOE_CUDA_OK(cudaMemsetAsync(P.row_gate, 0, 2 * align_up((size_t)D.Rmax * 4, 1024), stream));
     void *xg = base + W.xg, *dyg = base + W.dyg, *q = base + W.q, *k = base + W.k, *v = base + W.v, *o = base + W.o;
     void *dout = base + W.dout, *og = base + W.og, *dqkv = base + W.dqkv, *dxg = base + W.dxg;
     float *lse = (float*)(base + W.lse), *delta = (float*)(base + W.delta), *dgp = (float*)(base + W.dgp);
@@ -288,11 +286,12 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     UOE_LAUNCHED();
 
     // ---- router ----
+    DwrSum sum;
     if (use_gate) {
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, stream);
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, &sum, stream);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
     }
-    return launch_combine(D, dy, dxg, P, residual, false, dx, stream, use_gate ? rs.rvec : nullptr);
+    return launch_combine(D, dy, dxg, P, residual, false, dx, stream, use_gate ? rs.rvec : nullptr, sum);
 }

@@ -51,3 +51,25 @@ def test_rotary_positions_of_routed_rows(name, entry):
     ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
     ref = orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False, d_rope=d_rope)
     assert rel_inf(to_f64(y), ref) <= TOL
+
+
+# one pass over x for dW_r and dx: every column-block width, row segments (patches above 64 rows), one-row patches,
+# more experts than the widest register tile but one, a width that no block divides
+@pytest.mark.parametrize("kw", [dict(B=2, m=3, L=390, L_valid=301, d=200, n=20, k=5, c=2), dict(B=5, m=33, L=33, L_valid=31, d=640, n=9, k=3, c=8),
+                                dict(B=1, m=4, L=64, L_valid=64, d=72, n=3, k=1, c=1), dict(B=40, m=9, L=216, L_valid=216, d=384, n=8, k=2, c=3),
+                                dict(B=3, m=2, L=130, L_valid=130, d=2048, n=16, k=4, c=2)],
+                         ids=lambda k: f"d{k['d']}n{k['n']}")
+def test_router_gradients_of_the_balance_loss(kw):
+    """Tolerance: the stored dx is bfloat16 (2^-9), dW_r float32; 2e-2 of the largest value as for the other gradients."""
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(dtype="bf16", d_ff=0, H=0, **kw)
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w).f64 * 20, w.dtype)
+    prob = problem_of(w, "mlp")
+    xd, Wrd = to_dev(x), to_dev(Wr)
+    r = uoe.uoe_route(prob, xd, Wrd)
+    dloss = gen.normal(7, 0, (w.B,)).astype(np.float32)
+    dx, dWr = uoe.uoe_route_balance_backward(prob, xd, Wrd, r.p_patch, 0.05, torch.from_numpy(dloss).cuda())
+    ref_dx, ref_dWr = orc.balance_loss_backward(x.f64, Wr.f64, w.m, w.L_valid, w.k, 0.05, dloss.astype(np.float64))
+    assert rel_inf(to_f64(dx), ref_dx) <= TOL
+    assert rel_inf(to_f64(dWr), ref_dWr) <= TOL
+    assert np.all(to_f64(dx)[:, w.L_valid:] == 0)
