@@ -1,6 +1,7 @@
 // Internal launch interface between the entry points (route.cu, mlp.cu, smha.cu, api.cu) and the kernels.
 #pragma once
 #include "common.cuh"
+#include "wgrad_stream.cuh"
 
 namespace uoe {
 
@@ -257,22 +258,37 @@ inline int gemm_bf16_bn(int N) { return (N % 256 == 0) ? 256 : (N % 128 == 0 ? 1
 // Per-expert weight gradient over ragged row counts:  dW[e] [M, N] (float32, overwritten) =
 // sum over the rows r of expert e's region of  P[r, 0:M]^T  Q[r, 0:N]   (P [rows, M], Q [rows, N], bf16).
 // Rows of a region beyond its real rows must be zero in P or Q.
-// `part`: scratch of wgrad_scratch_bytes(n, M, N, rows_max) bytes for the split-K partial outputs (may be null when
-// that is 0; with null the contraction is never split).
-size_t wgrad_scratch_bytes(int n, int M, int N, long long rows_max);
 // Gathered operands (Eq. 18 inside the weight-gradient contraction): with gather_p (gather_q) the pointer P (Q) is
 // the source tensor [Bm patches, l_p, M (N)] and routed row r is row r % l_p of patch src_patch[r / l_p]
-// (-1 = zero rows).  Needs every 64-row K block to be whole slabs inside whole patches, with regions (multiples of
-// 128 rows) starting on patch boundaries:
-inline bool wgrad_can_gather(int l_p) { return l_p >= 16 && 128 % l_p == 0; }
+// (-1 = zero rows).  Needs regions (multiples of 128 rows) that start on patch boundaries.
+//
+// Large matrices (at least two 256 x 256 tiles per SM): one launch per gradient, 256 x 256 tiles, longest first.
+bool wgrad_large(int n, int M, int N);
+inline bool wgrad_large_can_gather(int l_p) { return l_p >= 16 && 128 % l_p == 0; }
 struct WgradGather {
     bool gather_p = false, gather_q = false;
     const int* src_patch = nullptr;
     int l_p = 64, Bm = 0;
 };
-uoe_status launch_wgrad_bf16(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
-                             long long rows_max, const char* label, int* status, cudaStream_t s, float* part = nullptr,
-                             const WgradGather& g = WgradGather());
+uoe_status launch_wgrad_large(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
+                              long long rows_max, const char* label, int* status, cudaStream_t s,
+                              const WgradGather& g = WgradGather());
+// All others: up to two gradients in one launch, cut into equal pieces over the SMs (wgrad_stream_tcgen05.cu).  `part`:
+// scratch of wgrad_stream_scratch_bytes(); *reduce receives what remains to be added by launch_wgrad_reduce or in the
+// spare CTAs of launch_router_backward.
+struct WStreamProblem {
+    const void *P, *Q;
+    int M, N;
+    bool gather_p, gather_q;
+    float* out[3];          // [n, M, out_cols] each: the columns of the gradient, out_cols at a time
+    int out_cols;
+    bool transposed;        // out[0] is [n, N, M]
+};
+size_t wgrad_stream_scratch_bytes();
+uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int* offsets, int n, long long rows_max,
+                               const int* src_patch, int l_p, int Bm, float* part, const char* label, int* status, cudaStream_t s,
+                               WReduce* reduce);
+uoe_status launch_wgrad_reduce(const WReduce& r, cudaStream_t s);
 uoe_status launch_gemm_f32(const GemmArgs& g, cudaStream_t s);
 
 // Scratch of the router half of a backward pass (all float32).
@@ -287,7 +303,7 @@ RouterBwdScratch router_backward_scratch(const Dims& D, char* base);
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
                                   const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
-                                  cudaStream_t stream);
+                                  cudaStream_t stream, const WReduce& reduce = WReduce());
 uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s);
 
 // Eq. 38-39 in one kernel for narrow experts (bf16, d_e = 256, d <= 512): z = phi(A W1[e]) W2[e] with the hidden tile

@@ -22,14 +22,19 @@ constexpr int kThreads = 256;
 // softmax Jacobians of Eq. 14 and 21:  G[b,j,i] = dlogit_patch[b,i,j]/cnt_j + dlogit_samp[b,i]/L_valid.
 // Latency-bound (a sample's partials are a few KB to a few hundred KB); one launch instead of a slab-sum kernel and a
 // Jacobian kernel whose sums over a slot list were one thread's serial loop.
-constexpr int kGradThreads = 512;
+constexpr int kGradThreads = kReduceThreads;
 __global__ void __launch_bounds__(kGradThreads)
 router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restrict__ pair_row,
                    const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
                    const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
-                   int l_p, int Lv, float* __restrict__ G) {
+                   int l_p, int Lv, float* __restrict__ G, int B,
+                   const __grid_constant__ WReduce reduce /* CTAs past the samples add up cut weight-gradient tiles */) {
     pdl_trigger();
     pdl_wait();
+    if (blockIdx.x >= B) {
+        wgrad_reduce(reduce, (int)blockIdx.x - B);
+        return;
+    }
     extern __shared__ float sm[];
     float* pp = sm;                 // [n][m] patch gate
     float* dpp = sm + n * m;        // [n][m] its gradient
@@ -309,6 +314,11 @@ balance_bwd_kernel(const float* __restrict__ p_patch, const float* __restrict__ 
 
 struct BwdWs { size_t plan, dyg, xg, dh, ag, dxg, dgp, G, rvec, wpart, wgpart, total; int nt; };
 
+// dy and x gathered inside the consumers' TMA loads (else copied into routed buffers first)
+bool bwd_can_gather(const Dims& D) {
+    return can_fuse_gather(D) && (!wgrad_large(D.n, D.d, D.d_e) || wgrad_large_can_gather(D.l_p));
+}
+
 BwdWs bwd_ws(const Dims& D) {
     WsCarver w;
     w.take(kStatusBytes);
@@ -316,7 +326,7 @@ BwdWs bwd_ws(const Dims& D) {
     r.nt = D.d_e / gemm_bf16_bn(D.d_e > 0 ? D.d_e : 64);
     if (r.nt < 1) r.nt = 1;
     r.plan = w.take(plan_bytes(D, true));
-    const bool fused = can_fuse_gather(D) && wgrad_can_gather(D.l_p);      // dy and x gathered inside the consumers' TMA loads
+    const bool fused = bwd_can_gather(D);      // dy and x gathered inside the consumers' TMA loads
     r.dyg = fused ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.xg = fused ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.dh = w.take((size_t)D.Rmax * D.d_e * D.esize);
@@ -326,10 +336,7 @@ BwdWs bwd_ws(const Dims& D) {
     r.G = w.take((size_t)D.B * D.m * D.n * sizeof(float));
     r.rvec = w.take((size_t)D.B * D.m * D.d * sizeof(float));
     r.wpart = w.take((size_t)apply_shape(D).splits * D.d * D.n * sizeof(float));
-    {   // split-K partials, sized for the larger of the two weight gradients
-        const size_t s1 = wgrad_scratch_bytes(D.n, D.d, D.d_e, D.Rmax), s2 = wgrad_scratch_bytes(D.n, D.d_e, D.d, D.Rmax);
-        r.wgpart = w.take((s1 > s2 ? s1 : s2) + 1024);
-    }
+    r.wgpart = w.take(wgrad_large(D.n, D.d, D.d_e) ? 0 : wgrad_stream_scratch_bytes());
     r.total = w.off;
     return r;
 }
@@ -343,7 +350,7 @@ BwdWs bwd_ws(const Dims& D) {
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
                                   const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
-                                  cudaStream_t stream) {
+                                  cudaStream_t stream, const WReduce& reduce) {
     if (!D.bf16) return UOE_ERR_UNSUPPORTED;
     const size_t smem = ((size_t)2 * D.n * D.m + (size_t)D.k * D.c) * sizeof(float);
     if ((size_t)2 * D.n * D.m * sizeof(float) > 40 * 1024) return UOE_ERR_UNSUPPORTED;
@@ -352,8 +359,8 @@ uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r,
     if (so != UOE_OK) return so;
     {
         ProfScope ps("router_grad", stream);
-        launch_k(router_grad_kernel, dim3(D.B), dim3(kGradThreads), smem, stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
-                 p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, rs.G);
+        launch_k(router_grad_kernel, dim3(D.B + reduce.blocks), dim3(kGradThreads), smem, stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
+                 p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, rs.G, D.B, reduce);
     }
     UOE_LAUNCHED();
     const ApplyShape a = apply_shape(D);
@@ -427,27 +434,36 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
     st = launch_plan(D, expert_idx, patch_idx, gate, expert_offsets, P, status, stream, use_gate);
     if (st != UOE_OK) return st;
     // Eq. 18 for dy and x: either inside the TMA loads of the kernels that consume them, or as routed copies
-    const bool fused = can_fuse_gather(D) && wgrad_can_gather(D.l_p);
+    const bool fused = bwd_can_gather(D);
     if (!fused) {
         st = launch_gather(D, dy, patch_idx, expert_offsets, P, dyg, stream);
         if (st != UOE_OK) return st;
         st = launch_gather(D, x, patch_idx, expert_offsets, P, xg, stream);
         if (st != UOE_OK) return st;
     }
-    WgradGather gq, gp;          // dW2 = ag^T dy_g (Q gathered), dW1 = x_g^T dh (P gathered)
-    if (fused) {
-        gq.gather_q = true; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m;
-        gp.gather_p = true; gp.src_patch = P.src_patch; gp.l_p = D.l_p; gp.Bm = D.B * D.m;
-    }
-
     GemmArgs ga{dyg, W2, nullptr, dh, nullptr, expert_offsets, D.n, D.d, D.d_e, prob->act, true, D.Rmax};
     ga.label = "bwd_da_dh";
     ga.bwd = true; ga.bwd_h = saved_h; ga.row_gate = P.row_gate; ga.row_valid = P.row_valid; ga.dg_part = dgp; ga.C1 = ag;
     if (fused) { ga.gather_x = dy; ga.src_patch = P.src_patch; ga.l_p = D.l_p; ga.Bm = D.B * D.m; }
     st = launch_gemm_bf16(ga, status, stream);
     if (st != UOE_OK) return st;
-    st = launch_wgrad_bf16(ag, fused ? dy : dyg, dW2, expert_offsets, D.n, D.d_e, D.d, D.Rmax, "wgrad_W2", status, stream,
-                           wgrad_scratch_bytes(D.n, D.d_e, D.d, D.Rmax) ? (float*)(base + W.wgpart) : nullptr, gq);
+    // dW2 = ag^T dy_g, dW1 = x_g^T dh
+    WReduce reduce;
+    if (wgrad_large(D.n, D.d, D.d_e)) {
+        WgradGather gq, gp;
+        if (fused) {
+            gq.gather_q = true; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m;
+            gp.gather_p = true; gp.src_patch = P.src_patch; gp.l_p = D.l_p; gp.Bm = D.B * D.m;
+        }
+        st = launch_wgrad_large(ag, fused ? dy : dyg, dW2, expert_offsets, D.n, D.d_e, D.d, D.Rmax, "wgrad_W2", status, stream, gq);
+        if (st != UOE_OK) return st;
+        st = launch_wgrad_large(fused ? x : xg, dh, dW1, expert_offsets, D.n, D.d, D.d_e, D.Rmax, "wgrad_W1", status, stream, gp);
+    } else {
+        const WStreamProblem probs[2] = {{ag, fused ? dy : dyg, D.d_e, D.d, false, fused, {dW2, nullptr, nullptr}, D.d, false},
+                                         {fused ? x : xg, dh, D.d, D.d_e, fused, false, {dW1, nullptr, nullptr}, D.d_e, false}};
+        st = launch_wgrad_stream(probs, 2, expert_offsets, D.n, D.Rmax, P.src_patch, D.l_p, D.B * D.m, (float*)(base + W.wgpart),
+                                 "wgrad_mlp", status, stream, &reduce);
+    }
     if (st != UOE_OK) return st;
     // patches of 128 tokens: dx_g and the combine are one kernel walked by output patch, after the router's term is known
     const bool patch_major = gemm2_patch_can(D, P, nullptr);
@@ -457,17 +473,15 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
         st = launch_gemm_bf16(gx, status, stream);
         if (st != UOE_OK) return st;
     }
-    st = launch_wgrad_bf16(fused ? x : xg, dh, dW1, expert_offsets, D.n, D.d, D.d_e, D.Rmax, "wgrad_W1", status, stream,
-                           wgrad_scratch_bytes(D.n, D.d, D.d_e, D.Rmax) ? (float*)(base + W.wgpart) : nullptr, gp);
-    if (st != UOE_OK) return st;
-
     DwrSum sum;
     if (use_gate) {
         RouterBwdScratch rs{G, rvec, wpart};
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, &sum, stream);
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, &sum, stream, reduce);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
+        st = launch_wgrad_reduce(reduce, stream);
+        if (st != UOE_OK) return st;
     }
     // dx = dy (selective residual) + the routed input gradients (the gate is already inside dh) + router term
     if (patch_major) {

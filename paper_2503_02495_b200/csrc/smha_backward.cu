@@ -102,34 +102,8 @@ concat_qkv_kernel(const uint4* __restrict__ Wq, const uint4* __restrict__ Wk, co
     }
 }
 
-// dWcat [n*d, 3 d_g] -> dWq, dWk, dWv [n*d, d_g];  dWoT [n, d, d_g] -> dWo [n, d_g, d]   (float32)
-__global__ void __launch_bounds__(kThreads)
-finalize_wgrads_kernel(const float* __restrict__ dWcat, const float* __restrict__ dWoT, float* __restrict__ dWq,
-                       float* __restrict__ dWk, float* __restrict__ dWv, float* __restrict__ dWo, int n, int d, int d_g) {
-    pdl_trigger();
-    pdl_wait();
-    const long long per = (long long)n * d * d_g;
-    const long long total = 4 * per;
-    for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < total; q += (long long)gridDim.x * kThreads) {
-        const int which = (int)(q / per);
-        const long long e = q % per;
-        if (which < 3) {
-            const long long r = e / d_g;
-            const int cc = (int)(e % d_g);
-            const float v = dWcat[r * 3 * d_g + which * d_g + cc];
-            (which == 0 ? dWq : (which == 1 ? dWk : dWv))[e] = v;
-        } else {                 // e indexes dWo [n, d_g, d]
-            const int dd = (int)(e % d);
-            const long long t = e / d;
-            const int cc = (int)(t % d_g);
-            const long long ex = t / d_g;
-            dWo[e] = dWoT[(ex * d + dd) * d_g + cc];
-        }
-    }
-}
-
 struct SmhaBwdWs {
-    size_t plan, xg, dyg, q, k, v, o, dout, og, dqkv, dxg, lse, delta, dgp, wcat, dwcat, dwot, router, wgpart, total;
+    size_t plan, xg, dyg, q, k, v, o, dout, og, dqkv, dxg, lse, delta, dgp, wcat, router, wgpart, total;
 };
 
 SmhaBwdWs smha_bwd_ws(const Dims& D) {
@@ -139,7 +113,7 @@ SmhaBwdWs smha_bwd_ws(const Dims& D) {
     const int heads = D.d_g > 0 ? D.d_g / 64 : 1;
     const size_t rg = (size_t)D.Rmax * D.d_g * D.esize;
     r.plan = w.take(plan_bytes(D, true));
-    const bool fused = can_fuse_gather(D) && wgrad_can_gather(D.l_p);      // x and dy gathered inside the consumers' TMA loads
+    const bool fused = can_fuse_gather(D);      // x and dy gathered inside the consumers' TMA loads
     r.xg = fused ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.dyg = fused ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.q = w.take(rg); r.k = w.take(rg); r.v = w.take(rg); r.o = w.take(rg); r.dout = w.take(rg); r.og = w.take(rg);
@@ -149,13 +123,8 @@ SmhaBwdWs smha_bwd_ws(const Dims& D) {
     r.delta = w.take((size_t)D.Rmax * heads * 4);
     r.dgp = w.take((size_t)D.Rmax * heads * 4);
     r.wcat = w.take((size_t)D.n * D.d * 3 * D.d_g * D.esize);
-    r.dwcat = w.take((size_t)D.n * D.d * 3 * D.d_g * 4);
-    r.dwot = w.take((size_t)D.n * D.d * D.d_g * 4);
     r.router = w.take(router_backward_scratch_bytes(D));
-    {   // split-K partials, sized for the larger of the two weight gradients
-        const size_t s1 = wgrad_scratch_bytes(D.n, D.d, 3 * D.d_g, D.Rmax), s2 = wgrad_scratch_bytes(D.n, D.d, D.d_g, D.Rmax);
-        r.wgpart = w.take((s1 > s2 ? s1 : s2) + 1024);
-    }
+    r.wgpart = w.take(wgrad_stream_scratch_bytes());
     r.total = w.off;
     return r;
 }
@@ -201,18 +170,14 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     void *dout = base + W.dout, *og = base + W.og, *dqkv = base + W.dqkv, *dxg = base + W.dxg;
     float *lse = (float*)(base + W.lse), *delta = (float*)(base + W.delta), *dgp = (float*)(base + W.dgp);
     void* wcat = base + W.wcat;
-    float *dwcat = (float*)(base + W.dwcat), *dwot = (float*)(base + W.dwot);
     const RouterBwdScratch rs = router_backward_scratch(D, base + W.router);
     const long long rowb = (long long)D.d_g * D.esize;
 
     st = launch_plan(D, expert_idx, patch_idx, gate, expert_offsets, P, status, stream, use_gate, v, rowb);
     if (st != UOE_OK) return st;
     // Eq. 18 for x and dy: either inside the TMA loads of the kernels that consume them, or as routed copies
-    const bool fused = can_fuse_gather(D) && wgrad_can_gather(D.l_p);
-    WgradGather gp;
-    if (fused) {
-        gp.gather_p = true; gp.src_patch = P.src_patch; gp.l_p = D.l_p; gp.Bm = D.B * D.m;
-    } else {
+    const bool fused = can_fuse_gather(D);
+    if (!fused) {
         st = launch_gather(D, x, patch_idx, expert_offsets, P, xg, stream);
         if (st != UOE_OK) return st;
         st = launch_gather(D, dy, patch_idx, expert_offsets, P, dyg, stream);
@@ -254,10 +219,6 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
                  (const float*)P.row_valid, delta, dgp, expert_offsets, D.n, heads, D.d_g);
     }
     UOE_LAUNCHED();
-    st = launch_wgrad_bf16(fused ? dy : dyg, og, dwot, expert_offsets, D.n, D.d, D.d_g, D.Rmax, "wgrad_Wo", status, stream,
-                           wgrad_scratch_bytes(D.n, D.d, D.d_g, D.Rmax) ? (float*)(base + W.wgpart) : nullptr, gp);
-    if (st != UOE_OK) return st;
-
     // ---- attention backward ----
     __nv_bfloat16* dq = (__nv_bfloat16*)dqkv;
     st = launch_attention_backward(D, q, k, v, dout, lse, delta, dq, dq + D.d_g, dq + 2 * D.d_g, 3 * D.d_g, P.pair_row,
@@ -275,23 +236,23 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     gx.label = "bwd_dx_att";
     st = launch_gemm_bf16(gx, status, stream);
     if (st != UOE_OK) return st;
-    st = launch_wgrad_bf16(fused ? x : xg, dqkv, dwcat, expert_offsets, D.n, D.d, 3 * D.d_g, D.Rmax, "wgrad_Wqkv", status, stream,
-                           wgrad_scratch_bytes(D.n, D.d, 3 * D.d_g, D.Rmax) ? (float*)(base + W.wgpart) : nullptr, gp);
+    // d[W^q W^k W^v] = x_g^T [dq dk dv], column blocks straight to the three outputs; dW^o^T = dy_g^T og, written transposed
+    WReduce reduce;
+    const WStreamProblem probs[2] = {{fused ? x : xg, dqkv, D.d, 3 * D.d_g, fused, false, {dWq, dWk, dWv}, D.d_g, false},
+                                     {fused ? dy : dyg, og, D.d, D.d_g, fused, false, {dWo, nullptr, nullptr}, D.d_g, true}};
+    st = launch_wgrad_stream(probs, 2, expert_offsets, D.n, D.Rmax, P.src_patch, D.l_p, D.B * D.m, (float*)(base + W.wgpart),
+                             "wgrad_att", status, stream, &reduce);
     if (st != UOE_OK) return st;
-    {
-        ProfScope ps("finalize_wgrads", stream);
-        launch_k(finalize_wgrads_kernel, dim3(256), dim3(kThreads), 0, stream, (const float*)dwcat, (const float*)dwot, dWq, dWk,
-                 dWv, dWo, D.n, D.d, D.d_g);
-    }
-    UOE_LAUNCHED();
 
     // ---- router ----
     DwrSum sum;
     if (use_gate) {
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, &sum, stream);
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, &sum, stream, reduce);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
+        st = launch_wgrad_reduce(reduce, stream);
+        if (st != UOE_OK) return st;
     }
     return launch_combine(D, dy, dxg, P, residual, false, dx, stream, use_gate ? rs.rvec : nullptr, sum);
 }

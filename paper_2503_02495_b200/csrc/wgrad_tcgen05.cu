@@ -4,10 +4,10 @@
 // operands are "MN-major" for the MMA: a K step is 64 consecutive rows, each row contributing 128 bytes
 // (64 elements) per swizzled box.
 //
-// Persistent CTAs walk (expert, 128-row tile of M, BN-column tile of N); warp roles and the two-buffer
-// TMEM accumulator are the same as in the forward grouped GEMM.  The output is float32 and overwritten
-// (each epilogue warp stages [32 rows x 32 columns] in swizzled shared memory and issues one TMA tensor
-// store); an expert with no rows gets zeros.
+// This file: matrices large enough for at least two 256 x 256 output tiles per SM (the others, and every SMHA gradient, are
+// in wgrad_stream_tcgen05.cu).  Persistent CTAs walk (expert, 256 x 256 tile); warp roles are those of the forward
+// grouped GEMM, with one accumulator set (all of TMEM).  The output is float32 and overwritten (each epilogue warp stages
+// [32 rows x 32 columns] in swizzled shared memory and issues one TMA tensor store); an expert with no rows gets zeros.
 // A tile's cost is its expert's row count, so the tile list is ordered by descending row count and handed out
 // longest first: a CTA's first tile is its own index, every further one comes from a counter in the workspace's
 // control block that the producer warp advances when it is ready for more work (greedy list scheduling: the CTAs
@@ -28,23 +28,22 @@ constexpr int A_BLOCK_BYTES = BM * BK * 2;
 constexpr int kSchedSlots = 4;       // tiles the producer may run ahead of the slowest consumer
 constexpr int kSchedWord = 64;       // words [64, 66) of the workspace's control block: next tile, CTAs finished
 
-// MT = 2: 256 x BN output tiles (two 128-row accumulators fed by the same Q stage), one accumulator set
-// drained by eight epilogue warps; MT = 1: 128 x BN tiles with two accumulator sets.
-template <int BN, int MT> struct WCfg {
+// 256 x 256 output tiles: two 128-row accumulators fed by the same Q stage, one accumulator set drained by eight warps
+constexpr int BN = 256, MT = 2;
+struct WCfg {
     static constexpr int A_BYTES = MT * A_BLOCK_BYTES;
     static constexpr int B_BYTES = BN * BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = (MT == 2) ? 3 : ((BN == 256) ? 4 : (BN == 128 ? 6 : 8));
-    static constexpr int NACC = (MT == 2) ? 1 : 2;
+    static constexpr int STAGES = 3;
     static constexpr int TMEM_COLS = 2 * BN;
-    static constexpr int EPI_WARPS = 4 * MT;
+    static constexpr int EPI_WARPS = 8;
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int STG_BYTES = 32 * 128;
     static constexpr int SMEM = STAGES * STAGE + 1024 + 1024 + EPI_WARPS * STG_BYTES;
 };
 
 struct WCtl {
-    uint64_t full[8], empty[8], tfull[2], tempty[2];
+    uint64_t full[WCfg::STAGES], empty[WCfg::STAGES], tfull, tempty;
     uint32_t tmem_base;
     int abort_flag;
     int offs[34];
@@ -53,14 +52,13 @@ struct WCtl {
     int sched_tile[kSchedSlots];   // tiles handed from the producer warp to the MMA thread and the epilogue warps
 };
 
-template <int BN, int MT>
-__global__ void __launch_bounds__(WCfg<BN, MT>::THREADS, 1)
+__global__ void __launch_bounds__(WCfg::THREADS, 1)
 wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
              const __grid_constant__ CUtensorMap tmW, const int* __restrict__ offsets, int n, int M, int N,
-             int ksplit, int* status, int gather_p, int gather_q, const int* __restrict__ src_patch, int l_p, int Bm,
+             int* status, int gather_p, int gather_q, const int* __restrict__ src_patch, int l_p, int Bm,
              int* __restrict__ sched /* [2], zero between launches */) {
     pdl_trigger();
-    using Cf = WCfg<BN, MT>;
+    using Cf = WCfg;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     WCtl* ctl = (WCtl*)(smem + Cf::STAGES * Cf::STAGE);
@@ -69,7 +67,8 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cf::STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tfull[a], 1); mbar_init(&ctl->tempty[a], 32 * Cf::EPI_WARPS); }
+        mbar_init(&ctl->tfull, 1);
+        mbar_init(&ctl->tempty, 32 * Cf::EPI_WARPS);
         for (int q = 0; q < kSchedSlots; ++q) { mbar_init(&ctl->sfull[q], 1); mbar_init(&ctl->sempty[q], 1 + Cf::EPI_WARPS); }
         ctl->abort_flag = 0;
         fence_barrier_init();
@@ -97,20 +96,14 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
     constexpr int TM = MT * BM;
     const int m_tiles = M / TM, n_tiles = N / BN;
     const int per_expert = m_tiles * n_tiles;
-    const int total_tiles = n * per_expert * ksplit;
-    // tile -> expert, output tile, and the slice [kb_lo, kb_lo + kb_cnt) of the expert's 64-row K blocks that split
-    // `ks` of the contraction covers (ksplit = 1: all of them); split ks writes its own copy of the output
-    auto decode = [&](int tile, int& e, int& m0, int& n0, int& ks, int& kb_lo, int& kb_cnt) {
-        ks = tile % ksplit;
-        const int t2 = tile / ksplit;
-        e = ctl->perm[t2 / per_expert];
-        const int rem = t2 % per_expert;
+    const int total_tiles = n * per_expert;
+    // tile -> expert, output tile, number of 64-row K blocks
+    auto decode = [&](int tile, int& e, int& m0, int& n0, int& num_kb) {
+        e = ctl->perm[tile / per_expert];
+        const int rem = tile % per_expert;
         m0 = (rem / n_tiles) * TM;
         n0 = (rem % n_tiles) * BN;
-        const int num_kb = (ctl->offs[e + 1] - ctl->offs[e]) / BK;
-        const int per = (num_kb + ksplit - 1) / ksplit;
-        kb_lo = ks * per;
-        kb_cnt = max(0, min(num_kb, kb_lo + per) - kb_lo);
+        num_kb = (ctl->offs[e + 1] - ctl->offs[e]) / BK;
     };
 
     // Consumer side of the tile hand-off (one thread per consumer warp calls it): the next tile of this CTA, or a value
@@ -153,9 +146,9 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
             tile = __shfl_sync(0xffffffffu, tile, 0);
             if (++slot == kSchedSlots) { slot = 0; sphase ^= 1; }
             if (tile >= total_tiles) break;
-            int e, m0, n0, ks, kb_lo, num_kb;
-            decode(tile, e, m0, n0, ks, kb_lo, num_kb);
-            const int r0 = ctl->offs[e] + kb_lo * BK;
+            int e, m0, n0, num_kb;
+            decode(tile, e, m0, n0, num_kb);
+            const int r0 = ctl->offs[e];
             const int patch_end = gathers ? (r0 + num_kb * BK + l_p - 1) >> lp_shift : 0;     // routed patches of this tile's rows
             int win0 = r0 >> lp_shift;
             int win = (gathers && win0 + lane < patch_end) ? src_patch[win0 + lane] : 0;
@@ -214,7 +207,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = instr_desc_bf16(BM, BN, true, true);
-            int stage = 0, acc = 0;
+            int stage = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool stop = false;
             int slot = 0;
@@ -222,11 +215,11 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
             while (!stop) {
                 const int tile = next_tile(slot, sphase);
                 if (tile >= total_tiles) break;
-                int e, m0, n0, ks, kb_lo, num_kb;
-                decode(tile, e, m0, n0, ks, kb_lo, num_kb);
-                if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
+                int e, m0, n0, num_kb;
+                decode(tile, e, m0, n0, num_kb);
+                if (!mbar_wait(&ctl->tempty, acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * BN;
+                const uint32_t d_tmem = tmem_base;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
                     tc_fence_after();
@@ -244,14 +237,13 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
                     if (++stage == Cf::STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (stop) break;
-                mma_commit(&ctl->tfull[acc]);
-                if (++acc == Cf::NACC) { acc = 0; acc_phase ^= 1; }
+                mma_commit(&ctl->tfull);
+                acc_phase ^= 1;
             }
         }
     } else {
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
-        int acc = 0;
         uint32_t acc_phase = 0;
         int slot = 0;
         uint32_t sphase = 0;
@@ -260,13 +252,13 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
             if (lane == 0) tile = next_tile(slot, sphase);
             tile = __shfl_sync(0xffffffffu, tile, 0);
             if (tile >= total_tiles) break;
-            int e, m0, n0, ks, kb_lo, num_kb;
-            decode(tile, e, m0, n0, ks, kb_lo, num_kb);
-            const bool ready = mbar_wait(&ctl->tfull[acc], acc_phase, abort_flag, status) && !*abort_flag;
+            int e, m0, n0, num_kb;
+            decode(tile, e, m0, n0, num_kb);
+            const bool ready = mbar_wait(&ctl->tfull, acc_phase, abort_flag, status) && !*abort_flag;
             if (!__all_sync(0xffffffffu, ready)) break;
             tc_fence_after();
-            const int wrow0 = (ks * n + e) * M + m0 + half * BM + quarter * 32;   // first row of this warp's piece in [ksplit*n*M, N]
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (MT == 2 ? half * BN : acc * BN);
+            const int wrow0 = e * M + m0 + half * BM + quarter * 32;   // first row of this warp's piece in [n*M, N]
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * BN;
             uint8_t* stg = smem + Cf::STAGES * Cf::STAGE + 1024 + (warp - 2) * Cf::STG_BYTES;
             // the TMEM read of the next piece is in flight while this one is staged and stored
             uint32_t v[32];
@@ -290,8 +282,8 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
                 if (lane == 0) { tma_store_2d(&tmW, stg, n0 + ch * 32, wrow0); bulk_commit(); }
             }
             tc_fence_before();
-            mbar_arrive(&ctl->tempty[acc]);
-            if (++acc == Cf::NACC) { acc = 0; acc_phase ^= 1; }
+            mbar_arrive(&ctl->tempty);
+            acc_phase ^= 1;
         }
     }
     if (warp >= 2 && lane == 0) bulk_wait_all();
@@ -311,28 +303,11 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
     }
 }
 
-// dW = sum over the K splits of their partial outputs, ascending split order.  float4 pieces.
-__global__ void __launch_bounds__(256)
-wgrad_reduce_kernel(const float4* __restrict__ part, float4* __restrict__ dW, long long vecs, int ksplit) {
-    pdl_trigger();
-    pdl_wait();
-    for (long long q = (long long)blockIdx.x * 256 + threadIdx.x; q < vecs; q += (long long)gridDim.x * 256) {
-        float4 a = part[q];
-        for (int s = 1; s < ksplit; ++s) {
-            const float4 t = part[(long long)s * vecs + q];
-            a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
-        }
-        dW[q] = a;
-    }
-}
-
-template <int BN, int MT>
 uoe_status launch_w(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
-                    long long rows_max, const char* label, int* status, cudaStream_t s, int ksplit, float* part,
-                    const WgradGather& g) {
-    using Cf = WCfg<BN, MT>;
+                    long long rows_max, const char* label, int* status, cudaStream_t s, const WgradGather& g) {
+    using Cf = WCfg;
     static DeviceOnce once;
-    auto kern = wgrad_kernel<BN, MT>;
+    auto kern = wgrad_kernel;
     {
         const uoe_status st = smem_opt_in(once, kern, Cf::SMEM);
         if (st != UOE_OK) return st;
@@ -353,63 +328,33 @@ uoe_status launch_w(const void* P, const void* Q, float* dW, const int* offsets,
         return make_tmap(tm, base, 3, dims, str, box);
     };
     if (!operand_map(&tmP, P, M, MT * BM, g.gather_p) || !operand_map(&tmQ, Q, N, BN, g.gather_q)) return UOE_ERR_CUDA;
-    CUtensorMap tmW;      // the output (or the per-split partial outputs) as [ksplit*n*M, N] float32, [32 x 32] pieces
+    CUtensorMap tmW;      // the output as [n*M, N] float32, [32 x 32] pieces
     {
-        const uint64_t dims[2] = {(uint64_t)N, (uint64_t)ksplit * n * M};
+        const uint64_t dims[2] = {(uint64_t)N, (uint64_t)n * M};
         const uint64_t str[1] = {(uint64_t)N * 4};
         const uint32_t wbox[2] = {32, 32};
-        if (!make_tmap(&tmW, ksplit > 1 ? part : dW, 2, dims, str, wbox, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return UOE_ERR_CUDA;
+        if (!make_tmap(&tmW, dW, 2, dims, str, wbox, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return UOE_ERR_CUDA;
     }
-    const long long tiles = (long long)n * (M / (MT * BM)) * (N / BN) * ksplit;
+    const long long tiles = (long long)n * (M / (MT * BM)) * (N / BN);
     int grid = (int)(tiles < sm_count() ? tiles : sm_count());
     ProfScope ps(label, s);
-    launch_k(kern, grid, dim3(Cf::THREADS), Cf::SMEM, s, tmP, tmQ, tmW, offsets, n, M, N, ksplit, status, g.gather_p ? 1 : 0,
+    launch_k(kern, grid, dim3(Cf::THREADS), Cf::SMEM, s, tmP, tmQ, tmW, offsets, n, M, N, status, g.gather_p ? 1 : 0,
              g.gather_q ? 1 : 0, g.src_patch, g.l_p, g.Bm, status + kSchedWord);
     UOE_LAUNCHED();
-    if (ksplit > 1) {
-        const long long vecs = (long long)n * M * N / 4;
-        launch_k(wgrad_reduce_kernel, dim3((unsigned)((vecs + 255) / 256 < 1184 ? (vecs + 255) / 256 : 1184)), dim3(256), 0, s,
-                 (const float4*)part, (float4*)dW, vecs, ksplit);
-        UOE_LAUNCHED();
-    }
     return UOE_OK;
 }
 
 }  // namespace
 
-// How many ways the contraction is split: weight gradients with few output tiles (small M x N per expert) leave most
-// SMs idle and give each busy one a long serial K loop, so their rows are split across CTAs into partial outputs
-// that a second kernel adds in a fixed order.  1 = no split.
-int wgrad_ksplit(int n, int M, int N, long long rows_max) {
-    const int bn = gemm_bf16_bn(N);
-    const long long tiles = (long long)n * (M / BM) * (N / bn);
-    if (tiles < 1 || n < 1 || tiles >= sm_count()) return 1;      // (shapes the kernel does not cover are refused later)
-    long long ks = (2ll * sm_count() + tiles - 1) / tiles;
-    const long long avg_kb = rows_max / ((long long)n * BK);        // 64-row K blocks per expert on average
-    if (ks > avg_kb / 4) ks = avg_kb / 4;                            // at least four K blocks per split
-    if (ks > 32) ks = 32;
-    return ks < 2 ? 1 : (int)ks;
-}
+// 256 x 256 tiles keep every SM busy with at least two of them; below that the matrices go to wgrad_stream_kernel.
+bool wgrad_large(int n, int M, int N) { return M % 256 == 0 && N % 256 == 0 && (long long)n * (M / 256) * (N / 256) >= 2 * sm_count(); }
 
-size_t wgrad_scratch_bytes(int n, int M, int N, long long rows_max) {
-    const int ks = wgrad_ksplit(n, M, N, rows_max);
-    return ks > 1 ? (size_t)ks * n * M * N * sizeof(float) : 0;
-}
-
-uoe_status launch_wgrad_bf16(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
-                             long long rows_max, const char* label, int* status, cudaStream_t s, float* part,
-                             const WgradGather& g) {
+uoe_status launch_wgrad_large(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
+                              long long rows_max, const char* label, int* status, cudaStream_t s, const WgradGather& g) {
     if (!status) return UOE_ERR_INVALID_ARG;       // the tile counters live in the control block behind the status word
-    if (M % BM != 0 || N % 64 != 0 || n > 32) return UOE_ERR_UNSUPPORTED;
-    if ((g.gather_p || g.gather_q) && (!g.src_patch || !wgrad_can_gather(g.l_p))) return UOE_ERR_INVALID_ARG;
-    const int bn = gemm_bf16_bn(N);
-    const int ks = part ? wgrad_ksplit(n, M, N, rows_max) : 1;
-    // 256-row output tiles when the weight matrices are large enough to keep every SM busy with them
-    if (bn == 256 && M % 256 == 0 && (long long)n * (M / 256) * (N / 256) >= 2 * sm_count())
-        return launch_w<256, 2>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, 1, nullptr, g);
-    if (bn == 256) return launch_w<256, 1>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, ks, part, g);
-    if (bn == 128) return launch_w<128, 1>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, ks, part, g);
-    return launch_w<64, 1>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, ks, part, g);
+    if (M % 256 != 0 || N % 256 != 0 || n > 32) return UOE_ERR_UNSUPPORTED;
+    if ((g.gather_p || g.gather_q) && (!g.src_patch || !wgrad_large_can_gather(g.l_p))) return UOE_ERR_INVALID_ARG;
+    return launch_w(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, g);
 }
 
 }  // namespace uoe

@@ -73,3 +73,34 @@ def test_router_gradients_of_the_balance_loss(kw):
     assert rel_inf(to_f64(dx), ref_dx) <= TOL
     assert rel_inf(to_f64(dWr), ref_dWr) <= TOL
     assert np.all(to_f64(dx)[:, w.L_valid:] == 0)
+
+
+# weight gradients cut into equal pieces over the SMs: ragged column tiles, 8-row slabs, one expert whose tiles are cut into
+# many pieces, experts without rows, routed copies, and the pass without gates (the cut tiles added by their own launch)
+def _bwd(**kw):
+    base = dict(B=3, L=96, L_valid=96, m=6, c=3, d=128, n=4, k=2, d_ff=512, H=4, d_h=64, dtype="bf16", w_std=0.05)
+    base.update(kw)
+    return gen.tiny(**base)
+
+
+WGRAD_CASES = {
+    "ragged_columns_patch8": (_bwd(B=5, L=64, L_valid=61, m=8, c=5, d=640, n=3, k=2, d_ff=3 * 128, H=9), True),
+    "one_expert_many_pieces": (_bwd(B=6, L=1024, L_valid=1000, m=8, c=8, d=128, n=1, k=1, d_ff=384, H=1), True),
+    "experts_without_rows": (_bwd(B=2, n=12, k=1, d_ff=12 * 128, H=12), True),
+    "routed_copies": (_bwd(B=4, L=140, L_valid=133, m=7, c=4, d=256, n=3, k=2, d_ff=3 * 256, H=6), True),
+    "no_gates": (_bwd(B=7, L=256, L_valid=256, m=8, c=6, d=384, n=2, k=2, d_ff=2 * 256, H=2), False),
+}
+
+
+@pytest.mark.parametrize("half", ["mlp", "att"])
+@pytest.mark.parametrize("name", list(WGRAD_CASES))
+def test_weight_gradients_cut_into_pieces(name, half):
+    from tests.test_gpu_mlp_backward import _run as run_mlp
+    from tests.test_gpu_smha_backward import _run as run_att
+    w, use_gate = WGRAD_CASES[name]
+    got, ref = (run_mlp(w, False, use_gate) if half == "mlp" else run_att(w, False, use_gate))[:2]
+    for g, r in zip(got, ref[:len(got)]):
+        if np.abs(r).max() > 0:
+            assert rel_inf(g, r) <= TOL
+        else:
+            assert np.all(g == 0)
