@@ -11,6 +11,17 @@ bool g_prof_on = false;
 std::vector<ProfRec> g_prof;
 }  // namespace
 
+int sm_count() {
+    static DeviceValue cache;
+    const int dev = current_device();
+    if (cache.has(dev)) return cache.get(dev);
+    int v = 148;
+    if (dev >= 0) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    if (v <= 0) v = 148;
+    if (dev >= 0) cache.set(dev, v);
+    return v;
+}
+
 ProfScope::ProfScope(const char* name, cudaStream_t s) : slot(-1), stream(s) {
     if (!g_prof_on || !name) return;
     ProfRec r{name, nullptr, nullptr};

@@ -30,6 +30,8 @@
 #include "tc.cuh"
 #include "tmap.cuh"
 
+#include <type_traits>
+
 namespace uoe {
 namespace {
 
@@ -58,6 +60,8 @@ template <int BN, int MT, bool BWD = false, bool PAIR = false> struct Cfg {
     static constexpr int SMEM = STAGES * STAGE + 1024 /*align slack*/ + 1024 /*barriers, offsets*/ + EPI_WARPS * STG_BYTES;
 };
 
+struct NoRope {};                  // what a kernel without the rotation takes in its place
+
 struct Ctl {                       // lives behind the stage ring
     uint64_t full[8], empty[8], tfull[2], tempty[2];
     uint32_t tmem_base;
@@ -66,7 +70,7 @@ struct Ctl {                       // lives behind the stage ring
     int tstart[34];                // first row tile of each expert (prefix sum), tstart[n] = number of row tiles
 };
 
-template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR>
+template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR, bool ROPE>
 __global__ void __launch_bounds__(Cfg<BN, MT, BWD, PAIR>::THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                  const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
@@ -79,7 +83,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmX, const SrcMap smap, int l_p, int Bm,
                  const __grid_constant__ CUtensorMap tmC0, const __grid_constant__ CUtensorMap tmC1,
                  const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmPre,
-                 const __grid_constant__ Rope rope /* pair0 < 32: matrices 0 and 1 hold 64-wide heads to be rotated */) {
+                 const __grid_constant__ typename std::conditional<ROPE, Rope, NoRope>::type rope /* matrices 0 and 1 hold 64-wide heads to be rotated */) {
     pdl_trigger();
     using Cf = Cfg<BN, MT, BWD, PAIR>;
     extern __shared__ uint8_t smem_raw[];
@@ -307,8 +311,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const int mat = (tile % n_tiles) / n_tiles_mat, col0 = ((tile % n_tiles) % n_tiles_mat) * BN;
             const CUtensorMap* tmC = mat == 0 ? &tmC0 : (mat == 1 ? &tmC1 : &tmC2);
             int tok = -1;                                    // position of this thread's row in its sample
-            if (!BWD && rope.pair0 < 32 && half < blocks)    // (two dependent look-ups, under the tile's main loop)
-                tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e]);
+            if constexpr (ROPE) {                            // (two dependent look-ups, under the tile's main loop)
+                if (half < blocks) tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e]);
+            }
             const bool ready = mbar_wait(&ctl->tfull[acc], acc_phase, abort_flag, status) && !*abort_flag;
             if (!__all_sync(0xffffffffu, ready)) break;      // warp-uniform: tcgen05.ld below is warp-collective
             tc_fence_after();
@@ -364,16 +369,18 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 for (int q = 0; q < 8; ++q) f[8 * q8 + q] += bv[q];
                             }
                         }
-                        if (rope.pair0 < 32 && (SIDE3 ? g : mat) < 2) {
-                            // Eq. 32 on the float32 accumulators: the head's last channels, two MUFU operations per pair
+                        if constexpr (ROPE) {
+                            if ((SIDE3 ? g : mat) < 2) {
+                                // Eq. 32 on the float32 accumulators: the head's last channels, two MUFU operations per pair
 #pragma unroll
-                            for (int p = 0; p < 32; ++p) {
-                                if (p >= rope.pair0) {
-                                    float cs, sn;
-                                    rope_angle(rope, p, (float)max(tok, 0), cs, sn);
-                                    const float a0 = f[2 * p], a1 = f[2 * p + 1];
-                                    f[2 * p] = a0 * cs - a1 * sn;
-                                    f[2 * p + 1] = a0 * sn + a1 * cs;
+                                for (int p = 0; p < 32; ++p) {
+                                    if (p >= rope.pair0) {
+                                        float cs, sn;
+                                        rope_angle(rope, p, (float)max(tok, 0), cs, sn);
+                                        const float a0 = f[2 * p], a1 = f[2 * p + 1];
+                                        f[2 * p] = a0 * cs - a1 * sn;
+                                        f[2 * p + 1] = a0 * sn + a1 * cs;
+                                    }
                                 }
                             }
                         }
@@ -408,12 +415,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
 }
 
-template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR = false>
+template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR = false, bool ROPE = false>
 uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     using Cf = Cfg<BN, MT, BWD, PAIR>;
     static DeviceOnce once;
     static DeviceValue pairs_cache;    // CTA pairs that can be resident at once, per device
-    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, BWD, MT, PAIR>;
+    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, BWD, MT, PAIR, ROPE>;
     {
         const uoe_status st = smem_opt_in(once, kern, Cf::SMEM);
         if (st != UOE_OK) return st;
@@ -484,16 +491,18 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
         if constexpr (PAIR) return launch_k_pairs(a...);
         else return launch_k(a...);
     };
+    typename std::conditional<ROPE, Rope, NoRope>::type rope;
+    if constexpr (ROPE) rope = *g.rope;
     launch(kern, dim3(grid), dim3(Cf::THREADS), (size_t)Cf::SMEM, s, tmA, tmB[0], tmB[1], tmB[2], (__nv_bfloat16*)g.C, (__nv_bfloat16*)g.C1,
                                              (__nv_bfloat16*)g.C2, (__nv_bfloat16*)g.pre, g.offsets, g.n, g.K, g.N,
                                              nmat, g.act, status, (const __nv_bfloat16*)g.bwd_h, g.row_gate, g.row_valid,
                                              g.dg_part, (const __nv_bfloat16*)g.bias, g.blk_scale, tmX, smap, g.l_p, g.Bm, tmC[0],
-                                             tmC[1], tmC[2], tmPre, g.rope ? *g.rope : Rope());
+                                             tmC[1], tmC[2], tmPre, rope);
     UOE_LAUNCHED();
     return UOE_OK;
 }
 
-template <bool B_KMAJOR, bool BWD>
+template <bool B_KMAJOR, bool BWD, bool ROPE = false>
 uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
     const int bn = gemm_bf16_bn(g.N);
     // 256-row tiles pay off when every SM still gets several of them and the K loop is long enough to be
@@ -505,12 +514,12 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
         if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 1, true>(g, status, s);
     }
     if constexpr (!BWD) {
-        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 1, true>(g, status, s);
-        if (bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 2>(g, status, s);
+        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 1, true, ROPE>(g, status, s);
+        if (bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 2, false, ROPE>(g, status, s);
     }
-    if (bn == 256) return launch_one<256, B_KMAJOR, BWD, 1>(g, status, s);
-    if (bn == 128) return launch_one<128, B_KMAJOR, BWD, 1>(g, status, s);
-    return launch_one<64, B_KMAJOR, BWD, 1>(g, status, s);
+    if (bn == 256) return launch_one<256, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
+    if (bn == 128) return launch_one<128, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
+    return launch_one<64, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
 }
 
 }  // namespace
@@ -518,7 +527,8 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
 uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
     if (g.K % BK != 0 || g.N % 64 != 0 || g.nmat > 3) return UOE_ERR_UNSUPPORTED;
     if ((g.bias || g.blk_scale) && (g.bwd || g.nmat > 1)) return UOE_ERR_UNSUPPORTED;      // a bias row per expert, a factor per block: plain forward GEMMs only
-    if (g.rope && g.rope->pair0 < 32 && (g.nmat != 3 || g.bwd)) return UOE_ERR_UNSUPPORTED;
+    const bool rope = g.rope && g.rope->pair0 < 32;      // (kernels of its own: the rotation's code would sit in every epilogue loop)
+    if (rope && (g.nmat != 3 || g.bwd || g.b_kmajor)) return UOE_ERR_UNSUPPORTED;
     if (g.nmat > 1 && g.pre) return UOE_ERR_UNSUPPORTED;
     if (g.gather_x && ((!g.src_patch && !g.map.on()) || g.l_p < 8 || g.l_p % 8 != 0 || BM % g.l_p != 0)) return UOE_ERR_INVALID_ARG;
     if (g.rows_max % BM != 0 || g.n > 31) return UOE_ERR_UNSUPPORTED;
@@ -527,7 +537,9 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
             return UOE_ERR_INVALID_ARG;
         return dispatch<true, true>(g, status, s);
     }
-    if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre) return launch_one<192, false, false, 1>(g, status, s);
+    if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre)
+        return rope ? launch_one<192, false, false, 1, false, true>(g, status, s) : launch_one<192, false, false, 1>(g, status, s);
+    if (rope) return dispatch<false, false, true>(g, status, s);
     if (g.b_kmajor) return dispatch<true, false>(g, status, s);
     return dispatch<false, false>(g, status, s);
 }

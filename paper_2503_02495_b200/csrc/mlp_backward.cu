@@ -23,7 +23,7 @@ constexpr int kThreads = 256;
 // Latency-bound (a sample's partials are a few KB to a few hundred KB); one launch instead of a slab-sum kernel and a
 // Jacobian kernel whose sums over a slot list were one thread's serial loop.
 constexpr int kGradThreads = kReduceThreads;
-__global__ void __launch_bounds__(kGradThreads)
+__global__ void __launch_bounds__(kGradThreads, 2)
 router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restrict__ pair_row,
                    const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
                    const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
@@ -262,15 +262,17 @@ ApplyShape apply_shape(const Dims& D) {
 template <bool SPREAD>
 void launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, const void* W_r, const float* G, float* rvec,
                          float* part, void* dx, cudaStream_t s) {
-    auto go = [&](auto kern) {
-        launch_k(kern, dim3(a.col_blocks, a.splits), dim3(a.CW), (size_t)kSlices * a.CW * sizeof(float), s, (const __nv_bfloat16*)x,
+    auto go = [&](SpreadOnce& once, auto kern) {
+        const size_t smem = spread_smem(once, kern, (long long)a.col_blocks * a.splits, (size_t)kSlices * a.CW * sizeof(float));
+        launch_k(kern, dim3(a.col_blocks, a.splits), dim3(a.CW), smem, s, (const __nv_bfloat16*)x,
                  (const __nv_bfloat16*)W_r, G, rvec, part, (__nv_bfloat16*)dx, D.B * D.m * a.nseg, D.L, D.Lv, D.d, D.n, D.m, D.l_p, a.nseg,
                  a.RT, a.per);
     };
     ProfScope ps("router_apply", s);
-    if (D.n <= 8) go(router_apply_kernel<8, SPREAD>);
-    else if (D.n <= 16) go(router_apply_kernel<16, SPREAD>);
-    else go(router_apply_kernel<32, SPREAD>);
+    static SpreadOnce once[3];
+    if (D.n <= 8) go(once[0], router_apply_kernel<8, SPREAD>);
+    else if (D.n <= 16) go(once[1], router_apply_kernel<16, SPREAD>);
+    else go(once[2], router_apply_kernel<32, SPREAD>);
 }
 
 // Gradient of the load-balancing loss (Eq. 42-44) with respect to the router logits.  grid B, 128 threads, dynamic
@@ -354,12 +356,13 @@ uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r,
     if (!D.bf16) return UOE_ERR_UNSUPPORTED;
     const size_t smem = ((size_t)2 * D.n * D.m + (size_t)D.k * D.c) * sizeof(float);
     if ((size_t)2 * D.n * D.m * sizeof(float) > 40 * 1024) return UOE_ERR_UNSUPPORTED;
-    static DeviceOnce once;
-    const uoe_status so = smem_opt_in(once, router_grad_kernel, 80 * 1024);      // k c <= n m: at most 60 KB
+    static SpreadOnce once;
+    const uoe_status so = smem_opt_in(once.opt_in, router_grad_kernel, 160 * 1024);      // k c <= n m: at most 60 KB
     if (so != UOE_OK) return so;
+    const int grad_ctas = D.B + reduce.blocks;
     {
         ProfScope ps("router_grad", stream);
-        launch_k(router_grad_kernel, dim3(D.B + reduce.blocks), dim3(kGradThreads), smem, stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
+        launch_k(router_grad_kernel, dim3(grad_ctas), dim3(kGradThreads), spread_smem(once, router_grad_kernel, grad_ctas, smem), stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
                  p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, rs.G, D.B, reduce);
     }
     UOE_LAUNCHED();

@@ -577,7 +577,11 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
         W.nchunks, W.rsplit, W.rows_per_cta, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch, expert_offsets, ctl, \
         tickets, masks, plan
 #define UOE_ROUTE_LAUNCH(T, TICKET, NT, SMEM) \
-        launch_k(route_kernel<T, TICKET, NT>, grid, dim3(NT), SMEM, stream, UOE_ROUTE_ARGS(T))
+        [&] { \
+            static SpreadOnce once; \
+            return launch_k(route_kernel<T, TICKET, NT>, grid, dim3(NT), spread_smem(once, route_kernel<T, TICKET, NT>, grid.x, SMEM), \
+                            stream, UOE_ROUTE_ARGS(T)); \
+        }()
     cudaError_t e;
     if (W.per_sample) {
         static DeviceOnce once_bf16, once_f32;

@@ -204,7 +204,7 @@ gather_kernel(const uint4* __restrict__ src, const int* __restrict__ patch_idx, 
 // ---------------------------------------------------------------------------------------------
 // combine: grid (B*m, row groups)
 // ---------------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, bool BWD /* the backward's combine: rvec and sum */>
 __global__ void __launch_bounds__(kThreads)
 combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __restrict__ inv_row,
                const float* __restrict__ inv_gate, T* __restrict__ y, int L, int Lv, int d, int m, int k,
@@ -215,7 +215,7 @@ combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __re
                int patches, const DwrSum sum /* total > 0: the CTAs past the patches add up dW_r (backward) */) {
     pdl_trigger();
     pdl_wait();
-    if (blockIdx.x >= patches) {
+    if (BWD && blockIdx.x >= patches) {
         if (blockIdx.y == 0) dwr_sum(sum, (int)blockIdx.x - patches);
         return;
     }
@@ -270,7 +270,7 @@ combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __re
                     }
                 }
             }
-            if (rvec) {
+            if (BWD && rvec) {
                 const float* rp = rvec + (size_t)bj * d + (size_t)cv * V;
 #pragma unroll
                 for (int v = 0; v < V; v += 4) {
@@ -379,8 +379,9 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
     if (nsplit < 1) nsplit = 1;
     if (nsplit > 128) nsplit = 128;
     dim3 grid(n_slabs + D.n + (tail ? 1 : 0), nsplit);
+    static SpreadOnce once;
     ProfScope ps("gather", s);
-    launch_k(gather_kernel, grid, dim3(kThreads), 0, s, (const uint4*)src, patch_idx, offsets, P.pair_row, P.expert_end,
+    launch_k(gather_kernel, grid, dim3(kThreads), spread_smem(once, gather_kernel, (long long)grid.x * grid.y, 0), s, (const uint4*)src, patch_idx, offsets, P.pair_row, P.expert_end,
                                             (uint4*)dst, n_slabs, D.k, D.c, D.m, slab_vecs, row_vecs, D.l_p, D.n,
                                             (uint4*)tail, tail_row_bytes / 16, D.Rmax);
     UOE_LAUNCHED();
@@ -399,26 +400,28 @@ uoe_status launch_combine(const Dims& D, const void* x, const void* z, const Pla
     if (rows_per_cta > D.l_p) rows_per_cta = D.l_p;
     dim3 grid(D.B * D.m + dwr_sum_blocks(sum), (D.l_p + rows_per_cta - 1) / rows_per_cta);
     const bool ident = P.inv_relative && P.identity_patches && P.gate != nullptr;
+    const long long ctas = (long long)grid.x * grid.y;
     ProfScope ps("combine", s);
-    if (D.bf16)
-        launch_k(combine_kernel<__nv_bfloat16>, grid, dim3(kThreads), 0, s, 
-            (const __nv_bfloat16*)x, (const __nv_bfloat16*)z, P.inv_row, P.inv_gate, (__nv_bfloat16*)y, D.L, D.Lv,
-            D.d, D.m, D.k, D.l_p, residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta, rvec,
-            P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr, ident ? P.gate : (const float*)nullptr, D.c, D.B * D.m, sum);
-    else
-        launch_k(combine_kernel<float>, grid, dim3(kThreads), 0, s, (const float*)x, (const float*)z, P.inv_row, P.inv_gate,
-                                                       (float*)y, D.L, D.Lv, D.d, D.m, D.k, D.l_p,
-                                                       residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta, rvec,
-                                                       P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr,
-                                                       ident ? P.gate : (const float*)nullptr, D.c, D.B * D.m, sum);
+    auto go = [&](SpreadOnce& once, auto kern, auto elem) {
+        using T = decltype(elem);
+        launch_k(kern, grid, dim3(kThreads), spread_smem(once, kern, ctas, 0), s, (const T*)x, (const T*)z, (const int*)P.inv_row,
+                 (const float*)P.inv_gate, (T*)y, D.L, D.Lv, D.d, D.m, D.k, D.l_p, residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta,
+                 rvec, P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr, ident ? P.gate : (const float*)nullptr, D.c,
+                 D.B * D.m, sum);
+    };
+    static SpreadOnce once[3];
+    if (!D.bf16) go(once[0], combine_kernel<float, false>, float());
+    else if (rvec || sum.total > 0) go(once[1], combine_kernel<__nv_bfloat16, true>, __nv_bfloat16());
+    else go(once[2], combine_kernel<__nv_bfloat16, false>, __nv_bfloat16());
     UOE_LAUNCHED();
     return UOE_OK;
 }
 
 uoe_status launch_gemm_f32(const GemmArgs& g, cudaStream_t s) {
     dim3 grid((unsigned)((g.rows_max + BM - 1) / BM), (g.N + BN - 1) / BN);
+    static SpreadOnce once;
     ProfScope ps(g.label, s);
-    launch_k(gemm_f32_kernel, grid, dim3(256), 0, s, (const float*)g.A, (const float*)g.W, (const float*)g.bias, (float*)g.C,
+    launch_k(gemm_f32_kernel, grid, dim3(256), spread_smem(once, gemm_f32_kernel, (long long)grid.x * grid.y, 0), s, (const float*)g.A, (const float*)g.W, (const float*)g.bias, (float*)g.C,
                                          (float*)g.pre, g.offsets, g.n, g.K, g.N, g.act, g.b_kmajor ? 1 : 0);
     UOE_LAUNCHED();
     return UOE_OK;

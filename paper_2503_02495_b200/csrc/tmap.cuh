@@ -77,16 +77,4 @@ inline bool make_tmap(CUtensorMap* out, const void* base, int rank, const uint64
     return true;
 }
 
-// SM count of the current device (cached per device).
-inline int sm_count() {
-    static DeviceValue cache;
-    const int dev = current_device();
-    if (cache.has(dev)) return cache.get(dev);
-    int v = 148;
-    if (dev >= 0) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    if (v <= 0) v = 148;
-    if (dev >= 0) cache.set(dev, v);
-    return v;
-}
-
 }  // namespace uoe

@@ -23,6 +23,11 @@ struct WReduce {
 
 constexpr int kReduceThreads = 512;
 
+// A tile counts as at least this many K blocks: writing its 128 KB out takes about as long, and an expert with few or no
+// rows has as many tiles as any other (uncounted, one CTA wrote all of an empty expert's zeros: 78 us instead of 50 for
+// the MLP half at B = 4, L = 2048, d = 1024, d_e = 512, n = 8 with one expert unused).
+constexpr int kMinTileKb = 4;
+
 #ifdef __CUDACC__
 struct WSched {
     int n, total, Q;          // cost of the line, cost of a piece
@@ -32,14 +37,14 @@ struct WSched {
 // A tile's part inside one piece.
 struct WFrag {
     int p, e, m0, n0, cols;            // problem, expert, first row and column of the tile, its columns
-    int kb_lo, kb_hi, kb_real;         // K blocks of this part; kb_real = 0: the expert has no rows, the tile is zero
+    int kb_lo, kb_hi;                  // K blocks of this part (none: the part is zero)
     int c_first, c_last;               // pieces that hold parts of the tile
 };
 
 // One warp builds it (n <= 32).
 __device__ __forceinline__ void wsched_build(WSched& s, const int* offs, int n, const WProblem* prob, int nprob, int pieces, int lane) {
     const int kb = lane < n ? (offs[lane + 1] - offs[lane]) / 64 : 0;
-    const int kb1 = lane < n ? max(kb, 1) : 0;
+    const int kb1 = lane < n ? max(kb, kMinTileKb) : 0;
     int incl = kb1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -65,14 +70,13 @@ __device__ __forceinline__ void wsched_build(WSched& s, const int* offs, int n, 
 }
 // The tile of problem p, expert e, index t within the expert; its place on the line.
 __device__ __forceinline__ void wsched_tile(const WSched& s, const WProblem& pr, int p, int e, int t, WFrag& f, int& begin, int& cost) {
-    const int kb1 = max(s.kb[e], 1);
+    const int kb1 = max(s.kb[e], kMinTileKb);
     cost = kb1 * pr.w;
     begin = s.base[p][e] + t * cost;
     f.p = p; f.e = e;
     f.m0 = (t / pr.n_tiles) * 128;
     f.n0 = (t % pr.n_tiles) * pr.BN;
     f.cols = min(pr.BN, pr.N - f.n0);
-    f.kb_real = s.kb[e];
     f.c_first = begin / s.Q;
     f.c_last = (begin + (kb1 - 1) * pr.w) / s.Q;
 }
@@ -85,13 +89,17 @@ __device__ __forceinline__ bool wsched_next(const WSched& s, const WProblem* pro
         int e = 0;
         while (pos >= s.base[p][e + 1]) ++e;
         const WProblem& pr = prob[p];
-        const int cost1 = max(s.kb[e], 1) * pr.w;
+        const int cost1 = max(s.kb[e], kMinTileKb) * pr.w;
         int begin, cost;
         wsched_tile(s, pr, p, e, (pos - s.base[p][e]) / cost1, f, begin, cost);
         f.kb_lo = (pos - begin + pr.w - 1) / pr.w;
         f.kb_hi = min(cost / pr.w, (min(end, begin + cost) - begin + pr.w - 1) / pr.w);
         pos = begin + cost;
-        if (f.kb_lo < f.kb_hi) return true;
+        if (f.kb_lo < f.kb_hi) {
+            f.kb_lo = min(f.kb_lo, s.kb[e]);
+            f.kb_hi = min(f.kb_hi, s.kb[e]);
+            return true;
+        }
     }
     return false;
 }
@@ -126,31 +134,33 @@ __device__ __forceinline__ void wgrad_reduce(const WReduce& r, int blk) {
     // lanes over (row, four columns) so that both the reads and the row-major writes are whole sectors; a transposed
     // output takes lanes over rows
     const int lr = pr.transposed ? lane : lane >> 3, lq = pr.transposed ? 0 : lane & 7;
-    float4 acc[8];
-    for (int c = f.c_first; c <= f.c_last; ++c) {
-        const float4* src = base + wsched_slot(f, c) * (size_t)(128 * 256 / 4);
-        float4 t[8];
+    const int col = f.n0 + ch * 32, which = pr.transposed ? 0 : col / pr.out_cols;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {            // half the piece at a time: few enough registers for two CTAs per SM
+        float4 acc[4];
+        for (int c = f.c_first; c <= f.c_last; ++c) {
+            const float4* src = base + wsched_slot(f, c) * (size_t)(128 * 256 / 4);
+            float4 t[4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) t[q] = pr.transposed ? src[q * 128 + lr] : src[lq * 128 + q * 4 + lr];
+            for (int q = 0; q < 4; ++q) t[q] = pr.transposed ? src[(4 * h + q) * 128 + lr] : src[lq * 128 + (4 * h + q) * 4 + lr];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            if (c == f.c_first) acc[q] = t[q];
-            else { acc[q].x += t[q].x; acc[q].y += t[q].y; acc[q].z += t[q].z; acc[q].w += t[q].w; }
+            for (int q = 0; q < 4; ++q) {
+                if (c == f.c_first) acc[q] = t[q];
+                else { acc[q].x += t[q].x; acc[q].y += t[q].y; acc[q].z += t[q].z; acc[q].w += t[q].w; }
+            }
         }
-    }
-    const int col = f.n0 + ch * 32;
-    if (pr.transposed) {
-        float* o = pr.out[0] + ((size_t)f.e * pr.N + col) * pr.M + f.m0 + quarter * 32 + lr;
+        if (pr.transposed) {
+            float* o = pr.out[0] + ((size_t)f.e * pr.N + col + 16 * h) * pr.M + f.m0 + quarter * 32 + lr;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            o[(size_t)(4 * q) * pr.M] = acc[q].x; o[(size_t)(4 * q + 1) * pr.M] = acc[q].y;
-            o[(size_t)(4 * q + 2) * pr.M] = acc[q].z; o[(size_t)(4 * q + 3) * pr.M] = acc[q].w;
+            for (int q = 0; q < 4; ++q) {
+                o[(size_t)(4 * q) * pr.M] = acc[q].x; o[(size_t)(4 * q + 1) * pr.M] = acc[q].y;
+                o[(size_t)(4 * q + 2) * pr.M] = acc[q].z; o[(size_t)(4 * q + 3) * pr.M] = acc[q].w;
+            }
+        } else {
+            float* o = pr.out[which] + ((size_t)f.e * pr.M + f.m0 + quarter * 32) * pr.out_cols + (col - which * pr.out_cols) + lq * 4;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) *(float4*)(o + (size_t)((4 * h + q) * 4 + lr) * pr.out_cols) = acc[q];
         }
-    } else {
-        const int which = col / pr.out_cols;
-        float* o = pr.out[which] + ((size_t)f.e * pr.M + f.m0 + quarter * 32) * pr.out_cols + (col - which * pr.out_cols) + lq * 4;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) *(float4*)(o + (size_t)(q * 4 + lr) * pr.out_cols) = acc[q];
     }
 }
 #endif

@@ -97,7 +97,7 @@ wgrad_stream_kernel(const __grid_constant__ WArgs a) {
         const int lp_shift = __ffs(a.l_p) - 1;               // gathered operands: l_p is a power of two that divides 128
         WFrag f;
         for (int pos = c * sc.Q; !stop && wsched_next(sc, a.prob, c, pos, f);) {
-            if (f.kb_real == 0) continue;
+            if (f.kb_lo >= f.kb_hi) continue;
             const WProblem& pr = a.prob[f.p];
             const WMaps& tm = a.maps[f.p];
             const WOperand &op = a.p[f.p], &oq = a.q[f.p];
@@ -174,7 +174,7 @@ wgrad_stream_kernel(const __grid_constant__ WArgs a) {
                 if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN_MAX;
-                for (int kb = f.kb_lo; kb < f.kb_hi && f.kb_real > 0; ++kb) {
+                for (int kb = f.kb_lo; kb < f.kb_hi; ++kb) {
                     if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
                     tc_fence_after();
                     const uint32_t sp = smem_u32(smem + stage * STAGE), sq = sp + P_BYTES;
@@ -208,7 +208,7 @@ wgrad_stream_kernel(const __grid_constant__ WArgs a) {
 #pragma unroll 1
             for (int ch = wsel; ch < f.cols / 32; ch += 2) {
                 uint32_t v[32];
-                if (f.kb_real > 0) {
+                if (f.kb_lo < f.kb_hi) {
                     tmem_ld32(taddr + ch * 32, v);
                     tmem_ld_wait();
                 } else {
@@ -345,7 +345,8 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
 uoe_status launch_wgrad_reduce(const WReduce& r, cudaStream_t s) {
     if (r.blocks == 0) return UOE_OK;
     ProfScope ps("wgrad_reduce", s);
-    launch_k(wgrad_reduce_kernel, dim3(r.blocks), dim3(kReduceThreads), 0, s, r);
+    static SpreadOnce once;
+    launch_k(wgrad_reduce_kernel, dim3(r.blocks), dim3(kReduceThreads), spread_smem(once, wgrad_reduce_kernel, r.blocks, 0), s, r);
     UOE_LAUNCHED();
     return UOE_OK;
 }
