@@ -785,8 +785,7 @@ Rope rope_of(const Dims& D, const PlanPtrs& P, const int* patch_idx) {
         r.hi[p] = (float)turns;
         r.lo[p] = (float)(turns - (double)r.hi[p]);
     }
-    r.map = src_map_of(D, P, patch_idx);
-    r.map.slot_pair = P.slot_pair; r.map.patch_idx = patch_idx; r.map.expert_end = P.expert_end;
+    r.map = row_map_of(D, P, patch_idx);
     return r;
 }
 

@@ -121,6 +121,13 @@ struct Rope {
     float hi[32], lo[32];              // turns per token of channel pair p: 10000^(-2 (p - pair0) / d_rope) / (2 pi)
 };
 Rope rope_of(const Dims& D, const PlanPtrs& P, const int* patch_idx);
+// The same map through slot_pair whichever kernel wrote the plan (for source_row: any patch length, single rows).
+inline SrcMap row_map_of(const Dims& D, const PlanPtrs& P, const int* patch_idx) {
+    SrcMap g = src_map_of(D, P, patch_idx);
+    g.src_patch = nullptr;
+    g.slot_pair = P.slot_pair; g.patch_idx = patch_idx; g.expert_end = P.expert_end;
+    return g;
+}
 #ifdef __CUDACC__
 // (cos, sin) of channel pair p of the token at position t
 __device__ __forceinline__ void rope_angle(const Rope& rp, int p, float t, float& cs, float& sn) {
@@ -128,14 +135,20 @@ __device__ __forceinline__ void rope_angle(const Rope& rp, int p, float t, float
     const float frac = (r - rintf(r)) + fmaf(t, rp.lo[p], fmaf(t, rp.hi[p], -r));     // fraction of a turn, in [-1/2, 1/2]
     __sincosf(frac * 6.283185307179586f, &sn, &cs);
 }
-// Position in its sample of the token at routed row r of expert e's region; -1 on padding rows and unused slots.
-__device__ __forceinline__ int token_of(const SrcMap& g, int r, int e, int off_e) {
+// Row of the source tensor [B*m*l_p rows] that routed row r of expert e's region holds; -1 on padding rows and unused
+// slots.  Any patch length (through slot_pair).
+__device__ __forceinline__ int source_row(const SrcMap& g, int r, int e, int off_e) {
     if (r >= g.expert_end[e]) return -1;
     const int rel = r - off_e, l_a = g.c * g.l_p;
     const int pair = g.slot_pair[(size_t)e * g.B + rel / l_a];
     const int u = (rel % l_a) / g.l_p;
     const int pj = g.n_elig >= 0 ? (u < g.n_elig ? u : -1) : g.patch_idx[(size_t)pair * g.c + u];
-    return pj >= 0 && pj < g.m ? pj * g.l_p + rel % g.l_p : -1;
+    return pj >= 0 && pj < g.m ? ((pair / g.k) * g.m + pj) * g.l_p + rel % g.l_p : -1;
+}
+// Position of that token in its sample, or -1.
+__device__ __forceinline__ int token_of(const SrcMap& g, int r, int e, int off_e) {
+    const int row = source_row(g, r, e, off_e);
+    return row < 0 ? -1 : row % (g.m * g.l_p);
 }
 // Source patch (index into the [Bm patches] view of the source tensor) of the l_p-row block that starts at routed row
 // r inside the region of expert e (first row off_e); Bm (out of range: the loads return zeros) for padding rows and
@@ -235,8 +248,9 @@ struct GemmArgs {
     //   C  [r,:] = row_gate[r] * u * phi'(h)         (gradient w.r.t. the pre-activation)
     //   C1 [r,:] = row_gate[r] * phi(h)              (gated activation, operand of the weight gradient)
     //   dg_part[r, column tile] = row_valid[r] * sum over the tile's columns of u * phi(h)
-    // bf16 path, gathered A (Eq. 18 inside the GEMM): if gather_x is not null, A is ignored and row block q of a
-    // tile is loaded from patch src_patch[tile*128/l_p + q] of gather_x [Bm patches, l_p, K]
+    // gathered A (Eq. 18 inside the GEMM): if gather_x is not null, A is ignored and, on the bf16 path, row block q of a
+    // tile is loaded from patch src_patch[tile*128/l_p + q] of gather_x [Bm patches, l_p, K]; the float32 path takes single
+    // rows through `map` (row_map_of)
     const void* gather_x = nullptr;
     const int* src_patch = nullptr;
     int l_p = 0, Bm = 0;

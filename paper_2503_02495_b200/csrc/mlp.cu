@@ -1,6 +1,6 @@
 // uoe_mlp_forward: UoME forward (Eq. 37-40) as plan -> gather (Eq. 18) -> grouped GEMM1 + phi (Eq. 38)
-// -> grouped GEMM2 (Eq. 39) -> weighted combine (Eq. 20 / 40).  On the bf16 path the gather happens inside the
-// first GEMM's loads, and for narrow experts (d_e = 256, d <= 512) both GEMMs are one kernel.
+// -> grouped GEMM2 (Eq. 39) -> weighted combine (Eq. 20 / 40).  The gather happens inside the first GEMM's loads (bf16: for
+// patch lengths that tile 128 rows), and for narrow experts (d_e = 256, d <= 512) both GEMMs are one kernel.
 #include "kernels.cuh"
 
 namespace uoe {
@@ -12,7 +12,7 @@ static MlpFwdWs mlp_fwd_ws(const Dims& D) {
     w.take(kStatusBytes);
     MlpFwdWs r;
     r.plan = w.take(plan_bytes(D));
-    r.xg = can_fuse_gather(D) ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);     // the GEMM gathers x itself
+    r.xg = can_fuse_gather(D) || !D.bf16 ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);     // the GEMM gathers x itself
     r.a = mlp_can_fuse(D) ? 0 : w.take((size_t)D.Rmax * D.d_e * D.esize);          // the fused kernel keeps the hidden tile on chip
     r.z = w.take((size_t)D.Rmax * D.d * D.esize);
     r.total = w.off;
@@ -23,7 +23,7 @@ size_t mlp_fwd_workspace_bytes(const Dims& D) { return mlp_fwd_ws(D).total; }
 
 size_t mlp_fwd_buffer_bytes(const Dims& D, size_t* xg, size_t* a, size_t* z) {
     WsCarver w;
-    *xg = can_fuse_gather(D) ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
+    *xg = can_fuse_gather(D) || !D.bf16 ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     *a = mlp_can_fuse(D) ? 0 : w.take((size_t)D.Rmax * D.d_e * D.esize);
     *z = w.take((size_t)D.Rmax * D.d * D.esize);
     return w.off;
@@ -39,14 +39,14 @@ uoe_status uoe::mlp_forward_run(const Dims& D, const uoe_problem* prob, const vo
                                 cudaStream_t stream) {
     uoe_status st;
     void *xg = bufs.xg, *a = bufs.a, *z = bufs.z;
-    const bool fused = can_fuse_gather(D);
+    const bool fused = can_fuse_gather(D) || !D.bf16;
     if (!fused) {
         st = launch_gather(D, x, patch_idx, expert_offsets, P, xg, stream);
         if (st != UOE_OK) return st;
     }
 
     GemmArgs g1{xg, W1, b1, a, saved_h, expert_offsets, D.n, D.d, D.d_e, prob->act, false, D.Rmax};
-    const SrcMap map = src_map_of(D, P, patch_idx);
+    const SrcMap map = D.bf16 ? src_map_of(D, P, patch_idx) : row_map_of(D, P, patch_idx);
     if (fused) { g1.gather_x = x; g1.map = map; g1.l_p = D.l_p; g1.Bm = D.B * D.m; }
     GemmArgs g2{a, W2, b2, z, nullptr, expert_offsets, D.n, D.d_e, D.d, UOE_ACT_IDENTITY, false, D.Rmax};
     g1.label = "gemm1_act";

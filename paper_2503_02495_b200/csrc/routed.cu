@@ -284,69 +284,141 @@ combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __re
 }
 
 // ---------------------------------------------------------------------------------------------
-// float32 grouped GEMM (FFMA): 64x64 tile, 16-deep K step, 4x4 outputs per thread
+// float32 grouped GEMM on the FFMA pipes: TM x TN tile, MT x NT outputs per thread, KG groups of threads that share
+// the tile and take the BK-deep K steps' columns in turn (their sums are added in group order at the end).  A three-stage
+// cp.async ring; A is kept [row][k] and read four k at a time, its rows dealt round robin to the threads so that the
+// reads of a warp hit different banks.  A may be gathered: single rows of x, any patch length (Eq. 18).
+// Two shapes.  Large problems: 128 x 64, 8 x 8 per thread (FFMA-bound: 16 multiply-adds per 16-byte shared-memory read).
+// Small ones, where the chain of K steps and idle SMs are the bound: 32 x 32 with four K groups (256 x 256 matrices over
+// 512 rows: 128 CTAs, each thread 64 of the 256 k's).
 // ---------------------------------------------------------------------------------------------
-constexpr int BM = 64, BN = 64, BK = 16;
+template <int TM, int TN, int MT, int NT, int KG, int BK> struct F32Cfg {
+    static constexpr int GROUP = (TM / MT) * (TN / NT);          // threads of a K group
+    static constexpr int THREADS = GROUP * KG;
+    static constexpr int LDA = BK + 4;                           // floats per A row: adjacent rows start four banks apart
+    static constexpr int STAGE = TM * LDA + BK * TN;             // floats
+    static constexpr int STAGES = 3;
+    static constexpr int RED = KG > 1 ? (KG - 1) * TM * TN : 0;
+    static constexpr int SMEM = (STAGES * STAGE > RED ? STAGES * STAGE : RED) * 4 + TM * 4;
+    static_assert(128 % TM == 0 && BK % (4 * KG) == 0 && NT % 4 == 0, "tile shape");
+};
 
-__global__ void __launch_bounds__(256)
+template <int TM, int TN, int MT, int NT, int KG, int BK>
+__global__ void __launch_bounds__(F32Cfg<TM, TN, MT, NT, KG, BK>::THREADS)
 gemm_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
                 float* __restrict__ C, float* __restrict__ pre, const int* __restrict__ offsets, int n, int K, int N,
-                int act, int b_kmajor) {
+                int act, int gathered, const SrcMap map) {
+    using Cf = F32Cfg<TM, TN, MT, NT, KG, BK>;
     pdl_trigger();
     pdl_wait();
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
-    const int total_rows = offsets[n];
-    const int row0 = blockIdx.x * BM;
-    if (row0 >= total_rows) return;
+    extern __shared__ __align__(16) float s_ring[];
+    int* s_src = (int*)(s_ring + (Cf::SMEM - TM * 4) / 4);       // source row of every tile row, -1 = zeros
+    const int row0 = blockIdx.x * TM, col0 = blockIdx.y * TN, tid = threadIdx.x;
+    if (row0 >= offsets[n]) return;
     int e = 0;
-    while (e + 1 < n && row0 >= offsets[e + 1]) ++e;       // regions are multiples of 128 rows: no tile straddles
-    const int col0 = blockIdx.y * BN;
+    while (e + 1 < n && row0 >= offsets[e + 1]) ++e;             // regions are multiples of 128 rows: no tile straddles
+    for (int r = tid; r < TM; r += Cf::THREADS) s_src[r] = gathered ? source_row(map, row0 + r, e, offsets[e]) : row0 + r;
+    __syncthreads();
     const float* We = W + (size_t)e * K * N;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int idx = threadIdx.x; idx < BM * BK; idx += 256) {
-            const int r = idx / BK, kk = idx % BK;
-            As[kk][r] = (k0 + kk < K) ? A[(size_t)(row0 + r) * K + k0 + kk] : 0.f;
+    const int steps = (K + BK - 1) / BK;
+
+    auto copy = [](float* dst, const float* src, bool valid) {   // 16 bytes, zero-filled when not valid
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                     :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
+    };
+    auto load = [&](int step) {
+        if (step < steps) {
+            float* sa = s_ring + (step % Cf::STAGES) * Cf::STAGE;
+            float* sb = sa + TM * Cf::LDA;
+            const int k0 = step * BK;
+            for (int q = tid; q < TM * BK / 4; q += Cf::THREADS) {
+                const int r = q / (BK / 4), kk = (q % (BK / 4)) * 4;
+                const int src = s_src[r];
+                const bool ok = src >= 0 && k0 + kk < K;
+                copy(sa + r * Cf::LDA + kk, ok ? A + (size_t)src * K + k0 + kk : A, ok);
+            }
+            for (int q = tid; q < BK * TN / 4; q += Cf::THREADS) {
+                const int kk = q / (TN / 4), cc = (q % (TN / 4)) * 4;
+                const bool ok = k0 + kk < K && col0 + cc < N;
+                copy(sb + kk * TN + cc, ok ? We + (size_t)(k0 + kk) * N + col0 + cc : We, ok);
+            }
         }
-        for (int idx = threadIdx.x; idx < BK * BN; idx += 256) {
-            int kk, cc;
-            if (b_kmajor) { cc = idx / BK; kk = idx % BK; } else { kk = idx / BN; cc = idx % BN; }
-            float v = 0.f;
-            if (k0 + kk < K && col0 + cc < N)
-                v = b_kmajor ? We[(size_t)(col0 + cc) * K + k0 + kk] : We[(size_t)(k0 + kk) * N + col0 + cc];
-            Bs[kk][cc] = v;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int st = 0; st < Cf::STAGES - 1; ++st) load(st);
+
+    const int g = tid / Cf::GROUP, t = tid % Cf::GROUP;
+    constexpr int TX = TN / NT, TY = TM / MT;
+    const int tx = t % TX, ty = t / TX;
+    float acc[MT][NT] = {};
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" :: "n"(Cf::STAGES - 2) : "memory");
+        __syncthreads();                      // this step has landed for every thread, and the step before it has been read
+        load(step + Cf::STAGES - 1);
+        const float* sa = s_ring + (step % Cf::STAGES) * Cf::STAGE;
+        const float* sb = sa + TM * Cf::LDA;
+#pragma unroll
+        for (int q = 0; q < BK / (4 * KG); ++q) {
+            const int kk = (q * KG + g) * 4;
+            float4 a[MT];
+#pragma unroll
+            for (int i = 0; i < MT; ++i) a[i] = *(const float4*)(sa + (i * TY + ty) * Cf::LDA + kk);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float b[NT];
+#pragma unroll
+                for (int j = 0; j < NT / 4; ++j) {
+                    const float4 v = *(const float4*)(sb + (kk + u) * TN + j * (TN / (NT / 4)) + tx * 4);
+                    b[4 * j] = v.x; b[4 * j + 1] = v.y; b[4 * j + 2] = v.z; b[4 * j + 3] = v.w;
+                }
+#pragma unroll
+                for (int i = 0; i < MT; ++i) {
+                    const float av = u == 0 ? a[i].x : (u == 1 ? a[i].y : (u == 2 ? a[i].z : a[i].w));
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) acc[i][j] = fmaf(av, b[j], acc[i][j]);
+                }
+            }
+        }
+    }
+    if (KG > 1) {                             // add the K groups' sums in group order
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (g > 0) {
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
+#pragma unroll
+                for (int j = 0; j < NT; ++j) s_ring[((g - 1) * MT * NT + i * NT + j) * Cf::GROUP + t] = acc[i][j];
         }
         __syncthreads();
+        if (g > 0) return;
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float a[4], bb[4];
+        for (int q = 0; q < KG - 1; ++q)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+            for (int i = 0; i < MT; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
-        }
-        __syncthreads();
+                for (int j = 0; j < NT; ++j) acc[i][j] += s_ring[(q * MT * NT + i * NT + j) * Cf::GROUP + t];
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const size_t r = (size_t)row0 + ty * 4 + i;
+    for (int j = 0; j < NT / 4; ++j) {
+        const int cc = col0 + j * (TN / (NT / 4)) + tx * 4;
+        if (cc >= N) continue;                // N is a multiple of four
+        float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bias) bv = *(const float4*)(bias + (size_t)e * N + cc);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int cc = col0 + tx * 4 + j;
-            if (cc >= N) continue;
-            float v = acc[i][j];
-            if (bias) v += bias[(size_t)e * N + cc];
-            if (pre) pre[r * N + cc] = v;
-            C[r * N + cc] = act_apply(v, act);
+        for (int i = 0; i < MT; ++i) {
+            const size_t o = (size_t)(row0 + i * TY + ty) * N + cc;
+            float4 v = make_float4(acc[i][4 * j] + bv.x, acc[i][4 * j + 1] + bv.y, acc[i][4 * j + 2] + bv.z, acc[i][4 * j + 3] + bv.w);
+            if (pre) *(float4*)(pre + o) = v;
+            v.x = act_apply(v.x, act); v.y = act_apply(v.y, act); v.z = act_apply(v.z, act); v.w = act_apply(v.w, act);
+            *(float4*)(C + o) = v;
         }
     }
 }
+
+// 128 x 64 tiles from here on (a little over one per SM); below, 32 x 32 tiles.  Whole forward, us with the large / small tiles
+// (256 x 256 experts): 76 tiles 71 / 47, 140 tiles 70 / 64;  512 x 384 experts, 400 tiles 218 / 246, 800 tiles 390 / 475.
+// (64 x 64 tiles with scalar copies, the only shape before: 177, 165, 414, 703.)
+constexpr long long kF32LargeTiles = 160;
 
 }  // namespace
 
@@ -418,11 +490,25 @@ uoe_status launch_combine(const Dims& D, const void* x, const void* z, const Pla
 }
 
 uoe_status launch_gemm_f32(const GemmArgs& g, cudaStream_t s) {
-    dim3 grid((unsigned)((g.rows_max + BM - 1) / BM), (g.N + BN - 1) / BN);
-    static SpreadOnce once;
+    if (g.b_kmajor || g.nmat != 1 || (g.K & 3) || (g.N & 3)) return UOE_ERR_UNSUPPORTED;
     ProfScope ps(g.label, s);
-    launch_k(gemm_f32_kernel, grid, dim3(256), spread_smem(once, gemm_f32_kernel, (long long)grid.x * grid.y, 0), s, (const float*)g.A, (const float*)g.W, (const float*)g.bias, (float*)g.C,
-                                         (float*)g.pre, g.offsets, g.n, g.K, g.N, g.act, g.b_kmajor ? 1 : 0);
+    auto go = [&](SpreadOnce& once, auto kern, int tm, int tn, int threads, int smem) {
+        const uoe_status st = smem_opt_in(once.opt_in, kern, 160 * 1024);
+        if (st != UOE_OK) return st;
+        const dim3 grid((unsigned)((g.rows_max + tm - 1) / tm), (g.N + tn - 1) / tn);
+        launch_k(kern, grid, dim3(threads), spread_smem(once, kern, (long long)grid.x * grid.y, (size_t)smem), s,
+                 (const float*)(g.gather_x ? g.gather_x : g.A), (const float*)g.W, (const float*)g.bias, (float*)g.C, (float*)g.pre,
+                 g.offsets, g.n, g.K, g.N, g.act, g.gather_x ? 1 : 0, g.map);
+        return UOE_OK;
+    };
+    using Large = F32Cfg<128, 64, 8, 8, 1, 16>;
+    using Small = F32Cfg<32, 32, 4, 4, 4, 32>;
+    static SpreadOnce once[2];
+    const long long large_tiles = g.rows_max / 128 * ((g.N + 63) / 64);
+    const uoe_status st = large_tiles >= kF32LargeTiles
+                              ? go(once[0], gemm_f32_kernel<128, 64, 8, 8, 1, 16>, 128, 64, Large::THREADS, Large::SMEM)
+                              : go(once[1], gemm_f32_kernel<32, 32, 4, 4, 4, 32>, 32, 32, Small::THREADS, Small::SMEM);
+    if (st != UOE_OK) return st;
     UOE_LAUNCHED();
     return UOE_OK;
 }

@@ -104,3 +104,28 @@ def test_weight_gradients_cut_into_pieces(name, half):
             assert rel_inf(g, r) <= TOL
         else:
             assert np.all(g == 0)
+
+
+# float32 grouped GEMM: both tile shapes, ragged K and N, patches that do not tile 128 rows, biases, padding rows.  Tolerance:
+# sums of at most 256 fp32 products, 2^-24 * sqrt(256) relative per output, 1e-5 of the largest value leaves ten times that.
+F32_CASES = {
+    "small_tiles": dict(B=3, m=5, L=65, L_valid=60, d=52, n=3, k=2, c=3, d_ff=3 * 28),
+    "large_tiles": dict(B=40, m=10, L=170, L_valid=165, d=200, n=3, k=2, c=5, d_ff=3 * 132),
+    "large_whole_samples": dict(B=48, m=2, L=128, L_valid=128, d=256, n=4, k=2, c=2, d_ff=4 * 256),
+}
+
+
+@pytest.mark.parametrize("name", list(F32_CASES))
+def test_float32_experts_with_biases(name):
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(H=0, act="gelu_tanh", w_std=0.1, **F32_CASES[name])
+    x, Wr = gen.make_x(w), gen.make_router(w)
+    W1, W2 = gen.make_mlp_weights(w)
+    b1, b2 = gen.store(gen.normal(5, 1, (w.n, w.d_e), 0.3), "f32"), gen.store(gen.normal(5, 2, (w.n, w.d), 0.3), "f32")
+    prob = problem_of(w, "mlp", residual=False)
+    xd = to_dev(x)
+    r = uoe.uoe_route(prob, xd, to_dev(Wr))
+    y = uoe.uoe_mlp_forward(prob, xd, to_dev(W1), to_dev(W2), r, b1=to_dev(b1), b2=to_dev(b2))
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    ref = orc.mlp_forward(x.f64, W1.f64, W2.f64, ro, w.act, residual=False, b1=b1.f64, b2=b2.f64)
+    assert rel_inf(to_f64(y), ref) <= 1e-5
