@@ -28,11 +28,13 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
                    const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
                    const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
                    int l_p, int Lv, float* __restrict__ G, int B,
-                   const __grid_constant__ WReduce reduce /* CTAs past the samples add up cut weight-gradient tiles */) {
+                   const __grid_constant__ WReduce reduce /* reduce.blocks further CTAs add up cut weight-gradient tiles */) {
     pdl_trigger();
     pdl_wait();
-    if (blockIdx.x >= B) {
-        wgrad_reduce(reduce, (int)blockIdx.x - B);
+    // the samples first where they are few (their slab sums are long chains), last where they would hold the additions up
+    const int b = B <= 64 ? (int)blockIdx.x : (int)blockIdx.x - reduce.blocks;
+    if (b < 0 || b >= B) {
+        wgrad_reduce(reduce, b < 0 ? (int)blockIdx.x : b - B);
         return;
     }
     extern __shared__ float sm[];
@@ -40,7 +42,7 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
     float* dpp = sm + n * m;        // [n][m] its gradient
     float* dg = sm + 2 * n * m;     // [k][c] gradient of the combine weight of every slot
     __shared__ float ps[32], dls[32], dps[32];
-    const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int idx = tid; idx < n * m; idx += kGradThreads) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
     if (tid < 32) { ps[tid] = tid < n ? p_samp[(size_t)b * n + tid] : 0.f; dps[tid] = 0.f; }
     const int len = l_p * nt;

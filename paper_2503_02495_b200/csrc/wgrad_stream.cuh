@@ -18,7 +18,8 @@ struct WReduce {
     const int* offsets = nullptr;
     const float* part = nullptr;
     int n = 0, nprob = 0, pieces = 0, blocks = 0;
-    int blocks_per_tile[2] = {0, 0};
+    int per = 1;              // blocks per tile
+    int by_cut = 0;           // blocks are counted by piece boundary (more tiles than pieces), else by tile
 };
 
 constexpr int kReduceThreads = 512;
@@ -107,8 +108,10 @@ __device__ __forceinline__ bool wsched_next(const WSched& s, const WProblem* pro
 // last (the tile goes on).
 __device__ __forceinline__ size_t wsched_slot(const WFrag& f, int c) { return (size_t)c * 2 + (c > f.c_first ? 0 : 1); }
 
-// Adds the parts of every cut tile in ascending order.  Block `blk` of kReduceThreads threads: a [32 x 32] piece of one tile
-// per warp.
+// Adds the parts of every cut tile in ascending order.  r.per blocks of kReduceThreads threads for a tile, half a [32 x 32]
+// piece per warp.  The blocks are counted by tile or, when there are more tiles than pieces, by the boundaries between
+// pieces: each cuts at most one tile, whose first boundary does the work.  Bound by the latency of the part loads: two
+// parts are in flight per warp (one part and a whole piece per warp: 32 us instead of 21 for the image block's MLP half).
 __device__ __forceinline__ void wgrad_reduce(const WReduce& r, int blk) {
     __shared__ WSched s;
     __shared__ int offs[34];
@@ -120,47 +123,66 @@ __device__ __forceinline__ void wgrad_reduce(const WReduce& r, int blk) {
         wsched_build(s, offs, r.n, r.prob, r.nprob, r.pieces, lane);
     }
     __syncthreads();
-    const int blocks0 = r.n * r.prob[0].m_tiles * r.prob[0].n_tiles * r.blocks_per_tile[0];
-    const int p = blk >= blocks0 ? 1 : 0;
-    const WProblem& pr = r.prob[p];
-    const int rel = p ? blk - blocks0 : blk, tile = rel / r.blocks_per_tile[p], per_e = pr.m_tiles * pr.n_tiles;
     WFrag f;
-    int begin, cost;
-    wsched_tile(s, pr, p, tile / per_e, tile % per_e, f, begin, cost);
-    const int piece = (rel % r.blocks_per_tile[p]) * (kReduceThreads / 32) + warp;
-    const int quarter = piece & 3, ch = piece >> 2;
+    int p = 0, begin, cost;
+    if (r.by_cut) {
+        const int c = 1 + blk / r.per, pos = c * s.Q;
+        if (pos >= s.total) return;
+        p = pos >= s.base[0][s.n] ? 1 : 0;
+        int e = 0;
+        while (pos >= s.base[p][e + 1]) ++e;
+        wsched_tile(s, r.prob[p], p, e, (pos - s.base[p][e]) / (max(s.kb[e], kMinTileKb) * r.prob[p].w), f, begin, cost);
+        if (f.c_first != c - 1) return;
+    } else {
+        const int tiles0 = r.n * r.prob[0].m_tiles * r.prob[0].n_tiles;
+        int tile = blk / r.per;
+        if (tile >= tiles0) { p = 1; tile -= tiles0; }
+        const int per_e = r.prob[p].m_tiles * r.prob[p].n_tiles;
+        wsched_tile(s, r.prob[p], p, tile / per_e, tile % per_e, f, begin, cost);
+    }
+    const WProblem& pr = r.prob[p];
+    const int piece = (blk % r.per) * (kReduceThreads / 32) + warp;
+    const int h = piece & 1, quarter = (piece >> 1) & 3, ch = piece >> 3;
     if (f.c_first == f.c_last || ch * 32 >= f.cols) return;
-    const float4* base = (const float4*)r.part + (size_t)ch * 8 * 128 + quarter * 32;
     // lanes over (row, four columns) so that both the reads and the row-major writes are whole sectors; a transposed
     // output takes lanes over rows
     const int lr = pr.transposed ? lane : lane >> 3, lq = pr.transposed ? 0 : lane & 7;
-    const int col = f.n0 + ch * 32, which = pr.transposed ? 0 : col / pr.out_cols;
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {            // half the piece at a time: few enough registers for two CTAs per SM
-        float4 acc[4];
-        for (int c = f.c_first; c <= f.c_last; ++c) {
-            const float4* src = base + wsched_slot(f, c) * (size_t)(128 * 256 / 4);
-            float4 t[4];
+    const int stride = pr.transposed ? 128 : 4;
+    const float4* base = (const float4*)r.part + (size_t)ch * 8 * 128 + quarter * 32 + (pr.transposed ? 4 * h * 128 : lq * 128 + 4 * h * 4) + lr;
+    auto part = [&](int c) { return base + wsched_slot(f, c) * (size_t)(128 * 256 / 4); };
+    float4 acc[4], t[4];
+    {
+        const float4 *s0 = part(f.c_first), *s1 = part(f.c_first + 1);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) t[q] = pr.transposed ? src[(4 * h + q) * 128 + lr] : src[lq * 128 + (4 * h + q) * 4 + lr];
+        for (int q = 0; q < 4; ++q) { acc[q] = s0[q * stride]; t[q] = s1[q * stride]; }
+    }
+    auto add = [&](const float4* v) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (c == f.c_first) acc[q] = t[q];
-                else { acc[q].x += t[q].x; acc[q].y += t[q].y; acc[q].z += t[q].z; acc[q].w += t[q].w; }
-            }
+        for (int q = 0; q < 4; ++q) { acc[q].x += v[q].x; acc[q].y += v[q].y; acc[q].z += v[q].z; acc[q].w += v[q].w; }
+    };
+    add(t);
+    for (int c = f.c_first + 2; c <= f.c_last; c += 2) {
+        const bool two = c < f.c_last;
+        const float4 *s0 = part(c), *s1 = part(two ? c + 1 : c);
+        float4 t1[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { t[q] = s0[q * stride]; t1[q] = s1[q * stride]; }
+        add(t);
+        if (two) add(t1);
+    }
+    const int col = f.n0 + ch * 32;
+    if (pr.transposed) {
+        float* o = pr.out[0] + ((size_t)f.e * pr.N + col + 16 * h) * pr.M + f.m0 + quarter * 32 + lr;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            o[(size_t)(4 * q) * pr.M] = acc[q].x; o[(size_t)(4 * q + 1) * pr.M] = acc[q].y;
+            o[(size_t)(4 * q + 2) * pr.M] = acc[q].z; o[(size_t)(4 * q + 3) * pr.M] = acc[q].w;
         }
-        if (pr.transposed) {
-            float* o = pr.out[0] + ((size_t)f.e * pr.N + col + 16 * h) * pr.M + f.m0 + quarter * 32 + lr;
+    } else {
+        const int which = col / pr.out_cols;
+        float* o = pr.out[which] + ((size_t)f.e * pr.M + f.m0 + quarter * 32) * pr.out_cols + (col - which * pr.out_cols) + lq * 4;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                o[(size_t)(4 * q) * pr.M] = acc[q].x; o[(size_t)(4 * q + 1) * pr.M] = acc[q].y;
-                o[(size_t)(4 * q + 2) * pr.M] = acc[q].z; o[(size_t)(4 * q + 3) * pr.M] = acc[q].w;
-            }
-        } else {
-            float* o = pr.out[which] + ((size_t)f.e * pr.M + f.m0 + quarter * 32) * pr.out_cols + (col - which * pr.out_cols) + lq * 4;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) *(float4*)(o + (size_t)((4 * h + q) * 4 + lr) * pr.out_cols) = acc[q];
-        }
+        for (int q = 0; q < 4; ++q) *(float4*)(o + (size_t)((4 * h + q) * 4 + lr) * pr.out_cols) = acc[q];
     }
 }
 #endif

@@ -333,11 +333,14 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     r.prob[0] = a.prob[0];
     r.prob[1] = a.prob[nprob - 1];
     r.offsets = offsets; r.part = part; r.n = n; r.nprob = nprob; r.pieces = a.pieces;
-    r.blocks = 0;
+    int tiles = 0, widest = 0;
     for (int i = 0; i < nprob; ++i) {
-        r.blocks_per_tile[i] = (a.prob[i].BN / 32 * 4 + kReduceThreads / 32 - 1) / (kReduceThreads / 32);
-        r.blocks += n * a.prob[i].m_tiles * a.prob[i].n_tiles * r.blocks_per_tile[i];
+        tiles += n * a.prob[i].m_tiles * a.prob[i].n_tiles;
+        if (a.prob[i].BN > widest) widest = a.prob[i].BN;
     }
+    r.per = (widest / 32 * 8 + kReduceThreads / 32 - 1) / (kReduceThreads / 32);
+    r.by_cut = tiles > a.pieces - 1 ? 1 : 0;
+    r.blocks = (r.by_cut ? a.pieces - 1 : tiles) * r.per;
     *reduce = r;
     return UOE_OK;
 }
