@@ -124,8 +124,8 @@ extern "C" uoe_status uoe_block_forward(const uoe_problem* att, const uoe_proble
         } else {
             st = route_run(att, cur, Wr_att, R, scratch, stream, nullptr);
             if (st != UOE_OK) return st;
-            st = launch_plan(Da, R.expert_idx, R.patch_idx, R.gate, R.expert_offsets, P, status, stream, true, B.v,
-                             (long long)Da.d_g * Da.esize);
+            st = launch_plan(Da, R.expert_idx, R.patch_idx, R.gate, R.expert_offsets, P, status, stream, true,
+                             PlanTails{{B.v, nullptr, nullptr, nullptr}, (long long)Da.d_g * Da.esize});
             if (st != UOE_OK) return st;
         }
         void* out_att = mlp ? u : y;

@@ -40,7 +40,10 @@ using namespace tc;
 constexpr int BM = 128, BK = 64;
 constexpr int A_BLOCK_BYTES = BM * BK * 2;     // 16 KB per 128-row block
 
-template <int BN, int MT, bool BWD = false, bool PAIR = false> struct Cfg {
+// what a tile's accumulator becomes: the forward's activation, the activation's backward, the attention output's backward
+enum Epilogue { kForward = 0, kActBackward = 1, kAttBackward = 2 };
+
+template <int BN, int MT, int EPI = kForward, bool PAIR = false> struct Cfg {
     static_assert(!PAIR || (MT == 1 && BN == 256), "CTA pairs: 128 rows and half of a 256-column B tile per CTA");
     static constexpr int UNIT = PAIR ? 2 : MT;                     // 128-row blocks per row tile
     static constexpr int A_BYTES = MT * A_BLOCK_BYTES;
@@ -54,7 +57,7 @@ template <int BN, int MT, bool BWD = false, bool PAIR = false> struct Cfg {
     static constexpr int TMEM_COLS = 2 * ACC_STRIDE;               // MT=1: two sets; MT=2: one set of two blocks
     // eight epilogue warps: with 256-row tiles one per (row block, TMEM lane quarter); with 128-row tiles two per lane
     // quarter, each draining half of the columns (the long backward epilogue keeps four: its registers would not fit)
-    static constexpr int EPI_WARPS = (MT == 2 || !BWD) ? 8 : 4;
+    static constexpr int EPI_WARPS = (MT == 2 || EPI != kActBackward) ? 8 : 4;
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int STG_BYTES = 32 * 128;                     // one epilogue warp's staging piece
     static constexpr int SMEM = STAGES * STAGE + 1024 /*align slack*/ + 1024 /*barriers, offsets*/ + EPI_WARPS * STG_BYTES;
@@ -70,8 +73,8 @@ struct Ctl {                       // lives behind the stage ring
     int tstart[34];                // first row tile of each expert (prefix sum), tstart[n] = number of row tiles
 };
 
-template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR, bool ROPE>
-__global__ void __launch_bounds__(Cfg<BN, MT, BWD, PAIR>::THREADS, 1)
+template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR, bool ROPE>
+__global__ void __launch_bounds__(Cfg<BN, MT, EPI, PAIR>::THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                  const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
                  __nv_bfloat16* __restrict__ C0, __nv_bfloat16* __restrict__ C1, __nv_bfloat16* __restrict__ C2,
@@ -83,9 +86,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmX, const SrcMap smap, int l_p, int Bm,
                  const __grid_constant__ CUtensorMap tmC0, const __grid_constant__ CUtensorMap tmC1,
                  const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmPre,
+                 int k_per_mat /* > 0: K block kb is 64 columns of weight tensor kb / k_per_mat (K-major weights, three tensors) */,
+                 const AttBwd att,
                  const __grid_constant__ typename std::conditional<ROPE, Rope, NoRope>::type rope /* matrices 0 and 1 hold 64-wide heads to be rotated */) {
     pdl_trigger();
-    using Cf = Cfg<BN, MT, BWD, PAIR>;
+    constexpr bool BWD = EPI == kActBackward;
+    using Cf = Cfg<BN, MT, EPI, PAIR>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     Ctl* ctl = (Ctl*)(smem + Cf::STAGES * Cf::STAGE);
@@ -105,8 +111,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         prefetch_tmap(&tmB0);
         prefetch_tmap(&tmX);
         prefetch_tmap(&tmC0);
-        if (nmat > 1 || BN == 192) { prefetch_tmap(&tmB1); prefetch_tmap(&tmB2); prefetch_tmap(&tmC1); prefetch_tmap(&tmC2); }
-        if (BWD) prefetch_tmap(&tmC1);
+        if (nmat > 1 || BN == 192 || k_per_mat > 0) { prefetch_tmap(&tmB1); prefetch_tmap(&tmB2); prefetch_tmap(&tmC1); prefetch_tmap(&tmC2); }
+        if (EPI != kForward) prefetch_tmap(&tmC1);
     }
     if (warp == 1) {
         if constexpr (PAIR) tmem_alloc_pair(&ctl->tmem_base, Cf::TMEM_COLS);
@@ -165,6 +171,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // set by the number of copies it issues.  W [n, K, N] is mapped as [n][N/64 column blocks][K][64], so a box holds
         // all the column blocks of a tile; the three side-by-side matrices take one copy each.
         constexpr int nbox_b = SIDE3 ? 3 : 1;
+        auto pick = [&](int q) { return q == 0 ? &tmB0 : (q == 1 ? &tmB1 : &tmB2); };
         const CUtensorMap* tmB_lane = lane == 0 ? &tmB0 : (lane == 1 ? &tmB1 : &tmB2);
         int e = 0;
         for (int tile = worker; tile < total_tiles && !stop; tile += workers) {
@@ -207,7 +214,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             else tma_load_2d_pair(sa_j, &tmA, k0, arow0, full0);
                         }
                         if (bx == 0) {
-                            if (B_KMAJOR) tma_load_3d_pair(sb_j, tmB, k0, bcol0, e, full0);
+                            if (B_KMAJOR) {
+                                const int kblk = kb * Cf::KSUB + j, q = k_per_mat > 0 ? kblk / k_per_mat : 0;
+                                tma_load_3d_pair(sb_j, k_per_mat > 0 ? pick(q) : tmB, (kblk - q * k_per_mat) * BK, bcol0, e, full0);
+                            }
                             else tma_load_4d_pair(sb_j, tmB, 0, k0, bcol0 / 64, e, full0);
                         }
                     }
@@ -218,7 +228,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                     if (lane < nbox_b) {
                         if (SIDE3) tma_load_4d(sb + lane * 8192, tmB_lane, 0, kb * BK, 0, e, &ctl->full[stage]);
-                        else if (B_KMAJOR) tma_load_3d(sb, tmB, kb * BK, col0, e, &ctl->full[stage]);
+                        else if (B_KMAJOR) {
+                            const int q = k_per_mat > 0 ? kb / k_per_mat : 0;
+                            tma_load_3d(sb, k_per_mat > 0 ? pick(q) : tmB, (kb - q * k_per_mat) * BK, col0, e, &ctl->full[stage]);
+                        }
                         else tma_load_4d(sb, tmB, 0, kb * BK, col0 / 64, e, &ctl->full[stage]);
                     }
                 }
@@ -349,6 +362,41 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         stage_store(ag, &tmC1, col0 + g * 64, wrow0);
                     }
                     dg_part[row * n_tiles_mat + (col0 / BN)] = rv * dsum;
+                } else if constexpr (EPI == kAttBackward) {
+                    // u = dy_g W^o^T of a 64-wide head, o the head's attention output, w the row's combine weight:
+                    // C = w u, C1 = w o, delta = w <u, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that
+                    // weigh nothing, whose o may never have been written)
+                    const float rg = row_gate[row], rv = row_valid[row];
+                    if (g_lo == 0 && (int)row >= att.expert_end[e]) {       // padding rows of dq, dk, dv: no other kernel writes them
+                        uint4* z = (uint4*)(att.dqkv + row * (3 * (size_t)N) + 3 * col0);
+                        for (int q = 0; q < 3 * BN / 8; ++q) z[q] = make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll 1
+                    for (int g = g_lo; g < g_hi; ++g) {
+                        uint32_t v[64];
+                        tmem_ld32(taddr + g * 64, v);
+                        tmem_ld32(taddr + g * 64 + 32, v + 32);
+                        const uint4* op = (const uint4*)(bwd_h + row * N + col0 + g * 64);
+                        uint4 ov[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) ov[q] = op[q];
+                        tmem_ld_wait();
+                        float u[64], o[64], dot = 0.f;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) unpack16<__nv_bfloat16>(ov[q], o + 8 * q);
+#pragma unroll
+                        for (int q = 0; q < 64; ++q) {
+                            u[q] = __uint_as_float(v[q]);
+                            dot = fmaf(u[q], o[q], dot);
+                            u[q] = rg != 0.f ? u[q] * rg : 0.f;
+                            o[q] = rg != 0.f ? o[q] * rg : 0.f;
+                        }
+                        stage_store(u, &tmC0, col0 + g * 64, wrow0);
+                        stage_store(o, &tmC1, col0 + g * 64, wrow0);
+                        const size_t h = row * (N / 64) + col0 / 64 + g;
+                        att.delta[h] = rg != 0.f ? rg * dot : 0.f;
+                        dg_part[h] = rv != 0.f ? dot : 0.f;
+                    }
                 } else {
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g) {
@@ -415,12 +463,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
 }
 
-template <int BN, bool B_KMAJOR, bool BWD, int MT, bool PAIR = false, bool ROPE = false>
+template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR = false, bool ROPE = false>
 uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
-    using Cf = Cfg<BN, MT, BWD, PAIR>;
+    using Cf = Cfg<BN, MT, EPI, PAIR>;
     static DeviceOnce once;
     static DeviceValue pairs_cache;    // CTA pairs that can be resident at once, per device
-    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, BWD, MT, PAIR, ROPE>;
+    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, EPI, MT, PAIR, ROPE>;
     {
         const uoe_status st = smem_opt_in(once, kern, Cf::SMEM);
         if (st != UOE_OK) return st;
@@ -454,8 +502,9 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     const void* Ws[3] = {g.W, g.W1 ? g.W1 : g.W, g.W2 ? g.W2 : g.W};
     for (int q = 0; q < 3; ++q) {
         if (B_KMAJOR) {       // W [n, N, K]
-            const uint64_t dims[3] = {(uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.n};
-            const uint64_t str[2] = {(uint64_t)g.K * 2, (uint64_t)g.K * g.N * 2};
+            const uint64_t Kw = g.k_mats > 0 ? g.K / g.k_mats : g.K;
+            const uint64_t dims[3] = {Kw, (uint64_t)g.N, (uint64_t)g.n};
+            const uint64_t str[2] = {Kw * 2, Kw * g.N * 2};
             const uint32_t box[3] = {BK, PAIR ? BN / 2 : BN, 1};
             if (!make_tmap(&tmB[q], Ws[q], 3, dims, str, box)) return UOE_ERR_CUDA;
         } else {              // W [n, K, N] as [n][N/64 column blocks][K][64]
@@ -497,12 +546,12 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
                                              (__nv_bfloat16*)g.C2, (__nv_bfloat16*)g.pre, g.offsets, g.n, g.K, g.N,
                                              nmat, g.act, status, (const __nv_bfloat16*)g.bwd_h, g.row_gate, g.row_valid,
                                              g.dg_part, (const __nv_bfloat16*)g.bias, g.blk_scale, tmX, smap, g.l_p, g.Bm, tmC[0],
-                                             tmC[1], tmC[2], tmPre, rope);
+                                             tmC[1], tmC[2], tmPre, g.k_mats > 0 ? g.K / g.k_mats / BK : 0, g.att, rope);
     UOE_LAUNCHED();
     return UOE_OK;
 }
 
-template <bool B_KMAJOR, bool BWD, bool ROPE = false>
+template <bool B_KMAJOR, int EPI, bool ROPE = false>
 uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
     const int bn = gemm_bf16_bn(g.N);
     // 256-row tiles pay off when every SM still gets several of them and the K loop is long enough to be
@@ -510,16 +559,16 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
     const long long tiles256 = (g.rows_max / 256) * (g.N / 256);
     // the backward epilogue is long: it stays on 128-row accumulators, whose drain overlaps the next tile's main loop,
     // and takes its 256-row tiles from CTA pairs when there are enough of them for every pair of SMs
-    if constexpr (BWD) {
-        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 1, true>(g, status, s);
+    if constexpr (EPI == kActBackward) {
+        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true>(g, status, s);
     }
-    if constexpr (!BWD) {
-        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 1, true, ROPE>(g, status, s);
-        if (bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, BWD, 2, false, ROPE>(g, status, s);
+    if constexpr (EPI == kForward) {
+        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true, ROPE>(g, status, s);
+        if (bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 2, false, ROPE>(g, status, s);
     }
-    if (bn == 256) return launch_one<256, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
-    if (bn == 128) return launch_one<128, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
-    return launch_one<64, B_KMAJOR, BWD, 1, false, ROPE>(g, status, s);
+    if (bn == 256) return launch_one<256, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
+    if (bn == 128) return launch_one<128, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
+    return launch_one<64, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
 }
 
 }  // namespace
@@ -535,13 +584,18 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
     if (g.bwd) {          // backward epilogue: weights are read K-major ([n, N, K])
         if (!g.b_kmajor || !g.bwd_h || !g.row_gate || !g.row_valid || !g.dg_part || !g.C1 || g.nmat > 1)
             return UOE_ERR_INVALID_ARG;
-        return dispatch<true, true>(g, status, s);
+        return dispatch<true, kActBackward>(g, status, s);
+    }
+    if (g.k_mats > 0 && (g.k_mats > 3 || !g.b_kmajor || g.nmat > 1 || g.K % (g.k_mats * BK) != 0)) return UOE_ERR_UNSUPPORTED;
+    if (g.att.delta) {    // attention output's backward
+        if (!g.b_kmajor || !g.bwd_h || !g.row_gate || !g.row_valid || !g.dg_part || !g.C1 || g.nmat > 1) return UOE_ERR_INVALID_ARG;
+        return dispatch<true, kAttBackward>(g, status, s);
     }
     if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre)
-        return rope ? launch_one<192, false, false, 1, false, true>(g, status, s) : launch_one<192, false, false, 1>(g, status, s);
-    if (rope) return dispatch<false, false, true>(g, status, s);
-    if (g.b_kmajor) return dispatch<true, false>(g, status, s);
-    return dispatch<false, false>(g, status, s);
+        return rope ? launch_one<192, false, kForward, 1, false, true>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
+    if (rope) return dispatch<false, kForward, true>(g, status, s);
+    if (g.b_kmajor) return dispatch<true, kForward>(g, status, s);
+    return dispatch<false, kForward>(g, status, s);
 }
 
 }  // namespace uoe

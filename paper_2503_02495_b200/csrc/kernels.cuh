@@ -172,10 +172,12 @@ __device__ __forceinline__ int src_of(const SrcMap& g, int r, int e, int off_e, 
 #endif
 
 // use_gate only matters for the per-row arrays of the backward (row_gate = gate or 1).
-// If tail is not null, rows [offsets[n], Rmax) of tail (rows of tail_row_bytes) are zero-filled.
+// Buffers in `tails` (rows of tails.row_bytes): the first 128 rows past the last expert region are zero-filled, as many as a
+// 128-row tile that starts inside the last region can reach.
+struct PlanTails { void* p[4] = {nullptr, nullptr, nullptr, nullptr}; long long row_bytes = 0; };
 uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_idx, const float* gate,
                        const int* offsets, const PlanPtrs& P, int* status, cudaStream_t s, bool use_gate = true,
-                       void* tail = nullptr, long long tail_row_bytes = 0);
+                       const PlanTails& tails = PlanTails());
 
 // Eq. 18 / 24: copy the selected patches of `src` [B,L,d] into the routed buffer `dst` [rows,d];
 // unused slots and the padding rows of each expert region are zero-filled.
@@ -222,6 +224,13 @@ uoe_status launch_dwr_sum(const DwrSum& sum, cudaStream_t s);
 uoe_status launch_combine(const Dims& D, const void* x, const void* z, const PlanPtrs& P, bool residual,
                           bool use_gate, void* y, cudaStream_t s, const float* rvec = nullptr, const DwrSum& sum = DwrSum());
 
+// Attention output's backward in a GEMM's epilogue (see GemmArgs::att).
+struct AttBwd {
+    float* delta = nullptr;              // [rows, heads]
+    const int* expert_end = nullptr;     // [n]
+    __nv_bfloat16* dqkv = nullptr;       // [rows, 3 N]
+};
+
 // Grouped GEMM over the routed rows: C[r,:] = epilogue(A[r,:] @ W[e(r)]) where e(r) is the expert whose
 // region holds row r.  W is [n, K, N] (b_kmajor = false: rows of K, N contiguous) or [n, N, K] (true).
 struct GemmArgs {
@@ -259,6 +268,12 @@ struct GemmArgs {
     // per 128-row block, Eq. 40 applied ahead of the second layer; `pre` keeps the unscaled pre-activation)
     const float* blk_scale = nullptr;
     const Rope* rope = nullptr;       // nmat = 3 (q, k, v of 64-wide heads): q and k are rotated before they are stored
+    // bf16 path, K-major weights, K split over k_mats weight tensors of the same shape (W, W1, W2: [n, N, K / k_mats] each)
+    int k_mats = 0;
+    // bf16 path, attention output's backward (att.delta set): with u = A @ W the gradient w.r.t. the attention output o
+    // (64-wide heads), o = bwd_h[r,:]:  C = w u, C1 = w o, delta[r, head] = w <u, o>, dg_part[r, head] = <u, o> (0 where
+    // row_valid is 0), w = row_gate[r]; the padding rows of att.dqkv are zeroed
+    AttBwd att;
     bool bwd = false;
     const void* bwd_h = nullptr;
     const float* row_gate = nullptr;

@@ -49,7 +49,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             const int* __restrict__ offsets, int B, int n, int k, int m, int c, int l_p,
             int* __restrict__ pair_row, int* __restrict__ inv_row, float* __restrict__ inv_gate,
             int* __restrict__ expert_end, int* status, float* __restrict__ row_gate, float* __restrict__ row_valid,
-            int Lv, int use_gate, int* __restrict__ src_patch, uint4* __restrict__ tail, long long tail_row_vecs,
+            int Lv, int use_gate, int* __restrict__ src_patch, const PlanTails tails,
             long long rows_max, int rows_given /* pair_row already holds every pair's first row (plan_rows_kernel) */,
             int* __restrict__ slot_pair) {
     pdl_trigger();
@@ -134,11 +134,13 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
                 for (int r = s_end[i] + tid; r < offs[i + 1]; r += NT) { row_gate[r] = 0.f; row_valid[r] = 0.f; }
         }
     }
-    if (tail) {
-        const long long r0 = offs[n];
-        const long long total = (rows_max - r0) * tail_row_vecs;
+    if (tails.row_bytes > 0) {
+        const long long r0 = offs[n], row_vecs = tails.row_bytes / 16;
+        const long long total = (min(rows_max, r0 + 128) - r0) * row_vecs;
         for (long long q = (long long)b * NT + tid; q < total; q += (long long)B * NT)
-            tail[r0 * tail_row_vecs + q] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (tails.p[i]) ((uint4*)tails.p[i])[r0 * row_vecs + q] = make_uint4(0, 0, 0, 0);
     }
     if (row_gate) {                          // per-row weights for the backward
         for (int idx = tid; idx < k * l_a; idx += NT) {
@@ -423,8 +425,7 @@ constexpr long long kF32LargeTiles = 160;
 }  // namespace
 
 uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_idx, const float* gate,
-                       const int* offsets, const PlanPtrs& P, int* status, cudaStream_t s, bool use_gate, void* tail,
-                       long long tail_row_bytes) {
+                       const int* offsets, const PlanPtrs& P, int* status, cudaStream_t s, bool use_gate, const PlanTails& tails) {
     const size_t smem = (size_t)D.k * D.c * 8;
     if (smem > 32 * 1024) return UOE_ERR_UNSUPPORTED;      // a sample's routing arrays live in shared memory
     const bool many = D.B > kPlanScanMaxB;
@@ -437,7 +438,7 @@ uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_id
     const int threads = (P.row_gate && (long long)D.k * D.l_a >= 4096) ? 512 : 128;      // the backward's per-row weights: k*l_a rows per sample
     launch_k(plan_kernel, dim3(D.B), dim3(threads), smem, s, expert_idx, patch_idx, gate, offsets, D.B, D.n, D.k, D.m, D.c, D.l_p,
                                     P.pair_row, P.inv_row, P.inv_gate, P.expert_end, status, P.row_gate, P.row_valid,
-                                    D.Lv, use_gate ? 1 : 0, P.src_patch, (uint4*)tail, tail_row_bytes / 16, D.Rmax, many ? 1 : 0, P.slot_pair);
+                                    D.Lv, use_gate ? 1 : 0, P.src_patch, tails, D.Rmax, many ? 1 : 0, P.slot_pair);
     UOE_LAUNCHED();
     return UOE_OK;
 }

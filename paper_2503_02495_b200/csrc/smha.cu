@@ -111,8 +111,8 @@ extern "C" uoe_status uoe_smha_forward(const uoe_problem* prob, const void* x, c
     const SmhaFwdBufs bufs{base + W.xg, base + W.q, base + W.k, base + W.v, base + W.o, base + W.z};
     // rows of v past the last expert region are never written by the projection but may sit inside the
     // last key tile of a pair: the plan kernel makes them finite (zero)
-    st = launch_plan(D, expert_idx, patch_idx, gate, expert_offsets, P, status, stream, true, bufs.v,
-                     (long long)D.d_g * D.esize);
+    st = launch_plan(D, expert_idx, patch_idx, gate, expert_offsets, P, status, stream, true,
+                     PlanTails{{bufs.v, nullptr, nullptr, nullptr}, (long long)D.d_g * D.esize});
     if (st != UOE_OK) return st;
     return smha_forward_run(D, prob, x, Wq, Wk, Wv, Wo, expert_idx, patch_idx, expert_offsets, P, bufs, y, lse, status, stream);
 }
