@@ -56,8 +56,8 @@ template <int BN, int MT, int EPI = kForward, bool PAIR = false> struct Cfg {
     static constexpr int ACC_STRIDE = (BN == 192) ? 256 : BN;      // TMEM columns between the two accumulator sets
     static constexpr int TMEM_COLS = 2 * ACC_STRIDE;               // MT=1: two sets; MT=2: one set of two blocks
     // eight epilogue warps: with 256-row tiles one per (row block, TMEM lane quarter); with 128-row tiles two per lane
-    // quarter, each draining half of the columns (the long backward epilogue keeps four: its registers would not fit)
-    static constexpr int EPI_WARPS = (MT == 2 || EPI != kActBackward) ? 8 : 4;
+    // quarter, each draining half of the columns
+    static constexpr int EPI_WARPS = 8;
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int STG_BYTES = 32 * 128;                     // one epilogue warp's staging piece
     static constexpr int SMEM = STAGES * STAGE + 1024 /*align slack*/ + 1024 /*barriers, offsets*/ + EPI_WARPS * STG_BYTES;
@@ -295,7 +295,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int wsel = (warp - 2) >> 2;
         const int half = PAIR ? rank : (MT == 2 ? wsel : 0);  // 128-row block this warp drains
         constexpr int G = BN / 64;                            // 64-column groups of the accumulator
-        constexpr bool SPLIT_COLS = MT == 1 && Cf::EPI_WARPS == 8;
+        constexpr bool SPLIT_COLS = MT == 1;
         const int g_lo = SPLIT_COLS ? wsel * ((G + 1) / 2) : 0;
         const int g_hi = SPLIT_COLS ? min(G, g_lo + (G + 1) / 2) : G;
         int acc = 0;
@@ -307,6 +307,16 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             return w;
         };
         uint8_t* stg = smem + Cf::STAGES * Cf::STAGE + 1024 + (warp - 2) * Cf::STG_BYTES;
+        auto stage_store_packed = [&](const uint32_t* f, const CUtensorMap* tm, int c0, int r0) {      // the same for bf16 pairs
+            if (lane == 0) bulk_wait_read();
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                *(uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = make_uint4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) { tma_store_2d(tm, stg, c0, r0); bulk_commit(); }
+        };
         // 64 values of this thread's row -> bf16 -> this warp's staging piece (row = lane, 128B swizzle) -> TMA store
         auto stage_store = [&](const float* f, const CUtensorMap* tm, int c0, int r0) {
             if (lane == 0) bulk_wait_read();          // the previous store has finished reading the piece
@@ -335,33 +345,44 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const size_t row = (size_t)wrow0 + lane;
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (MT == 2 ? half * BN : acc * Cf::ACC_STRIDE);
                 if constexpr (BWD) {
+                    // (32 columns at a time, kept packed until the 64-column pieces are complete: few enough registers for
+                    // eight warps; with four warps of 64 columns the image block's launch took 68 us)
                     const float rg = row_gate[row], rv = row_valid[row];
                     float dsum = 0.f;
 #pragma unroll 1
-                    for (int g = 0; g < BN / 64; ++g) {
-                        uint32_t v[64];
-                        tmem_ld32(taddr + g * 64, v);
-                        tmem_ld32(taddr + g * 64 + 32, v + 32);
+                    for (int g = g_lo; g < g_hi; ++g) {
+                        uint32_t pd[32], pa[32];             // dh and gated phi(h) of the piece, bf16 pairs
                         const uint4* hp = (const uint4*)(bwd_h + row * N + col0 + g * 64);
-                        uint4 hv[8];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) hv[q] = hp[q];
-                        tmem_ld_wait();
-                        float dh[64], ag[64];
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t v[32];
+                            tmem_ld32(taddr + g * 64 + c * 32, v);
+                            uint4 hv[4];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) unpack16<__nv_bfloat16>(hv[q], dh + 8 * q);     // h
-                        act_and_deriv_n<64>(dh, ag, dh, act);                                         // ag = phi(h), dh = phi'(h)
+                            for (int q = 0; q < 4; ++q) hv[q] = hp[c * 4 + q];
+                            tmem_ld_wait();
+                            float dh[32], ag[32];
 #pragma unroll
-                        for (int q = 0; q < 64; ++q) {
-                            const float u = __uint_as_float(v[q]);
-                            dsum = fmaf(u, ag[q], dsum);
-                            dh[q] = rg * u * dh[q];
-                            ag[q] = rg * ag[q];
+                            for (int q = 0; q < 4; ++q) unpack16<__nv_bfloat16>(hv[q], dh + 8 * q);     // h
+                            act_and_deriv_n<32>(dh, ag, dh, act);                                         // ag = phi(h), dh = phi'(h)
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) {
+                                const float u = __uint_as_float(v[q]);
+                                dsum = fmaf(u, ag[q], dsum);
+                                dh[q] = rg * u * dh[q];
+                                ag[q] = rg * ag[q];
+                            }
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) {
+                                pd[c * 16 + q] = pack_bf16x2(dh[2 * q], dh[2 * q + 1]);
+                                pa[c * 16 + q] = pack_bf16x2(ag[2 * q], ag[2 * q + 1]);
+                            }
                         }
-                        stage_store(dh, &tmC0, col0 + g * 64, wrow0);
-                        stage_store(ag, &tmC1, col0 + g * 64, wrow0);
+                        stage_store_packed(pd, &tmC0, col0 + g * 64, wrow0);
+                        stage_store_packed(pa, &tmC1, col0 + g * 64, wrow0);
                     }
-                    dg_part[row * n_tiles_mat + (col0 / BN)] = rv * dsum;
+                    constexpr int DG = dg_cols_per_tile(BN);
+                    if (wsel < DG) dg_part[row * (n_tiles_mat * DG) + (col0 / BN) * DG + wsel] = rv * dsum;
                 } else if constexpr (EPI == kAttBackward) {
                     // u = dy_g W^o^T of a 64-wide head, o the head's attention output, w the row's combine weight:
                     // C = w u, C1 = w o, delta = w <u, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that

@@ -281,8 +281,11 @@ struct GemmArgs {
     float* dg_part = nullptr;
 };
 
-// Column-tile width the bf16 grouped GEMM uses for N output columns (dg_part has N / that many columns).
+// Column-tile width the bf16 grouped GEMM uses for N output columns; dg_part has one column per tile, or two where a tile's
+// columns are shared by two epilogue warps.
 inline int gemm_bf16_bn(int N) { return (N % 256 == 0) ? 256 : (N % 128 == 0 ? 128 : 64); }
+__host__ __device__ constexpr int dg_cols_per_tile(int bn) { return bn >= 128 ? 2 : 1; }
+inline int gemm_dg_cols(int N) { return N / gemm_bf16_bn(N) * dg_cols_per_tile(gemm_bf16_bn(N)); }
 
 // Per-expert weight gradient over ragged row counts:  dW[e] [M, N] (float32, overwritten) =
 // sum over the rows r of expert e's region of  P[r, 0:M]^T  Q[r, 0:N]   (P [rows, M], Q [rows, N], bf16).

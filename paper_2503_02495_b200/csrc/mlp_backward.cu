@@ -327,7 +327,7 @@ BwdWs bwd_ws(const Dims& D) {
     WsCarver w;
     w.take(kStatusBytes);
     BwdWs r;
-    r.nt = D.d_e / gemm_bf16_bn(D.d_e > 0 ? D.d_e : 64);
+    r.nt = gemm_dg_cols(D.d_e);
     if (r.nt < 1) r.nt = 1;
     r.plan = w.take(plan_bytes(D, true));
     const bool fused = bwd_can_gather(D);      // dy and x gathered inside the consumers' TMA loads
