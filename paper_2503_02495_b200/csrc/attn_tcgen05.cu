@@ -6,7 +6,7 @@
 // one 128-query tile of one head of one pair; its keys come in 128-key tiles.
 //
 // Two kernels:
-//   attn_stream_kernel   many units (at least two per SM).  A persistent CTA (one per SM) holds two independent
+//   attn_stream_kernel   more units than SMs.  A persistent CTA (one per SM) holds two independent
 //     pipelines, each with its own TMA warp, its own MMA-issuing warp, four softmax warps (one thread per query row),
 //     its own Q buffer, two K/V stages, P buffer and TMEM columns, and each working units of its own:
 //       TMA warp      Q tile of the unit, then K and V of each key tile into the two-stage ring; with the fused output
@@ -20,7 +20,7 @@
 //     The pipelines only meet in the tensor and special-function units of their SM: while one computes exponentials
 //     or drains its output, the other's MMAs and loads run, and a pipeline's next Q, K, V are in flight while it
 //     still works the current unit.
-//   attn_tile_kernel     few units (fewer than two per SM): one CTA per unit, all eight warps on its softmax (two
+//   attn_tile_kernel     few units (at most one per SM): one CTA per unit, all eight warps on its softmax (two
 //     threads per query row), S of the next key tile issued behind P V, the output projection as one MMA group over
 //     all of TMEM.  With one unit per SM there is nothing to overlap a unit with, so the whole CTA works the unit.
 // Masks: the real keys of a pair are a prefix of its gathered order (patches ascending, pad tokens at
@@ -127,7 +127,21 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 
     // ---- the units of this pipeline ----
     const int n_units = a.pairs * a.heads * a.n_qt;
-    const int u_first = (int)blockIdx.x * 2 + g, u_step = 2 * (int)gridDim.x;
+    // With the causal mask a unit's work grows with its query tile: the units are taken heaviest tile first, dealt to the
+    // pipelines back and forth (every CTA's second pipeline counted from the other end), so that an SM gets about as much
+    // as any other.  Without it all units weigh the same and the query tiles of a (pair, head) stay together.
+    const int workers = 2 * (int)gridDim.x, worker = g == 0 ? (int)blockIdx.x : workers - 1 - (int)blockIdx.x;
+    auto unit_at = [&](int round, int& qt, int& head, int& pair) {
+        const int u = round * workers + ((round & 1) ? workers - 1 - worker : worker);
+        if (u >= n_units) return false;
+        if (a.causal) {
+            const int ph = a.pairs * a.heads;
+            qt = a.n_qt - 1 - u / ph; head = u % ph % a.heads; pair = u % ph / a.heads;
+        } else {
+            qt = u % a.n_qt; head = (u / a.n_qt) % a.heads; pair = u / (a.n_qt * a.heads);
+        }
+        return true;
+    };
     constexpr int t_first = 0, t_step = 1;
     auto kv_tiles = [&](int q0, int n_valid) {              // key tiles the unit has in all
         int kv_end = min(n_valid, a.l_a);
@@ -144,8 +158,8 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // =========================== TMA warp ===========================
         uint32_t q_cnt = 0, kv_cnt = 0;
         bool ok = true;
-        for (int u = u_first; u < n_units && ok; u += u_step) {
-            const int qt = u % a.n_qt, head = (u / a.n_qt) % a.heads, pair = u / (a.n_qt * a.heads);
+        int qt, head, pair;
+        for (int round = 0; ok && unit_at(round, qt, head, pair); ++round) {
             // real keys of this pair: sum over its slots of the real tokens in the slot's patch
             int nv = 0;
             for (int s0 = lane; s0 < a.c; s0 += 32) {
@@ -207,8 +221,8 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             constexpr uint32_t idesc_o = instr_desc_bf16(TQ, DH, false, true);
             uint32_t q_cnt = 0, kv_cnt = 0, acc_cnt = 0, p_cnt = 0, ready_cnt = 0;
             bool ok = true;
-            for (int u = u_first; u < n_units && ok; u += u_step) {
-                const int qt = u % a.n_qt;
+            int qt, head, pair;
+            for (int round = 0; ok && unit_at(round, qt, head, pair); ++round) {
                 ok = wait1(&pc->q_full, q_cnt & 1);
                 ++q_cnt;
                 if (!ok) break;
@@ -283,8 +297,8 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const int sw = trow & 7;
         uint32_t q_cnt = 0, acc_cnt = 0, o_cnt = 0;
         bool ok = true;
-        for (int u = u_first; u < n_units && ok; u += u_step) {
-            const int qt = u % a.n_qt, head = (u / a.n_qt) % a.heads;
+        int qt, head, pair;
+        for (int round = 0; ok && unit_at(round, qt, head, pair); ++round) {
             ok = __all_sync(0xffffffffu, wait(&pc->q_full, q_cnt & 1));
             ++q_cnt;
             if (!ok) break;
@@ -828,7 +842,9 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)D.d_h);
     ProfScope ps("attention", s);
     cudaError_t e;
-    if (units >= 2ll * sm_count()) {          // enough units to keep two pipelines per SM fed
+    // more units than SMs: two pipelines per SM (256 causal units of up to eight key tiles: 27 us, against 34 in two waves
+    // of one CTA per unit)
+    if (units > sm_count()) {
         AttnArgs a;
         a.O = (__nv_bfloat16*)o; a.Z = (__nv_bfloat16*)z; a.lse = lse;
         a.pair_row = pair_row; a.patch_idx = patch_idx; a.expert_idx = expert_idx;
@@ -841,7 +857,7 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
         if (fuse) e = launch_k(attn_stream_kernel<true>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
         else e = launch_k(attn_stream_kernel<false>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
     } else {
-        if (pairs > 65535) return UOE_ERR_UNSUPPORTED;      // (cannot happen: fewer than two units per SM)
+        if (pairs > 65535) return UOE_ERR_UNSUPPORTED;      // (cannot happen: at most one unit per SM)
         dim3 grid(n_qt, heads, (unsigned)pairs);
         if (fuse)
             e = launch_k(attn_tile_kernel<true>, grid, dim3(kTileThreads), TILE_SMEM_FUSED, s, tm[0], tm[1], tm[2], (__nv_bfloat16*)o, lse,
