@@ -18,13 +18,13 @@ namespace {
 constexpr int kScoreThreads = 256;
 
 // Selection for sample b by one CTA of NT threads (all threads call).  pp: n*m floats of shared memory.
-// Written for a short dependent chain (the router is latency-bound on all but the largest inputs): three phases
-// separated by CTA barriers, then the ticket.
+// Written for a short dependent chain (the router is latency-bound on all but the largest inputs): a CTA barrier between
+// the first phase and the others, then the ticket.
 //   A  a warp works 32/np2 patches at a time (np2 = n rounded up to a power of two), one lane per (patch, expert):
 //      adds the parts of the score in ascending order, softmax over the experts of the patch through segment
 //      shuffles (Eq. 14), first-stage counts of Eq. 15 when the capacity is dynamic; the raw scores are summed per
 //      expert on the side for the sample gate
-//   B  warp 0: sample gate (Eq. 21), top-k experts (Eq. 22); the other warps write p_patch
+//   B  every warp for itself: sample gate (Eq. 21), top-k experts (Eq. 22)
 //   C  a warp per chosen expert: top-c patches by rank counting (Eq. 17), gates, the inverse map of the plan
 // The CTA that completes the last sample (a ticket) turns every sample's expert set (one bit mask per sample, masks[B]
 // in the scratch area) into per-expert row offsets (Eq. 23) and, for the plan, each pair's first row.
@@ -39,9 +39,7 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
                               const float* local_scores = nullptr /* [m,n] in shared memory: used instead of `partial` */) {
     constexpr int NW = NT / 32;
     constexpr int kMaskCache = 1024;       // samples whose masks the last CTA keeps in shared memory
-    __shared__ float ps[32];               // sample gate
     __shared__ float s_raw[NW][32];        // per warp: sum over its patches of the raw scores, per expert
-    __shared__ int sel[32];                // chosen experts, ascending
     __shared__ int cnts[32];               // Eq. 16: patches each expert receives in the first routing stage; later: samples per expert
     __shared__ int s_last;
     __shared__ unsigned s_masks[kMaskCache];
@@ -90,7 +88,8 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
             const float e = valid ? expf(g - mx) : 0.f;
             float sum = e;
             for (int o = np2 >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            const float pr = e / sum;                    // (lanes outside the problem: 0/0, never used)
+            // (lanes outside the problem divide 1 by 1: a zero operand would send the whole warp through the division's slow path)
+            const float pr = (valid ? e : 1.f) / (valid ? sum : 1.f);
             if (valid) pp[i * m + j] = pr;
             if (dynamic_c) {                        // Eq. 15: every real patch goes to its k best experts (ties: lower index)
                 int rank = 0;
@@ -107,7 +106,10 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
     __syncthreads();
 
     // ---- B ----
-    if (warp == 0) {
+    for (int idx = tid; idx < n * m; idx += NT) p_patch[(size_t)b * n * m + idx] = pp[idx];
+    float ps;                                   // this lane's expert: sample gate
+    unsigned chosen;                            // the chosen experts
+    {
         float v = -INFINITY;
         if (lane < n) {                         // Eq. 21: mean over the real tokens, then W_r
             float s = 0.f;
@@ -122,29 +124,22 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
         float sum = e;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        const float pr = e / sum;
-        if (lane < n) { ps[lane] = pr; p_samp[(size_t)b * n + lane] = pr; }
+        ps = (lane < n ? e : 1.f) / sum;        // (lanes past the experts: not zero, for the division's fast path)
         // Eq. 22: rank = number of experts that beat this one (larger value, or equal with lower index)
         int rank = 0;
         if (!all_experts)
             for (int i = 0; i < n; ++i) {
-                const float w = __shfl_sync(0xffffffffu, pr, i);
-                rank += (w > pr) || (w == pr && i < lane);
+                const float w = __shfl_sync(0xffffffffu, ps, i);
+                rank += (w > ps) || (w == ps && i < lane);
             }
         const bool pick = lane < n && rank < k;
-        const unsigned mask = __ballot_sync(0xffffffffu, pick);
-        if (pick) {
-            const int s = __popc(mask & ((1u << lane) - 1u));
-            sel[s] = lane;
-            expert_idx[(size_t)b * k + s] = lane;
+        chosen = __ballot_sync(0xffffffffu, pick);
+        if (warp == 0) {
+            if (lane < n) p_samp[(size_t)b * n + lane] = ps;
+            if (pick) expert_idx[(size_t)b * k + __popc(chosen & ((1u << lane) - 1u))] = lane;
+            if (lane == 0) masks[b] = chosen;
         }
-        if (lane == 0) masks[b] = mask;
     }
-    if (NW == 1 || warp > 0) {
-        const int t0 = NW == 1 ? tid : tid - 32, nt = NW == 1 ? NT : NT - 32;
-        for (int idx = t0; idx < n * m; idx += nt) p_patch[(size_t)b * n * m + idx] = pp[idx];
-    }
-    __syncthreads();
 
     // ---- C ----
     int take = min(c, n_elig);
@@ -154,7 +149,9 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
         take = min(take, c_dyn);
     }
     for (int s = warp; s < k; s += NW) {            // Eq. 17 for the s-th chosen expert
-        const int i = sel[s];
+        const bool is_s = ((chosen >> lane) & 1u) && __popc(chosen & ((1u << lane) - 1u)) == s;
+        const int i = __ffs(__ballot_sync(0xffffffffu, is_s)) - 1;
+        const float p_i = __shfl_sync(0xffffffffu, ps, i);
         const float* v_i = pp + i * m;
         int* out_idx = patch_idx + ((size_t)b * k + s) * c;
         float* out_gate = gate + ((size_t)b * k + s) * c;
@@ -175,7 +172,7 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
             const bool pick = valid && rank < take;
             const unsigned mask = __ballot_sync(0xffffffffu, pick);
             const int pos = before + __popc(mask & ((1u << lane) - 1u));
-            const float g = use_gate ? ps[i] * v : 1.0f;
+            const float g = use_gate ? p_i * v : 1.0f;
             if (pick) {
                 out_idx[pos] = j;
                 out_gate[pos] = g;
@@ -218,10 +215,10 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
     if (tid == 0) {
         __threadfence();
         s_last = (atomicAdd(ticket, 1) == B - 1);
+        __threadfence();
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
     if (tid == 0) *ticket = 0;              // left at zero for the next call
     if (tid < 32) cnts[tid] = 0;
     __syncthreads();
@@ -298,7 +295,8 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     pdl_wait();
     constexpr int V = Vec16<T>::N;
     extern __shared__ uint4 s_dyn4[];
-    __shared__ __align__(16) float s_cs[NT * V];                    // column sums across row threads; later pooled columns, dot partials
+    __shared__ __align__(16) float s_cs[NT * V];                    // column sums across row threads; later over all rows
+    __shared__ float s_dot[NT / 32][32];
     __shared__ int s_mine;
     const int tid = threadIdx.x;
     const int nparts = nchunks * rsplit;
@@ -347,31 +345,30 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
                 for (int v = 0; v < V; ++v) cs[v] += f[v];
             }
         }
-        if (RT > 1) {                           // sum over the row threads, fixed order
 #pragma unroll
-            for (int v = 0; v < V; ++v) s_cs[tid * V + v] = cs[v];
+        for (int v = 0; v < V; ++v) s_cs[tid * V + v] = cs[v];
+        if (RT > 1) {                           // sum over the row threads, ascending; all threads take columns
             __syncthreads();
-            if (rt == 0)
-                for (int q = 1; q < RT; ++q)
-#pragma unroll
-                    for (int v = 0; v < V; ++v) cs[v] += s_cs[(q * CT + ct) * V + v];
+            for (int cc = tid; cc < CT * V; cc += NT) {
+                float a = s_cs[cc];
+                for (int q = 1; q < RT; ++q) a += s_cs[q * CT * V + cc];
+                s_cs[cc] = a;                   // (read by this thread alone until the next barrier)
+            }
         }
     }
 
-    // ---- score_part[bj, part, :] = column sums . W_r rows, out of shared memory; thread (group g, expert i) strides
-    //      over the CTA's columns ----
-    if (rt == 0 && col < d) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) s_cs[ct * V + v] = cs[v];       // the slot this thread itself wrote above: no one else reads it
-    }
+    // ---- score_part[bj, part, :] = column sums . W_r rows, out of shared memory: a lane per expert (np2 lanes), the lane
+    //      groups stride over the CTA's columns; sums meet through shuffles, then over the warps (0.75 us; as one thread's
+    //      sum over the groups 1.4) ----
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     {
-        const int groups = NT / n;
-        const int i = tid % n, g = tid / n;
+        const int np2 = n > 1 ? 1 << (32 - __clz(n - 1)) : 1;
+        const int groups = NT / np2;
+        const int i = tid % np2, g = tid / np2;
         const T* s_w = (const T*)s_dyn4;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        if (g < groups) {           // four independent chains, then the tail: a fixed summation order
+        if (i < n) {                // four independent chains, then the tail: a fixed summation order
             int cc = g;
             for (; cc + 3 * groups < cw; cc += 4 * groups) {
                 a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
@@ -381,14 +378,15 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
             }
             for (; cc < cw; cc += groups) a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
         }
-        __syncthreads();
-        s_cs[tid] = (a0 + a1) + (a2 + a3);
+        float a = (a0 + a1) + (a2 + a3);
+        for (int o = np2; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((tid & 31) < n) s_dot[tid >> 5][tid & 31] = a;
         __syncthreads();
         if (tid < n) {
             float sum = 0.f;
-            for (int q = 0; q < groups; ++q) sum += s_cs[q * n + tid];
+#pragma unroll
+            for (int q = 0; q < NT / 32; ++q) sum += s_dot[q][tid];
             scores[((size_t)bj * nparts + part) * n + tid] = sum;
-            __threadfence();
         }
     }
     if constexpr (TICKET) {
@@ -396,11 +394,11 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
         if (tid == 0) {
             __threadfence();
             s_mine = (atomicAdd(&sample_ticket[b], 1) == m * nparts - 1);
+            __threadfence();
             if (s_mine) sample_ticket[b] = 0;         // left at zero for the next call
         }
         __syncthreads();
         if (!s_mine) return;
-        __threadfence();
         // ---- this CTA completed sample b ----
         select_sample<NT>((float*)s_dyn4, scores, nparts, b, B, Lv, n, k, m, c, l_p, use_gate, expert_idx, patch_idx, gate, p_samp,
                           p_patch, offsets, masks, ctl + 1, plan);
@@ -482,7 +480,16 @@ route_sample_kernel(const T* __restrict__ x, const T* __restrict__ W_r, int B, i
         if (p < m * n) {
             const int j = p / n, i = p % n;
             const float* pj = s_pool + (size_t)j * d;
-            for (int cc = sub; cc < d; cc += parts) acc = fmaf(pj[cc], to_f32(s_w[cc * n + i]), acc);
+            float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            int cc = sub;
+            for (; cc + 3 * parts < d; cc += 4 * parts) {       // four independent chains (one: 4.3 us instead of 1.6)
+                acc = fmaf(pj[cc], to_f32(s_w[cc * n + i]), acc);
+                a1 = fmaf(pj[cc + parts], to_f32(s_w[(cc + parts) * n + i]), a1);
+                a2 = fmaf(pj[cc + 2 * parts], to_f32(s_w[(cc + 2 * parts) * n + i]), a2);
+                a3 = fmaf(pj[cc + 3 * parts], to_f32(s_w[(cc + 3 * parts) * n + i]), a3);
+            }
+            for (; cc < d; cc += parts) acc = fmaf(pj[cc], to_f32(s_w[cc * n + i]), acc);
+            acc = (acc + a1) + (a2 + a3);
         }
         for (int o = parts >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (p < m * n && sub == 0) s_sc[p] = acc;
