@@ -470,29 +470,32 @@ route_sample_kernel(const T* __restrict__ x, const T* __restrict__ W_r, int B, i
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    // ---- scores[j, i] = pooled patch j . W_r[:, i]: `parts` threads per score, columns dealt round robin, summed by a
-    //      fixed shuffle tree ----
-    int parts = 1;
-    while (parts < 32 && 2 * parts * m * n <= NT) parts <<= 1;
-    for (int p0 = 0; p0 < m * n; p0 += NT / parts) {
-        const int p = p0 + tid / parts, sub = tid % parts;
-        float acc = 0.f;
-        if (p < m * n) {
-            const int j = p / n, i = p % n;
-            const float* pj = s_pool + (size_t)j * d;
-            float a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            int cc = sub;
-            for (; cc + 3 * parts < d; cc += 4 * parts) {       // four independent chains (one: 4.3 us instead of 1.6)
-                acc = fmaf(pj[cc], to_f32(s_w[cc * n + i]), acc);
-                a1 = fmaf(pj[cc + parts], to_f32(s_w[(cc + parts) * n + i]), a1);
-                a2 = fmaf(pj[cc + 2 * parts], to_f32(s_w[(cc + 2 * parts) * n + i]), a2);
-                a3 = fmaf(pj[cc + 3 * parts], to_f32(s_w[(cc + 3 * parts) * n + i]), a3);
+    // ---- scores[j, i] = pooled patch j . W_r[:, i]: a warp per patch, a lane per expert and column group (np2 lanes per
+    //      group), four columns at a time, summed by a fixed shuffle tree (a thread per score and column slice issued
+    //      about eight instructions per product: 4.5 us at 14 patches, 6 experts, 384 columns) ----
+    {
+        const int warp = tid >> 5, lane = tid & 31;
+        const int np2 = n > 1 ? 1 << (32 - __clz(n - 1)) : 1;
+        const int i = lane % np2, seg = lane / np2, segs = 32 / np2;
+        for (int j = warp; j < m; j += NT / 32) {
+            const float4* pj = (const float4*)(s_pool + (size_t)j * d);
+            float a0 = 0.f, a1 = 0.f;
+            if (i < n) {
+                const T* w = s_w + i;
+#pragma unroll 4
+                for (int c4 = seg; c4 < d / 4; c4 += segs) {
+                    const float4 p = pj[c4];
+                    const T* wc = w + c4 * 4 * n;
+                    a0 = fmaf(p.x, to_f32(wc[0]), a0);
+                    a1 = fmaf(p.y, to_f32(wc[n]), a1);
+                    a0 = fmaf(p.z, to_f32(wc[2 * n]), a0);
+                    a1 = fmaf(p.w, to_f32(wc[3 * n]), a1);
+                }
             }
-            for (; cc < d; cc += parts) acc = fmaf(pj[cc], to_f32(s_w[cc * n + i]), acc);
-            acc = (acc + a1) + (a2 + a3);
+            float acc = a0 + a1;
+            for (int o = np2; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane < n) s_sc[j * n + lane] = acc;
         }
-        for (int o = parts >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (p < m * n && sub == 0) s_sc[p] = acc;
     }
     __syncthreads();
     select_sample<NT>(s_pp, nullptr, 1, b, B, Lv, n, k, m, c, l_p, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch, offsets,
