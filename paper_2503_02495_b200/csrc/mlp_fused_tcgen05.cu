@@ -6,16 +6,18 @@
 // write it to shared memory as the bf16 A operand of GEMM2, whose [128 x d] result goes back to TMEM and out by
 // TMA stores.  One persistent CTA per SM walks the 128-row tiles (expert regions are padded to 128 rows).
 //   warp 0      TMA producer: per 64-wide K step of GEMM1 an A block [128 x 64] (from a routed buffer, or gathered
-//               from x with one box per source patch, Eq. 18) and a W1 block [64 x 256]; then per 64-row K step of
-//               GEMM2 a W2 block [64 x up to 256]; one three-stage ring serves both, so W2 and the next tile's
-//               operands are fetched while the epilogue works
-//   warp 1      MMA issuer: tcgen05.mma 128 x 256 x 16 into TMEM columns [0, 256) (hidden tile), then
-//               128 x N x 16 into [256, 512) (output columns 0-255) and, for d > 256, into [0, 256) again (the
-//               hidden tile has been consumed by then)
+//               from x with one box per source patch, Eq. 18) and a W1 block [64 x 256]; then W2 in blocks of [64 rows x
+//               128 columns], three to a stage; one three-stage ring serves both, so W2 and the next tile's operands are
+//               fetched while the epilogue works
+//   warp 1      MMA issuer: tcgen05.mma 128 x 256 x 16 into TMEM columns [0, 256) (hidden tile); the output in chunks of
+//               128 columns, alternately into [256, 384) and [384, 512)
 //   warps 2-9   epilogue, two warps per TMEM lane quarter sharing the 64-column groups: hidden tile -> (optional
-//               store of the pre-activation) -> phi -> bf16 -> swizzled K-major tile in shared memory; output tile
-//               -> bf16 -> [32 x 64] pieces staged in the same shared memory (GEMM2 has finished reading it) -> TMA
-//               tensor stores
+//               store of the pre-activation) -> phi -> bf16 -> swizzled K-major tile in shared memory, 64 columns at a time
+//               (GEMM2 starts on the first); output chunk -> bf16 -> [32 x 32] pieces staged per warp -> TMA tensor stores
+// Bound by the chain load -> GEMM1 -> phi -> GEMM2 -> stores of a tile and by the L2 reads of its operands (98 KB of A, 393 KB
+// of weights at d = 384, 144 KB in flight).  The chunks let the write-out of a tile run under its own GEMM2 and the next
+// GEMM1, and three W2 blocks to a stage keep the whole ring in flight; with the output in two halves drained behind the
+// last MMA a tile took 11.7 us at d = 384 (a launch of one tile per SM 16.4 at d = 512, 11.5 at d = 256).
 #include "kernels.cuh"
 #include "tc.cuh"
 #include "tmap.cuh"
@@ -33,10 +35,15 @@ constexpr int STAGES = 3;
 constexpr int HID_BYTES = BM * DE * 2;            // 64 KB: phi(h) as four [128 x 64] swizzled tiles
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr int SMEM = STAGES * STAGE + HID_BYTES + 1024 /*align slack*/ + 1024 /*control*/;
+constexpr int NC = 128;                           // output columns of a chunk
+constexpr int BLK_BYTES = BK * NC * 2;            // 16 KB: a W2 block [64 x 128]
+constexpr int BLKS = STAGE / BLK_BYTES;           // W2 blocks per stage
+constexpr int PIECE_BYTES = 32 * 32 * 2;          // an epilogue warp's staging piece [32 rows x 32 columns]
+constexpr int SMEM = STAGES * STAGE + HID_BYTES + EPI_WARPS * PIECE_BYTES + 1024 /*align slack*/ + 1024 /*control*/;
+static_assert(SMEM <= 232448, "shared memory of one SM");
 
 struct FCtl {
-    uint64_t full[STAGES], empty[STAGES], bar_h, bar_a, bar_z, bar_done;
+    uint64_t full[STAGES], empty[STAGES], bar_h, bar_a[DE / 64], bar_z[2], bar_free[2];
     uint32_t tmem_base;
     int abort_flag;
     int offs[34];
@@ -54,16 +61,16 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sHid = smem + STAGES * STAGE;
-    FCtl* ctl = (FCtl*)(sHid + HID_BYTES);
+    uint8_t* sOut = sHid + HID_BYTES;
+    FCtl* ctl = (FCtl*)(sOut + EPI_WARPS * PIECE_BYTES);
     volatile int* abort_flag = &ctl->abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         mbar_init(&ctl->bar_h, 1);
-        mbar_init(&ctl->bar_a, 32 * EPI_WARPS);
-        mbar_init(&ctl->bar_z, 1);
-        mbar_init(&ctl->bar_done, 32 * EPI_WARPS);
+        for (int g = 0; g < DE / 64; ++g) mbar_init(&ctl->bar_a[g], 32 * EPI_WARPS / 2);
+        for (int q = 0; q < 2; ++q) { mbar_init(&ctl->bar_z[q], 1); mbar_init(&ctl->bar_free[q], 32 * EPI_WARPS); }
         ctl->abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmA);
@@ -95,8 +102,9 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t tmem_base = ctl->tmem_base;
     const int total_tiles = ctl->tstart[n];
     const int kb1 = d / BK;                     // K steps of GEMM1
-    constexpr int kb2 = DE / BK;                // K steps of GEMM2 (per output half)
-    const int nh = d > 256 ? 2 : 1;             // output halves of up to 256 columns
+    constexpr int kb2 = DE / BK;                // K steps of GEMM2 (per output chunk)
+    const int nc = (d + NC - 1) / NC;           // output chunks; the last may be 64 columns wide
+    const int nblk = nc * kb2;                  // W2 blocks: block q is K step q % kb2 of chunk q / kb2
 
     auto locate = [&](int tile, int& e, int& row0) {
         e = 0;
@@ -149,15 +157,18 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     tma_load_3d(sb + (lane - 16) * 8192, &tmW1, (lane - 16) * 64, kb * BK, e, &ctl->full[stage]);
                 advance();
             }
-            for (int j = 0; j < nh && !stop; ++j) {
-                const int nbox = min(256, d - j * 256) / 64;
-                for (int kb = 0; kb < kb2; ++kb) {
-                    if (!acquire((uint32_t)nbox * 8192)) { stop = true; break; }
-                    uint8_t* sb = smem + stage * STAGE + A_BYTES;
-                    if (lane < nbox) tma_load_3d(sb + lane * 8192, &tmW2, j * 256 + lane * 64, kb * BK, e, &ctl->full[stage]);
-                    advance();
-                    if (!looked && j * kb2 + kb + 1 == STAGES) { look_up(tile + gridDim.x); looked = true; }
-                }
+            for (int q0 = 0; q0 < nblk && !stop; q0 += BLKS) {
+                const int cnt = min(BLKS, nblk - q0);
+                uint32_t boxes = 0;                       // 64-column boxes of the stage
+#pragma unroll
+                for (int u = 0; u < BLKS; ++u)
+                    if (u < cnt) boxes += (d - ((q0 + u) / kb2) * NC) >= NC ? 2 : 1;
+                if (!acquire(boxes * 8192)) { stop = true; break; }
+                const int q = q0 + lane / 2, col = (q / kb2) * NC + (lane & 1) * 64;
+                if (lane < 2 * cnt && col < d)
+                    tma_load_3d(smem + stage * STAGE + (lane / 2) * BLK_BYTES + (lane & 1) * 8192, &tmW2, col, (q % kb2) * BK, e, &ctl->full[stage]);
+                advance();
+                if (!looked && q0 + BLKS >= min(nblk, 2 * BLKS)) { look_up(tile + gridDim.x); looked = true; }
             }
             if (!looked) look_up(tile + gridDim.x);
         }
@@ -166,53 +177,53 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (issued & (1u << s)) mbar_wait(&ctl->full[s], (issued_parity >> s) & 1, abort_flag, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
-            constexpr uint32_t idesc_h = instr_desc_bf16(BM, DE, false, true);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool stop = false;
-            int i = 0;                                   // tiles done by this CTA
-            for (int tile = blockIdx.x; tile < total_tiles && !stop; tile += gridDim.x, ++i) {
-                // d > 256: the hidden tile shares its TMEM columns with the second output half of the previous tile
-                if (nh == 2 && i > 0 && (!mbar_wait(&ctl->bar_done, (i - 1) & 1, abort_flag, status) || *abort_flag)) break;
+        // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+        const uint32_t el = elect_one();
+        constexpr uint32_t idesc_h = instr_desc_bf16(BM, DE, false, true);
+        int stage = 0;
+        uint32_t phase = 0;
+        bool stop = false;
+        int i = 0;                                   // tiles done by this CTA
+        uint32_t used = 0;                           // bit b: parity of the chunks put into output accumulator b so far
+        for (int tile = blockIdx.x; tile < total_tiles && !stop; tile += gridDim.x, ++i) {
+            // (the hidden accumulator is free: this thread has waited for phi of the previous tile's last columns)
+            for (int kb = 0; kb < kb1; ++kb) {
+                if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
                 tc_fence_after();
-                for (int kb = 0; kb < kb1; ++kb) {
-                    if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
+                const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
+#pragma unroll
+                for (int ks = 0; ks < BK / 16; ++ks)
+                    mma_bf16_elect(el, tmem_base, smem_desc(sa + ks * 32, 16, 1024), smem_desc(sb + ks * 2048, 8192, 1024), idesc_h,
+                             (kb | ks) != 0);
+                mma_commit_elect(el, &ctl->empty[stage]);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            if (stop) break;
+            mma_commit_elect(el, &ctl->bar_h);
+            const uint32_t ha = smem_u32(sHid);
+            for (int q0 = 0; q0 < nblk && !stop; q0 += BLKS) {
+                if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
+#pragma unroll 1
+                for (int q = q0; q < min(nblk, q0 + BLKS); ++q) {
+                    const int j = q / kb2, kb = q % kb2, buf = j & 1;
+                    // phi of hidden columns [64 kb, 64 kb + 64) is in shared memory; the accumulator has been drained
+                    if (j == 0 && (!mbar_wait(&ctl->bar_a[kb], i & 1, abort_flag, status) || *abort_flag)) { stop = true; break; }
+                    if (kb == 0) {
+                        if (!mbar_wait(&ctl->bar_free[buf], ((used >> buf) & 1) ^ 1, abort_flag, status) || *abort_flag) { stop = true; break; }
+                        used ^= 1u << buf;
+                    }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
+                    const uint32_t idesc_z = instr_desc_bf16(BM, min(NC, d - j * NC), false, true);
+                    const uint32_t sb = smem_u32(smem + stage * STAGE) + (q - q0) * BLK_BYTES;
 #pragma unroll
                     for (int ks = 0; ks < BK / 16; ++ks)
-                        mma_bf16(tmem_base, smem_desc(sa + ks * 32, 16, 1024), smem_desc(sb + ks * 2048, 8192, 1024), idesc_h,
-                                 (kb | ks) != 0);
-                    mma_commit(&ctl->empty[stage]);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                        mma_bf16_elect(el, tmem_base + 256 + buf * NC, smem_desc(ha + kb * (BM * 128) + ks * 32, 16, 1024),
+                                 smem_desc(sb + ks * 2048, 8192, 1024), idesc_z, (kb | ks) != 0);
+                    if (kb == kb2 - 1) mma_commit_elect(el, &ctl->bar_z[buf]);
                 }
                 if (stop) break;
-                mma_commit(&ctl->bar_h);
-                // phi(h) is in shared memory; d <= 256: the output columns [256, 512) of the previous tile are drained
-                if (!mbar_wait(&ctl->bar_a, i & 1, abort_flag, status) || *abort_flag) break;
-                if (nh == 1 && i > 0 && (!mbar_wait(&ctl->bar_done, (i - 1) & 1, abort_flag, status) || *abort_flag)) break;
-                tc_fence_after();
-                const uint32_t ha = smem_u32(sHid);
-                for (int j = 0; j < nh && !stop; ++j) {
-                    const int ncols = min(256, d - j * 256);
-                    const uint32_t idesc_z = instr_desc_bf16(BM, ncols, false, true);
-                    const uint32_t d_tmem = tmem_base + (j == 0 ? 256 : 0);
-                    for (int kb = 0; kb < kb2; ++kb) {
-                        if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
-                        tc_fence_after();
-                        const uint32_t sb = smem_u32(smem + stage * STAGE) + A_BYTES;
-#pragma unroll
-                        for (int ks = 0; ks < BK / 16; ++ks)
-                            mma_bf16(d_tmem, smem_desc(ha + kb * (BM * 128) + ks * 32, 16, 1024),
-                                     smem_desc(sb + ks * 2048, 8192, 1024), idesc_z, (kb | ks) != 0);
-                        mma_commit(&ctl->empty[stage]);
-                        if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                    }
-                }
-                if (stop) break;
-                mma_commit(&ctl->bar_z);
+                mma_commit_elect(el, &ctl->empty[stage]);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
     } else {
@@ -221,7 +232,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int wsel = (warp - 2) >> 2;
         const int trow = quarter * 32 + lane;                 // row of the tile = TMEM lane
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        uint8_t* stg = sHid + (warp - 2) * 4096;              // this warp's [32 x 64] staging piece (output phase)
+        uint8_t* stg = sOut + (warp - 2) * PIECE_BYTES;
+        uint32_t taken = 0;                                   // bit b: parity of the chunks taken from output accumulator b
         auto pack8 = [](const float* f) {
             uint4 w;
             w.x = pack_bf16x2(f[0], f[1]); w.y = pack_bf16x2(f[2], f[3]);
@@ -232,9 +244,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++i) {
             int e, row0;
             locate(tile, e, row0);
-            bool ready = mbar_wait(&ctl->bar_h, i & 1, abort_flag, status) && !*abort_flag;
-            // every warp's output pieces of the previous tile have left shared memory
-            if (i > 0) ready = mbar_wait(&ctl->bar_done, (i - 1) & 1, abort_flag, status) && ready && !*abort_flag;
+            const bool ready = mbar_wait(&ctl->bar_h, i & 1, abort_flag, status) && !*abort_flag;
+            // (the hidden tile in shared memory is free: the last chunk of the previous tile was waited for below)
             if (!__all_sync(0xffffffffu, ready)) break;      // warp-uniform: tcgen05.ld below is warp-collective
             tc_fence_after();
             // ---- hidden tile: phi, bf16, K-major swizzled [128 x 64] tiles ----
@@ -266,46 +277,53 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     *(uint4*)(sHid + g * (BM * 128) + trow * 128 + ((c ^ (trow & 7)) << 4)) = pack8(f + 8 * c);
+                fence_async_smem();              // generic-proxy writes -> visible to the tensor core
+                tc_fence_before();
+                mbar_arrive(&ctl->bar_a[g]);
             }
-            fence_async_smem();                  // generic-proxy writes -> visible to the tensor core
-            tc_fence_before();
-            mbar_arrive(&ctl->bar_a);
 
-            // ---- output tile ----
-            const bool zr = mbar_wait(&ctl->bar_z, i & 1, abort_flag, status) && !*abort_flag;
-            if (!__all_sync(0xffffffffu, zr)) break;
-            tc_fence_after();
+            // ---- output chunks ----
             const int wrow0 = row0 + quarter * 32;
+            bool zr = true;
 #pragma unroll 1
-            for (int g = wsel; g < d / 64; g += 2) {
-                const uint32_t col = g < 4 ? 256 + g * 64 : (g - 4) * 64;
+            for (int j = 0; j < nc; ++j) {
+                const int buf = j & 1, col0 = j * NC + wsel * 64;
+                zr = __all_sync(0xffffffffu, mbar_wait(&ctl->bar_z[buf], (taken >> buf) & 1, abort_flag, status) && !*abort_flag);
+                taken ^= 1u << buf;
+                if (!zr) break;
+                tc_fence_after();
                 uint32_t v[64];
-                tmem_ld32(t_lane + col, v);
-                tmem_ld32(t_lane + col + 32, v + 32);
-                tmem_ld_wait();
-                if (lane == 0) bulk_wait_read();          // the previous store has finished reading the piece
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    float f[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) f[q] = __uint_as_float(v[8 * c + q]);
-                    if (b2) {                                // the expert's bias row of the second layer
-                        float bv[8];
-                        unpack16<__nv_bfloat16>(*(const uint4*)(b2 + (size_t)e * d + g * 64 + 8 * c), bv);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) f[q] += bv[q];
-                    }
-                    *(uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = pack8(f);
+                if (col0 < d) {                           // (uniform over the warp)
+                    tmem_ld32(t_lane + 256 + buf * NC + wsel * 64, v);
+                    tmem_ld32(t_lane + 256 + buf * NC + wsel * 64 + 32, v + 32);
+                    tmem_ld_wait();
                 }
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) { tma_store_2d(&tmZ, stg, g * 64, wrow0); bulk_commit(); }
+                tc_fence_before();
+                mbar_arrive(&ctl->bar_free[buf]);
+                if (col0 >= d) continue;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (lane == 0) bulk_wait_read();      // the previous store has finished reading the piece
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        float f[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) f[q] = __uint_as_float(v[32 * h + 8 * c + q]);
+                        if (b2) {                            // the expert's bias row of the second layer
+                            float bv[8];
+                            unpack16<__nv_bfloat16>(*(const uint4*)(b2 + (size_t)e * d + col0 + 32 * h + 8 * c), bv);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) f[q] += bv[q];
+                        }
+                        *(uint4*)(stg + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = pack8(f);      // 64-byte swizzle
+                    }
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) { tma_store_2d(&tmZ, stg, col0 + 32 * h, wrow0); bulk_commit(); }
+                }
             }
-            if (lane == 0) bulk_wait_read();              // the pieces may be overwritten by the next hidden tile
-            __syncwarp();
-            tc_fence_before();
-            mbar_arrive(&ctl->bar_done);
+            if (!zr) break;
         }
     }
     if (warp >= 2 && lane == 0) bulk_wait_all();       // this warp's tensor stores are complete
@@ -356,11 +374,11 @@ uoe_status launch_mlp_fused(const Dims& D, const void* A, const void* W1, const 
         if (!make_tmap(&tmW1, W1, 3, dims1, str1, box)) return UOE_ERR_CUDA;
         if (!make_tmap(&tmW2, W2, 3, dims2, str2, box)) return UOE_ERR_CUDA;
     }
-    {                     // z as [rows_max, d], written in [32 rows x 64 columns] pieces
+    {                     // z as [rows_max, d], written in [32 rows x 32 columns] pieces
         const uint64_t dims[2] = {(uint64_t)D.d, (uint64_t)D.Rmax};
         const uint64_t str[1] = {(uint64_t)D.d * 2};
-        const uint32_t box[2] = {64, 32};
-        if (!make_tmap(&tmZ, z, 2, dims, str, box)) return UOE_ERR_CUDA;
+        const uint32_t box[2] = {32, 32};
+        if (!make_tmap(&tmZ, z, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B)) return UOE_ERR_CUDA;
     }
     const long long max_tiles = D.Rmax / BM;
     int grid = (int)(max_tiles < sm_count() ? max_tiles : sm_count());

@@ -128,6 +128,30 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  :: "r"(smem_u32(bar)) : "memory");
 }
 
+// Issue by a whole warp: the warp runs its control flow and addresses convergently (so that they stay in uniform registers)
+// and only the instruction itself is predicated on one elected lane.  Issued from inside a one-lane branch, every MMA first
+// moves its descriptors from vector to uniform registers one by one, which takes longer than a 128 x 128 x 16 MMA runs.
+__device__ __forceinline__ uint32_t elect_one() {          // 1 in one lane of the (converged) warp, 0 in the others
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }     // known to be uniform
+__device__ __forceinline__ void mma_bf16_elect(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                               bool accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
+}
+__device__ __forceinline__ void mma_commit_elect(uint32_t elected, uint64_t* bar) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 :: "r"(smem_u32(bar)), "r"(elected) : "memory");
+}
+
 // 32 lanes x 32 columns of fp32: thread t of the warp receives lane (base lane + t), columns c..c+31.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
     asm volatile(
