@@ -64,6 +64,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     __shared__ int s_nvalid;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t el = elect_one();                       // MMAs: issued by one lane of the converged warp 0
     const int tile = blockIdx.x, head = blockIdx.y, pair = blockIdx.z;
 
     if (warp == 0) tmem_alloc(&ctl->tmem_base, 512);       // S [0,128), dP [128,256), accumulators [256,384)
@@ -133,20 +134,21 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const int st = it & 1, cur = first + it;
         const int q_tile = DQ ? tile : cur, k_tile = DQ ? cur : tile;
         // ---- S = Q K^T, dP = dO V^T ----
-        if (tid == 0) {
+        if (warp == 0) {
             if (it == 0) ok = mbar_wait(&ctl->bar_fix, 0, abort_flag, status);
             ok = mbar_wait(&ctl->bar_ld[st], (it >> 1) & 1, abort_flag, status) && ok;
+            __syncwarp();
             tc_fence_after();
             const uint32_t f0 = smem_u32(sF0), f1 = smem_u32(sF1);
             const uint32_t s0 = smem_u32(sS0 + st * TILE_BYTES), s1 = smem_u32(sS1 + st * TILE_BYTES);
             const uint32_t qa = DQ ? f0 : s0, ka = DQ ? s0 : f0, doa = DQ ? f1 : s1, va = DQ ? s1 : f1;
 #pragma unroll
             for (int ks = 0; ks < DH / 16; ++ks)
-                mma_bf16(tmem_base, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
+                mma_bf16(el, tmem_base, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
 #pragma unroll
             for (int ks = 0; ks < DH / 16; ++ks)
-                mma_bf16(tmem_base + 128, smem_desc(doa + ks * 32, 16, 1024), smem_desc(va + ks * 32, 16, 1024), idesc_s, ks != 0);
-            mma_commit(&ctl->bar_s);
+                mma_bf16(el, tmem_base + 128, smem_desc(doa + ks * 32, 16, 1024), smem_desc(va + ks * 32, 16, 1024), idesc_s, ks != 0);
+            mma_commit(el, &ctl->bar_s);
         }
         ok = mbar_wait(&ctl->bar_s, it & 1, abort_flag, status);
         if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
@@ -207,27 +209,27 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         __syncthreads();
 
         // ---- accumulate: dQ += dS K   |   dV += P^T dO, dK += dS^T Q ----
-        if (tid == 0) {
+        if (warp == 0) {
             tc_fence_after();
             const uint32_t ds = smem_u32(sDS);
             const uint32_t s0 = smem_u32(sS0 + st * TILE_BYTES), s1 = smem_u32(sS1 + st * TILE_BYTES);
             if (DQ) {
 #pragma unroll
                 for (int ks = 0; ks < T / 16; ++ks)
-                    mma_bf16(tmem_base + 256, smem_desc(ds + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
+                    mma_bf16(el, tmem_base + 256, smem_desc(ds + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
                              smem_desc(s0 + ks * 2048, 8192, 1024), idesc_q, (it | ks) != 0);
             } else {
                 const uint32_t pp = smem_u32(sP);
 #pragma unroll
                 for (int ks = 0; ks < T / 16; ++ks)       // contraction over the 128 query rows, 16 per step
-                    mma_bf16(tmem_base + 320, smem_desc(pp + ks * 2048, TILE_BYTES, 1024),
+                    mma_bf16(el, tmem_base + 320, smem_desc(pp + ks * 2048, TILE_BYTES, 1024),
                              smem_desc(s1 + ks * 2048, 8192, 1024), idesc_t, (it | ks) != 0);
 #pragma unroll
                 for (int ks = 0; ks < T / 16; ++ks)
-                    mma_bf16(tmem_base + 256, smem_desc(ds + ks * 2048, TILE_BYTES, 1024),
+                    mma_bf16(el, tmem_base + 256, smem_desc(ds + ks * 2048, TILE_BYTES, 1024),
                              smem_desc(s0 + ks * 2048, 8192, 1024), idesc_t, (it | ks) != 0);
             }
-            if (it == n_it - 1) mma_commit(&ctl->bar_o);
+            if (it == n_it - 1) mma_commit(el, &ctl->bar_o);
         }
     }
 

@@ -216,76 +216,79 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         }
     } else if (role == 2) {
         // =========================== MMA warp ===========================
-        if (lane == 0) {
-            constexpr uint32_t idesc_s = instr_desc_bf16(TQ, TK, false, false);
-            constexpr uint32_t idesc_o = instr_desc_bf16(TQ, DH, false, true);
-            uint32_t q_cnt = 0, kv_cnt = 0, acc_cnt = 0, p_cnt = 0, ready_cnt = 0;
-            bool ok = true;
-            int qt, head, pair;
-            for (int round = 0; ok && unit_at(round, qt, head, pair); ++round) {
-                ok = wait1(&pc->q_full, q_cnt & 1);
-                ++q_cnt;
-                if (!ok) break;
-                const int n_kv = kv_tiles(qt * TQ, pc->n_valid);
-                if (t_first >= n_kv) { mbar_arrive(&pc->q_empty); continue; }
+        const uint32_t el = elect_one();
+        auto waitw = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait1(bar, parity)) != 0; };
+        constexpr uint32_t idesc_s = instr_desc_bf16(TQ, TK, false, false);
+        constexpr uint32_t idesc_o = instr_desc_bf16(TQ, DH, false, true);
+        uint32_t q_cnt = 0, kv_cnt = 0, acc_cnt = 0, p_cnt = 0, ready_cnt = 0;
+        bool ok = true;
+        int qt, head, pair;
+        for (int round = 0; ok && unit_at(round, qt, head, pair); ++round) {
+            ok = waitw(&pc->q_full, q_cnt & 1);
+            ++q_cnt;
+            if (!ok) break;
+            const int n_kv = kv_tiles(qt * TQ, pc->n_valid);
+            if (t_first >= n_kv) {
+                if (el) mbar_arrive(&pc->q_empty);
+                continue;
+            }
+            tc_fence_after();
+            const uint32_t qa = smem_u32(sQ), pa = smem_u32(sP);
+            // S of a key tile is issued as soon as its K has landed and the softmax warps have taken the previous S out
+            // of the accumulator -- ahead of the previous tile's P V, which has to wait for P -- so the next S is
+            // ready when the softmax warps come back for it
+            auto issue_s = [&](uint32_t stage_cnt, bool last) {
+                const int st = stage_cnt & 1;
+                if (!(waitw(&pc->kv_full[st], (stage_cnt >> 1) & 1) && waitw(&pc->acc_empty, (acc_cnt & 1) ^ 1))) return false;
                 tc_fence_after();
-                const uint32_t qa = smem_u32(sQ), pa = smem_u32(sP);
-                // S of a key tile is issued as soon as its K has landed and the softmax warps have taken the previous S out
-                // of the accumulator -- ahead of the previous tile's P V, which has to wait for P -- so the next S is
-                // ready when the softmax warps come back for it
-                auto issue_s = [&](uint32_t stage_cnt, bool last) {
-                    const int st = stage_cnt & 1;
-                    if (!(wait1(&pc->kv_full[st], (stage_cnt >> 1) & 1) && wait1(&pc->acc_empty, (acc_cnt & 1) ^ 1))) return false;
-                    tc_fence_after();
-                    const uint32_t ka = smem_u32(sKV + st * 2 * TILE_BYTES);
+                const uint32_t ka = smem_u32(sKV + st * 2 * TILE_BYTES);
 #pragma unroll
-                    for (int ks = 0; ks < DH / 16; ++ks)
-                        mma_bf16(tmem_pipe, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
-                    mma_commit(&pc->acc_full);
-                    ++acc_cnt;
-                    if (last) mma_commit(&pc->q_empty);       // the unit's last use of Q
-                    return true;
-                };
-                ok = issue_s(kv_cnt, t_first + t_step >= n_kv);
-                for (int t = t_first; t < n_kv && ok; t += t_step) {
+                for (int ks = 0; ks < DH / 16; ++ks)
+                    mma_bf16(el, tmem_pipe, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
+                mma_commit(el, &pc->acc_full);
+                ++acc_cnt;
+                if (last) mma_commit(el, &pc->q_empty);       // the unit's last use of Q
+                return true;
+            };
+            ok = issue_s(kv_cnt, t_first + t_step >= n_kv);
+            for (int t = t_first; t < n_kv && ok; t += t_step) {
+                const int st = kv_cnt & 1;
+                if (t + t_step < n_kv) {
+                    ok = issue_s(kv_cnt + 1, t + 2 * t_step >= n_kv);
+                    if (!ok) break;
+                }
+                ok = waitw(&pc->p_full, p_cnt & 1);
+                ++p_cnt;
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t va = smem_u32(sKV + st * 2 * TILE_BYTES) + TILE_BYTES;
+#pragma unroll
+                for (int ks = 0; ks < TK / 16; ++ks)
+                    mma_bf16(el, tmem_pipe + 128, smem_desc(pa + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
+                             smem_desc(va + ks * 2048, 8192, 1024), idesc_o, ks != 0);
+                mma_commit(el, &pc->o_full);
+                mma_commit(el, &pc->kv_empty[st]);
+                ++kv_cnt;
+            }
+            if (FUSE_O && ok) {
+                // z = o W^o_i (Eq. 35): the o tile sits where P was, chunk by chunk into the S accumulator
+                ok = waitw(&pc->o_ready, ready_cnt & 1);
+                ++ready_cnt;
+                for (int zc = 0; zc < n_zchunk && ok; ++zc) {
+                    const int nn = min(ZCHUNK, a.d - zc * ZCHUNK);
                     const int st = kv_cnt & 1;
-                    if (t + t_step < n_kv) {
-                        ok = issue_s(kv_cnt + 1, t + 2 * t_step >= n_kv);
-                        if (!ok) break;
-                    }
-                    ok = wait1(&pc->p_full, p_cnt & 1);
-                    ++p_cnt;
+                    ok = waitw(&pc->kv_full[st], (kv_cnt >> 1) & 1) && waitw(&pc->acc_empty, (acc_cnt & 1) ^ 1);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t va = smem_u32(sKV + st * 2 * TILE_BYTES) + TILE_BYTES;
+                    const uint32_t wa = smem_u32(sKV + st * 2 * TILE_BYTES);
+                    const uint32_t idesc_z = instr_desc_bf16(TQ, nn, false, true);
 #pragma unroll
-                    for (int ks = 0; ks < TK / 16; ++ks)
-                        mma_bf16(tmem_pipe + 128, smem_desc(pa + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
-                                 smem_desc(va + ks * 2048, 8192, 1024), idesc_o, ks != 0);
-                    mma_commit(&pc->o_full);
-                    mma_commit(&pc->kv_empty[st]);
+                    for (int ks = 0; ks < DH / 16; ++ks)
+                        mma_bf16(el, tmem_pipe, smem_desc(pa + ks * 32, 16, 1024), smem_desc(wa + ks * 2048, 8192, 1024), idesc_z, ks != 0);
+                    mma_commit(el, &pc->acc_full);
+                    mma_commit(el, &pc->kv_empty[st]);
+                    ++acc_cnt;
                     ++kv_cnt;
-                }
-                if (FUSE_O && ok) {
-                    // z = o W^o_i (Eq. 35): the o tile sits where P was, chunk by chunk into the S accumulator
-                    ok = wait1(&pc->o_ready, ready_cnt & 1);
-                    ++ready_cnt;
-                    for (int zc = 0; zc < n_zchunk && ok; ++zc) {
-                        const int nn = min(ZCHUNK, a.d - zc * ZCHUNK);
-                        const int st = kv_cnt & 1;
-                        ok = wait1(&pc->kv_full[st], (kv_cnt >> 1) & 1) && wait1(&pc->acc_empty, (acc_cnt & 1) ^ 1);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t wa = smem_u32(sKV + st * 2 * TILE_BYTES);
-                        const uint32_t idesc_z = instr_desc_bf16(TQ, nn, false, true);
-#pragma unroll
-                        for (int ks = 0; ks < DH / 16; ++ks)
-                            mma_bf16(tmem_pipe, smem_desc(pa + ks * 32, 16, 1024), smem_desc(wa + ks * 2048, 8192, 1024), idesc_z, ks != 0);
-                        mma_commit(&pc->acc_full);
-                        mma_commit(&pc->kv_empty[st]);
-                        ++acc_cnt;
-                        ++kv_cnt;
-                    }
                 }
             }
         }
@@ -523,6 +526,7 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int qt = blockIdx.x, head = blockIdx.y, pair = blockIdx.z;
     const int q0 = qt * TQ;
+    const uint32_t el = elect_one();                       // MMAs: issued by one lane of the converged warp 0
 
     if (warp == 0) tmem_alloc(&ctl->tmem_base, 512);       // S: two buffers, columns [0,128) and [128,256); O_t: [256,320)
     pdl_wait();                                             // from here on: data written by earlier kernels
@@ -588,15 +592,16 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     for (int it = 0; it < n_kv; ++it) {
         const int st = it & 1;
         // ---- S = Q K^T (issued here for the first tile only; later tiles are issued behind the previous P V) ----
-        if (tid == 0 && it == 0) {
+        if (warp == 0 && it == 0) {
             ok = mbar_wait(&ctl->bar_q, 0, abort_flag, status);
             ok = mbar_wait(&ctl->bar_kv[0], 0, abort_flag, status) && ok;
+            __syncwarp();
             tc_fence_after();
             const uint32_t qa = smem_u32(sQ), ka = smem_u32(sK);
 #pragma unroll
             for (int ks = 0; ks < DH / 16; ++ks)
-                mma_bf16(tmem_base, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
-            mma_commit(&ctl->bar_s);
+                mma_bf16(el, tmem_base, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s, ks != 0);
+            mma_commit(el, &ctl->bar_s);
         }
         ok = mbar_wait(&ctl->bar_s, it & 1, abort_flag, status);
         if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
@@ -653,24 +658,25 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         __syncthreads();
 
         // ---- O_t = P V, and behind it S of the next tile into the other S buffer (it runs under the O update) ----
-        if (tid == 0) {
+        if (warp == 0) {
             tc_fence_after();
             const uint32_t pa = smem_u32(sP), va = smem_u32(sV + st * TILE_BYTES);
 #pragma unroll
             for (int ks = 0; ks < TK / 16; ++ks)
-                mma_bf16(tmem_base + 256, smem_desc(pa + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
+                mma_bf16(el, tmem_base + 256, smem_desc(pa + (ks >> 2) * TILE_BYTES + (ks & 3) * 32, 16, 1024),
                          smem_desc(va + ks * 2048, 8192, 1024), idesc_o, ks != 0);
-            mma_commit(&ctl->bar_o);
+            mma_commit(el, &ctl->bar_o);
             if (it + 1 < n_kv) {
                 const int ns = (it + 1) & 1;
                 ok = mbar_wait(&ctl->bar_kv[ns], ((it + 1) >> 1) & 1, abort_flag, status) && ok;
+                __syncwarp();
                 tc_fence_after();
                 const uint32_t qa = smem_u32(sQ), ka = smem_u32(sK + ns * TILE_BYTES);
 #pragma unroll
                 for (int ks = 0; ks < DH / 16; ++ks)
-                    mma_bf16(tmem_base + ns * 128, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s,
+                    mma_bf16(el, tmem_base + ns * 128, smem_desc(qa + ks * 32, 16, 1024), smem_desc(ka + ks * 32, 16, 1024), idesc_s,
                              ks != 0);
-                mma_commit(&ctl->bar_s);
+                mma_commit(el, &ctl->bar_s);
             }
         }
         ok = mbar_wait(&ctl->bar_o, it & 1, abort_flag, status);
@@ -726,8 +732,9 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0 && !*abort_flag) {
+        if (warp == 0 && !*abort_flag) {
             ok = mbar_wait(&ctl->bar_w, 0, abort_flag, status);
+            __syncwarp();
             tc_fence_after();
             const uint32_t oa = smem_u32(sQ), wa = smem_u32(sW);
             for (int n0 = 0; n0 < d; n0 += 256) {            // up to 256 output columns per MMA
@@ -735,10 +742,10 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 const uint32_t idesc_z = instr_desc_bf16(TQ, nn, false, true);
 #pragma unroll
                 for (int ks = 0; ks < DH / 16; ++ks)
-                    mma_bf16(tmem_base + n0, smem_desc(oa + ks * 32, 16, 1024), smem_desc(wa + (n0 / 64) * 8192 + ks * 2048, 8192, 1024),
+                    mma_bf16(el, tmem_base + n0, smem_desc(oa + ks * 32, 16, 1024), smem_desc(wa + (n0 / 64) * 8192 + ks * 2048, 8192, 1024),
                              idesc_z, ks != 0);
             }
-            mma_commit(&ctl->bar_z);
+            mma_commit(el, &ctl->bar_z);
         }
         ok = mbar_wait(&ctl->bar_z, 0, abort_flag, status);
         if (__all_sync(0xffffffffu, ok && !*abort_flag)) {

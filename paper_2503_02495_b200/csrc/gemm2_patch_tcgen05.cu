@@ -151,39 +151,40 @@ gemm2_patch_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 if (issued & (1u << s)) mbar_wait(&ctl->full[s], (issued_parity >> s) & 1, abort_flag, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
-            constexpr uint32_t idesc = instr_desc_bf16(BM, BN, false, !B_KMAJOR);
-            int stage = 0, acc = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool stop = false;
-            int slot = 0;
-            uint32_t sphase = 0;
-            while (!stop) {
-                const int tile = next_tile(slot, sphase);
-                if (tile >= total_tiles) break;
-                const int p = tile / n_tiles;
-                int cnt = 0;
-                for (int s = 0; s < k; ++s) cnt += inv_row[(size_t)p * k + s] >= 0 ? 1 : 0;
-                if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
+        // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+        const uint32_t el = elect_one();
+        constexpr uint32_t idesc = instr_desc_bf16(BM, BN, false, !B_KMAJOR);
+        int stage = 0, acc = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        bool stop = false;
+        int slot = 0;
+        uint32_t sphase = 0;
+        while (!stop) {
+            int tile = 0;
+            if (lane == 0) tile = next_tile(slot, sphase);
+            tile = __shfl_sync(0xffffffffu, tile, 0);
+            if (tile >= total_tiles) break;
+            const int p = tile / n_tiles;
+            int cnt = 0;
+            for (int s = 0; s < k; ++s) cnt += inv_row[(size_t)p * k + s] >= 0 ? 1 : 0;
+            if (!mbar_wait_warp(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + acc * BN;
+            const int steps = cnt * kb_per;
+            for (int i = 0; i < steps; ++i) {
+                if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * BN;
-                const int steps = cnt * kb_per;
-                for (int i = 0; i < steps; ++i) {
-                    if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
-                    tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
+                const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
 #pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks)
-                        mma_bf16(d_tmem, smem_desc(sa + ks * 32, 16, 1024),
-                                 B_KMAJOR ? smem_desc(sb + ks * 32, 16, 1024) : smem_desc(sb + ks * 2048, 8192, 1024), idesc, (i | ks) != 0);
-                    mma_commit(&ctl->empty[stage]);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                }
-                if (stop) break;
-                mma_commit(&ctl->tfull[acc]);          // (no MMA issued for a patch nobody selected: arrives at once)
-                if (++acc == 2) { acc = 0; acc_phase ^= 1; }
+                for (int ks = 0; ks < BK / 16; ++ks)
+                    mma_bf16(el, d_tmem, smem_desc(sa + ks * 32, 16, 1024),
+                             B_KMAJOR ? smem_desc(sb + ks * 32, 16, 1024) : smem_desc(sb + ks * 2048, 8192, 1024), idesc, (i | ks) != 0);
+                mma_commit(el, &ctl->empty[stage]);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
+            if (stop) break;
+            mma_commit(el, &ctl->tfull[acc]);          // (no MMA issued for a patch nobody selected: arrives at once)
+            if (++acc == 2) { acc = 0; acc_phase ^= 1; }
         }
     } else {
         // ---------------- epilogue ----------------

@@ -245,8 +245,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (issued & (1u << s)) mbar_wait(&ctl->full[s], (issued_parity >> s) & 1, abort_flag, status);
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
-            // ---------------- MMA issuer ----------------
+        if (rank == 0) {
+            // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+            const uint32_t el = elect_one();
             constexpr uint32_t idesc = instr_desc_bf16(PAIR ? 2 * BM : BM, BN, false, !B_KMAJOR);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
@@ -255,11 +256,11 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int tile = worker; tile < total_tiles && !stop; tile += workers) {
                 int row0, blocks;
                 locate(tile / n_tiles, e, row0, blocks);
-                if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
+                if (!mbar_wait_warp(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * Cf::ACC_STRIDE;        // MT=2: acc is always 0, block h at column h*BN
                 for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
+                    if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                     tc_fence_after();
 #pragma unroll
                     for (int ks = 0; ks < Cf::KSUB * (BK / 16); ++ks) {
@@ -269,22 +270,22 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const uint64_t bd = B_KMAJOR ? smem_desc(sb + kq * 32, 16, 1024)
                                                      : smem_desc(sb + kq * 2048, 8192, 1024);
                         if constexpr (PAIR) {
-                            mma_bf16_pair(d_tmem, smem_desc(sa + kq * 32, 16, 1024), bd, idesc, (kb | ks) != 0);
+                            mma_bf16_pair(el, d_tmem, smem_desc(sa + kq * 32, 16, 1024), bd, idesc, (kb | ks) != 0);
                         } else {
 #pragma unroll
                             for (int h = 0; h < MT; ++h)
                                 if (h < blocks)
-                                    mma_bf16(d_tmem + h * BN, smem_desc(sa + h * A_BLOCK_BYTES + kq * 32, 16, 1024), bd, idesc,
+                                    mma_bf16(el, d_tmem + h * BN, smem_desc(sa + h * A_BLOCK_BYTES + kq * 32, 16, 1024), bd, idesc,
                                              (kb | ks) != 0);
                         }
                     }
-                    if constexpr (PAIR) mma_commit_pair(&ctl->empty[stage]);       // frees the stage in both CTAs
-                    else mma_commit(&ctl->empty[stage]);
+                    if constexpr (PAIR) mma_commit_pair(el, &ctl->empty[stage]);       // frees the stage in both CTAs
+                    else mma_commit(el, &ctl->empty[stage]);
                     if (++stage == Cf::STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (stop) break;
-                if constexpr (PAIR) mma_commit_pair(&ctl->tfull[acc]);
-                else mma_commit(&ctl->tfull[acc]);
+                if constexpr (PAIR) mma_commit_pair(el, &ctl->tfull[acc]);
+                else mma_commit(el, &ctl->tfull[acc]);
                 if (++acc == Cf::NACC) { acc = 0; acc_phase ^= 1; }
             }
         }

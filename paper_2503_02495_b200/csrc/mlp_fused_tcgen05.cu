@@ -64,7 +64,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     uint8_t* sOut = sHid + HID_BYTES;
     FCtl* ctl = (FCtl*)(sOut + EPI_WARPS * PIECE_BYTES);
     volatile int* abort_flag = &ctl->abort_flag;
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
@@ -188,28 +188,28 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int tile = blockIdx.x; tile < total_tiles && !stop; tile += gridDim.x, ++i) {
             // (the hidden accumulator is free: this thread has waited for phi of the previous tile's last columns)
             for (int kb = 0; kb < kb1; ++kb) {
-                if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
+                if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
 #pragma unroll
                 for (int ks = 0; ks < BK / 16; ++ks)
-                    mma_bf16_elect(el, tmem_base, smem_desc(sa + ks * 32, 16, 1024), smem_desc(sb + ks * 2048, 8192, 1024), idesc_h,
+                    mma_bf16(el, tmem_base, smem_desc(sa + ks * 32, 16, 1024), smem_desc(sb + ks * 2048, 8192, 1024), idesc_h,
                              (kb | ks) != 0);
-                mma_commit_elect(el, &ctl->empty[stage]);
+                mma_commit(el, &ctl->empty[stage]);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
             if (stop) break;
-            mma_commit_elect(el, &ctl->bar_h);
+            mma_commit(el, &ctl->bar_h);
             const uint32_t ha = smem_u32(sHid);
             for (int q0 = 0; q0 < nblk && !stop; q0 += BLKS) {
-                if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
+                if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
 #pragma unroll 1
                 for (int q = q0; q < min(nblk, q0 + BLKS); ++q) {
                     const int j = q / kb2, kb = q % kb2, buf = j & 1;
                     // phi of hidden columns [64 kb, 64 kb + 64) is in shared memory; the accumulator has been drained
-                    if (j == 0 && (!mbar_wait(&ctl->bar_a[kb], i & 1, abort_flag, status) || *abort_flag)) { stop = true; break; }
+                    if (j == 0 && !mbar_wait_warp(&ctl->bar_a[kb], i & 1, abort_flag, status)) { stop = true; break; }
                     if (kb == 0) {
-                        if (!mbar_wait(&ctl->bar_free[buf], ((used >> buf) & 1) ^ 1, abort_flag, status) || *abort_flag) { stop = true; break; }
+                        if (!mbar_wait_warp(&ctl->bar_free[buf], ((used >> buf) & 1) ^ 1, abort_flag, status)) { stop = true; break; }
                         used ^= 1u << buf;
                     }
                     tc_fence_after();
@@ -217,12 +217,12 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     const uint32_t sb = smem_u32(smem + stage * STAGE) + (q - q0) * BLK_BYTES;
 #pragma unroll
                     for (int ks = 0; ks < BK / 16; ++ks)
-                        mma_bf16_elect(el, tmem_base + 256 + buf * NC, smem_desc(ha + kb * (BM * 128) + ks * 32, 16, 1024),
+                        mma_bf16(el, tmem_base + 256 + buf * NC, smem_desc(ha + kb * (BM * 128) + ks * 32, 16, 1024),
                                  smem_desc(sb + ks * 2048, 8192, 1024), idesc_z, (kb | ks) != 0);
-                    if (kb == kb2 - 1) mma_commit_elect(el, &ctl->bar_z[buf]);
+                    if (kb == kb2 - 1) mma_commit(el, &ctl->bar_z[buf]);
                 }
                 if (stop) break;
-                mma_commit_elect(el, &ctl->empty[stage]);
+                mma_commit(el, &ctl->empty[stage]);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }

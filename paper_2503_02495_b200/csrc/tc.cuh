@@ -71,6 +71,12 @@ __device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity, v
     return mbar_wait(bar, parity, abort_flag, status);
 }
 
+// The same for a whole warp: true in every lane, or false in every lane (a wait ran out, or the CTA is winding down).  No
+// lane runs ahead of another's wait, so none can miss a phase.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status) && !*abort_flag);
+}
+
 // ---- TMA --------------------------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" :: "l"(m) : "memory");
@@ -114,20 +120,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
-}
-// The mbarrier gets one arrival when all MMAs issued so far by this thread have completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 :: "r"(smem_u32(bar)) : "memory");
-}
-
 // Issue by a whole warp: the warp runs its control flow and addresses convergently (so that they stay in uniform registers)
 // and only the instruction itself is predicated on one elected lane.  Issued from inside a one-lane branch, every MMA first
 // moves its descriptors from vector to uniform registers one by one, which takes longer than a 128 x 128 x 16 MMA runs.
@@ -136,9 +128,9 @@ __device__ __forceinline__ uint32_t elect_one() {          // 1 in one lane of t
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }     // known to be uniform
-__device__ __forceinline__ void mma_bf16_elect(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                               bool accumulate) {
+// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate
+__device__ __forceinline__ void mma_bf16(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         bool accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
@@ -146,7 +138,8 @@ __device__ __forceinline__ void mma_bf16_elect(uint32_t elected, uint32_t d_tmem
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
-__device__ __forceinline__ void mma_commit_elect(uint32_t elected, uint64_t* bar) {
+// The mbarrier gets one arrival when all MMAs issued so far by the elected lane have completed.
+__device__ __forceinline__ void mma_commit(uint32_t elected, uint64_t* bar) {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
                  "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
                  :: "r"(smem_u32(bar)), "r"(elected) : "memory");
@@ -214,20 +207,23 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t* slot_in_smem, uint32_t
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(taddr), "r"(ncols) : "memory");
 }
-__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
+__device__ __forceinline__ void mma_bf16_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              bool accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
-// one arrival on the barrier at this offset in each CTA of the pair when all MMAs issued so far by this thread have
+// one arrival on the barrier at this offset in each CTA of the pair when all MMAs issued so far by the elected lane have
 // completed (two commits, one per CTA: the second names the other CTA's barrier by its cluster address)
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 :: "r"(map_to_cta(bar, 0)) : "memory");
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 :: "r"(map_to_cta(bar, 1)) : "memory");
+__device__ __forceinline__ void mma_commit_pair(uint32_t elected, uint64_t* bar) {
+#pragma unroll
+    for (uint32_t r = 0; r < 2; ++r)
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                     :: "r"(map_to_cta(bar, r)), "r"(elected) : "memory");
 }
 
 // ---- descriptors ------------------------------------------------------------------------------

@@ -150,45 +150,44 @@ wgrad_stream_kernel(const __grid_constant__ WArgs a) {
                 if (issued & (1u << s)) mbar_wait(&ctl->full[s], (issued_parity >> s) & 1, abort_flag, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
-            int stage = 0, acc = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool stop = false;
-            WFrag f;
-            for (int pos = c * sc.Q; !stop && wsched_next(sc, a.prob, c, pos, f);) {
-                const WProblem& pr = a.prob[f.p];
-                const WOperand &op = a.p[f.p], &oq = a.q[f.p];
-                const uint32_t idesc = instr_desc_bf16(BM, f.cols, true, true);
-                // strides of a K-block's slabs: rows of a slab are consecutive, column blocks a slab's size apart; with
-                // eight-row slabs the second eight rows of a K step lie in the next slab
-                const int subp = op.gather ? op.sub : BK, subq = oq.gather ? oq.sub : BK, nbq = pr.BN / 64;
-                const uint32_t lbo_p = subp * 128, sbo_p = subp == 8 ? 2048 : 1024;
-                const uint32_t lbo_q = subq * 128, sbo_q = subq == 8 ? nbq * 1024 : 1024;
-                uint32_t po[BK / 16], qo[BK / 16];
+        // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
+        const uint32_t el = elect_one();
+        int stage = 0, acc = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        bool stop = false;
+        WFrag f;
+        for (int pos = c * sc.Q; !stop && wsched_next(sc, a.prob, c, pos, f);) {
+            const WProblem& pr = a.prob[f.p];
+            const WOperand &op = a.p[f.p], &oq = a.q[f.p];
+            const uint32_t idesc = instr_desc_bf16(BM, f.cols, true, true);
+            // strides of a K-block's slabs: rows of a slab are consecutive, column blocks a slab's size apart; with
+            // eight-row slabs the second eight rows of a K step lie in the next slab
+            const int subp = op.gather ? op.sub : BK, subq = oq.gather ? oq.sub : BK, nbq = pr.BN / 64;
+            const uint32_t lbo_p = subp * 128, sbo_p = subp == 8 ? 2048 : 1024;
+            const uint32_t lbo_q = subq * 128, sbo_q = subq == 8 ? nbq * 1024 : 1024;
+            uint32_t po[BK / 16], qo[BK / 16];
 #pragma unroll
-                for (int ks = 0; ks < BK / 16; ++ks) {
-                    po[ks] = (16 * ks / subp) * (subp * 256) + (16 * ks % subp) * 128;
-                    qo[ks] = (16 * ks / subq) * (subq * 128 * nbq) + (16 * ks % subq) * 128;
-                }
-                if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * BN_MAX;
-                for (int kb = f.kb_lo; kb < f.kb_hi; ++kb) {
-                    if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
-                    tc_fence_after();
-                    const uint32_t sp = smem_u32(smem + stage * STAGE), sq = sp + P_BYTES;
-#pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks)
-                        mma_bf16(d_tmem, smem_desc(sp + po[ks], lbo_p, sbo_p), smem_desc(sq + qo[ks], lbo_q, sbo_q), idesc,
-                                 kb > f.kb_lo || ks > 0);
-                    mma_commit(&ctl->empty[stage]);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
-                }
-                if (stop) break;
-                mma_commit(&ctl->tfull[acc]);
-                if (++acc == 2) { acc = 0; acc_phase ^= 1; }
+            for (int ks = 0; ks < BK / 16; ++ks) {
+                po[ks] = (16 * ks / subp) * (subp * 256) + (16 * ks % subp) * 128;
+                qo[ks] = (16 * ks / subq) * (subq * 128 * nbq) + (16 * ks % subq) * 128;
             }
+            if (!mbar_wait_warp(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + acc * BN_MAX;
+            for (int kb = f.kb_lo; kb < f.kb_hi; ++kb) {
+                if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
+                tc_fence_after();
+                const uint32_t sp = smem_u32(smem + stage * STAGE), sq = sp + P_BYTES;
+#pragma unroll
+                for (int ks = 0; ks < BK / 16; ++ks)
+                    mma_bf16(el, d_tmem, smem_desc(sp + po[ks], lbo_p, sbo_p), smem_desc(sq + qo[ks], lbo_q, sbo_q), idesc,
+                             kb > f.kb_lo || ks > 0);
+                mma_commit(el, &ctl->empty[stage]);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            if (stop) break;
+            mma_commit(el, &ctl->tfull[acc]);
+            if (++acc == 2) { acc = 0; acc_phase ^= 1; }
         }
     } else {
         // ---------------- write-out ----------------

@@ -205,41 +205,43 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
                 if (issued & (1u << s)) mbar_wait(&ctl->full[s], (issued_parity >> s) & 1, abort_flag, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc_bf16(BM, BN, true, true);
-            int stage = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool stop = false;
-            int slot = 0;
-            uint32_t sphase = 0;
-            while (!stop) {
-                const int tile = next_tile(slot, sphase);
-                if (tile >= total_tiles) break;
-                int e, m0, n0, num_kb;
-                decode(tile, e, m0, n0, num_kb);
-                if (!mbar_wait(&ctl->tempty, acc_phase ^ 1, abort_flag, status) || *abort_flag) break;
+        // MMA issuer: the whole warp, one elected lane issues
+        const uint32_t el = elect_one();
+        constexpr uint32_t idesc = instr_desc_bf16(BM, BN, true, true);
+        int stage = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        bool stop = false;
+        int slot = 0;
+        uint32_t sphase = 0;
+        while (!stop) {
+            int tile = 0;
+            if (lane == 0) tile = next_tile(slot, sphase);
+            tile = __shfl_sync(0xffffffffu, tile, 0);
+            if (tile >= total_tiles) break;
+            int e, m0, n0, num_kb;
+            decode(tile, e, m0, n0, num_kb);
+            if (!mbar_wait_warp(&ctl->tempty, acc_phase ^ 1, abort_flag, status)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base;
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base;
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!mbar_wait(&ctl->full[stage], phase, abort_flag, status) || *abort_flag) { stop = true; break; }
-                    tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + stage * Cf::STAGE);
-                    const uint32_t sb = sa + Cf::A_BYTES;
+                const uint32_t sa = smem_u32(smem + stage * Cf::STAGE);
+                const uint32_t sb = sa + Cf::A_BYTES;
 #pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks) {
-                        const uint64_t bd = smem_desc(sb + ks * 2048, 8192, 1024);
+                for (int ks = 0; ks < BK / 16; ++ks) {
+                    const uint64_t bd = smem_desc(sb + ks * 2048, 8192, 1024);
 #pragma unroll
-                        for (int h = 0; h < MT; ++h)
-                            mma_bf16(d_tmem + h * BN, smem_desc(sa + h * A_BLOCK_BYTES + ks * 2048, 8192, 1024), bd, idesc,
-                                     (kb | ks) != 0);
-                    }
-                    mma_commit(&ctl->empty[stage]);
-                    if (++stage == Cf::STAGES) { stage = 0; phase ^= 1; }
+                    for (int h = 0; h < MT; ++h)
+                        mma_bf16(el, d_tmem + h * BN, smem_desc(sa + h * A_BLOCK_BYTES + ks * 2048, 8192, 1024), bd, idesc,
+                                 (kb | ks) != 0);
                 }
-                if (stop) break;
-                mma_commit(&ctl->tfull);
-                acc_phase ^= 1;
+                mma_commit(el, &ctl->empty[stage]);
+                if (++stage == Cf::STAGES) { stage = 0; phase ^= 1; }
             }
+            if (stop) break;
+            mma_commit(el, &ctl->tfull);
+            acc_phase ^= 1;
         }
     } else {
         const int quarter = warp & 3;
