@@ -80,6 +80,7 @@ def work_table(w: gen.Workload):
         for name in ("bwd_da_dh", "bwd_dx", "wgrad_W1", "wgrad_W2"):
             t[name] = dict(flops=2 * R * d * de, bytes=(R * d + 2 * R * de + n * d * de) * s)
         t["wgrad_W1"]["bytes"] = t["wgrad_W2"]["bytes"] = (R * d + R * de) * s + n * d * de * 4
+        t["wgrad_mlp"] = {k: 2 * v for k, v in t["wgrad_W1"].items()}      # smaller matrices: both in one launch
         if patch_major(w):    # dx_g and the backward combine in one kernel: reads dh, W1 and dy, writes dx
             t["bwd_dx"] = dict(flops=2 * R * d * de, bytes=(R * de + n * d * de) * s + 2 * x_bytes)
         t["router_apply"] = dict(flops=0, bytes=x_bytes)
@@ -91,13 +92,10 @@ def work_table(w: gen.Workload):
         t["attention"] = dict(flops=att, bytes=4 * R * dg * s)
         t["out_proj"] = dict(flops=2 * R * dg * d, bytes=(R * dg + R * d + n * dg * d) * s)
     if w.H and w.backward:
-        # algorithmic work of the attention backward is five l_a x l_a contractions (dV, dP, dK, dQ and the
-        # rebuilt S); the dK/dV pass is credited with four of them, the dQ pass with one
-        t["attn_bwd_dkdv"] = dict(flops=2 * att, bytes=6 * R * dg * s)
-        t["attn_bwd_dq"] = dict(flops=att // 2, bytes=5 * R * dg * s)
+        # algorithmic work of the attention backward is five l_a x l_a contractions (dV, dP, dK, dQ and the rebuilt S)
+        t["attn_bwd"] = dict(flops=5 * att // 2, bytes=8 * R * dg * s)
         t["bwd_do"] = dict(flops=2 * R * d * dg, bytes=(R * d + R * dg + n * dg * d) * s)
-        t["wgrad_Wo"] = dict(flops=2 * R * d * dg, bytes=(R * d + R * dg) * s + n * d * dg * 4)
-        t["wgrad_Wqkv"] = dict(flops=6 * R * d * dg, bytes=(R * d + 3 * R * dg) * s + 3 * n * d * dg * 4)
+        t["wgrad_att"] = dict(flops=8 * R * d * dg, bytes=(2 * R * d + 4 * R * dg) * s + 4 * n * d * dg * 4)
         t["bwd_dx_att"] = dict(flops=6 * R * dg * d, bytes=(3 * R * dg + R * d + 3 * n * d * dg) * s)
     return t
 
@@ -112,8 +110,7 @@ def step_flops(w: gen.Workload) -> int:
     if w.H:
         f += t["qkv_proj"]["flops"] + t["attention"]["flops"] + t["out_proj"]["flops"]
     if w.H and w.backward:
-        f += t["attn_bwd_dkdv"]["flops"] + t["attn_bwd_dq"]["flops"] + t["bwd_do"]["flops"] + t["wgrad_Wo"]["flops"] + \
-            t["wgrad_Wqkv"]["flops"] + t["bwd_dx_att"]["flops"]
+        f += t["attn_bwd"]["flops"] + t["bwd_do"]["flops"] + t["wgrad_att"]["flops"] + t["bwd_dx_att"]["flops"]
     return f
 
 
@@ -663,7 +660,7 @@ def single_mode_of(dev, steps: int):
 
 
 TENSOR_KERNELS = ("gemm1_act", "gemm2", "mlp_fused", "qkv_proj", "out_proj", "attention", "bwd_da_dh", "bwd_dx", "wgrad_W1", "wgrad_W2",
-                  "attn_bwd_dkdv", "attn_bwd_dq", "bwd_do", "bwd_dx_att", "wgrad_Wo", "wgrad_Wqkv")
+                  "wgrad_mlp", "attn_bwd", "bwd_do", "bwd_dx_att", "wgrad_att")
 HBM_KERNELS = ("route", "gather", "combine", "router_apply")
 
 

@@ -129,3 +129,17 @@ def test_float32_experts_with_biases(name):
     ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
     ref = orc.mlp_forward(x.f64, W1.f64, W2.f64, ro, w.act, residual=False, b1=b1.f64, b2=b2.f64)
     assert rel_inf(to_f64(y), ref) <= 1e-5
+
+
+# attention backward: one tile (at most 128 tokens per pair), its edge, and blocks of 64 streamed past tiles of 128
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("l_p,c,L_valid", [(16, 8, 160), (8, 17, 260), (16, 4, 157), (32, 6, 250), (64, 5, 400), (1, 33, 40)],
+                         ids=lambda v: str(v))
+def test_attention_backward_tiles(l_p, c, L_valid, causal):
+    from tests.test_gpu_smha_backward import _run as run_att
+    m = max(c, -(-L_valid // l_p)) + 1
+    w = gen.tiny(B=3, L=m * l_p, L_valid=min(L_valid, m * l_p), m=m, c=c, d=128, n=3, k=2, d_ff=0, H=6, d_h=64, dtype="bf16",
+                 w_std=0.08, causal=causal)
+    got, ref = run_att(w, False)
+    for g, r in zip(got, ref[:len(got)]):
+        assert rel_inf(g, r) <= TOL
