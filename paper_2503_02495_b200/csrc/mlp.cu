@@ -12,7 +12,8 @@ static MlpFwdWs mlp_fwd_ws(const Dims& D) {
     w.take(kStatusBytes);
     MlpFwdWs r;
     r.plan = w.take(plan_bytes(D));
-    r.xg = can_fuse_gather(D) || !D.bf16 ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);     // the GEMM gathers x itself
+    // (the GEMM gathers x itself where patches tile 128 rows, and always in float32, whose workspace keeps the size it had)
+    r.xg = can_fuse_gather(D) ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.a = mlp_can_fuse(D) ? 0 : w.take((size_t)D.Rmax * D.d_e * D.esize);          // the fused kernel keeps the hidden tile on chip
     r.z = w.take((size_t)D.Rmax * D.d * D.esize);
     r.total = w.off;
