@@ -10,6 +10,7 @@
 //   dx_g = dh A^I_i^T                        grouped GEMM, then combined back with unit weights
 // Router: dgate -> dP_samp, dP_patch -> softmax Jacobians -> per-(sample, patch) logit gradient G, which
 // feeds dW_r (through the pooled token sums) and one more term of dx.
+#include "balance.cuh"
 #include "kernels.cuh"
 
 namespace uoe {
@@ -277,42 +278,32 @@ void launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, cons
     else go(once[2], router_apply_kernel<32, SPREAD>);
 }
 
-// Gradient of the load-balancing loss (Eq. 42-44) with respect to the router logits.  grid B, 128 threads, dynamic
-// shared memory n*m floats.  f_i (Eq. 43) is piecewise constant, so only P_i (Eq. 44) carries a gradient:
+// Gradient of the load-balancing loss (Eq. 42-44) with respect to the router logits.  grid B, dynamic shared memory
+// n (m + 1) floats.  f_i (Eq. 43) is piecewise constant, so only P_i (Eq. 44) carries a gradient:
 //   dL_b/dg_{i,j} = alpha f_i / l on the real patches;  G[b,j,i] = softmax Jacobian (Eq. 14) of that, / cnt_j.
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kBalanceThreads)
 balance_bwd_kernel(const float* __restrict__ p_patch, const float* __restrict__ dloss, int Lv, int n, int k, int m,
                    int l_p, float alpha, float* __restrict__ G) {
     pdl_trigger();
     pdl_wait();
-    extern __shared__ float pp[];          // [n][m]
+    extern __shared__ float s_gate[];
     __shared__ int cnts[32];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int n_elig = (Lv + l_p - 1) / l_p;
-    for (int idx = tid; idx < n * m; idx += 128) pp[idx] = p_patch[(size_t)b * n * m + idx];
-    if (tid < 32) cnts[tid] = 0;
-    __syncthreads();
-    for (int j = tid; j < n_elig; j += 128) {      // Eq. 15 / 43: patch j counts for its k best experts
-        for (int i = 0; i < n; ++i) {
-            const float v = pp[i * m + j];
-            int rank = 0;
-            for (int q = 0; q < n; ++q) {
-                const float w = pp[q * m + j];
-                rank += (w > v) || (w == v && q < i);
-            }
-            if (rank < k) atomicAdd(&cnts[i], 1);
-        }
-    }
-    __syncthreads();
     const float scale = dloss[b] * alpha * (float)n / ((float)k * (float)n_elig * (float)n_elig);     // dloss alpha (n / k l) / l
-    for (int j = tid; j < m; j += 128) {
+    balance_load(p_patch, b, n, m, s_gate);
+    __syncthreads();
+    balance_count(s_gate, n, k, m, n_elig, cnts, nullptr);
+    __syncthreads();
+    // scale cnts[i] is dL_b/dg of expert i; a thread per (patch, expert), in the order of G; the dot product over the experts is each thread's own
+    for (int idx = tid; idx < n * m; idx += kBalanceThreads) {
+        const int j = idx / n, i = idx - j * n;
         const int cnt = max(0, min(l_p, Lv - j * l_p));
         float dot = 0.f;
-        for (int i = 0; i < n; ++i) dot += pp[i * m + j] * scale * (float)cnts[i];
-        for (int i = 0; i < n; ++i) {
-            const float dl = pp[i * m + j] * (scale * (float)cnts[i] - dot);
-            G[((size_t)b * m + j) * n + i] = cnt > 0 ? dl / (float)cnt : 0.f;
-        }
+#pragma unroll 8
+        for (int q = 0; q < n; ++q) dot += s_gate[q * (m + 1) + j] * scale * (float)cnts[q];
+        const float dl = s_gate[i * (m + 1) + j] * (scale * (float)cnts[i] - dot);
+        G[(size_t)b * m * n + idx] = cnt > 0 ? dl / (float)cnt : 0.f;
     }
 }
 
@@ -518,7 +509,7 @@ extern "C" uoe_status uoe_route_balance_backward(const uoe_problem* prob, const 
     const RouterBwdScratch rs = router_backward_scratch(D, (char*)ws + kStatusBytes);
     {
         ProfScope ps("balance_bwd", stream);
-        launch_k(balance_bwd_kernel, dim3(D.B), dim3(128), (size_t)D.n * D.m * sizeof(float), stream, p_patch, dloss, D.Lv, D.n,
+        launch_k(balance_bwd_kernel, dim3(D.B), dim3(kBalanceThreads), (size_t)D.n * (D.m + 1) * sizeof(float), stream, p_patch, dloss, D.Lv, D.n,
                  D.k, D.m, D.l_p, alpha, rs.G);
     }
     UOE_LAUNCHED();

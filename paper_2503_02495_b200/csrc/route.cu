@@ -7,6 +7,7 @@
 //   CTA per sample.  Tickets and loads are reset by their last user, so a scratch area whose control block was
 //   zeroed once (uoe_workspace_init, or the static array of uoe_route_static) serves any number of calls of any shapes.
 // Also here: uoe_route_balance (Eq. 15-16, 42-44) and uoe_route_static.
+#include "balance.cuh"
 #include "kernels.cuh"
 
 namespace uoe {
@@ -296,7 +297,7 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     constexpr int V = Vec16<T>::N;
     extern __shared__ uint4 s_dyn4[];
     __shared__ __align__(16) float s_cs[NT * V];                    // column sums across row threads; later over all rows
-    __shared__ float s_dot[NT / 32][32];
+    __shared__ float s_dot[NT];
     __shared__ int s_mine;
     const int tid = threadIdx.x;
     const int nparts = nchunks * rsplit;
@@ -357,18 +358,17 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
         }
     }
 
-    // ---- score_part[bj, part, :] = column sums . W_r rows, out of shared memory: a lane per expert (np2 lanes), the lane
-    //      groups stride over the CTA's columns; sums meet through shuffles, then over the warps (0.75 us; as one thread's
-    //      sum over the groups 1.4) ----
+    // ---- score_part[bj, part, :] = column sums . W_r rows, out of shared memory: thread (group g, expert i) strides over
+    //      the CTA's columns, then a thread per expert adds the groups in ascending order, sixteen loads ahead of the adds
+    //      (0.85 us; with each load in front of its add 1.4) ----
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     {
-        const int np2 = n > 1 ? 1 << (32 - __clz(n - 1)) : 1;
-        const int groups = NT / np2;
-        const int i = tid % np2, g = tid / np2;
+        const int groups = NT / n;
+        const int i = tid % n, g = tid / n;
         const T* s_w = (const T*)s_dyn4;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        if (i < n) {                // four independent chains, then the tail: a fixed summation order
+        if (g < groups) {           // four independent chains, then the tail: a fixed summation order
             int cc = g;
             for (; cc + 3 * groups < cw; cc += 4 * groups) {
                 a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
@@ -378,14 +378,12 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
             }
             for (; cc < cw; cc += groups) a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
         }
-        float a = (a0 + a1) + (a2 + a3);
-        for (int o = np2; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if ((tid & 31) < n) s_dot[tid >> 5][tid & 31] = a;
+        s_dot[tid] = (a0 + a1) + (a2 + a3);
         __syncthreads();
         if (tid < n) {
             float sum = 0.f;
-#pragma unroll
-            for (int q = 0; q < NT / 32; ++q) sum += s_dot[q][tid];
+#pragma unroll 16
+            for (int q = 0; q < groups; ++q) sum += s_dot[q * n + tid];
             scores[((size_t)bj * nparts + part) * n + tid] = sum;
         }
     }
@@ -470,32 +468,28 @@ route_sample_kernel(const T* __restrict__ x, const T* __restrict__ W_r, int B, i
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    // ---- scores[j, i] = pooled patch j . W_r[:, i]: a warp per patch, a lane per expert and column group (np2 lanes per
-    //      group), four columns at a time, summed by a fixed shuffle tree (a thread per score and column slice issued
-    //      about eight instructions per product: 4.5 us at 14 patches, 6 experts, 384 columns) ----
-    {
-        const int warp = tid >> 5, lane = tid & 31;
-        const int np2 = n > 1 ? 1 << (32 - __clz(n - 1)) : 1;
-        const int i = lane % np2, seg = lane / np2, segs = 32 / np2;
-        for (int j = warp; j < m; j += NT / 32) {
-            const float4* pj = (const float4*)(s_pool + (size_t)j * d);
-            float a0 = 0.f, a1 = 0.f;
-            if (i < n) {
-                const T* w = s_w + i;
-#pragma unroll 4
-                for (int c4 = seg; c4 < d / 4; c4 += segs) {
-                    const float4 p = pj[c4];
-                    const T* wc = w + c4 * 4 * n;
-                    a0 = fmaf(p.x, to_f32(wc[0]), a0);
-                    a1 = fmaf(p.y, to_f32(wc[n]), a1);
-                    a0 = fmaf(p.z, to_f32(wc[2 * n]), a0);
-                    a1 = fmaf(p.w, to_f32(wc[3 * n]), a1);
-                }
+    // ---- scores[j, i] = pooled patch j . W_r[:, i]: `parts` threads per score, columns dealt round robin, summed by a
+    //      fixed shuffle tree.  Bound by instruction issue: two moving pointers, six instructions per product (columns
+    //      and rows indexed afresh for every product: 4.5 us at 14 patches, 6 experts, 384 columns) ----
+    int parts = 1;
+    while (parts < 32 && 2 * parts * m * n <= NT) parts <<= 1;
+    for (int p0 = 0; p0 < m * n; p0 += NT / parts) {
+        const int p = p0 + tid / parts, sub = tid & (parts - 1);
+        float acc = 0.f;
+        if (p < m * n) {
+            const int j = p / n;
+            const float* pc = s_pool + (size_t)j * d + sub;
+            const T* wc = s_w + sub * n + (p - j * n);
+            const int step = parts * n;
+#pragma unroll 8
+            for (int cc = sub; cc < d; cc += parts) {
+                acc = fmaf(*pc, to_f32(*wc), acc);
+                pc += parts;
+                wc += step;
             }
-            float acc = a0 + a1;
-            for (int o = np2; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane < n) s_sc[j * n + lane] = acc;
         }
+        for (int o = parts >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (p < m * n && sub == 0) s_sc[p] = acc;
     }
     __syncthreads();
     select_sample<NT>(s_pp, nullptr, 1, b, B, Lv, n, k, m, c, l_p, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch, offsets,
@@ -688,43 +682,30 @@ extern "C" uoe_status uoe_route(const uoe_problem* prob, const void* x, const vo
 // ------------------------------------------------------------------------------------------------
 namespace uoe {
 namespace {
-// grid B, 128 threads, dynamic shared memory n*m floats.
-__global__ void __launch_bounds__(128)
+// grid B, dynamic shared memory n (m + 1) floats.
+__global__ void __launch_bounds__(kBalanceThreads)
 balance_kernel(const float* __restrict__ p_patch, int Lv, int n, int k, int m, int l_p, float alpha,
                float* __restrict__ lb_loss, int* __restrict__ expert_count, int* __restrict__ c_dyn) {
     pdl_trigger();
     pdl_wait();
-    extern __shared__ float pp[];          // [n][m]
+    extern __shared__ float s_gate[];
     __shared__ int cnts[32];
-    __shared__ float Pm[32];
+    __shared__ float sums[32];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int n_elig = (Lv + l_p - 1) / l_p;       // patches holding at least one real token (a prefix)
-    for (int idx = tid; idx < n * m; idx += 128) pp[idx] = p_patch[(size_t)b * n * m + idx];
-    if (tid < 32) cnts[tid] = 0;
+    balance_load(p_patch, b, n, m, s_gate);
     __syncthreads();
-    for (int j = tid; j < n_elig; j += 128) {      // Eq. 15: patch j goes to its k best experts (ties: lower index)
-        for (int i = 0; i < n; ++i) {
-            const float v = pp[i * m + j];
-            int rank = 0;
-            for (int q = 0; q < n; ++q) {
-                const float w = pp[q * m + j];
-                rank += (w > v) || (w == v && q < i);
-            }
-            if (rank < k) atomicAdd(&cnts[i], 1);
-        }
-    }
-    if (tid < n) {                                  // Eq. 44: mean gate of expert i over the real patches, fixed order
-        float s = 0.f;
-        for (int j = 0; j < n_elig; ++j) s += pp[tid * m + j];
-        Pm[tid] = s / (float)n_elig;
-    }
+    balance_count(s_gate, n, k, m, n_elig, cnts, sums);
     __syncthreads();
     if (tid < n && expert_count) expert_count[(size_t)b * n + tid] = cnts[tid];
     if (tid == 0) {
         int cmax = 0;
         float loss = 0.f;
         const float fs = (float)n / ((float)k * (float)n_elig);                       // Eq. 43
-        for (int i = 0; i < n; ++i) { cmax = max(cmax, cnts[i]); loss += fs * (float)cnts[i] * Pm[i]; }
+        for (int i = 0; i < n; ++i) {
+            cmax = max(cmax, cnts[i]);
+            loss += fs * (float)cnts[i] * (sums[i] / (float)n_elig);                  // Eq. 44: mean gate over the real patches
+        }
         if (c_dyn) c_dyn[b] = cmax;                                                     // Eq. 16
         if (lb_loss) lb_loss[b] = alpha * loss;                                         // Eq. 42
     }
@@ -738,13 +719,13 @@ extern "C" uoe_status uoe_route_balance(const uoe_problem* prob, const float* p_
     uoe_status st = make_dims(prob, D);
     if (st != UOE_OK) return st;
     if (!p_patch || (!lb_loss && !expert_count && !c_dyn)) return UOE_ERR_INVALID_ARG;
-    const size_t smem = (size_t)D.n * D.m * sizeof(float);
-    if (smem > 36 * 1024) return UOE_ERR_UNSUPPORTED;
+    if ((size_t)D.n * D.m * sizeof(float) > 36 * 1024) return UOE_ERR_UNSUPPORTED;
+    const size_t smem = (size_t)D.n * (D.m + 1) * sizeof(float);
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     cudaError_t e;
     {
         ProfScope ps("route_balance", stream);
-        e = launch_k(balance_kernel, dim3(D.B), dim3(128), smem, stream, p_patch, D.Lv, D.n, D.k, D.m, D.l_p, alpha, lb_loss,
+        e = launch_k(balance_kernel, dim3(D.B), dim3(kBalanceThreads), smem, stream, p_patch, D.Lv, D.n, D.k, D.m, D.l_p, alpha, lb_loss,
                      expert_count, c_dyn);
     }
     if (e != cudaSuccess) return UOE_ERR_CUDA;

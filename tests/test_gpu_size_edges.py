@@ -75,6 +75,25 @@ def test_router_gradients_of_the_balance_loss(kw):
     assert np.all(to_f64(dx)[:, w.L_valid:] == 0)
 
 
+# a warp per expert (a second turn past sixteen), 32 patches per step: one expert, one patch, a step of one patch, all experts
+@pytest.mark.parametrize("n,k,m,L_valid", [(1, 1, 1, 3), (17, 4, 33, 130), (32, 32, 65, 260), (20, 1, 64, 256), (5, 2, 31, 121)])
+def test_loads_and_balance_loss(n, k, m, L_valid):
+    """Whole numbers exact on the gate values the GPU wrote; the loss is a float32 sum of at most 65 positive terms in
+    shuffle order (65 * 2^-24 = 4e-6 relative)."""
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(B=3, L=4 * m, L_valid=L_valid, m=m, c=1, d=64, n=n, k=k, d_ff=0, H=0, dtype="bf16")
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w).f64 * 20, w.dtype)
+    prob = problem_of(w, "mlp")
+    r = uoe.uoe_route(prob, to_dev(x), to_dev(Wr))
+    lb, cnt, cd = uoe.uoe_route_balance(prob, r.p_patch, alpha=0.01)
+    pp = r.p_patch.cpu().numpy().astype(np.float64)
+    pc = orc.patch_valid_counts(w.L, w.m, w.L_valid)
+    assert np.array_equal(cnt.cpu().numpy(), np.stack([orc.patch_expert_counts(pp[b], pc, k) for b in range(w.B)]))
+    assert np.array_equal(cd.cpu().numpy(), orc.dynamic_capacity(pp, pc, k))
+    ref = orc.balance_loss(pp, pc, k, alpha=0.01)
+    assert np.abs(lb.cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
 # weight gradients cut into equal pieces over the SMs: ragged column tiles, 8-row slabs, one expert whose tiles are cut into
 # many pieces, experts without rows, routed copies, and the pass without gates (the cut tiles added by their own launch)
 def _bwd(**kw):
