@@ -335,7 +335,7 @@ RouterBwdScratch router_backward_scratch(const Dims& D, char* base);
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
                                   const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
-                                  cudaStream_t stream, const WReduce& reduce = WReduce());
+                                  int* status, cudaStream_t stream, const WReduce& reduce = WReduce());
 uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s);
 
 // Eq. 38-39 in one kernel for narrow experts (bf16, d_e = 256, d <= 512): z = phi(A W1[e]) W2[e] with the hidden tile

@@ -12,9 +12,13 @@
 // feeds dW_r (through the pooled token sums) and one more term of dx.
 #include "balance.cuh"
 #include "kernels.cuh"
+#include "tc.cuh"
+#include "tmap.cuh"
 
 namespace uoe {
 namespace {
+
+using namespace tc;
 
 constexpr int kThreads = 256;
 
@@ -100,139 +104,139 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
 // What the router's logit gradient G [B*m, n] does to W_r and x, in one pass over x:
 //   dW_r[dd, i] = sum over (b, j) of pool[bj, dd] G[bj, i],  pool = sum of the real rows of patch bj
 //   rvec[bj, dd] = sum_i W_r[dd, i] G[bj, i], which every real token of the patch receives in dx
-// Bound by reading x once.  Grid (column blocks, splits), two CTAs per SM in all; a CTA has one thread per column of its
-// block and walks batches of eight slices: slice = (unit, row thread), where a unit is a patch or a segment of at most
-// 64 rows of a longer one, 16-byte loads, about eight rows per thread and batch, so a batch is 8 / RT units whose rows
-// are dealt to RT row threads.  The next batch's loads are in flight under this batch's arithmetic.  The sums meet in shared memory, then a thread adds its column's products: the pooled tensor
-// never reaches memory.  Every split leaves its own partial dW_r (dwr_sum adds them in split order).  SPREAD: the vector
-// is written to every row of dx at once instead of to rvec (the balance loss, whose whole dx it is).
-// Against a pooling kernel, one or two product kernels, a vector kernel and a spreading kernel (us, cold caches):
-// 23 instead of 58 at B = 256, L = 224, d = 384, n = 6;  9 instead of 22 at B = 16, L = 512, d = 512, n = 8;  77 as before
-// at B = 8, L = 4096, d = 4096, n = 16 (3.9 TB/s: two CTAs per SM do not cover the batch hand-offs there);  SPREAD 39
-// instead of 84 at B = 16, L = 2048, d = 1024, n = 16.
-constexpr int kSlices = 8;
+// Bound by reading x once.  Grid (blocks of 64 columns, splits of the patches), two CTAs per SM in all.  Every warp streams
+// for itself: it takes each eighth patch of its CTA's range through its own ring of TMA stages (at most 32 rows of 64
+// columns each), a lane adds two columns up over the rows and multiplies them, so no step waits for another warp and
+// the pooled tensor never reaches memory.  At the end the warps' dW_r meet in shared memory; every split leaves its own
+// partial (dwr_sum adds them in split order).  SPREAD: the vector is written to every row of dx at once instead of to
+// rvec (the balance loss, whose whole dx it is).
+// APPLY_FIGS
+constexpr int kApplyWarps = 8, kApplyCols = 64, kApplyRows = 32, kApplyStages = 8, kApplyRing = 3 * kApplyRows * kApplyCols * 2;
+struct ApplyArgs {
+    const __nv_bfloat16* W_r;
+    const float* G;
+    float *rvec, *part;
+    __nv_bfloat16* dx;
+    int* status;
+    int patches, Lv, d, n, m, l_p, nseg, seg_rows, per, stages;
+};
 template <int NMAX, bool SPREAD>
-__global__ void __launch_bounds__(320, NMAX > 16 ? 1 : 2)
-router_apply_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ W_r, const float* __restrict__ G,
-                    float* __restrict__ rvec, float* __restrict__ part, __nv_bfloat16* __restrict__ dx, int units, int L, int Lv,
-                    int d, int n, int m, int l_p, int nseg, int RT, int batches_per_cta) {
+__global__ void __launch_bounds__(32 * kApplyWarps, NMAX > 16 ? 1 : 2)
+router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], boxes of [seg_rows, 64] */, const ApplyArgs a) {
     pdl_trigger();
-    extern __shared__ float s_pool[];                // [kSlices][CW] column sums; SPREAD: then [kSlices / RT][CW] bfloat16
-    __shared__ float sG[kSlices * NMAX];
-    const int CW = blockDim.x, tid = threadIdx.x;    // CW: a multiple of 64
-    const int c0 = blockIdx.x * CW;
-    const int ct = tid % (CW / 8), slice = tid / (CW / 8);
-    const int PB = kSlices / RT;                     // units per batch
-    const int seg_rows = (l_p + nseg - 1) / nseg;
-    const int my_q = slice / RT, my_rt = slice % RT;
-    const int col = c0 + ct * 8, dd = c0 + tid;
-    pdl_wait();
-    float acc[NMAX], w[NMAX];
-#pragma unroll
-    for (int i = 0; i < NMAX; ++i) {
-        acc[i] = 0.f;
-        w[i] = (i < n && dd < d) ? __bfloat162float(W_r[(size_t)dd * n + i]) : 0.f;
+    extern __shared__ uint8_t s_raw[];
+    __shared__ uint64_t full[kApplyWarps][kApplyStages];
+    __shared__ int s_abort;
+    __shared__ __align__(16) float sG[kApplyWarps][NMAX];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n = a.n, d = a.d, nseg = a.nseg, unit_bytes = a.seg_rows * kApplyCols * 2;
+    uint8_t* smem = (uint8_t*)(((uintptr_t)s_raw + 127) & ~(uintptr_t)127);
+    uint8_t* ring = smem + warp * a.stages * unit_bytes;
+    volatile int* abort_flag = &s_abort;
+    if (tid == 0) s_abort = 0;
+    if (lane == 0) {
+        for (int s = 0; s < a.stages; ++s) mbar_init(&full[warp][s], 1);
+        fence_barrier_init();
+        prefetch_tmap(&xmap);
     }
-    const int q_lo = blockIdx.y * batches_per_cta * PB, q_hi = min(units, q_lo + batches_per_cta * PB);
-    // the loads of a batch: this thread's first eight rows, and its share of the batch's G (at most four values)
-    uint4 ld[8];
-    float gv[4];
-    int rows = 0, rows_all = 0;                     // real rows of the unit, all its rows
-    const __nv_bfloat16* base = nullptr;
-    auto issue = [&](int q0) {
-        rows = rows_all = 0;
-        const int unit = q0 + my_q;
-        if (my_q < PB && unit < q_hi && col < d) {
-            const int bj = nseg == 1 ? unit : unit / nseg, b = bj / m, s0 = nseg == 1 ? 0 : (unit - bj * nseg) * seg_rows;
-            const int r0 = (bj - b * m) * l_p + s0;      // first row in the sample
-            rows_all = min(seg_rows, l_p - s0);
-            rows = max(0, min(rows_all, Lv - r0));
-            base = x + ((size_t)b * L + r0) * d + col;
+    __syncthreads();
+    const int c0 = blockIdx.x * kApplyCols, dd = c0 + 2 * lane;       // this lane's columns: dd and dd + 1 (d is a multiple of eight)
+    const int first = blockIdx.y * a.per + warp, end = min(a.patches, (int)(blockIdx.y + 1) * a.per);
+    int ip = first, is = 0, st_in = 0;                // the next copy: patch, segment, stage
+    auto issue = [&]() {
+        if (ip >= end) return;
+        if (lane == 0) {
+            mbar_arrive_expect_tx(&full[warp][st_in], (uint32_t)unit_bytes);
+            tma_load_2d(ring + st_in * unit_bytes, &xmap, c0, ip * a.l_p + is * a.seg_rows, &full[warp][st_in]);
         }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (my_rt + u * RT < rows) ld[u] = ld_stream16(base + (size_t)(my_rt + u * RT) * d);
-        const int ng = min(PB, q_hi - q0) * n;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (tid + u * CW < ng)
-                gv[u] = nseg == 1 ? G[(size_t)q0 * n + tid + u * CW] : G[(size_t)((q0 + (tid + u * CW) / n) / nseg) * n + (tid + u * CW) % n];
+        if (++st_in == a.stages) st_in = 0;
+        if (++is == nseg) { is = 0; ip += kApplyWarps; }
     };
-    if (q_lo < q_hi) issue(q_lo);
-    for (int q0 = q_lo; q0 < q_hi; q0 += PB) {
-        const int nb = min(PB, q_hi - q0), rows_q = rows, rows_all_q = rows_all;
-        __nv_bfloat16* dx_base = SPREAD ? dx + (base - x) : nullptr;
-        {   // ---- column sums of this thread's slice ----
-            float cs[8];
+    pdl_wait();
+    for (int s = 0; s < a.stages; ++s) issue();
+    float g_next = first < end && lane < n ? a.G[(size_t)first * n + lane] : 0.f;
+    float acc[2][NMAX], w[2][NMAX];
 #pragma unroll
-            for (int v = 0; v < 8; ++v) cs[v] = 0.f;
-            auto add = [&](const uint4& t) {
-                float f[8];
-                unpack16<__nv_bfloat16>(t, f);
+    for (int v = 0; v < 2; ++v)
 #pragma unroll
-                for (int v = 0; v < 8; ++v) cs[v] += f[v];
-            };
+        for (int i = 0; i < NMAX; ++i) {
+            acc[v][i] = 0.f;
+            w[v][i] = (i < n && dd < d) ? __bfloat162float(a.W_r[(size_t)(dd + v) * n + i]) : 0.f;
+        }
+    int st = 0;                                       // the stage that is read next
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int patch = first; ok && patch < end; patch += kApplyWarps) {
+        const int j = patch % a.m, real = max(0, min(a.l_p, a.Lv - j * a.l_p));
+        float p[2] = {0.f, 0.f};
+        for (int seg = 0; seg < nseg; ++seg) {
+            ok = mbar_wait_warp(&full[warp][st], phase, abort_flag, a.status);
+            if (!ok) break;
+            const int rows = min(a.seg_rows, real - seg * a.seg_rows);
+            const uint8_t* src = ring + st * unit_bytes + lane * 4;
+            auto add = [&](uint32_t t) { p[0] += __uint_as_float(t << 16); p[1] += __uint_as_float(t & 0xffff0000u); };
+            int r = 0;
+            for (; r + 7 < rows; r += 8) {
+                uint32_t t[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (my_rt + u * RT < rows) add(ld[u]);
-            int r = my_rt + 8 * RT;
-            for (; r + 3 * RT < rows; r += 4 * RT) {
-                uint4 t[4];
+                for (int u = 0; u < 8; ++u) t[u] = *(const uint32_t*)(src + (r + u) * (kApplyCols * 2));
 #pragma unroll
-                for (int u = 0; u < 4; ++u) t[u] = ld_stream16(base + (size_t)(r + u * RT) * d);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) add(t[u]);
+                for (int u = 0; u < 8; ++u) add(t[u]);
             }
-            for (; r < rows; r += RT) add(ld_stream16(base + (size_t)r * d));
-#pragma unroll
-            for (int v = 0; v < 8; v += 4)
-                *(float4*)(s_pool + slice * CW + ct * 8 + v) = make_float4(cs[v], cs[v + 1], cs[v + 2], cs[v + 3]);
+            for (; r < rows; ++r) add(*(const uint32_t*)(src + r * (kApplyCols * 2)));
+            __syncwarp();                             // the stage has been read
+            issue();
+            if (++st == a.stages) { st = 0; phase ^= 1; }
         }
+        if (!ok) break;
+        if (lane < NMAX) sG[warp][lane] = g_next;     // zero past the experts
+        __syncwarp();
+        g_next = patch + kApplyWarps < end && lane < n ? a.G[(size_t)(patch + kApplyWarps) * n + lane] : 0.f;
+        float rv[2] = {0.f, 0.f};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int idx = tid + u * CW;
-            if (idx < nb * n) sG[(idx / n) * NMAX + idx % n] = gv[u];
-        }
-        __syncthreads();
-        if (q0 + PB < q_hi) issue(q0 + PB);
-        float rv[kSlices];
+        for (int i = 0; i < NMAX; i += 4) {
+            const float4 g4 = *(const float4*)(&sG[warp][i]);
+            const float g[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
-        for (int q = 0; q < kSlices; ++q) {          // (unrolled over the largest batch so that rv stays in registers)
-            rv[q] = 0.f;
-            if (q < nb) {
-                float p = 0.f;
-                for (int rt = 0; rt < RT; ++rt) p += s_pool[(q * RT + rt) * CW + tid];
-                float a = 0.f;
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int i = 0; i < NMAX; ++i) {
-                    if (i < n) {
-                        const float g = sG[q * NMAX + i];
-                        acc[i] = fmaf(p, g, acc[i]);
-                        a = fmaf(w[i], g, a);
-                    }
+                for (int v = 0; v < 2; ++v) {
+                    acc[v][i + q] = fmaf(p[v], g[q], acc[v][i + q]);
+                    rv[v] = fmaf(w[v][i + q], g[q], rv[v]);
                 }
-                rv[q] = a;
-                if (!SPREAD && dd < d && (nseg == 1 || (q0 + q) % nseg == 0)) rvec[(size_t)(nseg == 1 ? q0 + q : (q0 + q) / nseg) * d + dd] = a;
-            }
         }
-        __syncthreads();
-        if (SPREAD) {
-            __nv_bfloat16* s_rv = (__nv_bfloat16*)s_pool;
-#pragma unroll
-            for (int q = 0; q < kSlices; ++q)
-                if (q < nb) s_rv[q * CW + tid] = __float2bfloat16(rv[q]);
-            __syncthreads();
-            if (my_q < nb && col < d) {
-                const uint4 v = *(const uint4*)(s_rv + my_q * CW + ct * 8);
-                for (int r = my_rt; r < rows_all_q; r += RT) st_stream16(dx_base + (size_t)r * d, r < rows_q ? v : make_uint4(0, 0, 0, 0));
+        __syncwarp();
+        if (dd < d) {
+            if (!SPREAD) *(float2*)(a.rvec + (size_t)patch * d + dd) = make_float2(rv[0], rv[1]);
+            else {
+                const __nv_bfloat162 t = __floats2bfloat162_rn(rv[0], rv[1]);
+                __nv_bfloat16* o = a.dx + (size_t)patch * a.l_p * d + dd;
+#pragma unroll 8
+                for (int r = 0; r < a.l_p; ++r, o += d) __stcs((uint32_t*)o, r < real ? *(const uint32_t*)&t : 0u);
             }
-            __syncthreads();
         }
     }
-    if (dd < d) {
+    if (!ok && lane == 0)                             // winding down: let this warp's own copies land before the CTA exits
+        for (int s = 0; s < a.stages; ++s) {          // (stages without a copy in flight just run out of polls)
+            mbar_wait(&full[warp][st], phase, abort_flag, a.status);
+            if (++st == a.stages) { st = 0; phase ^= 1; }
+        }
+    if (!__syncthreads_and(ok)) return;               // (uniform) a copy did not arrive
+    // ---- the warps' sums, ascending ----
+    float* red = (float*)smem;                        // [warps][64 columns][NMAX + 1]
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
 #pragma unroll
         for (int i = 0; i < NMAX; ++i)
-            if (i < n) part[((size_t)blockIdx.y * d + dd) * n + i] = acc[i];
+            if (i < n) red[(warp * kApplyCols + 2 * lane + v) * (NMAX + 1) + i] = acc[v][i];
+    __syncthreads();
+    const int outs = min(kApplyCols, d - c0) * n;
+    for (int idx = tid; idx < outs; idx += 32 * kApplyWarps) {
+        const int cc = idx / n, i = idx - cc * n;
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < kApplyWarps; ++q) sum += red[(q * kApplyCols + cc) * (NMAX + 1) + i];
+        a.part[((size_t)blockIdx.y * d + c0) * n + idx] = sum;
     }
 }
 
@@ -243,39 +247,46 @@ dwr_sum_kernel(const DwrSum s) {
     dwr_sum(s, blockIdx.x);
 }
 
-// Column block, row threads and splits of router_apply_kernel for a problem.
-struct ApplyShape { int CW, RT, nseg, col_blocks, splits, per; };
+// Segments, stages and splits of router_apply_kernel for a problem.
+struct ApplyShape { int nseg, seg_rows, stages, col_blocks, splits, per; };
 ApplyShape apply_shape(const Dims& D) {
     ApplyShape a;
-    a.CW = D.d < 256 ? (D.d + 63) / 64 * 64 : 256;
-    for (int cw : {256, 320, 192, 128})
-        if (D.d % cw == 0) { a.CW = cw; break; }
-    a.col_blocks = (D.d + a.CW - 1) / a.CW;
-    // rows of a patch are dealt to as many threads as leave each about eight rows, one batch of loads
-    a.nseg = (D.l_p + 63) / 64;
-    a.RT = 1;
-    while (a.RT < kSlices && (D.l_p + a.nseg - 1) / a.nseg >= 16 * a.RT) a.RT *= 2;
-    const int PB = kSlices / a.RT, batches = (D.B * D.m * a.nseg + PB - 1) / PB;
+    a.col_blocks = (D.d + kApplyCols - 1) / kApplyCols;
+    a.nseg = (D.l_p + kApplyRows - 1) / kApplyRows;
+    a.seg_rows = (D.l_p + a.nseg - 1) / a.nseg;
+    a.stages = kApplyRing / (a.seg_rows * kApplyCols * 2);         // 12 KB in flight per warp
+    if (a.stages > kApplyStages) a.stages = kApplyStages;
+    const int patches = D.B * D.m;
     const int cap = 2 * 148 / a.col_blocks > 1 ? 2 * 148 / a.col_blocks : 1;        // two CTAs per SM: one full wave
-    a.splits = batches < cap ? batches : cap;
-    a.per = (batches + a.splits - 1) / a.splits;
-    a.splits = (batches + a.per - 1) / a.per;
+    a.per = (patches + cap - 1) / cap;
+    a.splits = (patches + a.per - 1) / a.per;
     return a;
 }
 template <bool SPREAD>
-void launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, const void* W_r, const float* G, float* rvec,
-                         float* part, void* dx, cudaStream_t s) {
-    auto go = [&](SpreadOnce& once, auto kern) {
-        const size_t smem = spread_smem(once, kern, (long long)a.col_blocks * a.splits, (size_t)kSlices * a.CW * sizeof(float));
-        launch_k(kern, dim3(a.col_blocks, a.splits), dim3(a.CW), smem, s, (const __nv_bfloat16*)x,
-                 (const __nv_bfloat16*)W_r, G, rvec, part, (__nv_bfloat16*)dx, D.B * D.m * a.nseg, D.L, D.Lv, D.d, D.n, D.m, D.l_p, a.nseg,
-                 a.RT, a.per);
+uoe_status launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, const void* W_r, const float* G, float* rvec,
+                               float* part, void* dx, int* status, cudaStream_t s) {
+    CUtensorMap xmap;
+    const uint64_t dims[2] = {(uint64_t)D.d, (uint64_t)D.B * D.L}, str[1] = {(uint64_t)D.d * 2};
+    const uint32_t box[2] = {(uint32_t)kApplyCols, (uint32_t)a.seg_rows};
+    if (!make_tmap(&xmap, x, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_NONE)) return UOE_ERR_CUDA;
+    ApplyArgs p;
+    p.W_r = (const __nv_bfloat16*)W_r; p.G = G; p.rvec = rvec; p.part = part; p.dx = (__nv_bfloat16*)dx; p.status = status;
+    p.patches = D.B * D.m; p.Lv = D.Lv; p.d = D.d; p.n = D.n; p.m = D.m; p.l_p = D.l_p; p.nseg = a.nseg;
+    p.seg_rows = a.seg_rows; p.per = a.per; p.stages = a.stages;
+    auto go = [&](SpreadOnce& once, auto kern, int nmax) {
+        const uoe_status so = smem_opt_in(once.opt_in, kern, 160 * 1024);
+        if (so != UOE_OK) return so;
+        const size_t ring = (size_t)kApplyWarps * a.stages * a.seg_rows * kApplyCols * 2;
+        const size_t red = (size_t)kApplyWarps * kApplyCols * (nmax + 1) * 4;
+        launch_k(kern, dim3(a.col_blocks, a.splits), dim3(32 * kApplyWarps),
+                 spread_smem(once, kern, (long long)a.col_blocks * a.splits, (ring > red ? ring : red) + 128), s, xmap, p);
+        return UOE_OK;
     };
     ProfScope ps("router_apply", s);
     static SpreadOnce once[3];
-    if (D.n <= 8) go(once[0], router_apply_kernel<8, SPREAD>);
-    else if (D.n <= 16) go(once[1], router_apply_kernel<16, SPREAD>);
-    else go(once[2], router_apply_kernel<32, SPREAD>);
+    if (D.n <= 8) return go(once[0], router_apply_kernel<8, SPREAD>, 8);
+    if (D.n <= 16) return go(once[1], router_apply_kernel<16, SPREAD>, 16);
+    return go(once[2], router_apply_kernel<32, SPREAD>, 32);
 }
 
 // Gradient of the load-balancing loss (Eq. 42-44) with respect to the router logits.  grid B, dynamic shared memory
@@ -345,7 +356,7 @@ BwdWs bwd_ws(const Dims& D) {
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
                                   const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
-                                  cudaStream_t stream, const WReduce& reduce) {
+                                  int* status, cudaStream_t stream, const WReduce& reduce) {
     if (!D.bf16) return UOE_ERR_UNSUPPORTED;
     const size_t smem = ((size_t)2 * D.n * D.m + (size_t)D.k * D.c) * sizeof(float);
     if ((size_t)2 * D.n * D.m * sizeof(float) > 40 * 1024) return UOE_ERR_UNSUPPORTED;
@@ -360,7 +371,8 @@ uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r,
     }
     UOE_LAUNCHED();
     const ApplyShape a = apply_shape(D);
-    launch_router_apply<false>(D, a, x, W_r, rs.G, rs.rvec, rs.wpart, nullptr, stream);
+    const uoe_status st = launch_router_apply<false>(D, a, x, W_r, rs.G, rs.rvec, rs.wpart, nullptr, status, stream);
+    if (st != UOE_OK) return st;
     UOE_LAUNCHED();
     *sum = DwrSum{rs.wpart, dW_r, D.d * D.n, a.splits};
     return UOE_OK;
@@ -472,7 +484,7 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
     DwrSum sum;
     if (use_gate) {
         RouterBwdScratch rs{G, rvec, wpart};
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, &sum, stream, reduce);
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, W.nt, rs, dW_r, &sum, status, stream, reduce);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
@@ -514,7 +526,8 @@ extern "C" uoe_status uoe_route_balance_backward(const uoe_problem* prob, const 
     }
     UOE_LAUNCHED();
     const ApplyShape a = apply_shape(D);
-    launch_router_apply<true>(D, a, x, W_r, rs.G, nullptr, rs.wpart, dx, stream);
+    st = launch_router_apply<true>(D, a, x, W_r, rs.G, nullptr, rs.wpart, dx, (int*)ws, stream);
+    if (st != UOE_OK) return st;
     UOE_LAUNCHED();
     return launch_dwr_sum(DwrSum{rs.wpart, dW_r, D.d * D.n, a.splits}, stream);
 }

@@ -151,7 +151,7 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     // ---- router ----
     DwrSum sum;
     if (use_gate) {
-        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, &sum, stream, reduce);
+        st = launch_router_backward(D, x, W_r, expert_idx, patch_idx, p_samp, p_patch, P, dgp, heads, rs, dW_r, &sum, status, stream, reduce);
         if (st != UOE_OK) return st;
     } else {
         UOE_CUDA_OK(cudaMemsetAsync(dW_r, 0, (size_t)D.d * D.n * sizeof(float), stream));
