@@ -110,7 +110,29 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
 // the pooled tensor never reaches memory.  At the end the warps' dW_r meet in shared memory; every split leaves its own
 // partial (dwr_sum adds them in split order).  SPREAD: the vector is written to every row of dx at once instead of to
 // rvec (the balance loss, whose whole dx it is).
-// APPLY_FIGS
+// Against CTA-wide batches (16-byte loads a batch ahead in registers, sums through shared memory, two to four CTA barriers
+// per batch: a chain of barriers and 750 instructions per warp and batch, the same through TMA stages), us, cold caches:
+// B = 256, L = 224, d = 384, n = 6: 20.8 -> 17.0;  B = 16, L = 512, d = 512, n = 8: 8.8 -> 6.7;  B = 4, L = 2048, d = 1024,
+// n = 8: 10.5 -> 8.2;  B = 8, L = 4096, d = 4096, n = 16: 70 -> 48 (5.5 TB/s);  SPREAD, B = 16, L = 2048, d = 1024,
+// n = 16: 34 -> 24.4.  (A pooling kernel, product kernels and a vector or spreading kernel before that: 58, 22, -, 77, 84.)
+// Two float32 additions or multiply-adds in one instruction, each rounded as the single one is.
+__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void f2_add(unsigned long long& a, unsigned long long b) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+}
+__device__ __forceinline__ void f2_fma(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
 constexpr int kApplyWarps = 8, kApplyCols = 64, kApplyRows = 32, kApplyStages = 8, kApplyRing = 3 * kApplyRows * kApplyCols * 2;
 struct ApplyArgs {
     const __nv_bfloat16* W_r;
@@ -127,7 +149,7 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], b
     extern __shared__ uint8_t s_raw[];
     __shared__ uint64_t full[kApplyWarps][kApplyStages];
     __shared__ int s_abort;
-    __shared__ __align__(16) float sG[kApplyWarps][NMAX];
+    __shared__ __align__(16) float2 sG[kApplyWarps][NMAX];              // (g, g)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n = a.n, d = a.d, nseg = a.nseg, unit_bytes = a.seg_rows * kApplyCols * 2;
     uint8_t* smem = (uint8_t*)(((uintptr_t)s_raw + 127) & ~(uintptr_t)127);
@@ -155,26 +177,25 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], b
     pdl_wait();
     for (int s = 0; s < a.stages; ++s) issue();
     float g_next = first < end && lane < n ? a.G[(size_t)first * n + lane] : 0.f;
-    float acc[2][NMAX], w[2][NMAX];
+    unsigned long long acc[NMAX], w[NMAX];            // pairs over the two columns
 #pragma unroll
-    for (int v = 0; v < 2; ++v)
-#pragma unroll
-        for (int i = 0; i < NMAX; ++i) {
-            acc[v][i] = 0.f;
-            w[v][i] = (i < n && dd < d) ? __bfloat162float(a.W_r[(size_t)(dd + v) * n + i]) : 0.f;
-        }
+    for (int i = 0; i < NMAX; ++i) {
+        const bool in = i < n && dd < d;
+        acc[i] = 0ull;
+        w[i] = in ? f2_pack(__bfloat162float(a.W_r[(size_t)dd * n + i]), __bfloat162float(a.W_r[(size_t)(dd + 1) * n + i])) : 0ull;
+    }
     int st = 0;                                       // the stage that is read next
     uint32_t phase = 0;
     bool ok = true;
     for (int patch = first; ok && patch < end; patch += kApplyWarps) {
         const int j = patch % a.m, real = max(0, min(a.l_p, a.Lv - j * a.l_p));
-        float p[2] = {0.f, 0.f};
+        unsigned long long p = 0ull;
         for (int seg = 0; seg < nseg; ++seg) {
             ok = mbar_wait_warp(&full[warp][st], phase, abort_flag, a.status);
             if (!ok) break;
             const int rows = min(a.seg_rows, real - seg * a.seg_rows);
             const uint8_t* src = ring + st * unit_bytes + lane * 4;
-            auto add = [&](uint32_t t) { p[0] += __uint_as_float(t << 16); p[1] += __uint_as_float(t & 0xffff0000u); };
+            auto add = [&](uint32_t t) { f2_add(p, f2_pack(__uint_as_float(t << 16), __uint_as_float(t & 0xffff0000u))); };
             int r = 0;
             for (; r + 7 < rows; r += 8) {
                 uint32_t t[8];
@@ -189,30 +210,32 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], b
             if (++st == a.stages) { st = 0; phase ^= 1; }
         }
         if (!ok) break;
-        if (lane < NMAX) sG[warp][lane] = g_next;     // zero past the experts
+        if (lane < NMAX) sG[warp][lane] = make_float2(g_next, g_next);     // zero past the experts
         __syncwarp();
         g_next = patch + kApplyWarps < end && lane < n ? a.G[(size_t)(patch + kApplyWarps) * n + lane] : 0.f;
-        float rv[2] = {0.f, 0.f};
+        unsigned long long rv2 = 0ull;
 #pragma unroll
-        for (int i = 0; i < NMAX; i += 4) {
-            const float4 g4 = *(const float4*)(&sG[warp][i]);
-            const float g[4] = {g4.x, g4.y, g4.z, g4.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    acc[v][i + q] = fmaf(p[v], g[q], acc[v][i + q]);
-                    rv[v] = fmaf(w[v][i + q], g[q], rv[v]);
-                }
+        for (int i = 0; i < NMAX; i += 2) {
+            const ulonglong2 g = *(const ulonglong2*)(&sG[warp][i]);
+            f2_fma(acc[i], p, g.x);
+            f2_fma(rv2, w[i], g.x);
+            f2_fma(acc[i + 1], p, g.y);
+            f2_fma(rv2, w[i + 1], g.y);
         }
         __syncwarp();
-        if (dd < d) {
-            if (!SPREAD) *(float2*)(a.rvec + (size_t)patch * d + dd) = make_float2(rv[0], rv[1]);
-            else {
-                const __nv_bfloat162 t = __floats2bfloat162_rn(rv[0], rv[1]);
-                __nv_bfloat16* o = a.dx + (size_t)patch * a.l_p * d + dd;
-#pragma unroll 8
-                for (int r = 0; r < a.l_p; ++r, o += d) __stcs((uint32_t*)o, r < real ? *(const uint32_t*)&t : 0u);
+        const float2 rv = f2_unpack(rv2);
+        if (!SPREAD) {
+            if (dd < d) *(float2*)(a.rvec + (size_t)patch * d + dd) = rv;
+        } else {                                      // four lanes' columns to one: a store covers four rows
+            const __nv_bfloat162 t2 = __floats2bfloat162_rn(rv.x, rv.y);
+            const uint32_t t = *(const uint32_t*)&t2;
+            const int q = 4 * (lane & 7), col = c0 + 8 * (lane & 7);
+            const uint4 v = make_uint4(__shfl_sync(0xffffffffu, t, q), __shfl_sync(0xffffffffu, t, q + 1),
+                                       __shfl_sync(0xffffffffu, t, q + 2), __shfl_sync(0xffffffffu, t, q + 3));
+            if (col < d) {
+                __nv_bfloat16* o = a.dx + ((size_t)patch * a.l_p + (lane >> 3)) * d + col;
+#pragma unroll 4
+                for (int r = lane >> 3; r < a.l_p; r += 4, o += (size_t)4 * d) st_stream16(o, r < real ? v : make_uint4(0, 0, 0, 0));
             }
         }
     }
@@ -225,10 +248,12 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], b
     // ---- the warps' sums, ascending ----
     float* red = (float*)smem;                        // [warps][64 columns][NMAX + 1]
 #pragma unroll
-    for (int v = 0; v < 2; ++v)
-#pragma unroll
-        for (int i = 0; i < NMAX; ++i)
-            if (i < n) red[(warp * kApplyCols + 2 * lane + v) * (NMAX + 1) + i] = acc[v][i];
+    for (int i = 0; i < NMAX; ++i)
+        if (i < n) {
+            const float2 t = f2_unpack(acc[i]);
+            red[(warp * kApplyCols + 2 * lane) * (NMAX + 1) + i] = t.x;
+            red[(warp * kApplyCols + 2 * lane + 1) * (NMAX + 1) + i] = t.y;
+        }
     __syncthreads();
     const int outs = min(kApplyCols, d - c0) * n;
     for (int idx = tid; idx < outs; idx += 32 * kApplyWarps) {
