@@ -224,6 +224,33 @@ __device__ __forceinline__ void unpack16(const uint4& v, float* f) {
     }
 }
 
+// Two float32 additions or multiply-adds in one instruction, each rounded as the single one is.
+__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void f2_add(unsigned long long& a, unsigned long long b) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+}
+__device__ __forceinline__ void f2_fma(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// acc[pairs of elements] += the elements of v.
+template <typename T>
+__device__ __forceinline__ void f2_add16(unsigned long long* acc, const uint4& v) {
+    float f[Vec16<T>::N];
+    unpack16<T>(v, f);
+#pragma unroll
+    for (int i = 0; i < Vec16<T>::N / 2; ++i) f2_add(acc[i], f2_pack(f[2 * i], f[2 * i + 1]));
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&t);

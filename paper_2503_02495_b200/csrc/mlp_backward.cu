@@ -115,24 +115,6 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
 // B = 256, L = 224, d = 384, n = 6: 20.8 -> 17.0;  B = 16, L = 512, d = 512, n = 8: 8.8 -> 6.7;  B = 4, L = 2048, d = 1024,
 // n = 8: 10.5 -> 8.2;  B = 8, L = 4096, d = 4096, n = 16: 70 -> 48 (5.5 TB/s);  SPREAD, B = 16, L = 2048, d = 1024,
 // n = 16: 34 -> 24.4.  (A pooling kernel, product kernels and a vector or spreading kernel before that: 58, 22, -, 77, 84.)
-// Two float32 additions or multiply-adds in one instruction, each rounded as the single one is.
-__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ void f2_add(unsigned long long& a, unsigned long long b) {
-    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
-}
-__device__ __forceinline__ void f2_fma(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 constexpr int kApplyWarps = 8, kApplyCols = 64, kApplyRows = 32, kApplyStages = 8, kApplyRing = 3 * kApplyRows * kApplyCols * 2;
 struct ApplyArgs {
     const __nv_bfloat16* W_r;

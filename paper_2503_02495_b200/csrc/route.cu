@@ -272,7 +272,7 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
     }
 }
 
-// Scoring (Eq. 13, 21) and selection, in one kernel or two.  Grid B*m * nchunks * rsplit, column chunk fastest: a CTA
+// Scoring (Eq. 13, 21) and selection, in one kernel or two.  Grid (nchunks * rsplit, m, B), column chunk fastest: a CTA
 // takes one column chunk of one row slice of a patch (CT threads span the columns of the chunk, 16 bytes each, NT/CT
 // span rows).  CTAs that run at the same time cover neighbouring chunks of the same rows, so together they read x
 // linearly.  The CTA first asks for the rows of W_r that belong to its columns (cp.async into shared memory, landing
@@ -291,7 +291,7 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
              int* __restrict__ expert_idx, int* __restrict__ patch_idx, float* __restrict__ gate,
              float* __restrict__ p_samp, float* __restrict__ p_patch, int* __restrict__ offsets,
              int* __restrict__ ctl /* word 1: ticket */, int* __restrict__ sample_ticket /* [B] */, unsigned* __restrict__ masks /* [B] */,
-             const PlanPtrs plan /* all null: no plan is written */) {
+             const PlanPtrs plan /* all null: no plan is written */, int b0 /* first sample of the launch */) {
     pdl_trigger();
     pdl_wait();
     constexpr int V = Vec16<T>::N;
@@ -301,10 +301,9 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     __shared__ int s_mine;
     const int tid = threadIdx.x;
     const int nparts = nchunks * rsplit;
-    const int bj = blockIdx.x / nparts;
-    const int b = bj / m, j = bj % m;
-    const int part = blockIdx.x % nparts;
-    const int chunk = part % nchunks, rs = part / nchunks;
+    const int b = b0 + blockIdx.z, j = blockIdx.y, bj = b * m + j;
+    const int part = blockIdx.x;
+    const int rs = rsplit > 1 ? part / nchunks : 0, chunk = part - rs * nchunks;
     const int c0 = chunk * CT * V, cw = min(CT * V, d - c0);          // this CTA's columns: [c0, c0 + cw)
 
     {   // the W_r rows of these columns: cw * n consecutive elements (cw and the rows' start are multiples of V elements)
@@ -316,14 +315,15 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     }
 
     // ---- column sums of this CTA's rows ----
-    const int ct = tid % CT, rt = tid / CT, RT = NT / CT;
+    const int ct_log = __ffs(CT) - 1;                                 // (CT is a power of two)
+    const int ct = tid & (CT - 1), rt = tid >> ct_log, RT = NT >> ct_log;
     const int col = c0 + ct * V;
-    float cs[V];
+    unsigned long long cs[V / 2];                                     // pairs of columns
     {
         const int row_lo = rs * rows_per_cta;
         const int rows = min(max(0, min(l_p, Lv - j * l_p)), row_lo + rows_per_cta);      // this slice: [row_lo, rows)
 #pragma unroll
-        for (int v = 0; v < V; ++v) cs[v] = 0.f;
+        for (int v = 0; v < V / 2; ++v) cs[v] = 0ull;
         if (col < d) {
             const T* base = x + ((size_t)b * L + (size_t)j * l_p) * d + col;
             int r = row_lo + rt;
@@ -332,22 +332,12 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
 #pragma unroll
                 for (int u = 0; u < 8; ++u) q[u] = ld_stream16(base + (size_t)(r + u * RT) * d);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    float f[V];
-                    unpack16<T>(q[u], f);
-#pragma unroll
-                    for (int v = 0; v < V; ++v) cs[v] += f[v];
-                }
+                for (int u = 0; u < 8; ++u) f2_add16<T>(cs, q[u]);
             }
-            for (; r < rows; r += RT) {
-                float f[V];
-                unpack16<T>(ld_stream16(base + (size_t)r * d), f);
-#pragma unroll
-                for (int v = 0; v < V; ++v) cs[v] += f[v];
-            }
+            for (; r < rows; r += RT) f2_add16<T>(cs, ld_stream16(base + (size_t)r * d));
         }
 #pragma unroll
-        for (int v = 0; v < V; ++v) s_cs[tid * V + v] = cs[v];
+        for (int v = 0; v < V / 2; v += 2) *(ulonglong2*)(s_cs + tid * V + 2 * v) = make_ulonglong2(cs[v], cs[v + 1]);
         if (RT > 1) {                           // sum over the row threads, ascending; all threads take columns
             __syncthreads();
             for (int cc = tid; cc < CT * V; cc += NT) {
@@ -365,18 +355,22 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     __syncthreads();
     {
         const int groups = NT / n;
-        const int i = tid % n, g = tid / n;
-        const T* s_w = (const T*)s_dyn4;
+        const int g = tid / n, i = tid - g * n;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
         if (g < groups) {           // four independent chains, then the tail: a fixed summation order
+            const float* pc = s_cs + g;                       // moving pointers: six instructions per product
+            const T* pw = (const T*)s_dyn4 + g * n + i;
+            const int step = groups * n;
             int cc = g;
             for (; cc + 3 * groups < cw; cc += 4 * groups) {
-                a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
-                a1 = fmaf(s_cs[cc + groups], to_f32(s_w[(cc + groups) * n + i]), a1);
-                a2 = fmaf(s_cs[cc + 2 * groups], to_f32(s_w[(cc + 2 * groups) * n + i]), a2);
-                a3 = fmaf(s_cs[cc + 3 * groups], to_f32(s_w[(cc + 3 * groups) * n + i]), a3);
+                a0 = fmaf(pc[0], to_f32(pw[0]), a0);
+                a1 = fmaf(pc[groups], to_f32(pw[step]), a1);
+                a2 = fmaf(pc[2 * groups], to_f32(pw[2 * step]), a2);
+                a3 = fmaf(pc[3 * groups], to_f32(pw[3 * step]), a3);
+                pc += 4 * groups;
+                pw += 4 * step;
             }
-            for (; cc < cw; cc += groups) a0 = fmaf(s_cs[cc], to_f32(s_w[cc * n + i]), a0);
+            for (; cc < cw; cc += groups, pc += groups, pw += step) a0 = fmaf(*pc, to_f32(*pw), a0);
         }
         s_dot[tid] = (a0 + a1) + (a2 + a3);
         __syncthreads();
@@ -578,14 +572,17 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
     float* scores = (float*)(base + W.scores);
     const int use_gate = ((flags & UOE_FLAG_GATE) ? 1 : 0) | ((flags & UOE_FLAG_DYNAMIC_C) ? 2 : 0) |
                          ((flags & UOE_FLAG_GENERAL_PATH) ? 4 : 0);                                       // selection flags
-    dim3 grid((unsigned)(D.B * D.m * W.nchunks * W.rsplit));
+    constexpr int kGridZ = 65535;      // samples per launch of route_kernel (more than that: more launches)
+    int b0 = 0;
+    dim3 grid((unsigned)(W.nchunks * W.rsplit), (unsigned)D.m, (unsigned)(D.B < kGridZ ? D.B : kGridZ));
+    const long long ctas = (long long)grid.x * grid.y * grid.z;
 #define UOE_ROUTE_ARGS(T) (const T*)x, (const T*)W_r, scores, D.B, D.L, D.Lv, D.d, D.n, D.k, D.m, D.c, D.l_p, W.CT, \
         W.nchunks, W.rsplit, W.rows_per_cta, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch, expert_offsets, ctl, \
-        tickets, masks, plan
+        tickets, masks, plan, b0
 #define UOE_ROUTE_LAUNCH(T, TICKET, NT, SMEM) \
         [&] { \
             static SpreadOnce once; \
-            return launch_k(route_kernel<T, TICKET, NT>, grid, dim3(NT), spread_smem(once, route_kernel<T, TICKET, NT>, grid.x, SMEM), \
+            return launch_k(route_kernel<T, TICKET, NT>, grid, dim3(NT), spread_smem(once, route_kernel<T, TICKET, NT>, ctas, SMEM), \
                             stream, UOE_ROUTE_ARGS(T)); \
         }()
     cudaError_t e;
@@ -609,9 +606,12 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
     }
     {
         ProfScope ps(profile ? "route" : nullptr, stream);
-        if (W.small_ctas) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, 64, W.smem) : UOE_ROUTE_LAUNCH(float, false, 64, W.smem);
-        else if (W.two_kernels) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, kScoreThreads, W.smem) : UOE_ROUTE_LAUNCH(float, false, kScoreThreads, W.smem);
-        else e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, true, kScoreThreads, smem0) : UOE_ROUTE_LAUNCH(float, true, kScoreThreads, smem0);
+        for (e = cudaSuccess; e == cudaSuccess && b0 < D.B; b0 += kGridZ) {
+            if (D.B - b0 < kGridZ) grid.z = (unsigned)(D.B - b0);
+            if (W.small_ctas) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, 64, W.smem) : UOE_ROUTE_LAUNCH(float, false, 64, W.smem);
+            else if (W.two_kernels) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, kScoreThreads, W.smem) : UOE_ROUTE_LAUNCH(float, false, kScoreThreads, W.smem);
+            else e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, true, kScoreThreads, smem0) : UOE_ROUTE_LAUNCH(float, true, kScoreThreads, smem0);
+        }
     }
 #undef UOE_ROUTE_LAUNCH
 #undef UOE_ROUTE_ARGS
