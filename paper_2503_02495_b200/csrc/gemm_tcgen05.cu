@@ -349,7 +349,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     // (32 columns at a time, kept packed until the 64-column pieces are complete: few enough registers for
                     // eight warps; with four warps of 64 columns the image block's launch took 68 us)
                     const float rg = row_gate[row], rv = row_valid[row];
-                    float dsum = 0.f;
+                    const unsigned long long rg2 = f2_pack(rg, rg);
+                    unsigned long long dsum2 = 0ull;
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g) {
                         uint32_t pd[32], pa[32];             // dh and gated phi(h) of the piece, bf16 pairs
@@ -367,23 +368,24 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             for (int q = 0; q < 4; ++q) unpack16<__nv_bfloat16>(hv[q], dh + 8 * q);     // h
                             act_and_deriv_n<32>(dh, ag, dh, act);                                         // ag = phi(h), dh = phi'(h)
 #pragma unroll
-                            for (int q = 0; q < 32; ++q) {
-                                const float u = __uint_as_float(v[q]);
-                                dsum = fmaf(u, ag[q], dsum);
-                                dh[q] = rg * u * dh[q];
-                                ag[q] = rg * ag[q];
-                            }
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) {
-                                pd[c * 16 + q] = pack_bf16x2(dh[2 * q], dh[2 * q + 1]);
-                                pa[c * 16 + q] = pack_bf16x2(ag[2 * q], ag[2 * q + 1]);
+                            for (int q = 0; q < 16; ++q) {         // in pairs: the launch is bound by its epilogue's instructions
+                                const unsigned long long u = f2_pack(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1]));
+                                const unsigned long long a = f2_pack(ag[2 * q], ag[2 * q + 1]);
+                                f2_fma(dsum2, u, a);
+                                const float2 dv = f2_unpack(f2_mul(f2_mul(rg2, u), f2_pack(dh[2 * q], dh[2 * q + 1])));
+                                const float2 av = f2_unpack(f2_mul(rg2, a));
+                                pd[c * 16 + q] = pack_bf16x2(dv.x, dv.y);
+                                pa[c * 16 + q] = pack_bf16x2(av.x, av.y);
                             }
                         }
                         stage_store_packed(pd, &tmC0, col0 + g * 64, wrow0);
                         stage_store_packed(pa, &tmC1, col0 + g * 64, wrow0);
                     }
                     constexpr int DG = dg_cols_per_tile(BN);
-                    if (wsel < DG) dg_part[row * (n_tiles_mat * DG) + (col0 / BN) * DG + wsel] = rv * dsum;
+                    if (wsel < DG) {
+                        const float2 ds = f2_unpack(dsum2);
+                        dg_part[row * (n_tiles_mat * DG) + (col0 / BN) * DG + wsel] = rv * (ds.x + ds.y);
+                    }
                 } else if constexpr (EPI == kAttBackward) {
                     // u = dy_g W^o^T of a 64-wide head, o the head's attention output, w the row's combine weight:
                     // C = w u, C1 = w o, delta = w <u, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that
