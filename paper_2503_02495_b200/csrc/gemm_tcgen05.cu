@@ -308,15 +308,22 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             return w;
         };
         uint8_t* stg = smem + Cf::STAGES * Cf::STAGE + 1024 + (warp - 2) * Cf::STG_BYTES;
-        auto stage_store_packed = [&](const uint32_t* f, const CUtensorMap* tm, int c0, int r0) {      // the same for bf16 pairs
+        // the backward epilogues: 32 columns of both outputs at a time (bf16 pairs), half of the staging piece each with 64-byte
+        // rows: one wait per 32 columns, for stores that were issued a whole chunk's arithmetic ago
+        // (one output after the other through the whole piece, each waiting for the store before it: activation backward of
+        // the image block 60 us, 45 now; wide block 37 and 31; whole training steps 731 -> 714 and 556 -> 547)
+        auto stage_both = [&](const uint32_t* f0, const uint32_t* f1, int c0, int r0) {
             if (lane == 0) bulk_wait_read();
             __syncwarp();
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                *(uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = make_uint4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
+            for (int c = 0; c < 4; ++c) {
+                const int at = lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4);
+                *(uint4*)(stg + at) = make_uint4(f0[4 * c], f0[4 * c + 1], f0[4 * c + 2], f0[4 * c + 3]);
+                *(uint4*)(stg + 2048 + at) = make_uint4(f1[4 * c], f1[4 * c + 1], f1[4 * c + 2], f1[4 * c + 3]);
+            }
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) { tma_store_2d(tm, stg, c0, r0); bulk_commit(); }
+            if (lane == 0) { tma_store_2d(&tmC0, stg, c0, r0); tma_store_2d(&tmC1, stg + 2048, c0, r0); bulk_commit(); }
         };
         // 64 values of this thread's row -> bf16 -> this warp's staging piece (row = lane, 128B swizzle) -> TMA store
         auto stage_store = [&](const float* f, const CUtensorMap* tm, int c0, int r0) {
@@ -338,48 +345,55 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if constexpr (ROPE) {                            // (two dependent look-ups, under the tile's main loop)
                 if (half < blocks) tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e]);
             }
+            const int wrow0 = row0 + half * BM + quarter * 32;           // first row of this warp's piece
+            const size_t row = (size_t)wrow0 + lane;
+            // the backward epilogues' second operand (h or o): 32 columns ahead, the first ones under the tile's main loop
+            [[maybe_unused]] float rg = 0.f, rv = 0.f;
+            [[maybe_unused]] uint4 hv[4];
+            [[maybe_unused]] const uint4* hp = nullptr;
+            if constexpr (EPI != kForward) {
+                if (half < blocks) {
+                    rg = row_gate[row]; rv = row_valid[row];
+                    hp = (const uint4*)(bwd_h + row * N + col0);
+                    if (g_lo < g_hi) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) hv[q] = hp[g_lo * 8 + q];
+                    }
+                }
+            }
             const bool ready = mbar_wait(&ctl->tfull[acc], acc_phase, abort_flag, status) && !*abort_flag;
             if (!__all_sync(0xffffffffu, ready)) break;      // warp-uniform: tcgen05.ld below is warp-collective
             tc_fence_after();
             if (half < blocks) {
-                const int wrow0 = row0 + half * BM + quarter * 32;       // first row of this warp's piece
-                const size_t row = (size_t)wrow0 + lane;
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (MT == 2 ? half * BN : acc * Cf::ACC_STRIDE);
                 if constexpr (BWD) {
-                    // (32 columns at a time, kept packed until the 64-column pieces are complete: few enough registers for
-                    // eight warps; with four warps of 64 columns the image block's launch took 68 us)
-                    const float rg = row_gate[row], rv = row_valid[row];
                     const unsigned long long rg2 = f2_pack(rg, rg);
                     unsigned long long dsum2 = 0ull;
 #pragma unroll 1
-                    for (int g = g_lo; g < g_hi; ++g) {
-                        uint32_t pd[32], pa[32];             // dh and gated phi(h) of the piece, bf16 pairs
-                        const uint4* hp = (const uint4*)(bwd_h + row * N + col0 + g * 64);
+                    for (int ch = 2 * g_lo; ch < 2 * g_hi; ++ch) {
+                        uint32_t v[32];
+                        tmem_ld32(taddr + ch * 32, v);
+                        float dh[32], ag[32];
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            uint32_t v[32];
-                            tmem_ld32(taddr + g * 64 + c * 32, v);
-                            uint4 hv[4];
+                        for (int q = 0; q < 4; ++q) unpack16<__nv_bfloat16>(hv[q], dh + 8 * q);     // h
+                        if (ch + 1 < 2 * g_hi) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) hv[q] = hp[c * 4 + q];
-                            tmem_ld_wait();
-                            float dh[32], ag[32];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) unpack16<__nv_bfloat16>(hv[q], dh + 8 * q);     // h
-                            act_and_deriv_n<32>(dh, ag, dh, act);                                         // ag = phi(h), dh = phi'(h)
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) {         // in pairs: the launch is bound by its epilogue's instructions
-                                const unsigned long long u = f2_pack(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1]));
-                                const unsigned long long a = f2_pack(ag[2 * q], ag[2 * q + 1]);
-                                f2_fma(dsum2, u, a);
-                                const float2 dv = f2_unpack(f2_mul(f2_mul(rg2, u), f2_pack(dh[2 * q], dh[2 * q + 1])));
-                                const float2 av = f2_unpack(f2_mul(rg2, a));
-                                pd[c * 16 + q] = pack_bf16x2(dv.x, dv.y);
-                                pa[c * 16 + q] = pack_bf16x2(av.x, av.y);
-                            }
+                            for (int q = 0; q < 4; ++q) hv[q] = hp[ch * 4 + 4 + q];
                         }
-                        stage_store_packed(pd, &tmC0, col0 + g * 64, wrow0);
-                        stage_store_packed(pa, &tmC1, col0 + g * 64, wrow0);
+                        act_and_deriv_n<32>(dh, ag, dh, act);                                         // ag = phi(h), dh = phi'(h)
+                        tmem_ld_wait();
+                        uint32_t pd[16], pa[16];                   // dh and gated phi(h), bf16 pairs
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {             // in pairs: the launch is bound by its epilogue's instructions
+                            const unsigned long long u = f2_pack(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1]));
+                            const unsigned long long a = f2_pack(ag[2 * q], ag[2 * q + 1]);
+                            f2_fma(dsum2, u, a);
+                            const float2 dv = f2_unpack(f2_mul(f2_mul(rg2, u), f2_pack(dh[2 * q], dh[2 * q + 1])));
+                            const float2 av = f2_unpack(f2_mul(rg2, a));
+                            pd[q] = pack_bf16x2(dv.x, dv.y);
+                            pa[q] = pack_bf16x2(av.x, av.y);
+                        }
+                        stage_both(pd, pa, col0 + ch * 32, wrow0);
                     }
                     constexpr int DG = dg_cols_per_tile(BN);
                     if (wsel < DG) {
@@ -390,33 +404,36 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     // u = dy_g W^o^T of a 64-wide head, o the head's attention output, w the row's combine weight:
                     // C = w u, C1 = w o, delta = w <u, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that
                     // weigh nothing, whose o may never have been written)
-                    const float rg = row_gate[row], rv = row_valid[row];
                     if (g_lo == 0 && (int)row >= att.expert_end[e]) {       // padding rows of dq, dk, dv: no other kernel writes them
                         uint4* z = (uint4*)(att.dqkv + row * (3 * (size_t)N) + 3 * col0);
                         for (int q = 0; q < 3 * BN / 8; ++q) z[q] = make_uint4(0, 0, 0, 0);
                     }
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g) {
-                        uint32_t v[64];
-                        tmem_ld32(taddr + g * 64, v);
-                        tmem_ld32(taddr + g * 64 + 32, v + 32);
-                        const uint4* op = (const uint4*)(bwd_h + row * N + col0 + g * 64);
-                        uint4 ov[8];
+                        float dot = 0.f;
+#pragma unroll 1
+                        for (int ch = 2 * g; ch < 2 * g + 2; ++ch) {
+                            uint32_t v[32];
+                            tmem_ld32(taddr + ch * 32, v);
+                            float o[32];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) ov[q] = op[q];
-                        tmem_ld_wait();
-                        float u[64], o[64], dot = 0.f;
+                            for (int q = 0; q < 4; ++q) unpack16<__nv_bfloat16>(hv[q], o + 8 * q);
+                            if (ch + 1 < 2 * g_hi) {
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) unpack16<__nv_bfloat16>(ov[q], o + 8 * q);
+                                for (int q = 0; q < 4; ++q) hv[q] = hp[ch * 4 + 4 + q];
+                            }
+                            tmem_ld_wait();
+                            uint32_t pu[16], po[16];
 #pragma unroll
-                        for (int q = 0; q < 64; ++q) {
-                            u[q] = __uint_as_float(v[q]);
-                            dot = fmaf(u[q], o[q], dot);
-                            u[q] = rg != 0.f ? u[q] * rg : 0.f;
-                            o[q] = rg != 0.f ? o[q] * rg : 0.f;
+                            for (int q = 0; q < 16; ++q) {
+                                const float u0 = __uint_as_float(v[2 * q]), u1 = __uint_as_float(v[2 * q + 1]);
+                                dot = fmaf(u0, o[2 * q], dot);
+                                dot = fmaf(u1, o[2 * q + 1], dot);
+                                pu[q] = rg != 0.f ? pack_bf16x2(u0 * rg, u1 * rg) : 0u;
+                                po[q] = rg != 0.f ? pack_bf16x2(o[2 * q] * rg, o[2 * q + 1] * rg) : 0u;
+                            }
+                            stage_both(pu, po, col0 + ch * 32, wrow0);
                         }
-                        stage_store(u, &tmC0, col0 + g * 64, wrow0);
-                        stage_store(o, &tmC1, col0 + g * 64, wrow0);
                         const size_t h = row * (N / 64) + col0 / 64 + g;
                         att.delta[h] = rg != 0.f ? rg * dot : 0.f;
                         dg_part[h] = rv != 0.f ? dot : 0.f;
@@ -545,8 +562,11 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
         const uint64_t str[1] = {(uint64_t)g.N * 2};
         const uint32_t box[2] = {64, 32};
         const void* Cs[3] = {g.C, g.C1 ? g.C1 : g.C, g.C2 ? g.C2 : g.C};
+        const uint32_t box_bwd[2] = {32, 32};             // the backward epilogues' pieces
         for (int q = 0; q < 3; ++q)
-            if (!make_tmap(&tmC[q], Cs[q], 2, dims, str, box)) return UOE_ERR_CUDA;
+            if (!(EPI == kForward ? make_tmap(&tmC[q], Cs[q], 2, dims, str, box)
+                                  : make_tmap(&tmC[q], Cs[q], 2, dims, str, box_bwd, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B)))
+                return UOE_ERR_CUDA;
         if (!make_tmap(&tmPre, g.pre ? g.pre : g.C, 2, dims, str, box)) return UOE_ERR_CUDA;
     }
     long long max_tiles = ((g.rows_max / BM + Cf::UNIT - 1) / Cf::UNIT + g.n) * (BN == 192 ? 1 : (g.N / BN) * nmat);
