@@ -325,15 +325,19 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             __syncwarp();
             if (lane == 0) { tma_store_2d(&tmC0, stg, c0, r0); tma_store_2d(&tmC1, stg + 2048, c0, r0); bulk_commit(); }
         };
-        // 64 values of this thread's row -> bf16 -> this warp's staging piece (row = lane, 128B swizzle) -> TMA store
+        // the forward epilogue: 32 columns of this thread's row -> bf16 -> one half of the staging piece (64-byte rows) -> TMA
+        // store; the halves take turns, so a chunk waits for the store before the last one only
+        int stg_half = 0;
         auto stage_store = [&](const float* f, const CUtensorMap* tm, int c0, int r0) {
-            if (lane == 0) bulk_wait_read();          // the previous store has finished reading the piece
+            if (lane == 0) bulk_wait_read_but_one();
             __syncwarp();
+            uint8_t* p = stg + stg_half * 2048;
+            stg_half ^= 1;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) *(uint4*)(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = pack8(f + 8 * c);
+            for (int c = 0; c < 4; ++c) *(uint4*)(p + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = pack8(f + 8 * c);
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) { tma_store_2d(tm, stg, c0, r0); bulk_commit(); }
+            if (lane == 0) { tma_store_2d(tm, p, c0, r0); bulk_commit(); }
         };
         int e = 0;
         for (int tile = worker; tile < total_tiles; tile += workers) {
@@ -440,18 +444,20 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 } else {
 #pragma unroll 1
-                    for (int g = g_lo; g < g_hi; ++g) {
-                        uint32_t v[64];
-                        tmem_ld32(taddr + g * 64, v);
-                        tmem_ld32(taddr + g * 64 + 32, v + 32);
+                    for (int g = g_lo; g < g_hi; ++g)
+#pragma unroll (ROPE ? 2 : 1)
+                    for (int c = 0; c < 2; ++c) {
+                        const int col = g * 64 + c * 32;             // in the tile
+                        uint32_t v[32];
+                        tmem_ld32(taddr + col, v);
                         tmem_ld_wait();
-                        float f[64];
+                        float f[32];
 #pragma unroll
-                        for (int q = 0; q < 64; ++q) f[q] = __uint_as_float(v[q]);
+                        for (int q = 0; q < 32; ++q) f[q] = __uint_as_float(v[q]);
                         if (bias) {                                  // the expert's bias row (the in-place bias of the batched product)
-                            const uint4* bp = (const uint4*)(bias + (size_t)e * N + (SIDE3 ? 0 : col0) + g * 64);
+                            const uint4* bp = (const uint4*)(bias + (size_t)e * N + (SIDE3 ? 0 : col0) + col);
 #pragma unroll
-                            for (int q8 = 0; q8 < 8; ++q8) {
+                            for (int q8 = 0; q8 < 4; ++q8) {
                                 float bv[8];
                                 unpack16<__nv_bfloat16>(bp[q8], bv);
 #pragma unroll
@@ -462,10 +468,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             if ((SIDE3 ? g : mat) < 2) {
                                 // Eq. 32 on the float32 accumulators: the head's last channels, two MUFU operations per pair
 #pragma unroll
-                                for (int p = 0; p < 32; ++p) {
-                                    if (p >= rope.pair0) {
+                                for (int p = 0; p < 16; ++p) {
+                                    if (c * 16 + p >= rope.pair0) {
                                         float cs, sn;
-                                        rope_angle(rope, p, (float)max(tok, 0), cs, sn);
+                                        rope_angle(rope, c * 16 + p, (float)max(tok, 0), cs, sn);
                                         const float a0 = f[2 * p], a1 = f[2 * p + 1];
                                         f[2 * p] = a0 * cs - a1 * sn;
                                         f[2 * p + 1] = a0 * sn + a1 * cs;
@@ -473,15 +479,15 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 }
                             }
                         }
-                        if (pre) stage_store(f, &tmPre, col0 + g * 64, wrow0);
-                        act_apply_n<64>(f, act);
+                        if (pre) stage_store(f, &tmPre, col0 + col, wrow0);
+                        act_apply_n<32>(f, act);
                         if (blk_scale) {
                             const float sc = blk_scale[(row0 + half * BM) >> 7];
 #pragma unroll
-                            for (int q = 0; q < 64; ++q) f[q] *= sc;
+                            for (int q = 0; q < 32; ++q) f[q] *= sc;
                         }
-                        if (SIDE3) stage_store(f, g == 0 ? &tmC0 : (g == 1 ? &tmC1 : &tmC2), 0, wrow0);
-                        else stage_store(f, tmC, col0 + g * 64, wrow0);
+                        if (SIDE3) stage_store(f, g == 0 ? &tmC0 : (g == 1 ? &tmC1 : &tmC2), c * 32, wrow0);
+                        else stage_store(f, tmC, col0 + col, wrow0);
                     }
                 }
             }
@@ -560,14 +566,14 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     {
         const uint64_t dims[2] = {(uint64_t)g.N, (uint64_t)g.rows_max};
         const uint64_t str[1] = {(uint64_t)g.N * 2};
-        const uint32_t box[2] = {64, 32};
+        const uint32_t box[2] = {32, 32};
         const void* Cs[3] = {g.C, g.C1 ? g.C1 : g.C, g.C2 ? g.C2 : g.C};
-        const uint32_t box_bwd[2] = {32, 32};             // the backward epilogues' pieces
+        auto out_map = [&](CUtensorMap* tm, const void* p) {
+            return make_tmap(tm, p, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B);
+        };
         for (int q = 0; q < 3; ++q)
-            if (!(EPI == kForward ? make_tmap(&tmC[q], Cs[q], 2, dims, str, box)
-                                  : make_tmap(&tmC[q], Cs[q], 2, dims, str, box_bwd, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B)))
-                return UOE_ERR_CUDA;
-        if (!make_tmap(&tmPre, g.pre ? g.pre : g.C, 2, dims, str, box)) return UOE_ERR_CUDA;
+            if (!out_map(&tmC[q], Cs[q])) return UOE_ERR_CUDA;
+        if (!out_map(&tmPre, g.pre ? g.pre : g.C)) return UOE_ERR_CUDA;
     }
     long long max_tiles = ((g.rows_max / BM + Cf::UNIT - 1) / Cf::UNIT + g.n) * (BN == 192 ? 1 : (g.N / BN) * nmat);
     const int walkers = PAIR ? max_pairs : sm_count();

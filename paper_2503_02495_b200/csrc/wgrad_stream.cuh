@@ -7,7 +7,7 @@ namespace uoe {
 // One family of weight-gradient matrices [M, N], one per expert.
 struct WProblem {
     int M, N, BN, m_tiles, n_tiles;
-    int w;                    // cost of one 64-row K block of a tile (128-byte row pieces loaded)
+    int w;                    // cost of one 64-row K block of a tile (tile_shape)
     int transposed;           // out[0] is [n, N, M]
     int out_cols;             // columns per output tensor (N, or N / 3 with three tensors side by side)
     float* out[3];            // [n, M, out_cols]

@@ -13,7 +13,7 @@
 // than two thirds are the same for every width (kStepCost).  The tiles
 // of both problems form one line, cut into equal pieces, one per CTA (one CTA per SM), whatever the load of the experts.
 // A tile inside one piece is written straight to its output; a tile cut by pieces leaves one partial tile per piece in
-// the scratch, and wgrad_reduce adds them in ascending order (in spare CTAs of the combine that ends the pass, or as a
+// the scratch, and wgrad_reduce adds them in ascending order (in spare CTAs of router_grad_kernel, or as a
 // launch of its own).  No CTA waits for another, every sum has a fixed order.
 //   warp 0      TMA producer, four-stage ring (P block [64 x 128], Q block [64 x BN])
 //   warp 1      MMA issuer: tcgen05.mma 128 x BN x 16, two accumulator sets (the write-out of a tile runs under the next)
