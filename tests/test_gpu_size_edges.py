@@ -94,6 +94,24 @@ def test_loads_and_balance_loss(n, k, m, L_valid):
     assert np.abs(lb.cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max()
 
 
+def test_more_samples_than_a_grid_dimension_holds():
+    """Scores of 65541 samples take two launches, the ticket runs through both.  Tolerance 2e-6: softmax values at most 1 from
+    float32 sums of 33 * 16 bfloat16 products (528 * 2^-24 * |logit| below 1, divided by 33 tokens)."""
+    import paper_2503_02495_b200 as uoe
+    B, L, d, n, k = 65541, 33, 16, 4, 2
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(B, L, d, device="cuda", generator=g).bfloat16()
+    Wr = (0.5 * torch.randn(d, n, device="cuda", generator=g)).bfloat16()
+    r = uoe.uoe_route(uoe.Problem(B=B, L=L, L_valid=L, d=d, n=n, k=k, m=1, c=1, dtype="bf16"), x, Wr)
+    ref = torch.softmax(x.double().mean(1) @ Wr.double(), dim=1)
+    assert (r.p_samp.double() - ref).abs().max() <= 2e-6
+    assert (r.p_patch.reshape(B, n).double() - ref).abs().max() <= 2e-6
+    picked = ref.gather(1, r.expert_idx.long())
+    assert (picked.min(1).values >= ref.topk(k, dim=1).values.min(1).values - 2e-6).all()
+    rows = torch.bincount(r.expert_idx.flatten().long(), minlength=n) * L
+    assert torch.equal(r.expert_offsets.long().diff(), (rows + 127) // 128 * 128)
+
+
 # weight gradients cut into equal pieces over the SMs: ragged column tiles, 8-row slabs, one expert whose tiles are cut into
 # many pieces, experts without rows, routed copies, and the pass without gates (the cut tiles added by their own launch)
 def _bwd(**kw):
