@@ -406,15 +406,18 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 } else if constexpr (EPI == kAttBackward) {
                     // u = dy_g W^o^T of a 64-wide head, o the head's attention output, w the row's combine weight:
-                    // C = w u, C1 = w o, delta = w <u, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that
-                    // weigh nothing, whose o may never have been written)
+                    // C = w u, C1 = w o, delta = <C, o>, gate gradient = <u, o> on real tokens (exact zeros on rows that
+                    // weigh nothing, whose o may never have been written).  delta is taken from C as it is stored: the
+                    // attention backward subtracts it from <C, v_j> of every key, and what C's rounding adds to both cancels
+                    // only if it is the same rounding (with w <u, o> in its place the error of dW^q and dW^k was 1.1 to 2.3
+                    // times as large where the tokens of a sample have a mean in common)
                     if (g_lo == 0 && (int)row >= att.expert_end[e]) {       // padding rows of dq, dk, dv: no other kernel writes them
                         uint4* z = (uint4*)(att.dqkv + row * (3 * (size_t)N) + 3 * col0);
                         for (int q = 0; q < 3 * BN / 8; ++q) z[q] = make_uint4(0, 0, 0, 0);
                     }
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g) {
-                        float dot = 0.f;
+                        float dot = 0.f, dot_c = 0.f;
 #pragma unroll 1
                         for (int ch = 2 * g; ch < 2 * g + 2; ++ch) {
                             uint32_t v[32];
@@ -434,12 +437,14 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 dot = fmaf(u0, o[2 * q], dot);
                                 dot = fmaf(u1, o[2 * q + 1], dot);
                                 pu[q] = rg != 0.f ? pack_bf16x2(u0 * rg, u1 * rg) : 0u;
+                                dot_c = fmaf(__uint_as_float(pu[q] << 16), o[2 * q], dot_c);
+                                dot_c = fmaf(__uint_as_float(pu[q] & 0xffff0000u), o[2 * q + 1], dot_c);
                                 po[q] = rg != 0.f ? pack_bf16x2(o[2 * q] * rg, o[2 * q + 1] * rg) : 0u;
                             }
                             stage_both(pu, po, col0 + ch * 32, wrow0);
                         }
                         const size_t h = row * (N / 64) + col0 / 64 + g;
-                        att.delta[h] = rg != 0.f ? rg * dot : 0.f;
+                        att.delta[h] = rg != 0.f ? dot_c : 0.f;
                         dg_part[h] = rv != 0.f ? dot : 0.f;
                     }
                 } else {

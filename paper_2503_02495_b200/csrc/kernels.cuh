@@ -271,7 +271,7 @@ struct GemmArgs {
     // bf16 path, K-major weights, K split over k_mats weight tensors of the same shape (W, W1, W2: [n, N, K / k_mats] each)
     int k_mats = 0;
     // bf16 path, attention output's backward (att.delta set): with u = A @ W the gradient w.r.t. the attention output o
-    // (64-wide heads), o = bwd_h[r,:]:  C = w u, C1 = w o, delta[r, head] = w <u, o>, dg_part[r, head] = <u, o> (0 where
+    // (64-wide heads), o = bwd_h[r,:]:  C = w u, C1 = w o, delta[r, head] = <C as stored, o>, dg_part[r, head] = <u, o> (0 where
     // row_valid is 0), w = row_gate[r]; the padding rows of att.dqkv are zeroed
     AttBwd att;
     bool bwd = false;

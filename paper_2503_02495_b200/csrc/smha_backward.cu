@@ -5,7 +5,7 @@
 // In routed-row space, for the rows r of pair (b, i) with combine weight w_r (0 on pad-token rows):
 //   q, k, v = x_g W^{q,k,v}_i ; o, lse = attention(q, k, v)              recomputed (Eq. 28-34)
 //   do_raw  = dy_g W^o_i^T                                               grouped GEMM (K-major weights), whose epilogue makes
-//   dgate(patch) = sum_r <do_raw_r, o_r> ;  do = w do_raw ; og = w o ;  delta_{r,h} = sum_{c in head h} do o
+//   dgate(patch) = sum_r <do_raw_r, o_r> ;  do = w do_raw ; og = w o ;  delta_{r,h} = sum_{c in head h} do o (do as rounded)
 //             (as a kernel of its own this was another pass over do_raw, o, do and og: 20 us for the image block, B = 256)
 //   dq, dk, dv = attention backward(q, k, v, do, lse, delta)             -> one buffer [rows, 3 d_g]
 //   dx_g = [dq dk dv] [W^q_i W^k_i W^v_i]^T                              one grouped GEMM, K = 3 d_g, weights read in place

@@ -131,3 +131,37 @@ def test_smha_forward_and_backward_on_dynamic_capacity_routing():
     ref = orc.smha_backward(x.f64, Wq.f64, Wk.f64, Wv.f64, Wo.f64, Wr.f64, ro, dy.f64, w.d_h, True, False, True)
     for nm, g, rr in zip(NAMES, got, ref[:6]):
         assert rel_inf(to_f64(g), rr) <= TOL, nm
+
+
+@pytest.mark.parametrize("use_gate", [False, True])
+@pytest.mark.parametrize("l_p", [8, 32])          # 48 tokens per pair: one tile; 192: blocks streamed past tiles
+def test_score_gradients_vanish_for_equal_tokens(l_p, use_gate):
+    """Where a sample's tokens are all equal, so are its values: dP - delta is <do, v> - <do, o> with o = v and the gradient of
+    the scores is zero, if both products take do with the same rounding.  What may remain is the order of two float32 sums
+    of 64 products each, 2 * 64 * 2^-23 of the sum of their magnitudes; do rounded for one of them only (2^-9 per product)
+    leaves some thirty times that, all with one sign since every row of a sample gets the same dy."""
+    import paper_2503_02495_b200 as uoe
+    w = _w(B=3, L=12 * l_p, L_valid=12 * l_p, m=12, c=6, n=2, k=2, H=4)
+    x = gen.store(np.repeat(gen.normal(3, 1, (w.B, 1, w.d)), w.L, axis=1), "bf16")
+    dy = gen.store(np.repeat(gen.normal(3, 2, (w.B, 1, w.d)), w.L, axis=1), "bf16")
+    Wr = gen.make_router(w, "att")
+    ws = gen.make_attn_weights(w)
+    Wq, Wk, Wv, Wo = (t.f64 for t in ws)
+    prob = problem_of(w, "att", residual=False, gate=use_gate)
+    xd, Wrd = to_dev(x), to_dev(Wr)
+    r = uoe.uoe_route(prob, xd, Wrd)
+    _, dWq, dWk, *_ = uoe.uoe_smha_backward(prob, xd, *(to_dev(t) for t in ws), Wrd, r, to_dev(dy))
+    bound = np.zeros((2,) + Wq.shape)
+    for b in range(w.B):
+        for s in range(w.k):
+            e, gates = int(r.expert_idx[b, s]), to_f64(r.gate)[b, s]
+            xb = x.f64[b, 0]
+            q, k, v, do = xb @ Wq[e], xb @ Wk[e], xb @ Wv[e], dy.f64[b, 0] @ Wo[e].T
+            for h in range(0, Wq.shape[2], 64):
+                rows = np.abs(do[h:h + 64] * v[h:h + 64]).sum() * l_p * gates.sum()
+                for t, other in enumerate((k, q)):
+                    bound[t, e][:, h:h + 64] += 2 * 64 * 2.0 ** -23 * rows / 8 * np.abs(np.outer(xb, other[h:h + 64]))
+    for got, lim in ((dWq, bound[0]), (dWk, bound[1])):
+        ratio = (np.abs(to_f64(got)) / (1.02 * lim + 1e-30)).max()
+        print(f"largest share of the bound: {ratio:.3f}")
+        assert ratio <= 1
