@@ -417,7 +417,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g) {
-                        float dot = 0.f, dot_c = 0.f;
+                        const unsigned long long rg2 = f2_pack(rg, rg);
+                        unsigned long long dot2 = 0ull, dot_c2 = 0ull;         // <u, o> and <C, o>, even and odd columns
 #pragma unroll 1
                         for (int ch = 2 * g; ch < 2 * g + 2; ++ch) {
                             uint32_t v[32];
@@ -433,19 +434,20 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             uint32_t pu[16], po[16];
 #pragma unroll
                             for (int q = 0; q < 16; ++q) {
-                                const float u0 = __uint_as_float(v[2 * q]), u1 = __uint_as_float(v[2 * q + 1]);
-                                dot = fmaf(u0, o[2 * q], dot);
-                                dot = fmaf(u1, o[2 * q + 1], dot);
-                                pu[q] = rg != 0.f ? pack_bf16x2(u0 * rg, u1 * rg) : 0u;
-                                dot_c = fmaf(__uint_as_float(pu[q] << 16), o[2 * q], dot_c);
-                                dot_c = fmaf(__uint_as_float(pu[q] & 0xffff0000u), o[2 * q + 1], dot_c);
-                                po[q] = rg != 0.f ? pack_bf16x2(o[2 * q] * rg, o[2 * q + 1] * rg) : 0u;
+                                const unsigned long long u = f2_pack(__uint_as_float(v[2 * q]), __uint_as_float(v[2 * q + 1]));
+                                const unsigned long long o2 = f2_pack(o[2 * q], o[2 * q + 1]);
+                                const float2 wu = f2_unpack(f2_mul(u, rg2)), wo = f2_unpack(f2_mul(o2, rg2));
+                                pu[q] = rg != 0.f ? pack_bf16x2(wu.x, wu.y) : 0u;
+                                po[q] = rg != 0.f ? pack_bf16x2(wo.x, wo.y) : 0u;
+                                f2_fma(dot2, u, o2);
+                                f2_fma(dot_c2, f2_pack(__uint_as_float(pu[q] << 16), __uint_as_float(pu[q] & 0xffff0000u)), o2);
                             }
                             stage_both(pu, po, col0 + ch * 32, wrow0);
                         }
                         const size_t h = row * (N / 64) + col0 / 64 + g;
-                        att.delta[h] = rg != 0.f ? dot_c : 0.f;
-                        dg_part[h] = rv != 0.f ? dot : 0.f;
+                        const float2 dot = f2_unpack(dot2), dot_c = f2_unpack(dot_c2);
+                        att.delta[h] = rg != 0.f ? dot_c.x + dot_c.y : 0.f;
+                        dg_part[h] = rv != 0.f ? dot.x + dot.y : 0.f;
                     }
                 } else {
 #pragma unroll 1
