@@ -23,8 +23,9 @@ struct PlanPtrs {
     float* row_gate = nullptr;   // [Rmax]   backward only: combine weight of each routed row (0 on pad-token rows and unused slots)
     float* row_valid = nullptr;  // [Rmax]   backward only: 1 on rows that hold a real token, else 0
     int* src_patch = nullptr;    // [Rmax/l_p] source patch (b*m + j) of every l_p-row block of the routed buffers, -1 = zero rows
-    int* slot_pair = nullptr;    // [n,B]    pair (b*k + s) of the q-th sample in expert i's region (with the plan written by the
-                                 //          router kernel it also replaces src_patch, which that plan does not fill)
+    int* slot_pair = nullptr;    // which pair (b*k + s) a place in an expert's region belongs to.  Plan written by the router
+                                 //          kernel: [n,B], the q-th sample of expert i (it also replaces src_patch, which that
+                                 //          plan does not fill); by plan_kernel: indexed by row, pair_slot_by_row
     bool inv_relative = false;   // inv_row holds offsets from pair_row (plan written by the router kernel)
     // plan written by the router kernel, whole samples per expert (every chosen expert takes every patch that holds a
     // real token, Eq. 21-26): slot u of a pair is patch u, so inv_row, inv_gate and patch_idx are neither written nor
@@ -63,10 +64,19 @@ uoe_status route_run(const uoe_problem* prob, const void* x, const void* W_r, co
 inline bool can_fuse_gather(const Dims& D) {
     return D.bf16 && D.l_p % 8 == 0 && 128 % D.l_p == 0 && D.d % 64 == 0;
 }
+// Index into slot_pair as plan_kernel fills it, for the q-th pair of a region that begins at row `off`.  With 2^shift <= l_a
+// a region spans at least 2^shift rows per pair, so off >> shift grows by at least one per pair from region to region and no
+// two pairs share an entry, however many slots of a caller's routing name one expert ([n,B] has room for one per sample).
+inline int pair_slot_shift(int l_a) { int s = 0; while ((2 << s) <= l_a && s < 30) ++s; return s; }
+__host__ __device__ inline size_t pair_slot_by_row(int off, int q, int shift) { return (size_t)(off >> shift) + q; }
+inline size_t slot_pair_entries(const Dims& D) {
+    const size_t by_sample = (size_t)D.n * D.B, by_row = (size_t)(D.Rmax >> pair_slot_shift(D.l_a)) + 1;
+    return by_sample > by_row ? by_sample : by_row;
+}
 inline size_t plan_bytes(const Dims& D, bool with_rows = false) {
     return align_up((size_t)D.B * D.k * 4, 1024) + 2 * align_up((size_t)D.B * D.m * D.k * 4, 1024) + 1024 +
            (with_rows ? 2 * align_up((size_t)D.Rmax * 4, 1024) : 0) + align_up((size_t)(D.Rmax / D.l_p + 1) * 4, 1024) +
-           align_up((size_t)D.n * D.B * 4, 1024);
+           align_up(slot_pair_entries(D) * 4, 1024);
 }
 inline PlanPtrs plan_ptrs(const Dims& D, char* base, bool with_rows = false) {
     PlanPtrs p;
@@ -93,10 +103,11 @@ inline PlanPtrs plan_ptrs(const Dims& D, char* base, bool with_rows = false) {
 // pair that owns the block (slot_pair) and that pair's selected patches (patch_idx).
 struct SrcMap {
     const int* src_patch = nullptr;
-    const int* slot_pair = nullptr;    // [n,B]
+    const int* slot_pair = nullptr;    // as in PlanPtrs
     const int* patch_idx = nullptr;    // [B,k,c]
     const int* expert_end = nullptr;   // [n]
     int B = 0, k = 0, c = 0, m = 0, l_p = 0;
+    int slot_shift = -1;               // >= 0: slot_pair as plan_kernel fills it (pair_slot_by_row)
     int n_elig = -1;                   // >= 0: slot u of a pair is patch u for u < n_elig (whole samples per expert), patch_idx is not read
     __host__ __device__ bool on() const { return src_patch != nullptr || slot_pair != nullptr; }
 };
@@ -126,6 +137,7 @@ inline SrcMap row_map_of(const Dims& D, const PlanPtrs& P, const int* patch_idx)
     SrcMap g = src_map_of(D, P, patch_idx);
     g.src_patch = nullptr;
     g.slot_pair = P.slot_pair; g.patch_idx = patch_idx; g.expert_end = P.expert_end;
+    if (!P.inv_relative) g.slot_shift = pair_slot_shift(D.l_a);
     return g;
 }
 #ifdef __CUDACC__
@@ -140,7 +152,9 @@ __device__ __forceinline__ void rope_angle(const Rope& rp, int p, float t, float
 __device__ __forceinline__ int source_row(const SrcMap& g, int r, int e, int off_e) {
     if (r >= g.expert_end[e]) return -1;
     const int rel = r - off_e, l_a = g.c * g.l_p;
-    const int pair = g.slot_pair[(size_t)e * g.B + rel / l_a];
+    const int q = rel / l_a;
+    const int pair = g.slot_pair[g.slot_shift >= 0 ? pair_slot_by_row(off_e, q, g.slot_shift) : (size_t)e * g.B + q];
+    if (pair < 0 || pair >= g.B * g.k) return -1;      // rows that a slot left out of the plan left without a pair
     const int u = (rel % l_a) / g.l_p;
     const int pj = g.n_elig >= 0 ? (u < g.n_elig ? u : -1) : g.patch_idx[(size_t)pair * g.c + u];
     return pj >= 0 && pj < g.m ? ((pair / g.k) * g.m + pj) * g.l_p + rel % g.l_p : -1;

@@ -70,7 +70,8 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
     __syncthreads();
     // gate = P_samp * P_patch: a warp per chosen expert, lanes over its slots
     for (int s = warp; s < k; s += kGradThreads / 32) {
-        const int i = expert_idx[(size_t)b * k + s];
+        int i = expert_idx[(size_t)b * k + s];
+        i = (unsigned)i < (unsigned)n ? i : 0;            // (the plan kernel has reported an index out of range)
         float acc = 0.f;
         for (int u = lane; u < c; u += 32) {
             const int j = patch_idx[((size_t)b * k + s) * c + u];

@@ -9,14 +9,15 @@ constexpr int kThreads = 256;
 
 // ---------------------------------------------------------------------------------------------
 // pair rows for many samples: one CTA passes over expert_idx [B,k] once, a warp per expert, 32 samples per step,
-// and writes where every (sample, slot) pair's rows start (samples ascending inside an expert's region).  O(B k)
-// work in all, where plan_kernel's own scan of the earlier samples is O(B k) per sample.
+// and writes where every (sample, slot) pair's rows start (samples, then slots ascending inside an expert's region) and
+// the table that leads back from there.  O(B k) work in all, where plan_kernel's own scan of the earlier samples is
+// O(B k) per sample.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPlanScanMaxB = 512;        // up to here every sample's CTA scans the earlier samples itself
 
 __global__ void __launch_bounds__(1024)
 plan_rows_kernel(const int* __restrict__ expert_idx, const int* __restrict__ offsets, int B, int n, int k, int l_a,
-                 int* __restrict__ pair_row, int* status) {
+                 int* __restrict__ pair_row, int* __restrict__ slot_pair, int slot_shift, int rows_max) {
     pdl_trigger();
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -25,16 +26,23 @@ plan_rows_kernel(const int* __restrict__ expert_idx, const int* __restrict__ off
         int running = 0;
         for (int b0 = 0; b0 < B; b0 += 32) {
             const int b = b0 + lane;
-            int slot = -1;
+            unsigned slots = 0;                 // this sample's slots that name expert i (a caller's routing may repeat one)
             if (b < B)
-                for (int s = 0; s < k; ++s) {
-                    const int e = expert_idx[(size_t)b * k + s];
-                    if (e < 0 || e >= n) set_status(status, UOE_ERR_DEVICE_INDEX);
-                    if (e == i) slot = s;
-                }
-            const unsigned ball = __ballot_sync(0xffffffffu, slot >= 0);
-            if (slot >= 0) pair_row[(size_t)b * k + slot] = off_i + (running + __popc(ball & ((1u << lane) - 1u))) * l_a;
-            running += __popc(ball);
+                for (int s = 0; s < k; ++s)
+                    if (expert_idx[(size_t)b * k + s] == i) slots |= 1u << s;
+            int incl = __popc(slots);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            int q = running + incl - __popc(slots);
+            for (unsigned left = slots; left; left &= left - 1, ++q) {
+                const int pair = b * k + __ffs(left) - 1, row = off_i + q * l_a;
+                pair_row[pair] = row;
+                if (row >= 0 && row <= rows_max - l_a) slot_pair[pair_slot_by_row(off_i, q, slot_shift)] = pair;
+            }
+            running += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
 }
@@ -50,13 +58,15 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             int* __restrict__ pair_row, int* __restrict__ inv_row, float* __restrict__ inv_gate,
             int* __restrict__ expert_end, int* status, float* __restrict__ row_gate, float* __restrict__ row_valid,
             int Lv, int use_gate, int* __restrict__ src_patch, const PlanTails tails,
-            long long rows_max, int rows_given /* pair_row already holds every pair's first row (plan_rows_kernel) */,
-            int* __restrict__ slot_pair) {
+            long long rows_max, int rows_given /* pair_row and slot_pair are already there (plan_rows_kernel) */,
+            int* __restrict__ slot_pair, int slot_shift) {
     pdl_trigger();
     pdl_wait();
     extern __shared__ int s_dyn[];
     int* s_pi = s_dyn;                         // [k*c] patch indices of this sample
     float* s_g = (float*)(s_dyn + k * c);      // [k*c] gates
+    // A slot that names no expert is reported and given the last rows that hold a pair, so that whatever goes by pairs stays
+    // inside the buffers (its sample's results mean nothing; no other sample reads those rows).
     __shared__ int my_e[32], prow[32], hist[33], offs[34];
     const int b = blockIdx.x, tid = threadIdx.x, NT = blockDim.x;      // NT: 128 or 512 (long per-row arrays)
     const int l_a = c * l_p;
@@ -65,7 +75,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
     // ---- one round of loads ----
     if (tid < k) {
         int e = expert_idx[b * k + tid];
-        if (e < 0 || e >= n) { set_status(status, UOE_ERR_DEVICE_INDEX); e = 0; }
+        if (e < 0 || e >= n) { set_status(status, UOE_ERR_DEVICE_INDEX); e = -1; }
         my_e[tid] = e;
     }
     if (tid <= n) offs[tid] = offsets[tid];
@@ -90,20 +100,26 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
     }
     __syncthreads();
     if (tid < k) {
-        const int row = rows_given ? pair_row[b * k + tid] : offs[my_e[tid]] + hist[my_e[tid]] * l_a;
+        const int e = my_e[tid];
+        // pairs of this expert in front of this one: of earlier samples, and of this one (a caller's routing may repeat an expert)
+        const unsigned same = __match_any_sync(k < 32 ? (1u << k) - 1u : 0xffffffffu, e);
+        int row = (int)rows_max - l_a;
+        if (e >= 0) {
+            const int q = hist[e] + __popc(same & ((1u << tid) - 1u));
+            row = rows_given ? pair_row[b * k + tid] : offs[e] + q * l_a;
+            if (!rows_given) slot_pair[pair_slot_by_row(offs[e], q, slot_shift)] = b * k + tid;
+        }
         prow[tid] = row;
-        if (!rows_given) pair_row[b * k + tid] = row;
-        slot_pair[(size_t)my_e[tid] * B + (row - offs[my_e[tid]]) / l_a] = b * k + tid;
+        pair_row[b * k + tid] = row;
     }
     __syncthreads();
     for (int idx = tid; idx < m * k; idx += NT) {          // inverse map: which routed rows feed patch j
         const int j = idx / k, s = idx % k;
-        int row = -1;
-        float g = 0.f;
+        int slot = -1;
         for (int u = 0; u < c; ++u)
-            if (s_pi[s * c + u] == j) { row = prow[s] + u * l_p; g = s_g[s * c + u]; }
-        inv_row[((size_t)b * m + j) * k + s] = row;
-        inv_gate[((size_t)b * m + j) * k + s] = g;
+            if (s_pi[s * c + u] == j) slot = u;
+        inv_row[((size_t)b * m + j) * k + s] = slot >= 0 ? prow[s] + slot * l_p : -1;
+        inv_gate[((size_t)b * m + j) * k + s] = slot >= 0 ? s_g[s * c + slot] : 0.f;
     }
     // source patch of every l_p-row block (used when the GEMM gathers its own A operand)
     for (int idx = tid; idx < k * c; idx += NT) {
@@ -123,7 +139,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             __syncthreads();
             if (tid < n) expert_end[tid] = s_end[tid];
         } else {
-            if (tid < k) atomicAdd(&hist[my_e[tid]], 1);
+            if (tid < k && my_e[tid] >= 0) atomicAdd(&hist[my_e[tid]], 1);
             __syncthreads();
             if (tid < n) s_end[tid] = expert_end[tid] = offs[tid] + hist[tid] * l_a;
         }
@@ -431,14 +447,15 @@ uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_id
     const bool many = D.B > kPlanScanMaxB;
     if (many) {
         ProfScope ps("plan_rows", s);
-        launch_k(plan_rows_kernel, dim3(1), dim3(1024), 0, s, expert_idx, offsets, D.B, D.n, D.k, D.l_a, P.pair_row, status);
+        launch_k(plan_rows_kernel, dim3(1), dim3(1024), 0, s, expert_idx, offsets, D.B, D.n, D.k, D.l_a, P.pair_row, P.slot_pair,
+                 pair_slot_shift(D.l_a), (int)D.Rmax);
         UOE_LAUNCHED();
     }
     ProfScope ps("plan", s);
     const int threads = (P.row_gate && (long long)D.k * D.l_a >= 4096) ? 512 : 128;      // the backward's per-row weights: k*l_a rows per sample
     launch_k(plan_kernel, dim3(D.B), dim3(threads), smem, s, expert_idx, patch_idx, gate, offsets, D.B, D.n, D.k, D.m, D.c, D.l_p,
                                     P.pair_row, P.inv_row, P.inv_gate, P.expert_end, status, P.row_gate, P.row_valid,
-                                    D.Lv, use_gate ? 1 : 0, P.src_patch, tails, D.Rmax, many ? 1 : 0, P.slot_pair);
+                                    D.Lv, use_gate ? 1 : 0, P.src_patch, tails, D.Rmax, many ? 1 : 0, P.slot_pair, pair_slot_shift(D.l_a));
     UOE_LAUNCHED();
     return UOE_OK;
 }
