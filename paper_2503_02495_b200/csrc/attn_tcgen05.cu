@@ -229,6 +229,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (!ok) break;
             const int n_kv = kv_tiles(qt * TQ, pc->n_valid);
             if (t_first >= n_kv) {
+                __syncwarp();                 // every lane has read n_valid, which the TMA warp overwrites after the arrival
                 if (el) mbar_arrive(&pc->q_empty);
                 continue;
             }

@@ -96,3 +96,21 @@ def test_expert_out_of_range_is_reported_by_the_backward(half, bad):
     with pytest.raises(layer.uoe.UoeError) as ei:
         layer.backward(gen.make_dy(w))
     assert ei.value.status == 6
+
+
+# more units than SMs (two pipelines per SM), with the output projection inside the kernel and without
+@pytest.mark.parametrize("heads", [1, 2])
+@pytest.mark.parametrize("B", [240])
+def test_pairs_without_a_patch(B, heads):
+    """Every third pair has only unused slots: no keys, no rows to add, no gradient; the others are not disturbed."""
+    w = _att(B=B, L=48, L_valid=45, m=3, c=2, n=2, H=2 * heads)
+    layer = Layer(w, "att")
+    patch = layer.r.patch_idx.cpu().numpy().copy()
+    patch.reshape(B * w.k, w.c)[::3] = -1
+    ro = layer.use(layer.r.expert_idx.cpu().numpy(), patch)
+    for _ in range(3):
+        assert rel_inf(to_f64(layer.forward()), layer.reference(ro)) <= 2e-2
+    dy = gen.make_dy(w)
+    ref = orc.smha_backward(layer.x.f64, *[q.f64 for q in layer.ws], layer.Wr.f64, ro, dy.f64, w.d_h, w.causal, False)
+    for g, r in zip(layer.backward(dy), ref):
+        assert rel_inf(to_f64(g), r) <= 2e-2
