@@ -558,12 +558,14 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
     int kv_end = min(n_valid, l_a);
     if (causal) kv_end = min(kv_end, q0 + TQ);
-    const int n_kv = (kv_end + TK - 1) / TK;               // >= 1: every pair holds a real token
+    const int n_kv = (kv_end + TK - 1) / TK;               // 0 for a pair without a patch: then nothing waits for Q either
     const int col_h = head * DH;
 
     if (tid == 0) {
-        mbar_arrive_expect_tx(&ctl->bar_q, TILE_BYTES);
-        tma_load_2d(sQ, &tmQ, col_h, row_base + q0, &ctl->bar_q);
+        if (n_kv > 0) {
+            mbar_arrive_expect_tx(&ctl->bar_q, TILE_BYTES);
+            tma_load_2d(sQ, &tmQ, col_h, row_base + q0, &ctl->bar_q);
+        }
         for (int t = 0; t < 2 && t < n_kv; ++t) {
             mbar_arrive_expect_tx(&ctl->bar_kv[t], 2 * TILE_BYTES);
             tma_load_2d(sK + t * TILE_BYTES, &tmK, col_h, row_base + t * TK, &ctl->bar_kv[t]);
@@ -783,7 +785,7 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         }
     }
     if (tid == 0 && *abort_flag) {           // let copies that may still be in flight land (bounded)
-        mbar_wait(&ctl->bar_q, 0, abort_flag, status);
+        if (n_kv > 0) mbar_wait(&ctl->bar_q, 0, abort_flag, status);
         for (int t = 0; t < 2 && t < n_kv; ++t) mbar_try_wait(&ctl->bar_kv[t], 0);
         if (FUSE_O) mbar_wait(&ctl->bar_w, 0, abort_flag, status);
     }

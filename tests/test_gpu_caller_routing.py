@@ -98,9 +98,9 @@ def test_expert_out_of_range_is_reported_by_the_backward(half, bad):
     assert ei.value.status == 6
 
 
-# more units than SMs (two pipelines per SM), with the output projection inside the kernel and without
+# few units (a CTA each) and more units than SMs (two pipelines per SM), with the output projection inside the kernel and without
 @pytest.mark.parametrize("heads", [1, 2])
-@pytest.mark.parametrize("B", [240])
+@pytest.mark.parametrize("B", [12, 240])
 def test_pairs_without_a_patch(B, heads):
     """Every third pair has only unused slots: no keys, no rows to add, no gradient; the others are not disturbed."""
     w = _att(B=B, L=48, L_valid=45, m=3, c=2, n=2, H=2 * heads)
