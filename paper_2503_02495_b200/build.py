@@ -27,7 +27,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
     sources = sorted(f for f in os.listdir(SRC) if f.endswith(".cu"))
-    headers = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith(".cuh")]
+    headers = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith((".cuh", ".h"))]
     headers.append(os.path.join(ROOT, "include", "uoe.h"))
     objs, jobs = [], []
     for f in sources:

@@ -1,13 +1,14 @@
 // The line of output tiles that wgrad_stream_kernel cuts into equal pieces, and the addition of the partial tiles.
 #pragma once
 #include "common.cuh"
+#include "wgrad_line.h"
 
 namespace uoe {
 
 // One family of weight-gradient matrices [M, N], one per expert.
 struct WProblem {
     int M, N, BN, m_tiles, n_tiles;
-    int w;                    // cost of one 64-row K block of a tile (tile_shape)
+    int w;                    // cost of one 64-row K block of a tile (wgrad_tile_shape)
     int transposed;           // out[0] is [n, N, M]
     int out_cols;             // columns per output tensor (N, or N / 3 with three tensors side by side)
     float* out[3];            // [n, M, out_cols]
@@ -23,11 +24,6 @@ struct WReduce {
 };
 
 constexpr int kReduceThreads = 512;
-
-// A tile counts as at least this many K blocks: writing its 128 KB out takes about as long, and an expert with few or no
-// rows has as many tiles as any other (uncounted, one CTA wrote all of an empty expert's zeros: 78 us instead of 50 for
-// the MLP half at B = 4, L = 2048, d = 1024, d_e = 512, n = 8 with one expert unused).
-constexpr int kMinTileKb = 4;
 
 #ifdef __CUDACC__
 struct WSched {

@@ -11,7 +11,7 @@
 //
 // Work split: an output tile is 128 x BN (BN <= 256); its cost is its 64-row K blocks times the time of one, of which more
 // than two thirds are the same for every width (kStepCost).  The tiles
-// of both problems form one line, cut into equal pieces, one per CTA (one CTA per SM), whatever the load of the experts.
+// of both problems form one line (wgrad_line.h), cut into equal pieces, one per CTA (one CTA per SM), whatever the load of the experts.
 // A tile inside one piece is written straight to its output; a tile cut by pieces leaves one partial tile per piece in
 // the scratch, and wgrad_reduce adds them in ascending order (in spare CTAs of router_grad_kernel, or as a
 // launch of its own).  No CTA waits for another, every sum has a fixed order.
@@ -28,15 +28,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BK = 64, BN_MAX = 256;
+constexpr int BM = kLineBM, BK = kLineBK, BN_MAX = kLineBNMax;
 constexpr int P_BYTES = BM * BK * 2, Q_BYTES = BN_MAX * BK * 2, STAGE = P_BYTES + Q_BYTES;
 constexpr int STAGES = 4;
 constexpr int EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS, STG_BYTES = 32 * 128;
 constexpr int CTL_BYTES = 2048;
-// The cost of a K block is kStepCost plus one per 64 columns of either operand: a block takes 1000 to 1500 cycles, most
-// of it the round trip of its copies whatever their width.  With the bytes alone as the cost (no constant part) the
-// pieces of narrow tiles were the last to end: image block, training 749 us -> 742, language-model block 279 -> 277.
-constexpr int kStepCost = 16;
 constexpr int SMEM = STAGES * STAGE + 1024 /*align slack*/ + CTL_BYTES + EPI_WARPS * STG_BYTES;
 
 struct SCtl {
@@ -264,15 +260,6 @@ wgrad_reduce_kernel(const __grid_constant__ WReduce r) {
     wgrad_reduce(r, blockIdx.x);
 }
 
-// Column tiles of at most 256, as equal as 64-wide blocks allow.
-void tile_shape(WProblem& p) {
-    p.n_tiles = (p.N + BN_MAX - 1) / BN_MAX;
-    p.BN = (p.N / 64 + p.n_tiles - 1) / p.n_tiles * 64;
-    p.n_tiles = (p.N + p.BN - 1) / p.BN;
-    p.m_tiles = p.M / BM;
-    p.w = kStepCost + (BM + p.BN) / 64;
-}
-
 }  // namespace
 
 size_t wgrad_stream_scratch_bytes() { return (size_t)2 * 148 * BM * BN_MAX * sizeof(float); }
@@ -289,7 +276,9 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     WArgs a;
     a.offsets = offsets; a.src_patch = src_patch; a.part = part; a.status = status;
     a.n = n; a.nprob = nprob; a.l_p = l_p > 0 ? l_p : 64; a.Bm = Bm;
-    long long cost = 0;                                       // bound on the whole line
+    a.pieces = sm_count() < 148 ? sm_count() : 148;
+    WTileShape shape[2];
+    int wmax = 0;
     for (int i = 0; i < nprob; ++i) {
         const WStreamProblem& in = probs[i];
         if (in.M % BM != 0 || in.N % 64 != 0) return UOE_ERR_UNSUPPORTED;
@@ -298,8 +287,9 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
         p.M = in.M; p.N = in.N; p.transposed = in.transposed ? 1 : 0;
         p.out_cols = in.out_cols > 0 ? in.out_cols : in.N;
         for (int q = 0; q < 3; ++q) p.out[q] = in.out[q];
-        tile_shape(p);
-        cost += (long long)p.m_tiles * p.n_tiles * p.w * (rows_max / BK + n);
+        const WTileShape t = shape[i] = wgrad_tile_shape(in.M, in.N);
+        p.BN = t.BN; p.m_tiles = t.m_tiles; p.n_tiles = t.n_tiles; p.w = t.w;
+        if (t.w > wmax) wmax = t.w;
         const int sub = l_p < BK ? l_p : BK;
         auto operand = [&](WOperand& o, CUtensorMap* tm, const void* base, int cols, int nblk, bool gather) {
             o.gather = gather ? 1 : 0; o.sub = gather ? sub : BK; o.nslab = BK / o.sub;
@@ -326,8 +316,7 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
             else if (!make_tmap(&a.maps[i].out[q], o, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return UOE_ERR_CUDA;
         }
     }
-    if (cost >= 0x7fffffffll) return UOE_ERR_UNSUPPORTED;
-    a.pieces = sm_count() < 148 ? sm_count() : 148;
+    if (!wgrad_line_fits(wgrad_line_bound(shape, nprob, n, rows_max), wmax, a.pieces)) return UOE_ERR_UNSUPPORTED;
     {
         ProfScope ps(label, s);
         launch_k(wgrad_stream_kernel, dim3(a.pieces), dim3(THREADS), (size_t)SMEM, s, a);

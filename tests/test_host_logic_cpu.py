@@ -13,3 +13,13 @@ def test_per_device_setup_bookkeeping(tmp_path):
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     assert r.stdout.strip() == "ok"
+
+
+def test_bound_on_the_weight_gradient_line(tmp_path):
+    exe = str(tmp_path / "wgrad_line_check")
+    src = os.path.join(ROOT, "tests", "host", "wgrad_line_check.cpp")
+    inc = os.path.join(ROOT, "paper_2503_02495_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", inc, src, "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout.strip() == "ok"
