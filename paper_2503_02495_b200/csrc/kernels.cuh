@@ -330,7 +330,7 @@ struct WStreamProblem {
     int out_cols;
     bool transposed;        // out[0] is [n, N, M]
 };
-size_t wgrad_stream_scratch_bytes();
+size_t wgrad_stream_scratch_bytes(const int (*mn)[2] /* [M, N] of each gradient */, int nprob, int n, long long rows_max);
 uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int* offsets, int n, long long rows_max,
                                const int* src_patch, int l_p, int Bm, float* part, const char* label, int* status, cudaStream_t s,
                                WReduce* reduce);

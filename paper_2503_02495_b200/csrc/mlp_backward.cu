@@ -350,7 +350,8 @@ BwdWs bwd_ws(const Dims& D) {
     r.G = w.take((size_t)D.B * D.m * D.n * sizeof(float));
     r.rvec = w.take((size_t)D.B * D.m * D.d * sizeof(float));
     r.wpart = w.take((size_t)apply_shape(D).splits * D.d * D.n * sizeof(float));
-    r.wgpart = w.take(wgrad_large(D.n, D.d, D.d_e) ? 0 : wgrad_stream_scratch_bytes());
+    const int grads[2][2] = {{D.d_e, D.d}, {D.d, D.d_e}};
+    r.wgpart = w.take(wgrad_large(D.n, D.d, D.d_e) ? 0 : wgrad_stream_scratch_bytes(grads, 2, D.n, D.Rmax));
     r.total = w.off;
     return r;
 }

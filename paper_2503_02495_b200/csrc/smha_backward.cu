@@ -47,7 +47,8 @@ SmhaBwdWs smha_bwd_ws(const Dims& D) {
     r.delta = w.take((size_t)D.Rmax * heads * 4);
     r.dgp = w.take((size_t)D.Rmax * heads * 4);
     r.router = w.take(router_backward_scratch_bytes(D));
-    r.wgpart = w.take(wgrad_stream_scratch_bytes());
+    const int grads[2][2] = {{D.d, 3 * D.d_g}, {D.d, D.d_g}};
+    r.wgpart = w.take(wgrad_stream_scratch_bytes(grads, 2, D.n, D.Rmax));
     r.total = w.off;
     return r;
 }

@@ -35,9 +35,27 @@ inline long long wgrad_line_bound(const WTileShape* t, int nprob, int n, long lo
     for (int p = 0; p < nprob; ++p) cost += (long long)t[p].m_tiles * t[p].n_tiles * t[p].w * (rows_max / kLineBK + (long long)kMinTileKb * n);
     return cost;
 }
+// Pieces (one CTA each, at most one per SM of 148) that the line can fill when every piece is at least kMinPieceKb K blocks
+// of the widest tile: what is launched, and what the scratch of cut tiles is sized for.
+constexpr int kMaxPieces = 148, kMinPieceKb = 4;
+inline int wgrad_pieces(long long bound, int wmax, int sms) {
+    const long long least = (long long)kMinPieceKb * wmax, fill = (bound + least - 1) / least;
+    const int cap = sms < kMaxPieces ? sms : kMaxPieces;
+    return fill < 1 ? 1 : (fill < cap ? (int)fill : cap);
+}
+// Floats of that scratch: two parts of a tile per piece, each as wide as the widest tile.
+inline long long wgrad_part_floats(int widest) { return (long long)kLineBM * widest; }
+inline long long wgrad_scratch_floats(const WTileShape* t, int nprob, int n, long long rows_max) {
+    int wmax = 0, widest = 0;
+    for (int p = 0; p < nprob; ++p) {
+        if (t[p].w > wmax) wmax = t[p].w;
+        if (t[p].BN > widest) widest = t[p].BN;
+    }
+    return 2 * wgrad_part_floats(widest) * wgrad_pieces(wgrad_line_bound(t, nprob, n, rows_max), wmax, kMaxPieces);
+}
 // Whether the line and the piece ends, multiples of a piece that is rounded up, fit the kernel's 32-bit positions.
 inline bool wgrad_line_fits(long long bound, int wmax, int pieces) {
-    const long long rounded = bound + pieces, least = 4ll * wmax * pieces;      // pieces * Q, Q = max(ceil(line / pieces), 4 wmax)
+    const long long rounded = bound + pieces, least = (long long)kMinPieceKb * wmax * pieces;      // pieces * Q, Q = max(ceil(line / pieces), kMinPieceKb wmax)
     return (rounded > least ? rounded : least) + wmax < 0x7fffffffll;
 }
 

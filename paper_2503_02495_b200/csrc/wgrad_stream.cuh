@@ -20,6 +20,7 @@ struct WReduce {
     const float* part = nullptr;
     int n = 0, nprob = 0, pieces = 0, blocks = 0;
     int per = 1;              // blocks per tile
+    int part_floats = 0;      // of a part of a tile in the scratch
     int by_cut = 0;           // blocks are counted by piece boundary (more tiles than pieces), else by tile
 };
 
@@ -61,7 +62,7 @@ __device__ __forceinline__ void wsched_build(WSched& s, const int* offs, int n, 
     if (lane == 0) {
         s.n = n;
         s.total = start;
-        s.Q = max((start + pieces - 1) / pieces, 4 * wmax);      // at least four K blocks per piece
+        s.Q = max((start + pieces - 1) / pieces, kMinPieceKb * wmax);
     }
     __syncwarp();
 }
@@ -145,7 +146,7 @@ __device__ __forceinline__ void wgrad_reduce(const WReduce& r, int blk) {
     const int lr = pr.transposed ? lane : lane >> 3, lq = pr.transposed ? 0 : lane & 7;
     const int stride = pr.transposed ? 128 : 4;
     const float4* base = (const float4*)r.part + (size_t)ch * 8 * 128 + quarter * 32 + (pr.transposed ? 4 * h * 128 : lq * 128 + 4 * h * 4) + lr;
-    auto part = [&](int c) { return base + wsched_slot(f, c) * (size_t)(128 * 256 / 4); };
+    auto part = [&](int c) { return base + wsched_slot(f, c) * (size_t)(r.part_floats / 4); };
     float4 acc[4], t[4];
     {
         const float4 *s0 = part(f.c_first), *s1 = part(f.c_first + 1);

@@ -10,8 +10,8 @@
 // block.
 //
 // Work split: an output tile is 128 x BN (BN <= 256); its cost is its 64-row K blocks times the time of one, of which more
-// than two thirds are the same for every width (kStepCost).  The tiles
-// of both problems form one line (wgrad_line.h), cut into equal pieces, one per CTA (one CTA per SM), whatever the load of the experts.
+// than two thirds are the same for every width (kStepCost).  The tiles of both problems form one line (wgrad_line.h), cut
+// into equal pieces, one per CTA (one CTA per SM; fewer where the line is too short for that), whatever the load of the experts.
 // A tile inside one piece is written straight to its output; a tile cut by pieces leaves one partial tile per piece in
 // the scratch, and wgrad_reduce adds them in ascending order (in spare CTAs of router_grad_kernel, or as a
 // launch of its own).  No CTA waits for another, every sum has a fixed order.
@@ -54,7 +54,7 @@ struct WArgs {
     const int* src_patch;
     float* part;
     int* status;
-    int n, nprob, l_p, Bm, pieces;
+    int n, nprob, l_p, Bm, pieces, part_floats;
 };
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -204,7 +204,7 @@ wgrad_stream_kernel(const __grid_constant__ WArgs a) {
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN_MAX;
             const int row = quarter * 32 + lane;
-            float4* part = (float4*)(a.part + wsched_slot(f, c) * (size_t)(BM * BN_MAX));
+            float4* part = (float4*)(a.part + wsched_slot(f, c) * (size_t)a.part_floats);
 #pragma unroll 1
             for (int ch = wsel; ch < f.cols / 32; ch += 2) {
                 uint32_t v[32];
@@ -262,7 +262,11 @@ wgrad_reduce_kernel(const __grid_constant__ WReduce r) {
 
 }  // namespace
 
-size_t wgrad_stream_scratch_bytes() { return (size_t)2 * 148 * BM * BN_MAX * sizeof(float); }
+size_t wgrad_stream_scratch_bytes(const int (*mn)[2], int nprob, int n, long long rows_max) {
+    WTileShape t[2];
+    for (int i = 0; i < nprob; ++i) t[i] = wgrad_tile_shape(mn[i][0], mn[i][1]);
+    return (size_t)wgrad_scratch_floats(t, nprob, n, rows_max) * sizeof(float);
+}
 
 uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int* offsets, int n, long long rows_max,
                                const int* src_patch, int l_p, int Bm, float* part, const char* label, int* status, cudaStream_t s,
@@ -276,9 +280,8 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     WArgs a;
     a.offsets = offsets; a.src_patch = src_patch; a.part = part; a.status = status;
     a.n = n; a.nprob = nprob; a.l_p = l_p > 0 ? l_p : 64; a.Bm = Bm;
-    a.pieces = sm_count() < 148 ? sm_count() : 148;
     WTileShape shape[2];
-    int wmax = 0;
+    int wmax = 0, widest = 0;
     for (int i = 0; i < nprob; ++i) {
         const WStreamProblem& in = probs[i];
         if (in.M % BM != 0 || in.N % 64 != 0) return UOE_ERR_UNSUPPORTED;
@@ -290,6 +293,7 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
         const WTileShape t = shape[i] = wgrad_tile_shape(in.M, in.N);
         p.BN = t.BN; p.m_tiles = t.m_tiles; p.n_tiles = t.n_tiles; p.w = t.w;
         if (t.w > wmax) wmax = t.w;
+        if (t.BN > widest) widest = t.BN;
         const int sub = l_p < BK ? l_p : BK;
         auto operand = [&](WOperand& o, CUtensorMap* tm, const void* base, int cols, int nblk, bool gather) {
             o.gather = gather ? 1 : 0; o.sub = gather ? sub : BK; o.nslab = BK / o.sub;
@@ -316,7 +320,10 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
             else if (!make_tmap(&a.maps[i].out[q], o, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return UOE_ERR_CUDA;
         }
     }
-    if (!wgrad_line_fits(wgrad_line_bound(shape, nprob, n, rows_max), wmax, a.pieces)) return UOE_ERR_UNSUPPORTED;
+    const long long bound = wgrad_line_bound(shape, nprob, n, rows_max);
+    a.pieces = wgrad_pieces(bound, wmax, sm_count());
+    a.part_floats = (int)wgrad_part_floats(widest);
+    if (!wgrad_line_fits(bound, wmax, a.pieces)) return UOE_ERR_UNSUPPORTED;
     {
         ProfScope ps(label, s);
         launch_k(wgrad_stream_kernel, dim3(a.pieces), dim3(THREADS), (size_t)SMEM, s, a);
@@ -326,11 +333,9 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     r.prob[0] = a.prob[0];
     r.prob[1] = a.prob[nprob - 1];
     r.offsets = offsets; r.part = part; r.n = n; r.nprob = nprob; r.pieces = a.pieces;
-    int tiles = 0, widest = 0;
-    for (int i = 0; i < nprob; ++i) {
-        tiles += n * a.prob[i].m_tiles * a.prob[i].n_tiles;
-        if (a.prob[i].BN > widest) widest = a.prob[i].BN;
-    }
+    r.part_floats = a.part_floats;
+    int tiles = 0;
+    for (int i = 0; i < nprob; ++i) tiles += n * a.prob[i].m_tiles * a.prob[i].n_tiles;
     r.per = (widest / 32 * 8 + kReduceThreads / 32 - 1) / (kReduceThreads / 32);
     r.by_cut = tiles > a.pieces - 1 ? 1 : 0;
     r.blocks = (r.by_cut ? a.pieces - 1 : tiles) * r.per;

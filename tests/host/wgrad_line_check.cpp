@@ -34,6 +34,11 @@ int main() {
         if (!wgrad_line_fits(bound, wmax, pieces)) { ++refused; continue; }
         long long Q = (line + pieces - 1) / pieces;
         if (Q < 4ll * wmax) Q = 4ll * wmax;
+        // the pieces the line can fill are as long as with more of them, and hold the whole line
+        const int used = wgrad_pieces(bound, wmax, pieces);
+        long long Qu = (line + used - 1) / used;
+        if (Qu < 4ll * wmax) Qu = 4ll * wmax;
+        if (used > pieces || (Qu != Q && used < pieces) || used * Qu < line) { std::printf("%d of %d pieces\n", used, pieces); return 5; }
         if (pieces * Q > 0x7fffffffll || line + pieces > 0x7fffffffll) { std::printf("piece end %lld\n", pieces * Q); return 2; }
         full += bound < 0x7fffffffll / 2 ? 0 : 1;
     }

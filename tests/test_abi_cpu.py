@@ -92,3 +92,13 @@ def test_every_entry_point_validates_on_the_host(uoe):
     st = lib.uoe_route(ctypes.byref(huge), dummy, dummy, dummy, dummy, dummy, dummy, dummy, dummy, dummy,
                        ctypes.c_size_t(1 << 40), None)
     assert st == 2
+
+
+def test_backward_workspace_follows_the_problem(uoe):
+    """The scratch for cut weight-gradient tiles is bounded by the rows there are: a few 128-row tiles of work do not ask for
+    two tiles per SM (37 MB)."""
+    base = dict(B=1, L=64, L_valid=64, d=128, n=2, k=1, m=4, c=2)
+    assert uoe.uoe_workspace_bytes(uoe.Problem(**base, d_e=128), uoe.UOE_OP_MLP_BWD) < 2 << 20
+    assert uoe.uoe_workspace_bytes(uoe.Problem(**base, H=2, d_h=64), uoe.UOE_OP_SMHA_BWD) < 2 << 20
+    # widths the backward refuses can still be asked about
+    assert uoe.uoe_workspace_bytes(uoe.Problem(**base, d_e=8), uoe.UOE_OP_MLP_BWD) > 0
