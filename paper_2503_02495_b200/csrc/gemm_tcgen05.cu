@@ -347,7 +347,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const CUtensorMap* tmC = mat == 0 ? &tmC0 : (mat == 1 ? &tmC1 : &tmC2);
             int tok = -1;                                    // position of this thread's row in its sample
             if constexpr (ROPE) {                            // (two dependent look-ups, under the tile's main loop)
-                if (half < blocks) tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e]);
+                int b;
+                if (half < blocks) tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e], b);
             }
             const int wrow0 = row0 + half * BM + quarter * 32;           // first row of this warp's piece
             const size_t row = (size_t)wrow0 + lane;

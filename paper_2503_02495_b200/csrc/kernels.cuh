@@ -147,9 +147,9 @@ __device__ __forceinline__ void rope_angle(const Rope& rp, int p, float t, float
     const float frac = (r - rintf(r)) + fmaf(t, rp.lo[p], fmaf(t, rp.hi[p], -r));     // fraction of a turn, in [-1/2, 1/2]
     __sincosf(frac * 6.283185307179586f, &sn, &cs);
 }
-// Row of the source tensor [B*m*l_p rows] that routed row r of expert e's region holds; -1 on padding rows and unused
-// slots.  Any patch length (through slot_pair).
-__device__ __forceinline__ int source_row(const SrcMap& g, int r, int e, int off_e) {
+// Position in its sample, and the sample, of the token that routed row r of expert e's region holds; -1 on padding rows and
+// unused slots.  Any patch length (through slot_pair).
+__device__ __forceinline__ int token_of(const SrcMap& g, int r, int e, int off_e, int& b) {
     if (r >= g.expert_end[e]) return -1;
     const int rel = r - off_e, l_a = g.c * g.l_p;
     const int q = rel / l_a;
@@ -157,13 +157,16 @@ __device__ __forceinline__ int source_row(const SrcMap& g, int r, int e, int off
     if (pair < 0 || pair >= g.B * g.k) return -1;      // rows that a slot left out of the plan left without a pair
     const int u = (rel % l_a) / g.l_p;
     const int pj = g.n_elig >= 0 ? (u < g.n_elig ? u : -1) : g.patch_idx[(size_t)pair * g.c + u];
-    return pj >= 0 && pj < g.m ? ((pair / g.k) * g.m + pj) * g.l_p + rel % g.l_p : -1;
+    b = pair / g.k;
+    return pj >= 0 && pj < g.m ? pj * g.l_p + rel % g.l_p : -1;
 }
-// Position of that token in its sample, or -1.
-__device__ __forceinline__ int token_of(const SrcMap& g, int r, int e, int off_e) {
-    const int row = source_row(g, r, e, off_e);
-    return row < 0 ? -1 : row % (g.m * g.l_p);
+// That token's row of the source tensor [B*m*l_p rows] (there may be more than 2^31 of them), or -1.
+__device__ __forceinline__ long long source_row(const SrcMap& g, int r, int e, int off_e) {
+    int b = 0;
+    const int t = token_of(g, r, e, off_e, b);
+    return t < 0 ? -1 : (long long)b * (g.m * g.l_p) + t;
 }
+
 // Source patch (index into the [Bm patches] view of the source tensor) of the l_p-row block that starts at routed row
 // r inside the region of expert e (first row off_e); Bm (out of range: the loads return zeros) for padding rows and
 // unused slots.

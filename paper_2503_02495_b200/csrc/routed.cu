@@ -317,7 +317,8 @@ template <int TM, int TN, int MT, int NT, int KG, int BK> struct F32Cfg {
     static constexpr int STAGE = TM * LDA + BK * TN;             // floats
     static constexpr int STAGES = 3;
     static constexpr int RED = KG > 1 ? (KG - 1) * TM * TN : 0;
-    static constexpr int SMEM = (STAGES * STAGE > RED ? STAGES * STAGE : RED) * 4 + TM * 4;
+    static constexpr int SMEM = (STAGES * STAGE > RED ? STAGES * STAGE : RED) * 4 + TM * 8;
+    static_assert(STAGE % 2 == 0 && RED % 2 == 0, "the row indices behind the ring are 8-byte aligned");
     static_assert(128 % TM == 0 && BK % (4 * KG) == 0 && NT % 4 == 0, "tile shape");
 };
 
@@ -330,7 +331,7 @@ gemm_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, const 
     pdl_trigger();
     pdl_wait();
     extern __shared__ __align__(16) float s_ring[];
-    int* s_src = (int*)(s_ring + (Cf::SMEM - TM * 4) / 4);       // source row of every tile row, -1 = zeros
+    long long* s_src = (long long*)(s_ring + (Cf::SMEM - TM * 8) / 4);       // source row of every tile row, -1 = zeros
     const int row0 = blockIdx.x * TM, col0 = blockIdx.y * TN, tid = threadIdx.x;
     if (row0 >= offsets[n]) return;
     int e = 0;
@@ -351,7 +352,7 @@ gemm_f32_kernel(const float* __restrict__ A, const float* __restrict__ W, const 
             const int k0 = step * BK;
             for (int q = tid; q < TM * BK / 4; q += Cf::THREADS) {
                 const int r = q / (BK / 4), kk = (q % (BK / 4)) * 4;
-                const int src = s_src[r];
+                const long long src = s_src[r];
                 const bool ok = src >= 0 && k0 + kk < K;
                 copy(sa + r * Cf::LDA + kk, ok ? A + (size_t)src * K + k0 + kk : A, ok);
             }

@@ -180,3 +180,35 @@ def test_attention_backward_tiles(l_p, c, L_valid, causal):
     got, ref = run_att(w, False)
     for g, r in zip(got, ref[:len(got)]):
         assert rel_inf(g, r) <= TOL
+
+
+# more tokens than 2^31: 32768 + 40 samples of 65536 rows of 16 bytes (34 GB in, 34 GB out); the last samples are past the limit
+def _two_to_the_31(dtype):
+    import paper_2503_02495_b200 as uoe
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 100 << 30:
+        pytest.skip("needs 100 GB of device memory")
+    f32 = dtype == "f32"
+    prob = uoe.Problem(B=32768 + 40, L=65536, L_valid=65536, d=4 if f32 else 8, n=1, k=1, m=1024, c=1, d_e=4 if f32 else 0,
+                       dtype=dtype, gate=False, residual=False, act="identity")
+    x = torch.zeros(prob.B, prob.L, prob.d, dtype=prob.torch_dtype, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(2)
+    for b in (0, prob.B - 1):
+        x[b] = torch.randn(prob.L, prob.d, device="cuda", generator=g).to(prob.torch_dtype)
+    return uoe, prob, x, g
+
+
+def test_float32_rows_past_two_to_the_31():
+    """1e-6 of the largest value: sums of four float32 products, twice."""
+    uoe, prob, x, g = _two_to_the_31("f32")
+    W1, W2 = (torch.randn(1, 4, 4, device="cuda", generator=g) for _ in range(2))
+    patch = torch.randint(prob.m, (prob.B, 1, 1), device="cuda", generator=g).to(torch.int32)
+    rows = prob.B * prob.l_p
+    r = uoe.Routing(torch.zeros(prob.B, 1, dtype=torch.int32, device="cuda"), patch, torch.ones(prob.B, 1, 1, device="cuda"), None, None,
+                    torch.tensor([0, (rows + 127) // 128 * 128], dtype=torch.int32, device="cuda"))
+    y = uoe.uoe_mlp_forward(prob, x, W1, W2, r)
+    for b in (0, prob.B - 1):
+        t = int(patch[b]) * prob.l_p + torch.arange(prob.l_p, device="cuda")
+        ref = torch.zeros(prob.L, prob.d, dtype=torch.float64, device="cuda")
+        ref[t] = x[b, t].double() @ W1[0].double() @ W2[0].double()
+        assert (y[b].double() - ref).abs().max() <= 1e-6 * ref.abs().max()
