@@ -127,7 +127,7 @@ struct ApplyArgs {
 };
 template <int NMAX, bool SPREAD>
 __global__ void __launch_bounds__(32 * kApplyWarps, NMAX > 16 ? 1 : 2)
-router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], boxes of [seg_rows, 64] */, const ApplyArgs a) {
+router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B m, l_p, d], boxes of [seg_rows, 64] */, const ApplyArgs a) {
     pdl_trigger();
     extern __shared__ uint8_t s_raw[];
     __shared__ uint64_t full[kApplyWarps][kApplyStages];
@@ -152,7 +152,7 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B L, d], b
         if (ip >= end) return;
         if (lane == 0) {
             mbar_arrive_expect_tx(&full[warp][st_in], (uint32_t)unit_bytes);
-            tma_load_2d(ring + st_in * unit_bytes, &xmap, c0, ip * a.l_p + is * a.seg_rows, &full[warp][st_in]);
+            tma_load_3d(ring + st_in * unit_bytes, &xmap, c0, is * a.seg_rows, ip, &full[warp][st_in]);
         }
         if (++st_in == a.stages) st_in = 0;
         if (++is == nseg) { is = 0; ip += kApplyWarps; }
@@ -274,9 +274,9 @@ template <bool SPREAD>
 uoe_status launch_router_apply(const Dims& D, const ApplyShape& a, const void* x, const void* W_r, const float* G, float* rvec,
                                float* part, void* dx, int* status, cudaStream_t s) {
     CUtensorMap xmap;
-    const uint64_t dims[2] = {(uint64_t)D.d, (uint64_t)D.B * D.L}, str[1] = {(uint64_t)D.d * 2};
-    const uint32_t box[2] = {(uint32_t)kApplyCols, (uint32_t)a.seg_rows};
-    if (!make_tmap(&xmap, x, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_NONE)) return UOE_ERR_CUDA;
+    const uint64_t dims[3] = {(uint64_t)D.d, (uint64_t)D.l_p, (uint64_t)D.B * D.m}, str[2] = {(uint64_t)D.d * 2, (uint64_t)D.d * 2 * D.l_p};
+    const uint32_t box[3] = {(uint32_t)kApplyCols, (uint32_t)a.seg_rows, 1};
+    if (!make_tmap(&xmap, x, 3, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_NONE)) return UOE_ERR_CUDA;
     ApplyArgs p;
     p.W_r = (const __nv_bfloat16*)W_r; p.G = G; p.rvec = rvec; p.part = part; p.dx = (__nv_bfloat16*)dx; p.status = status;
     p.patches = D.B * D.m; p.Lv = D.Lv; p.d = D.d; p.n = D.n; p.m = D.m; p.l_p = D.l_p; p.nseg = a.nseg;

@@ -212,3 +212,21 @@ def test_float32_rows_past_two_to_the_31():
         ref = torch.zeros(prob.L, prob.d, dtype=torch.float64, device="cuda")
         ref[t] = x[b, t].double() @ W1[0].double() @ W2[0].double()
         assert (y[b].double() - ref).abs().max() <= 1e-6 * ref.abs().max()
+
+
+def test_router_gradient_of_rows_past_two_to_the_31():
+    """With one expert the balance loss has no gradient, so the gate is given: two experts, p and 1 - p of every patch.  dW_r is a
+    float32 sum over the last sample's 65536 rows, 2^-24 * sqrt(65536) relative; 1e-3 of the largest value."""
+    uoe, prob, x, g = _two_to_the_31("bf16")
+    prob.n = 2
+    p = torch.full((prob.B, 2, prob.m), 0.5, device="cuda")
+    p[:, 0] = 0.75
+    p[:, 1] = 0.25
+    dloss = torch.zeros(prob.B, device="cuda")
+    dloss[-1] = 1.0
+    dx, dWr = uoe.uoe_route_balance_backward(prob, x, torch.zeros(prob.d, 2, dtype=torch.bfloat16, device="cuda"), p, 1.0, dloss)
+    # every patch goes to expert 0: f = (2, 0), dL/dg = f / m, the softmax Jacobian leaves +-0.75 * 0.25 * 2 / m, per token / l_p
+    ref = x[-1].double().sum(0) * (0.75 * 0.25 * 2 / prob.m / prob.l_p)
+    assert (dWr[:, 0].double() - ref).abs().max() <= 1e-3 * ref.abs().max()
+    assert (dWr[:, 1].double() + ref).abs().max() <= 1e-3 * ref.abs().max()
+    assert (dx[-1] == 0).all()
