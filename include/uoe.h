@@ -164,7 +164,9 @@ uoe_status uoe_route_balance(const uoe_problem* prob, const float* p_patch, floa
  * softmax (Eq. 14) and the mean-pooled linear router (Eq. 13).  The paper gives no backward text.
  *   dx [B,L,d] in prob->dtype and dW_r [d,n] float32 are overwritten (add them to the layer's own gradients);
  *   dloss [B] float32; p_patch [B,n,m] as written by uoe_route for the same x and W_r.  bfloat16 only.
- * Workspace: uoe_workspace_bytes(prob, UOE_OP_BALANCE_BWD).  All pointers except prob are device pointers.
+ * Workspace: uoe_workspace_bytes(prob, UOE_OP_BALANCE_BWD), prepared with uoe_workspace_init like any other: a wait inside
+ * the kernel that runs out is reported in its status word (dx and dW_r are then incomplete).  All pointers except prob are
+ * device pointers.
  */
 uoe_status uoe_route_balance_backward(const uoe_problem* prob, const void* x, const void* W_r, const float* p_patch,
                                       float alpha, const float* dloss, void* dx, float* dW_r,

@@ -348,8 +348,11 @@ def uoe_route_balance(prob: Problem, p_patch, alpha: float = 1.0):
     return lb, cnt, cd
 
 
-def uoe_route_balance_backward(prob: Problem, x, W_r, p_patch, alpha: float, dloss, ws=None):
-    """(dx [B,L,d], dW_r [d,n] float32): gradient of sum(dloss * lb_loss) with respect to x and W_r."""
+def uoe_route_balance_backward(prob: Problem, x, W_r, p_patch, alpha: float, dloss, ws=None, check: bool = False):
+    """(dx [B,L,d], dW_r [d,n] float32): gradient of sum(dloss * lb_loss) with respect to x and W_r.
+
+    Its kernel waits for copies with a limit; check=True synchronises and raises if a wait ran out (by default the call stays
+    asynchronous and the status word of `ws`, if one is given, can be read later)."""
     _contig(x, prob.torch_dtype)
     _contig(W_r, prob.torch_dtype)
     _contig(p_patch, torch.float32)
@@ -361,6 +364,8 @@ def uoe_route_balance_backward(prob: Problem, x, W_r, p_patch, alpha: float, dlo
                                          ctypes.c_float(alpha), _ptr(dloss), _ptr(dx), _ptr(dW_r), _ptr(ws), ws.numel(),
                                          _stream())
     _check(st, "uoe_route_balance_backward")
+    if check:
+        _check(uoe_read_device_status(ws), "uoe_route_balance_backward (device)")
     return dx, dW_r
 
 

@@ -179,3 +179,21 @@ def test_route_balance_backward_matches_oracle(name):
     assert np.abs(got_dx - ref_dx).max() <= 2e-2 * np.abs(ref_dx).max()
     assert np.abs(dWr.cpu().numpy() - ref_dWr).max() <= 2e-2 * np.abs(ref_dWr).max()
     assert np.all(got_dx[:, w.L_valid:] == 0)
+
+
+def test_balance_backward_reports_the_workspace_status():
+    """A status in the workspace (here put there by the test) is raised when the call is asked to check, and only then."""
+    import paper_2503_02495_b200 as uoe
+    prob = uoe.Problem(B=2, L=32, L_valid=32, d=64, n=4, k=2, m=4, c=2)
+    x = torch.randn(2, 32, 64, device="cuda").bfloat16()
+    Wr = torch.randn(64, 4, device="cuda").bfloat16()
+    p = torch.softmax(torch.randn(2, 4, 4, device="cuda"), dim=1)
+    ws = uoe.alloc_workspace(prob, uoe.UOE_OP_BALANCE_BWD)
+    args = (prob, x, Wr, p, 0.1, torch.ones(2, device="cuda"))
+    want = uoe.uoe_route_balance_backward(*args, ws=ws, check=True)
+    ws[:4] = torch.tensor([5, 0, 0, 0], dtype=torch.uint8, device="cuda")
+    got = uoe.uoe_route_balance_backward(*args, ws=ws)
+    assert torch.equal(got[1], want[1])
+    with pytest.raises(uoe.UoeError) as ei:
+        uoe.uoe_route_balance_backward(*args, ws=ws, check=True)
+    assert ei.value.status == 5
