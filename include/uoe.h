@@ -23,9 +23,9 @@
  *     consecutive calls and stop them from overlapping).  A new workspace is prepared once with
  *     uoe_workspace_init; uoe_read_device_status clears the word after reporting an anomaly.
  *   - Devices and threads.  A process may use the library on several devices; kernel attributes and cached
- *     device properties are set up per device by the first call that needs them there.  That first call per
- *     device (of each entry point, uoe_route_static included) is not thread-safe; afterwards calls from several
- *     threads are safe as long as they use distinct workspaces.  uoe_profile_* is never thread-safe.
+ *     device properties are set up per device by the first call that needs them there.  Calls from several threads
+ *     are safe, first calls included, as long as they use distinct workspaces (and, for uoe_route_static, are
+ *     ordered on the device as described there).  uoe_profile_* is never thread-safe.
  *   - Element type: `dtype` selects float32 or bfloat16 storage for x, weights and y.  Products are
  *     accumulated in float32.  Routing probabilities and gates are always float32.
  *

@@ -744,19 +744,19 @@ extern "C" uoe_status uoe_route_balance(const uoe_problem* prob, const float* p_
 static __device__ __align__(256) unsigned char g_route_static_scratch[UOE_ROUTE_STATIC_SCRATCH_BYTES];
 
 namespace {
-unsigned char* g_route_static_ptr[kMaxDevices] = {};    // device address of the array, per device
+std::atomic<unsigned char*> g_route_static_ptr[kMaxDevices] = {};    // device address of the array, per device
 
 // In host code `g_route_static_scratch` is only a handle; the address a kernel can use comes from
 // cudaGetSymbolAddress, asked once per device with that device current.
 uoe_status route_static_base(unsigned char** out) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return UOE_ERR_CUDA;
-    if (!g_route_static_ptr[dev]) {
-        void* p = nullptr;
+    void* p = g_route_static_ptr[dev].load(std::memory_order_relaxed);
+    if (!p) {
         if (cudaGetSymbolAddress(&p, g_route_static_scratch) != cudaSuccess || !p) return UOE_ERR_CUDA;
-        g_route_static_ptr[dev] = (unsigned char*)p;
+        g_route_static_ptr[dev].store((unsigned char*)p, std::memory_order_relaxed);
     }
-    *out = g_route_static_ptr[dev];
+    *out = (unsigned char*)p;
     return UOE_OK;
 }
 }  // namespace

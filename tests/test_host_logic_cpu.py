@@ -23,3 +23,13 @@ def test_bound_on_the_weight_gradient_line(tmp_path):
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     assert r.stdout.strip() == "ok"
+
+
+def test_setup_bookkeeping_under_threads(tmp_path):
+    exe = str(tmp_path / "device_once_threads")
+    src = os.path.join(ROOT, "tests", "host", "device_once_threads.cpp")
+    inc = os.path.join(ROOT, "paper_2503_02495_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-g", "-Wall", "-Werror", "-pthread", "-fsanitize=thread", "-I", inc, src, "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout.strip() == "ok"
