@@ -572,6 +572,7 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
     float* scores = (float*)(base + W.scores);
     const int use_gate = ((flags & UOE_FLAG_GATE) ? 1 : 0) | ((flags & UOE_FLAG_DYNAMIC_C) ? 2 : 0) |
                          ((flags & UOE_FLAG_GENERAL_PATH) ? 4 : 0);                                       // selection flags
+    constexpr size_t kPlainSmem = 32 * 1024;      // with up to 14.2 KB of a kernel's own this stays below the 48 KB that need no opt-in
     constexpr int kGridZ = 65535;      // samples per launch of route_kernel (more than that: more launches)
     int b0 = 0;
     dim3 grid((unsigned)(W.nchunks * W.rsplit), (unsigned)D.m, (unsigned)(D.B < kGridZ ? D.B : kGridZ));
@@ -582,6 +583,7 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
 #define UOE_ROUTE_LAUNCH(T, TICKET, NT, SMEM) \
         [&] { \
             static SpreadOnce once; \
+            if (SMEM > kPlainSmem && smem_opt_in(once.opt_in, route_kernel<T, TICKET, NT>, 160 * 1024) != UOE_OK) return cudaErrorInvalidValue; \
             return launch_k(route_kernel<T, TICKET, NT>, grid, dim3(NT), spread_smem(once, route_kernel<T, TICKET, NT>, ctas, SMEM), \
                             stream, UOE_ROUTE_ARGS(T)); \
         }()

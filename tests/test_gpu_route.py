@@ -197,3 +197,17 @@ def test_balance_backward_reports_the_workspace_status():
     with pytest.raises(uoe.UoeError) as ei:
         uoe.uoe_route_balance_backward(*args, ws=ws, check=True)
     assert ei.value.status == 5
+
+
+@pytest.mark.parametrize("B,n,m,l_p", [(3, 32, 276, 4), (3, 32, 288, 4), (1, 9, 1024, 40)])
+def test_largest_gate_of_a_sample(B, n, m, l_p):
+    """n * m gate values up to the limit of 36 KB, few enough samples that scoring and selection are one kernel (its own shared
+    memory and the gate values exceed 48 KB together)."""
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(B=B, L=l_p * m, L_valid=l_p * m - 2, m=m, c=m // 3, d=64, n=n, k=5, d_ff=0, H=0, dtype="bf16")
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w).f64 * 20, w.dtype)
+    r = uoe.uoe_route(problem_of(w, "mlp"), to_dev(x), to_dev(Wr))
+    ref = orc.route(x.f64, Wr.f64, w.k, w.m, w.c, L_valid=w.L_valid)
+    assert np.abs(r.p_samp.cpu().numpy() - ref.p_samp).max() <= 2e-6
+    assert np.abs(r.p_patch.cpu().numpy() - ref.p_patch).max() <= 2e-6
+    check_routing(r, ref)
