@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "device_once.h"
 #include "uoe.h"
 
@@ -16,7 +18,7 @@ namespace uoe {
 // host side
 // ------------------------------------------------------------------------------------------------
 
-extern long long g_launch_count;   // kernels enqueued by this process (reported by uoe_launch_count)
+extern std::atomic<long long> g_launch_count;   // kernels enqueued by this process (reported by uoe_launch_count)
 
 #define UOE_CUDA_OK(expr)                                   \
     do {                                                    \
@@ -26,7 +28,7 @@ extern long long g_launch_count;   // kernels enqueued by this process (reported
 
 #define UOE_LAUNCHED()                                      \
     do {                                                    \
-        ++uoe::g_launch_count;                              \
+        uoe::g_launch_count.fetch_add(1, std::memory_order_relaxed); \
         if (cudaGetLastError() != cudaSuccess) return UOE_ERR_CUDA; \
     } while (0)
 

@@ -12,7 +12,7 @@
 
 namespace uoe {
 
-long long g_launch_count = 0;
+std::atomic<long long> g_launch_count{0};
 
 namespace {
 
@@ -613,12 +613,12 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
             if (W.small_ctas) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, 64, W.smem) : UOE_ROUTE_LAUNCH(float, false, 64, W.smem);
             else if (W.two_kernels) e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, false, kScoreThreads, W.smem) : UOE_ROUTE_LAUNCH(float, false, kScoreThreads, W.smem);
             else e = D.bf16 ? UOE_ROUTE_LAUNCH(__nv_bfloat16, true, kScoreThreads, smem0) : UOE_ROUTE_LAUNCH(float, true, kScoreThreads, smem0);
+            if (e == cudaSuccess) UOE_LAUNCHED();
         }
     }
 #undef UOE_ROUTE_LAUNCH
 #undef UOE_ROUTE_ARGS
     if (e != cudaSuccess) return UOE_ERR_CUDA;
-    UOE_LAUNCHED();
     if (!W.two_kernels) return UOE_OK;
     {
         ProfScope ps(profile ? "route_select" : nullptr, stream);

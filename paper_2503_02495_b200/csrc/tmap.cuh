@@ -38,7 +38,7 @@ struct TmapKeyHash {
     }
 };
 constexpr size_t kTmapCacheMax = 4096;
-inline long long& tmap_encode_count() { static long long n = 0; return n; }     // encodings done (cache misses), for tests
+inline std::atomic<long long>& tmap_encode_count() { static std::atomic<long long> n{0}; return n; }     // encodings done (cache misses), for tests
 
 // Tensor of `rank` dims (dims[0] innermost, contiguous), box of `box` elements, 128-byte swizzle.
 // strides_bytes[i] is the stride of dim i+1.

@@ -112,6 +112,15 @@ def test_more_samples_than_a_grid_dimension_holds():
     assert torch.equal(r.expert_offsets.long().diff(), (rows + 127) // 128 * 128)
 
 
+def test_every_launch_of_a_call_is_counted():
+    """Scores of more samples than a grid dimension holds: two launches."""
+    import paper_2503_02495_b200 as uoe
+    prob = uoe.Problem(B=65541, L=33, L_valid=33, d=16, n=4, k=2, m=1, c=1, dtype="bf16")
+    before = uoe.uoe_launch_count()
+    uoe.uoe_route(prob, torch.zeros(prob.B, 33, 16, dtype=torch.bfloat16, device="cuda"), torch.zeros(16, 4, dtype=torch.bfloat16, device="cuda"))
+    assert uoe.uoe_launch_count() - before == 2
+
+
 # weight gradients cut into equal pieces over the SMs: ragged column tiles, 8-row slabs, one expert whose tiles are cut into
 # many pieces, experts without rows, routed copies, and the pass without gates (the cut tiles added by their own launch)
 def _bwd(**kw):
