@@ -311,15 +311,15 @@ inline int gemm_dg_cols(int N) { return N / gemm_bf16_bn(N) * dg_cols_per_tile(g
 // the source tensor [Bm patches, l_p, M (N)] and routed row r is row r % l_p of patch src_patch[r / l_p]
 // (-1 = zero rows).  Needs regions (multiples of 128 rows) that start on patch boundaries.
 //
-// Large matrices (at least two 256 x 256 tiles per SM): one launch per gradient, 256 x 256 tiles, longest first.
-bool wgrad_large(int n, int M, int N);
-inline bool wgrad_large_can_gather(int l_p) { return l_p >= 16 && 128 % l_p == 0; }
+// Whole tiles: one launch per gradient, longest experts first.
+bool wgrad_large(int n, int M, int N);       // at least two 256 x 256 tiles per SM
+inline bool wgrad_whole_can_gather(int l_p) { return l_p >= 16 && 128 % l_p == 0; }
 struct WgradGather {
     bool gather_p = false, gather_q = false;
     const int* src_patch = nullptr;
     int l_p = 64, Bm = 0;
 };
-uoe_status launch_wgrad_large(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
+uoe_status launch_wgrad_whole(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
                               long long rows_max, const char* label, int* status, cudaStream_t s,
                               const WgradGather& g = WgradGather());
 // All others: up to two gradients in one launch, cut into equal pieces over the SMs (wgrad_stream_tcgen05.cu).  `part`:

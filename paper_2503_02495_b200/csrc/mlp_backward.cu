@@ -328,10 +328,28 @@ balance_bwd_kernel(const float* __restrict__ p_patch, const float* __restrict__ 
 
 struct BwdWs { size_t plan, dyg, xg, dh, ag, dxg, dgp, G, rvec, wpart, wgpart, total; int nt; };
 
-// dy and x gathered inside the consumers' TMA loads (else copied into routed buffers first)
-bool bwd_can_gather(const Dims& D) {
-    return can_fuse_gather(D) && (!wgrad_large(D.n, D.d, D.d_e) || wgrad_large_can_gather(D.l_p));
+// Which kernel takes the two weight gradients: whole tiles (wgrad_tcgen05.cu) or a line of tiles cut into equal pieces
+// (wgrad_stream_tcgen05.cu).  The pieces fill the SMs whatever the number of tiles, but at any moment the CTAs work all over
+// the line, so that operands larger than L2 (126 MB) are read from memory once per tile: 844 us against 574 for both gradients
+// at d = 1536, d_e = 896, n = 24, 82k routed rows; 454 against 330 at d = 2048, d_e = 1024, n = 8, 32k rows, x and dy gathered.
+// With fewer tiles than SMs, or operands in L2, whole tiles lose: n = 2, d = 512, d_e = 256, 32k rows, backward of the half 541
+// against 162; d = 1024, d_e = 512, n = 8, 8k rows 107 against 109, 32k rows 267 against 245.  The lines lie where the two were
+// equal over 1176 problems (n 2 to 24, d 512 to 4096, d_e 256 to 2048, 256 to 16384 rows per expert, gathered and copied):
+// tiles per SM, and the bytes of the two operands that are d wide.  Widths that are no multiple of 256 have 128-wide whole tiles,
+// a fifth slower out of L2.
+bool wgrad_whole(const Dims& D) {
+    if (wgrad_large(D.n, D.d, D.d_e)) return true;
+    const bool copies = !can_fuse_gather(D);
+    if (!copies && !wgrad_whole_can_gather(D.l_p)) return false;      // (copying the rows costs more)
+    auto tiles = [&](int M, int N) { return (long long)D.n * (M / 128) * (N / (N % 256 == 0 ? 256 : 128)); };
+    const double per_sm = (double)(tiles(D.d, D.d_e) + tiles(D.d_e, D.d)) / sm_count();
+    const double mb = 2.0 * (copies ? (double)D.Rmax : (double)D.B * D.L) * D.d * D.esize / 1e6;
+    if (D.d % 256 == 0 && D.d_e % 256 == 0) return (per_sm >= 1.5 && mb > 64) || (copies && per_sm >= 0.8 && mb > 126);
+    return per_sm >= 2.5 && mb > 115;
 }
+
+// dy and x gathered inside the consumers' TMA loads (else copied into routed buffers first)
+bool bwd_can_gather(const Dims& D) { return can_fuse_gather(D) && (!wgrad_whole(D) || wgrad_whole_can_gather(D.l_p)); }
 
 BwdWs bwd_ws(const Dims& D) {
     WsCarver w;
@@ -351,7 +369,7 @@ BwdWs bwd_ws(const Dims& D) {
     r.rvec = w.take((size_t)D.B * D.m * D.d * sizeof(float));
     r.wpart = w.take((size_t)apply_shape(D).splits * D.d * D.n * sizeof(float));
     const int grads[2][2] = {{D.d_e, D.d}, {D.d, D.d_e}};
-    r.wgpart = w.take(wgrad_large(D.n, D.d, D.d_e) ? 0 : wgrad_stream_scratch_bytes(grads, 2, D.n, D.Rmax));
+    r.wgpart = w.take(wgrad_whole(D) ? 0 : wgrad_stream_scratch_bytes(grads, 2, D.n, D.Rmax));
     r.total = w.off;
     return r;
 }
@@ -466,15 +484,15 @@ extern "C" uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, c
     if (st != UOE_OK) return st;
     // dW2 = ag^T dy_g, dW1 = x_g^T dh
     WReduce reduce;
-    if (wgrad_large(D.n, D.d, D.d_e)) {
+    if (wgrad_whole(D)) {
         WgradGather gq, gp;
         if (fused) {
             gq.gather_q = true; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m;
             gp.gather_p = true; gp.src_patch = P.src_patch; gp.l_p = D.l_p; gp.Bm = D.B * D.m;
         }
-        st = launch_wgrad_large(ag, fused ? dy : dyg, dW2, expert_offsets, D.n, D.d_e, D.d, D.Rmax, "wgrad_W2", status, stream, gq);
+        st = launch_wgrad_whole(ag, fused ? dy : dyg, dW2, expert_offsets, D.n, D.d_e, D.d, D.Rmax, "wgrad_W2", status, stream, gq);
         if (st != UOE_OK) return st;
-        st = launch_wgrad_large(fused ? x : xg, dh, dW1, expert_offsets, D.n, D.d, D.d_e, D.Rmax, "wgrad_W1", status, stream, gp);
+        st = launch_wgrad_whole(fused ? x : xg, dh, dW1, expert_offsets, D.n, D.d, D.d_e, D.Rmax, "wgrad_W1", status, stream, gp);
     } else {
         const WStreamProblem probs[2] = {{ag, fused ? dy : dyg, D.d_e, D.d, false, fused, {dW2, nullptr, nullptr}, D.d, false},
                                          {fused ? x : xg, dh, D.d, D.d_e, fused, false, {dW1, nullptr, nullptr}, D.d_e, false}};

@@ -4,9 +4,11 @@
 // operands are "MN-major" for the MMA: a K step is 64 consecutive rows, each row contributing 128 bytes
 // (64 elements) per swizzled box.
 //
-// This file: matrices large enough for at least two 256 x 256 output tiles per SM (the others, and every SMHA gradient, are
-// in wgrad_stream_tcgen05.cu).  Persistent CTAs walk (expert, 256 x 256 tile); warp roles are those of the forward
-// grouped GEMM, with one accumulator set (all of TMEM).  The output is float32 and overwritten (each epilogue warp stages
+// This file: whole output tiles, one gradient per launch, for matrices of many tiles whose operands do not stay in L2
+// (wgrad_whole in mlp_backward.cu says which; the others, and every SMHA gradient, are in wgrad_stream_tcgen05.cu).
+// Persistent CTAs walk (expert, tile): 256 x 256 where every SM gets at least two of them, else 128 x 256 or 128 x 128; all
+// CTAs work on neighbouring tiles of one or two experts at a time, so an operand block is read from memory once.  Warp roles
+// are those of the forward grouped GEMM.  The output is float32 and overwritten (each epilogue warp stages
 // [32 rows x 32 columns] in swizzled shared memory and issues one TMA tensor store); an expert with no rows gets zeros.
 // A tile's cost is its expert's row count, so the tile list is ordered by descending row count and handed out
 // longest first: a CTA's first tile is its own index, every further one comes from a counter in the workspace's
@@ -28,37 +30,39 @@ constexpr int A_BLOCK_BYTES = BM * BK * 2;
 constexpr int kSchedSlots = 4;       // tiles the producer may run ahead of the slowest consumer
 constexpr int kSchedWord = 64;       // words [64, 66) of the workspace's control block: next tile, CTAs finished
 
-// 256 x 256 output tiles: two 128-row accumulators fed by the same Q stage, one accumulator set drained by eight warps
-constexpr int BN = 256, MT = 2;
-struct WCfg {
+// MT = 2: 256 x BN output tiles (two 128-row accumulators fed by the same Q stage), one accumulator set drained by eight
+// warps; MT = 1: 128 x BN tiles with two accumulator sets.
+template <int BN, int MT> struct WCfg {
     static constexpr int A_BYTES = MT * A_BLOCK_BYTES;
     static constexpr int B_BYTES = BN * BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = 3;
+    static constexpr int STAGES = MT == 2 ? 3 : (BN == 256 ? 4 : (BN == 128 ? 6 : 8));
+    static constexpr int NACC = MT == 2 ? 1 : 2;
     static constexpr int TMEM_COLS = 2 * BN;
-    static constexpr int EPI_WARPS = 8;
+    static constexpr int EPI_WARPS = 4 * MT;
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int STG_BYTES = 32 * 128;
     static constexpr int SMEM = STAGES * STAGE + 1024 + 1024 + EPI_WARPS * STG_BYTES;
 };
 
 struct WCtl {
-    uint64_t full[WCfg::STAGES], empty[WCfg::STAGES], tfull, tempty;
+    uint64_t full[8], empty[8], tfull[2], tempty[2];
     uint32_t tmem_base;
     int abort_flag;
     int offs[34];
     int perm[32];                  // experts by descending row count
     uint64_t sfull[kSchedSlots], sempty[kSchedSlots];
-    int sched_tile[kSchedSlots];   // tiles handed from the producer warp to the MMA thread and the epilogue warps
+    int sched_tile[kSchedSlots];   // tiles handed from the producer warp to the MMA warp and the epilogue warps
 };
 
-__global__ void __launch_bounds__(WCfg::THREADS, 1)
+template <int BN, int MT>
+__global__ void __launch_bounds__(WCfg<BN, MT>::THREADS, 1)
 wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
              const __grid_constant__ CUtensorMap tmW, const int* __restrict__ offsets, int n, int M, int N,
              int* status, int gather_p, int gather_q, const int* __restrict__ src_patch, int l_p, int Bm,
              int* __restrict__ sched /* [2], zero between launches */) {
     pdl_trigger();
-    using Cf = WCfg;
+    using Cf = WCfg<BN, MT>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     WCtl* ctl = (WCtl*)(smem + Cf::STAGES * Cf::STAGE);
@@ -67,8 +71,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cf::STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-        mbar_init(&ctl->tfull, 1);
-        mbar_init(&ctl->tempty, 32 * Cf::EPI_WARPS);
+        for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tfull[a], 1); mbar_init(&ctl->tempty[a], 32 * Cf::EPI_WARPS); }
         for (int q = 0; q < kSchedSlots; ++q) { mbar_init(&ctl->sfull[q], 1); mbar_init(&ctl->sempty[q], 1 + Cf::EPI_WARPS); }
         ctl->abort_flag = 0;
         fence_barrier_init();
@@ -208,7 +211,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
         // MMA issuer: the whole warp, one elected lane issues
         const uint32_t el = elect_one();
         constexpr uint32_t idesc = instr_desc_bf16(BM, BN, true, true);
-        int stage = 0;
+        int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool stop = false;
         int slot = 0;
@@ -220,9 +223,9 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
             if (tile >= total_tiles) break;
             int e, m0, n0, num_kb;
             decode(tile, e, m0, n0, num_kb);
-            if (!mbar_wait_warp(&ctl->tempty, acc_phase ^ 1, abort_flag, status)) break;
+            if (!mbar_wait_warp(&ctl->tempty[acc], acc_phase ^ 1, abort_flag, status)) break;
             tc_fence_after();
-            const uint32_t d_tmem = tmem_base;
+            const uint32_t d_tmem = tmem_base + acc * BN;
             for (int kb = 0; kb < num_kb; ++kb) {
                 if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                 tc_fence_after();
@@ -240,12 +243,13 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
                 if (++stage == Cf::STAGES) { stage = 0; phase ^= 1; }
             }
             if (stop) break;
-            mma_commit(el, &ctl->tfull);
-            acc_phase ^= 1;
+            mma_commit(el, &ctl->tfull[acc]);
+            if (++acc == Cf::NACC) { acc = 0; acc_phase ^= 1; }
         }
     } else {
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
+        int acc = 0;
         uint32_t acc_phase = 0;
         int slot = 0;
         uint32_t sphase = 0;
@@ -256,11 +260,11 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
             if (tile >= total_tiles) break;
             int e, m0, n0, num_kb;
             decode(tile, e, m0, n0, num_kb);
-            const bool ready = mbar_wait(&ctl->tfull, acc_phase, abort_flag, status) && !*abort_flag;
+            const bool ready = mbar_wait(&ctl->tfull[acc], acc_phase, abort_flag, status) && !*abort_flag;
             if (!__all_sync(0xffffffffu, ready)) break;
             tc_fence_after();
             const int wrow0 = e * M + m0 + half * BM + quarter * 32;   // first row of this warp's piece in [n*M, N]
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * BN;
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (MT == 2 ? half : acc) * BN;
             uint8_t* stg = smem + Cf::STAGES * Cf::STAGE + 1024 + (warp - 2) * Cf::STG_BYTES;
             // the TMEM read of the next piece is in flight while this one is staged and stored
             uint32_t v[32];
@@ -284,8 +288,8 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
                 if (lane == 0) { tma_store_2d(&tmW, stg, n0 + ch * 32, wrow0); bulk_commit(); }
             }
             tc_fence_before();
-            mbar_arrive(&ctl->tempty);
-            acc_phase ^= 1;
+            mbar_arrive(&ctl->tempty[acc]);
+            if (++acc == Cf::NACC) { acc = 0; acc_phase ^= 1; }
         }
     }
     if (warp >= 2 && lane == 0) bulk_wait_all();
@@ -305,11 +309,12 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CU
     }
 }
 
+template <int BN, int MT>
 uoe_status launch_w(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
                     long long rows_max, const char* label, int* status, cudaStream_t s, const WgradGather& g) {
-    using Cf = WCfg;
+    using Cf = WCfg<BN, MT>;
     static DeviceOnce once;
-    auto kern = wgrad_kernel;
+    auto kern = wgrad_kernel<BN, MT>;
     {
         const uoe_status st = smem_opt_in(once, kern, Cf::SMEM);
         if (st != UOE_OK) return st;
@@ -348,15 +353,16 @@ uoe_status launch_w(const void* P, const void* Q, float* dW, const int* offsets,
 
 }  // namespace
 
-// 256 x 256 tiles keep every SM busy with at least two of them; below that the matrices go to wgrad_stream_kernel.
 bool wgrad_large(int n, int M, int N) { return M % 256 == 0 && N % 256 == 0 && (long long)n * (M / 256) * (N / 256) >= 2 * sm_count(); }
 
-uoe_status launch_wgrad_large(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
+uoe_status launch_wgrad_whole(const void* P, const void* Q, float* dW, const int* offsets, int n, int M, int N,
                               long long rows_max, const char* label, int* status, cudaStream_t s, const WgradGather& g) {
     if (!status) return UOE_ERR_INVALID_ARG;       // the tile counters live in the control block behind the status word
-    if (M % 256 != 0 || N % 256 != 0 || n > 32) return UOE_ERR_UNSUPPORTED;
-    if ((g.gather_p || g.gather_q) && (!g.src_patch || !wgrad_large_can_gather(g.l_p))) return UOE_ERR_INVALID_ARG;
-    return launch_w(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, g);
+    if (M % BM != 0 || N % BM != 0 || n > 32) return UOE_ERR_UNSUPPORTED;
+    if ((g.gather_p || g.gather_q) && (!g.src_patch || !wgrad_whole_can_gather(g.l_p))) return UOE_ERR_INVALID_ARG;
+    if (wgrad_large(n, M, N)) return launch_w<256, 2>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, g);
+    if (N % 256 == 0) return launch_w<256, 1>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, g);
+    return launch_w<128, 1>(P, Q, dW, offsets, n, M, N, rows_max, label, status, s, g);
 }
 
 }  // namespace uoe

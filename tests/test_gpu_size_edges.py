@@ -239,3 +239,49 @@ def test_router_gradient_of_rows_past_two_to_the_31():
     assert (dWr[:, 0].double() - ref).abs().max() <= 1e-3 * ref.abs().max()
     assert (dWr[:, 1].double() + ref).abs().max() <= 1e-3 * ref.abs().max()
     assert (dx[-1] == 0).all()
+
+
+# whole tiles (many of them, operands past L2): 128 x 256 gathered and from copies, 128 x 128 beside 128 x 256, experts without rows
+WHOLE_CASES = {
+    "gathered_256": dict(B=34, L=512, l_p=32, d=1024, n=16, k=4, c=8, d_e=512),
+    "copies_256": dict(B=24, L=480, l_p=24, d=1024, n=16, k=4, c=12, d_e=512),
+    "gathered_128": dict(B=72, L=512, l_p=64, d=896, n=12, k=2, c=3, d_e=1024),
+    "some_experts_idle": dict(B=48, L=512, l_p=16, d=1280, n=16, k=3, c=10, d_e=640, used=(0, 5, 6, 11, 15)),
+}
+
+
+@pytest.mark.parametrize("name", list(WHOLE_CASES))
+def test_weight_gradients_of_whole_tiles(name):
+    """Against float64 on the GPU with the identity as activation; the bfloat16 tolerance of the other gradients."""
+    import paper_2503_02495_b200 as uoe
+    kw = dict(WHOLE_CASES[name])
+    used, l_p = kw.pop("used", None), kw.pop("l_p")
+    p = uoe.Problem(**kw, m=kw["L"] // l_p, L_valid=kw["L"] - 5, act="identity", residual=False)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    rn = lambda *s, std=1.0: (std * torch.randn(*s, device="cuda", generator=g)).bfloat16()
+    x, dy, Wr = rn(p.B, p.L, p.d), rn(p.B, p.L, p.d), rn(p.d, p.n, std=0.05)
+    x[:, p.L_valid:] = 0
+    W1, W2 = rn(p.n, p.d, p.d_e, std=0.03), rn(p.n, p.d_e, p.d, std=0.03)
+    r = uoe.uoe_route(p, x, Wr)
+    if used:       # the same patches, the experts drawn from a few
+        pick = torch.stack([torch.tensor(used, device="cuda")[torch.randperm(len(used), device="cuda", generator=g)[:p.k]].sort().values for _ in range(p.B)])
+        r.expert_idx = pick.to(torch.int32)
+        rows = torch.bincount(pick.flatten(), minlength=p.n) * p.l_a
+        r.expert_offsets = torch.cat([rows.new_zeros(1), ((rows + 127) // 128 * 128).cumsum(0)]).to(torch.int32)
+    sh = uoe.alloc_saved_h(p)
+    uoe.uoe_mlp_forward(p, x, W1, W2, r, saved_h=sh)
+    uoe.uoe_profile_enable(True)
+    _, dW1, dW2, _ = uoe.uoe_mlp_backward(p, x, W1, W2, Wr, r, sh, dy)
+    uoe.uoe_profile_enable(False)
+    assert {"wgrad_W1", "wgrad_W2"} <= {label for label, _ in uoe.uoe_profile_records()}      # this case is one of whole tiles
+    tok = (r.patch_idx.long()[..., None] * l_p + torch.arange(l_p, device="cuda")).flatten(2)          # [B, k, l_a]
+    w = (r.gate.double().repeat_interleave(l_p, 2) * (tok < p.L_valid)).flatten(1)
+    for e in range(p.n):
+        b, s = (r.expert_idx == e).nonzero(as_tuple=True)
+        xe = x.double()[b[:, None], tok[b, s]].flatten(0, 1)
+        de = (dy.double()[b[:, None], tok[b, s]] * w.view(p.B, p.k, -1)[b, s][..., None]).flatten(0, 1)
+        for got, ref in ((dW1[e], xe.T @ (de @ W2[e].double().T)), (dW2[e], (xe @ W1[e].double()).T @ de)):
+            if len(b):
+                assert (got.double() - ref).abs().max() <= TOL * ref.abs().max()
+            else:
+                assert (got == 0).all()
