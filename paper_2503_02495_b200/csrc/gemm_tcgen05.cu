@@ -73,7 +73,7 @@ struct Ctl {                       // lives behind the stage ring
     int tstart[34];                // first row tile of each expert (prefix sum), tstart[n] = number of row tiles
 };
 
-template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR, bool ROPE>
+template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR, bool ROPE, int CW /* columns of a chunk of the forward epilogue */>
 __global__ void __launch_bounds__(Cfg<BN, MT, EPI, PAIR>::THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                  const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2,
@@ -325,16 +325,24 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             __syncwarp();
             if (lane == 0) { tma_store_2d(&tmC0, stg, c0, r0); tma_store_2d(&tmC1, stg + 2048, c0, r0); bulk_commit(); }
         };
-        // the forward epilogue: 32 columns of this thread's row -> bf16 -> one half of the staging piece (64-byte rows) -> TMA
-        // store; the halves take turns, so a chunk waits for the store before the last one only
-        int stg_half = 0;
+        // the forward epilogue: CW columns of this thread's row -> bf16 -> staging piece -> TMA store.  32 columns take one half of
+        // the piece (64-byte rows), and the halves take turns, so that a chunk waits for the store before the last one only; 64
+        // columns take all of it (whole 128-byte lines), and a chunk waits for the store before it.
+        [[maybe_unused]] int stg_half = 0;
         auto stage_store = [&](const float* f, const CUtensorMap* tm, int c0, int r0) {
-            if (lane == 0) bulk_wait_read_but_one();
+            if (lane == 0) {
+                if (CW == 32) bulk_wait_read_but_one();
+                else bulk_wait_read();
+            }
             __syncwarp();
-            uint8_t* p = stg + stg_half * 2048;
-            stg_half ^= 1;
+            uint8_t* p = stg;
+            if constexpr (CW == 32) {
+                p += stg_half * 2048;
+                stg_half ^= 1;
+            }
 #pragma unroll
-            for (int c = 0; c < 4; ++c) *(uint4*)(p + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = pack8(f + 8 * c);
+            for (int c = 0; c < CW / 8; ++c)
+                *(uint4*)(p + lane * (2 * CW) + ((CW == 32 ? c ^ ((lane >> 1) & 3) : c ^ (lane & 7)) << 4)) = pack8(f + 8 * c);
             fence_async_smem();
             __syncwarp();
             if (lane == 0) { tma_store_2d(tm, p, c0, r0); bulk_commit(); }
@@ -454,18 +462,19 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g)
 #pragma unroll (ROPE ? 2 : 1)
-                    for (int c = 0; c < 2; ++c) {
-                        const int col = g * 64 + c * 32;             // in the tile
-                        uint32_t v[32];
+                    for (int c = 0; c < 64 / CW; ++c) {
+                        const int col = g * 64 + c * CW;             // in the tile
+                        uint32_t v[CW];
                         tmem_ld32(taddr + col, v);
+                        if constexpr (CW == 64) tmem_ld32(taddr + col + 32, v + 32);
                         tmem_ld_wait();
-                        float f[32];
+                        float f[CW];
 #pragma unroll
-                        for (int q = 0; q < 32; ++q) f[q] = __uint_as_float(v[q]);
+                        for (int q = 0; q < CW; ++q) f[q] = __uint_as_float(v[q]);
                         if (bias) {                                  // the expert's bias row (the in-place bias of the batched product)
                             const uint4* bp = (const uint4*)(bias + (size_t)e * N + (SIDE3 ? 0 : col0) + col);
 #pragma unroll
-                            for (int q8 = 0; q8 < 4; ++q8) {
+                            for (int q8 = 0; q8 < CW / 8; ++q8) {
                                 float bv[8];
                                 unpack16<__nv_bfloat16>(bp[q8], bv);
 #pragma unroll
@@ -488,13 +497,13 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                         }
                         if (pre) stage_store(f, &tmPre, col0 + col, wrow0);
-                        act_apply_n<32>(f, act);
+                        act_apply_n<CW>(f, act);
                         if (blk_scale) {
                             const float sc = blk_scale[(row0 + half * BM) >> 7];
 #pragma unroll
-                            for (int q = 0; q < 32; ++q) f[q] *= sc;
+                            for (int q = 0; q < CW; ++q) f[q] *= sc;
                         }
-                        if (SIDE3) stage_store(f, g == 0 ? &tmC0 : (g == 1 ? &tmC1 : &tmC2), c * 32, wrow0);
+                        if (SIDE3) stage_store(f, g == 0 ? &tmC0 : (g == 1 ? &tmC1 : &tmC2), c * CW, wrow0);
                         else stage_store(f, tmC, col0 + col, wrow0);
                     }
                 }
@@ -518,12 +527,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
 }
 
-template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR = false, bool ROPE = false>
+template <int BN, bool B_KMAJOR, int EPI, int MT, bool PAIR = false, bool ROPE = false, int CW = 32>
 uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     using Cf = Cfg<BN, MT, EPI, PAIR>;
     static DeviceOnce once;
     static DeviceValue pairs_cache;    // CTA pairs that can be resident at once, per device
-    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, EPI, MT, PAIR, ROPE>;
+    auto kern = gemm_bf16_kernel<BN, B_KMAJOR, EPI, MT, PAIR, ROPE, CW>;
     {
         const uoe_status st = smem_opt_in(once, kern, Cf::SMEM);
         if (st != UOE_OK) return st;
@@ -574,10 +583,10 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     {
         const uint64_t dims[2] = {(uint64_t)g.N, (uint64_t)g.rows_max};
         const uint64_t str[1] = {(uint64_t)g.N * 2};
-        const uint32_t box[2] = {32, 32};
+        const uint32_t box[2] = {CW, 32};
         const void* Cs[3] = {g.C, g.C1 ? g.C1 : g.C, g.C2 ? g.C2 : g.C};
         auto out_map = [&](CUtensorMap* tm, const void* p) {
-            return make_tmap(tm, p, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B);
+            return make_tmap(tm, p, 2, dims, str, box, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CW == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
         };
         for (int q = 0; q < 3; ++q)
             if (!out_map(&tmC[q], Cs[q])) return UOE_ERR_CUDA;
@@ -609,7 +618,7 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
     return UOE_OK;
 }
 
-template <bool B_KMAJOR, int EPI, bool ROPE = false>
+template <bool B_KMAJOR, int EPI, bool ROPE = false, int CW = 32>
 uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
     const int bn = gemm_bf16_bn(g.N);
     // 256-row tiles pay off when every SM still gets several of them and the K loop is long enough to be
@@ -621,12 +630,12 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
         if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true>(g, status, s);
     }
     if constexpr (EPI == kForward) {
-        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true, ROPE>(g, status, s);
-        if (bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 2, false, ROPE>(g, status, s);
+        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true, ROPE, CW>(g, status, s);
+        if (CW == 32 && bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 2, false, ROPE>(g, status, s);
     }
-    if (bn == 256) return launch_one<256, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
-    if (bn == 128) return launch_one<128, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
-    return launch_one<64, B_KMAJOR, EPI, 1, false, ROPE>(g, status, s);
+    if (bn == 256) return launch_one<256, B_KMAJOR, EPI, 1, false, ROPE, CW>(g, status, s);
+    if (bn == 128) return launch_one<128, B_KMAJOR, EPI, 1, false, ROPE, CW>(g, status, s);
+    return launch_one<64, B_KMAJOR, EPI, 1, false, ROPE, CW>(g, status, s);
 }
 
 }  // namespace
@@ -649,9 +658,16 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
         if (!g.b_kmajor || !g.bwd_h || !g.row_gate || !g.row_valid || !g.dg_part || !g.C1 || g.nmat > 1) return UOE_ERR_INVALID_ARG;
         return dispatch<true, kAttBackward>(g, status, s);
     }
-    if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre)
-        return rope ? launch_one<192, false, kForward, 1, false, true>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
+    // With one or two K blocks the launch is its output: whole lines per store (64-column chunks).  Output projection of one head,
+    // 25600 rows x 1024 columns: 21 us in 32-column chunks, 19 so; K = 128, N = 1408, 67k rows, with the pre-activation: 82 and
+    // 68.  From four K blocks on the 32-column chunks are ahead (K = 256, N = 256, 32k rows: 25 us against 27).
+    const bool short_k = g.K <= 128;
+    if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre) {
+        if (rope) return launch_one<192, false, kForward, 1, false, true>(g, status, s);
+        return short_k ? launch_one<192, false, kForward, 1, false, false, 64>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
+    }
     if (rope) return dispatch<false, kForward, true>(g, status, s);
+    if (short_k) return g.b_kmajor ? dispatch<true, kForward, false, 64>(g, status, s) : dispatch<false, kForward, false, 64>(g, status, s);
     if (g.b_kmajor) return dispatch<true, kForward>(g, status, s);
     return dispatch<false, kForward>(g, status, s);
 }

@@ -285,3 +285,42 @@ def test_weight_gradients_of_whole_tiles(name):
                 assert (got.double() - ref).abs().max() <= TOL * ref.abs().max()
             else:
                 assert (got == 0).all()
+
+
+# one or two K blocks: whole lines per store of the forward epilogue, every tile width, CTA pairs, side-by-side projections
+@pytest.mark.parametrize("d,d_e,B", [(64, 64, 3), (128, 320, 3), (64, 1152, 5), (128, 512, 3), (128, 1280, 260)])
+def test_forward_of_short_contractions(d, d_e, B):
+    """The pre-activation and y against float64 on the GPU, the bfloat16 tolerance of the other outputs."""
+    import paper_2503_02495_b200 as uoe
+    p = uoe.Problem(B=B, L=256, L_valid=250, d=d, n=3, k=2, m=4, c=3, d_e=d_e, residual=False)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    rn = lambda *s, std=1.0: (std * torch.randn(*s, device="cuda", generator=g)).bfloat16()
+    x, Wr, W1, W2 = rn(p.B, p.L, d), rn(d, p.n, std=0.1), rn(p.n, d, d_e, std=0.1), rn(p.n, d_e, d, std=0.1)
+    b1, b2 = rn(p.n, d_e), rn(p.n, d)
+    x[:, p.L_valid:] = 0
+    r = uoe.uoe_route(p, x, Wr)
+    sh = uoe.alloc_saved_h(p)
+    y = uoe.uoe_mlp_forward(p, x, W1, W2, r, b1=b1, b2=b2, saved_h=sh)
+    tok = (r.patch_idx.long()[..., None] * p.l_p + torch.arange(p.l_p, device="cuda")).flatten(2)
+    ref = torch.zeros(p.B, p.L, d, dtype=torch.float64, device="cuda")
+    for e in range(p.n):
+        b, s = (r.expert_idx == e).nonzero(as_tuple=True)
+        h = x.double()[b[:, None], tok[b, s]] @ W1[e].double() + b1[e].double()
+        off = int(r.expert_offsets[e])
+        assert (sh[off:off + h.shape[0] * p.l_a].double() - h.flatten(0, 1)).abs().max() <= TOL * h.abs().max()
+        z = (torch.nn.functional.silu(h) @ W2[e].double() + b2[e].double()) * r.gate.double()[b, s].repeat_interleave(p.l_p, 1)[..., None]
+        ref.index_put_((b[:, None].expand(-1, p.l_a), tok[b, s]), z * (tok[b, s] < p.L_valid)[..., None], accumulate=True)
+    assert (y.double() - ref).abs().max() <= TOL * ref.abs().max()
+
+
+@pytest.mark.parametrize("d,heads", [(64, 1), (128, 1), (640, 1), (1088, 2), (1280, 1)])
+def test_attention_projections_of_short_contractions(d, heads):
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(B=3, L=96, L_valid=90, m=6, c=4, d=d, n=2, k=2, d_ff=0, H=2 * heads, d_h=64, dtype="bf16", w_std=0.05, causal=True)
+    x, Wr, ws = gen.make_x(w), gen.make_router(w, "att"), gen.make_attn_weights(w)
+    prob = problem_of(w, "att", residual=False)
+    r = uoe.uoe_route(prob, to_dev(x), to_dev(Wr))
+    y = uoe.uoe_smha_forward(prob, to_dev(x), *(to_dev(q) for q in ws), r)
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    ref = orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False)
+    assert rel_inf(to_f64(y), ref) <= TOL
