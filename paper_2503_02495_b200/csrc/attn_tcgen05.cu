@@ -6,7 +6,7 @@
 // one 128-query tile of one head of one pair; its keys come in 128-key tiles.
 //
 // Two kernels:
-//   attn_stream_kernel   more units than SMs.  A persistent CTA (one per SM) holds two independent
+//   attn_stream_kernel   many units (launch_attention says which of the two).  A persistent CTA (one per SM) holds two independent
 //     pipelines, each with its own TMA warp, its own MMA-issuing warp, four softmax warps (one thread per query row),
 //     its own Q buffer, two K/V stages, P buffer and TMEM columns, and each working units of its own:
 //       TMA warp      Q tile of the unit, then K and V of each key tile into the two-stage ring; with the fused output
@@ -20,7 +20,7 @@
 //     The pipelines only meet in the tensor and special-function units of their SM: while one computes exponentials
 //     or drains its output, the other's MMAs and loads run, and a pipeline's next Q, K, V are in flight while it
 //     still works the current unit.
-//   attn_tile_kernel     few units (at most one per SM): one CTA per unit, all eight warps on its softmax (two
+//   attn_tile_kernel     few units, or short ones: one CTA per unit, all eight warps on its softmax (two
 //     threads per query row), S of the next key tile issued behind P V, the output projection as one MMA group over
 //     all of TMEM.  With one unit per SM there is nothing to overlap a unit with, so the whole CTA works the unit.
 // Masks: the real keys of a pair are a prefix of its gathered order (patches ascending, pad tokens at
@@ -852,9 +852,13 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)D.d_h);
     ProfScope ps("attention", s);
     cudaError_t e;
-    // more units than SMs: two pipelines per SM (256 causal units of up to eight key tiles: 27 us, against 34 in two waves
-    // of one CTA per unit)
-    if (units > sm_count()) {
+    // Two pipelines per SM from two units per SM on, and below that from one, if a unit has four key tiles or more on average:
+    // then two waves of one CTA per unit take longer than one of pairs, with less they do not (whole attention forward, us,
+    // pairs / waves: 160 units of 16 key tiles 82 / 98, 256 causal ones of up to eight 87 / 90, 176 of four 56 / 58, 180 of three
+    // 54 / 55, 180 of two 52 / 52, 152 of one 74 / 70 with d = 1024).
+    const int n_kt = (D.l_a + TK - 1) / TK;
+    const double key_tiles = causal ? (n_kt + 1) / 2.0 : n_kt;
+    if (units >= 2ll * sm_count() || (units > sm_count() && key_tiles >= 4)) {
         AttnArgs a;
         a.O = (__nv_bfloat16*)o; a.Z = (__nv_bfloat16*)z; a.lse = lse;
         a.pair_row = pair_row; a.patch_idx = patch_idx; a.expert_idx = expert_idx;
@@ -867,7 +871,7 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
         if (fuse) e = launch_k(attn_stream_kernel<true>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
         else e = launch_k(attn_stream_kernel<false>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
     } else {
-        if (pairs > 65535) return UOE_ERR_UNSUPPORTED;      // (cannot happen: at most one unit per SM)
+        if (pairs > 65535) return UOE_ERR_UNSUPPORTED;      // (cannot happen: fewer than two units per SM)
         dim3 grid(n_qt, heads, (unsigned)pairs);
         if (fuse)
             e = launch_k(attn_tile_kernel<true>, grid, dim3(kTileThreads), TILE_SMEM_FUSED, s, tm[0], tm[1], tm[2], (__nv_bfloat16*)o, lse,
