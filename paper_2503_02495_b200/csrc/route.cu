@@ -491,9 +491,11 @@ route_sample_kernel(const T* __restrict__ x, const T* __restrict__ W_r, int B, i
 }
 
 // Selection as a kernel of its own (after a route_kernel launch without tickets): grid B, one CTA per sample.  One chain per
-// sample: 16 warps leave two turns of phase A to each at m = 64, n = 16 (11.6 us, cold caches; 8 warps 14.0).
-constexpr int kSelectThreads = 512;
-__global__ void __launch_bounds__(kSelectThreads)
+// sample: 16 warps leave two turns of phase A to each at m = 64, n = 16 (11.6 us, cold caches; 8 warps 14.0).  With more samples
+// than CTAs of 16 warps fit the machine twice per SM the warps of other samples fill the gaps: 8 warps (600 samples of four
+// patches, 8 experts: whole call 27.7 us, with 16 warps 31.4; 5000 samples of two 75 and 107).
+template <int NT>
+__global__ void __launch_bounds__(NT)
 route_select_kernel(const float* __restrict__ scores, int nparts, int B, int Lv, int n, int k, int m, int c, int l_p,
                     int use_gate, int* __restrict__ expert_idx, int* __restrict__ patch_idx, float* __restrict__ gate,
                     float* __restrict__ p_samp, float* __restrict__ p_patch, int* __restrict__ offsets,
@@ -501,7 +503,7 @@ route_select_kernel(const float* __restrict__ scores, int nparts, int B, int Lv,
     pdl_trigger();
     pdl_wait();
     extern __shared__ float s_sel[];
-    select_sample<kSelectThreads>(s_sel, scores, nparts, blockIdx.x, B, Lv, n, k, m, c, l_p, use_gate, expert_idx, patch_idx, gate,
+    select_sample<NT>(s_sel, scores, nparts, blockIdx.x, B, Lv, n, k, m, c, l_p, use_gate, expert_idx, patch_idx, gate,
                                  p_samp, p_patch, offsets, masks, ctl + 1, plan);
 }
 
@@ -623,9 +625,11 @@ uoe_status route_launch(const Dims& D, uint32_t flags, const void* x, const void
     {
         ProfScope ps(profile ? "route_select" : nullptr, stream);
         const size_t sel = (size_t)D.n * D.m * sizeof(float);
-        e = launch_k(route_select_kernel, dim3(D.B), dim3(kSelectThreads), sel, stream, (const float*)scores, W.nchunks * W.rsplit,
-                     D.B, D.Lv, D.n, D.k, D.m, D.c, D.l_p, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch,
-                     expert_offsets, ctl, masks, plan);
+        auto go = [&](auto kern, int threads) {
+            return launch_k(kern, dim3(D.B), dim3(threads), sel, stream, (const float*)scores, W.nchunks * W.rsplit, D.B, D.Lv, D.n, D.k, D.m,
+                            D.c, D.l_p, use_gate, expert_idx, patch_idx, gate, p_samp, p_patch, expert_offsets, ctl, masks, plan);
+        };
+        e = D.B <= 2 * sm_count() ? go(route_select_kernel<512>, 512) : go(route_select_kernel<256>, 256);
     }
     if (e != cudaSuccess) return UOE_ERR_CUDA;
     UOE_LAUNCHED();
