@@ -17,7 +17,7 @@ constexpr int kPlanScanMaxB = 512;        // up to here every sample's CTA scans
 
 __global__ void __launch_bounds__(1024)
 plan_rows_kernel(const int* __restrict__ expert_idx, const int* __restrict__ offsets, int B, int n, int k, int l_a,
-                 int* __restrict__ pair_row, int* __restrict__ slot_pair, int slot_shift, int rows_max) {
+                 int* __restrict__ pair_row, int* __restrict__ slot_pair, int slot_shift) {
     pdl_trigger();
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -30,19 +30,24 @@ plan_rows_kernel(const int* __restrict__ expert_idx, const int* __restrict__ off
             if (b < B)
                 for (int s = 0; s < k; ++s)
                     if (expert_idx[(size_t)b * k + s] == i) slots |= 1u << s;
-            int incl = __popc(slots);
+            const unsigned ball = __ballot_sync(0xffffffffu, slots != 0u);
+            int q = running + __popc(ball & ((1u << lane) - 1u));
+            running += __popc(ball);
+            if (__any_sync(0xffffffffu, slots & (slots - 1u))) {      // more than one slot of a sample: count slots, not samples
+                int incl = __popc(slots);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                q = running - __popc(ball) + incl - __popc(slots);
+                running += __shfl_sync(0xffffffffu, incl, 31) - __popc(ball);
             }
-            int q = running + incl - __popc(slots);
             for (unsigned left = slots; left; left &= left - 1, ++q) {
-                const int pair = b * k + __ffs(left) - 1, row = off_i + q * l_a;
-                pair_row[pair] = row;
-                if (row >= 0 && row <= rows_max - l_a) slot_pair[pair_slot_by_row(off_i, q, slot_shift)] = pair;
+                const int pair = b * k + __ffs(left) - 1;
+                pair_row[pair] = off_i + q * l_a;
+                slot_pair[pair_slot_by_row(off_i, q, slot_shift)] = pair;
             }
-            running += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
 }
@@ -110,7 +115,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             if (!rows_given) slot_pair[pair_slot_by_row(offs[e], q, slot_shift)] = b * k + tid;
         }
         prow[tid] = row;
-        pair_row[b * k + tid] = row;
+        if (!rows_given || e < 0) pair_row[b * k + tid] = row;
     }
     __syncthreads();
     for (int idx = tid; idx < m * k; idx += NT) {          // inverse map: which routed rows feed patch j
@@ -449,7 +454,7 @@ uoe_status launch_plan(const Dims& D, const int* expert_idx, const int* patch_id
     if (many) {
         ProfScope ps("plan_rows", s);
         launch_k(plan_rows_kernel, dim3(1), dim3(1024), 0, s, expert_idx, offsets, D.B, D.n, D.k, D.l_a, P.pair_row, P.slot_pair,
-                 pair_slot_shift(D.l_a), (int)D.Rmax);
+                 pair_slot_shift(D.l_a));
         UOE_LAUNCHED();
     }
     ProfScope ps("plan", s);
