@@ -630,7 +630,12 @@ uoe_status dispatch(const GemmArgs& g, int* status, cudaStream_t s) {
         if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true>(g, status, s);
     }
     if constexpr (EPI == kForward) {
-        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 1, true, ROPE, CW>(g, status, s);
+        if (bn == 256 && g.K % 128 == 0 && tiles256 >= 2 * sm_count()) {
+            if constexpr (!ROPE) {      // (a pair's main loop is shorter: the whole-line epilogue is the better one up to here)
+                if (g.K <= 512) return launch_one<256, B_KMAJOR, EPI, 1, true, false, 64>(g, status, s);
+            }
+            return launch_one<256, B_KMAJOR, EPI, 1, true, ROPE>(g, status, s);
+        }
         if (CW == 32 && bn == 256 && g.K >= 1024 && tiles256 >= 2 * sm_count()) return launch_one<256, B_KMAJOR, EPI, 2, false, ROPE>(g, status, s);
     }
     if (bn == 256) return launch_one<256, B_KMAJOR, EPI, 1, false, ROPE, CW>(g, status, s);
@@ -658,9 +663,9 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
         if (!g.b_kmajor || !g.bwd_h || !g.row_gate || !g.row_valid || !g.dg_part || !g.C1 || g.nmat > 1) return UOE_ERR_INVALID_ARG;
         return dispatch<true, kAttBackward>(g, status, s);
     }
-    // With one or two K blocks the launch is its output: whole lines per store (64-column chunks).  Output projection of one head,
-    // 25600 rows x 1024 columns: 21 us in 32-column chunks, 19 so; K = 128, N = 1408, 67k rows, with the pre-activation: 82 and
-    // 68.  From four K blocks on the 32-column chunks are ahead (K = 256, N = 256, 32k rows: 25 us against 27).
+    // With a short contraction the launch is its output: whole lines per store (64-column chunks).  Output projection of one
+    // head, 25600 rows x 1024 columns: 21 us in 32-column chunks, 19 so; K = 128, N = 1408, 67k rows, with the pre-activation: 82
+    // and 68; on CTA pairs 131k rows, N = 1024: K = 256 115 and 99, K = 384 117 and 107, K = 512 equal, K = 1024 213 and 224.
     const bool short_k = g.K <= 128;
     if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre) {
         if (rope) return launch_one<192, false, kForward, 1, false, true>(g, status, s);
