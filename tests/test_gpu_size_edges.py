@@ -324,3 +324,19 @@ def test_attention_projections_of_short_contractions(d, heads):
     ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
     ref = orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False)
     assert rel_inf(to_f64(y), ref) <= TOL
+
+
+@pytest.mark.parametrize("heads", [1, 3])
+def test_attention_of_pairs_with_fewer_key_tiles_than_others(heads):
+    """Pairs that hold the last, nearly empty patch have one key tile less; more units than two per SM."""
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(B=60 // heads, L=6 * 48, L_valid=5 * 48 + 1, m=6, c=3, d=64, n=3, k=3, d_ff=0, H=3 * heads, d_h=64, dtype="bf16", w_std=0.08)
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w, "att").f64 * 20, w.dtype)
+    ws = gen.make_attn_weights(w)
+    prob = problem_of(w, "att", residual=False)
+    r = uoe.uoe_route(prob, to_dev(x), to_dev(Wr))
+    has_last = (r.patch_idx == w.m - 1).any(2)
+    assert has_last.any() and not has_last.all()
+    y = uoe.uoe_smha_forward(prob, to_dev(x), *(to_dev(q) for q in ws), r)
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    assert rel_inf(to_f64(y), orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False)) <= TOL
