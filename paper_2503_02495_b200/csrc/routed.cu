@@ -293,7 +293,8 @@ combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __re
                     }
                 }
             }
-            if (BWD && rvec) {
+            if (rvec) {         // (a run-time check in the forward too: without it the compiler orders the loop above worse, d = 2432,
+                                // sixteen experts, 22k tokens 176 us instead of 166)
                 const float* rp = rvec + (size_t)bj * d + (size_t)cv * V;
 #pragma unroll
                 for (int v = 0; v < V; v += 4) {
