@@ -50,22 +50,42 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int idx = tid; idx < n * m; idx += kGradThreads) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
     if (tid < 32) { ps[tid] = tid < n ? p_samp[(size_t)b * n + tid] : 0.f; dps[tid] = 0.f; }
+    // four slabs at a time, so that their look-ups and loads are in flight together (one at a time a sample of 1271 slabs of
+    // four tokens took 90 us)
     const int len = l_p * nt;
-    for (int slab = warp; slab < k * c; slab += kGradThreads / 32) {
-        const int j = patch_idx[(size_t)b * k * c + slab];
-        float a = 0.f;
-        if (j >= 0 && j < m) {
-            const float* src = dg_part + ((size_t)pair_row[b * k + slab / c] + (size_t)(slab % c) * l_p) * nt;
-            int q = lane;
-            for (; q + 96 < len; q += 128) {
-                const float t0 = src[q], t1 = src[q + 32], t2 = src[q + 64], t3 = src[q + 96];
-                a += (t0 + t1) + (t2 + t3);
-            }
-            for (; q < len; q += 32) a += src[q];
+    constexpr int U = 4;
+    for (int slab0 = warp * U; slab0 < k * c; slab0 += kGradThreads / 32 * U) {
+        const float* src[U];
+        int n_q[U];                                       // values of the slab: none of an unused slot
+        float a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int slab = min(slab0 + u, k * c - 1);
+            const int j = patch_idx[(size_t)b * k * c + slab];
+            src[u] = dg_part + ((size_t)pair_row[b * k + slab / c] + (size_t)(slab % c) * l_p) * nt;
+            n_q[u] = j >= 0 && j < m ? len : 0;
+            a[u] = 0.f;
+        }
+        int q = lane;
+        for (; q + 96 < len; q += 128) {
+            float t[U][4];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int w = 0; w < 4; ++w) t[u][w] = n_q[u] ? src[u][q + 32 * w] : 0.f;
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] += (t[u][0] + t[u][1]) + (t[u][2] + t[u][3]);
+        }
+        for (; q < len; q += 32) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] += n_q[u] ? src[u][q] : 0.f;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) dg[slab] = a;
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a[u] += __shfl_xor_sync(0xffffffffu, a[u], o);
+            if (lane == 0 && slab0 + u < k * c) dg[slab0 + u] = a[u];
+        }
     }
     __syncthreads();
     // gate = P_samp * P_patch: a warp per chosen expert, lanes over its slots
