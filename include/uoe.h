@@ -26,6 +26,9 @@
  *     device properties are set up per device by the first call that needs them there.  Calls from several threads
  *     are safe, first calls included, as long as they use distinct workspaces (and, for uoe_route_static, are
  *     ordered on the device as described there).  uoe_profile_* is never thread-safe.
+ *   - Streams.  Calls on different streams may run at the same time.  Launches of about one to four small CTAs per SM ask
+ *     for shared memory they do not use, so that they spread over the SMs; while one runs, fewer CTAs of another stream
+ *     fit beside it.
  *   - Element type: `dtype` selects float32 or bfloat16 storage for x, weights and y.  Products are
  *     accumulated in float32.  Routing probabilities and gates are always float32.
  *

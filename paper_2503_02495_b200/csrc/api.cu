@@ -11,9 +11,8 @@ bool g_prof_on = false;
 std::vector<ProfRec> g_prof;
 }  // namespace
 
-int sm_count() {
+int sm_count(int dev) {
     static DeviceValue cache;
-    const int dev = current_device();
     if (cache.has(dev)) return cache.get(dev);
     int v = 148;
     if (dev >= 0) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);

@@ -209,8 +209,8 @@ __device__ __forceinline__ void attn_bwd_body(const BwdMaps& m, const BwdMaps& m
                 mma_bf16(el, tmem + 128, smem_desc(v_a + ks * 32, 16, 1024), smem_desc(do_a + ks * 32, 16, 1024), idesc_s, ks != 0);
             mma_commit(el, &ctl->bar_s);
         }
-        // statistics of the 128 queries meanwhile: in P's upper tile, which nothing uses before the exponentials; read into
-        // registers piece by piece below, behind a barrier of their own
+        // statistics of the 128 queries meanwhile: in dS's tiles, which are written only behind the barrier that follows the
+        // last read of them
         float* st = (float*)sDS;                                              // [lse * log2 e | delta][128], overwritten by dS last
         if (tid < T) { st[tid] = stat(a.lse, tid) * kLog2e; st[T + tid] = stat(a.delta, tid); }
         __syncthreads();

@@ -6,8 +6,8 @@
 // one 128-query tile of one head of one pair; its keys come in 128-key tiles.
 //
 // Two kernels:
-//   attn_stream_kernel   many units (launch_attention says which of the two).  A persistent CTA (one per SM) holds two independent
-//     pipelines, each with its own TMA warp, its own MMA-issuing warp, four softmax warps (one thread per query row),
+//   attn_stream_kernel   many units (launch_attention says which of the two).  A persistent CTA (one per SM) holds two
+//     independent pipelines, each with its own TMA warp, its own MMA-issuing warp, four softmax warps (one thread per query row),
 //     its own Q buffer, two K/V stages, P buffer and TMEM columns, and each working units of its own:
 //       TMA warp      Q tile of the unit, then K and V of each key tile into the two-stage ring; with the fused output
 //                     projection also the expert's W^o in 192-column chunks through the same ring
@@ -146,7 +146,6 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         }
         return true;
     };
-    constexpr int t_first = 0, t_step = 1;
     auto kv_tiles = [&](int q0, int n_valid) {              // key tiles the unit has in all
         int kv_end = min(n_valid, a.l_a);
         if (a.causal) kv_end = min(kv_end, q0 + TQ);
@@ -176,7 +175,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const int expert = FUSE_O ? a.expert_idx[pair] : 0;
             const int q0 = qt * TQ, col_h = head * DH;
             const int n_kv = kv_tiles(q0, nv);
-            const bool mine = t_first < n_kv;
+            const bool mine = n_kv > 0;
             if (lane == 0) {
                 ok = wait1(&pc->q_empty, (q_cnt & 1) ^ 1);
                 if (ok) {
@@ -189,7 +188,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     }
                 }
                 ++q_cnt;
-                for (int t = t_first; t < n_kv && ok; t += t_step) {
+                for (int t = 0; t < n_kv && ok; ++t) {
                     const int st = kv_cnt & 1;
                     ok = wait1(&pc->kv_empty[st], ((kv_cnt >> 1) & 1) ^ 1);
                     if (!ok) break;
@@ -232,7 +231,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             ++q_cnt;
             if (!ok) break;
             const int n_kv = kv_tiles(qt * TQ, pc->n_valid);
-            if (t_first >= n_kv) {
+            if (n_kv == 0) {
                 __syncwarp();                 // every lane has read n_valid, which the TMA warp overwrites after the arrival
                 if (el) mbar_arrive(&pc->q_empty);
                 continue;
@@ -255,11 +254,11 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 if (last) mma_commit(el, &pc->q_empty);       // the unit's last use of Q
                 return true;
             };
-            ok = issue_s(kv_cnt, t_first + t_step >= n_kv);
-            for (int t = t_first; t < n_kv && ok; t += t_step) {
+            ok = issue_s(kv_cnt, n_kv == 1);
+            for (int t = 0; t < n_kv && ok; ++t) {
                 const int st = kv_cnt & 1;
-                if (t + t_step < n_kv) {
-                    ok = issue_s(kv_cnt + 1, t + 2 * t_step >= n_kv);
+                if (t + 1 < n_kv) {
+                    ok = issue_s(kv_cnt + 1, t + 2 >= n_kv);
                     if (!ok) break;
                 }
                 ok = waitw(&pc->p_full, p_cnt & 1);
@@ -315,7 +314,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (lane == 0) mbar_arrive(&pc->q_empty);
             const int q0 = qt * TQ, qrow = q0 + trow;
             const int n_kv = kv_tiles(q0, n_valid);
-            if (t_first >= n_kv) continue;
+            if (n_kv == 0) continue;
             const int kv_lim = min(n_valid, a.l_a);
 
             float o_acc[DH];
@@ -340,7 +339,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 return true;
             };
 
-            for (int t = t_first; t < n_kv && ok; t += t_step) {
+            for (int t = 0; t < n_kv && ok; ++t) {
                 ok = __all_sync(0xffffffffu, wait(&pc->acc_full, acc_cnt & 1));
                 ++acc_cnt;
                 if (!ok) break;

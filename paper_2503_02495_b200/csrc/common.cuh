@@ -54,21 +54,24 @@ inline uoe_status smem_opt_in(DeviceOnce& once, K kern, int bytes) {
     return UOE_OK;
 }
 
-int sm_count();       // SMs of the current device (cached per device)
+int sm_count(int dev);      // SMs of a device (cached; 148 if it is not known)
+inline int sm_count() { return sm_count(current_device()); }
 
 // Dynamic shared memory to request for a launch of `ctas` small CTAs so that they spread evenly over the SMs.  Under
 // programmatic launch the CTAs of a kernel become resident as the CTAs of the kernel before it leave, and the first SMs
 // to come free would take as many as fit while others get none: a kernel of one or two CTAs per SM then runs packed on a
 // fraction of the machine.  Asking for so much shared memory that no more than ceil(ctas / SMs) fit keeps them apart
-// (language-model training step 351 -> 326 us, wide block 688 -> 676 us, ragged forward 87 -> 81 us).  Not for fewer CTAs
+// (passes in a CUDA graph, without and with: float32 forward 39.3 and 31.9 us, ragged block forward 74.7 and 70.2,
+// language-model block forward 72.2 and 70.1, its training step 244.7 and 242.5).  The reservation also keeps CTAs of other
+// streams away: of nine pairs of such graphs on two streams eight were as fast together as without it or faster (two float32
+// forwards 43.5 -> 34.5 us), two language-model block forwards were 7 % slower (103.6 -> 111).  Not for fewer CTAs
 // than half the SMs, where one per SM gains nothing and waits for an SM with the room (three 16-CTA kernels in a
 // row: 88 -> 95 us; a 64-CTA combine: +2 us), nor beyond four per SM, where the packing evens out.
 struct SpreadOnce { DeviceOnce opt_in; DeviceValue fixed; };      // one per kernel
 template <typename K>
 inline size_t spread_smem(SpreadOnce& once, K kern, long long ctas, size_t smem) {
-    const int sms = sm_count();
+    const int dev = current_device(), sms = sm_count(dev);
     if (ctas < sms / 2 || ctas > 4ll * sms) return smem;
-    const int dev = current_device();
     if (!once.fixed.has(dev)) {               // static shared memory of the kernel plus the system's share of a CTA
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || smem_opt_in(once.opt_in, kern, 160 * 1024) != UOE_OK) return smem;

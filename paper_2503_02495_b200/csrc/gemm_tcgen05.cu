@@ -8,9 +8,9 @@
 //   warp 0      TMA producer (lane 0 runs the pipeline; boxes of a stage that need separate copies are issued one per
 //               lane): A tile [MT*128 x 64] and B tile [64 x BN] per K step into a 128B-swizzled ring
 //   warp 1      MMA issuer: tcgen05.mma 128 x BN x 16 into TMEM accumulators
-//   warps 2..   epilogue: tcgen05.ld the accumulator (one row per thread), activation, bf16, then a
-//               [32 rows x 64 columns] piece per warp staged in swizzled shared memory and written with one
-//               TMA tensor store (full 128-byte lines instead of 16-byte scattered stores)
+//   warps 2..   epilogue: tcgen05.ld the accumulator (one row per thread), activation, bf16, then pieces of 32 rows x 32
+//               columns (64 where the contraction is short) per warp, staged in swizzled shared memory and written
+//               with one TMA tensor store each
 // Three tile shapes:
 //   MT = 1  128-row tiles, two TMEM accumulators: the epilogue of tile t overlaps the main loop of tile t+1
 //   PAIR    256-row tiles worked by a cluster of two CTAs (tcgen05 cta_group::2): CTA r of the pair loads row block r
@@ -578,7 +578,7 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
             if (!make_tmap(&tmB[q], Ws[q], 4, dims, str, box)) return UOE_ERR_CUDA;
         }
     }
-    // outputs as [rows_max, N], written in [32 rows x 64 columns] pieces
+    // outputs as [rows_max, N], written in [32 rows x CW columns] pieces
     CUtensorMap tmC[3], tmPre;
     {
         const uint64_t dims[2] = {(uint64_t)g.N, (uint64_t)g.rows_max};

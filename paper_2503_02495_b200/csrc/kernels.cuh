@@ -125,7 +125,7 @@ inline SrcMap src_map_of(const Dims& D, const PlanPtrs& P, const int* patch_idx)
 // turns per token, split in two floats, so that the reduction to one turn is exact to well below the result's rounding.
 // (As a kernel of its own the rotation was a second pass over q and k and two roundings, and its 128 CTAs of sine code
 // started, under programmatic launch, on the few SMs the projection left first: the wide block forward, B = 4, L = 2048,
-// d = 1024, 16 heads, took 343 us with it and takes 189 us with the rotation in the epilogue.)
+// d = 1024, 16 heads, took 343 us with it and takes 170 us with the rotation in the epilogue.)
 struct Rope {
     int pair0 = 32;                    // first rotated channel pair of a 64-wide head (32: nothing is rotated)
     SrcMap map;                        // where a routed row comes from (through slot_pair)

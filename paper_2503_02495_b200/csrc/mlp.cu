@@ -12,7 +12,8 @@ static MlpFwdWs mlp_fwd_ws(const Dims& D) {
     w.take(kStatusBytes);
     MlpFwdWs r;
     r.plan = w.take(plan_bytes(D));
-    // (the GEMM gathers x itself where patches tile 128 rows, and always in float32, whose workspace keeps the size it had)
+    // (the GEMM gathers x itself where patches tile 128 rows, and always in float32, where the bytes stay part of the stated
+    // size, Rmax * (2 d + d_e) floats and the plan, though nothing uses them any more)
     r.xg = can_fuse_gather(D) ? 0 : w.take((size_t)D.Rmax * D.d * D.esize);
     r.a = mlp_can_fuse(D) ? 0 : w.take((size_t)D.Rmax * D.d_e * D.esize);          // the fused kernel keeps the hidden tile on chip
     r.z = w.take((size_t)D.Rmax * D.d * D.esize);

@@ -282,10 +282,13 @@ ApplyShape apply_shape(const Dims& D) {
     a.col_blocks = (D.d + kApplyCols - 1) / kApplyCols;
     a.nseg = (D.l_p + kApplyRows - 1) / kApplyRows;
     a.seg_rows = (D.l_p + a.nseg - 1) / a.nseg;
-    a.stages = kApplyRing / (a.seg_rows * kApplyCols * 2);         // 12 KB in flight per warp
+    a.stages = kApplyRing / (a.seg_rows * kApplyCols * 2);         // 12 KB in flight per warp; less with patches of up to 11 rows,
+                                                                   // whose stages are capped
     if (a.stages > kApplyStages) a.stages = kApplyStages;
     const int patches = D.B * D.m;
-    const int cap = 2 * 148 / a.col_blocks > 1 ? 2 * 148 / a.col_blocks : 1;        // two CTAs per SM: one full wave
+    // a full wave at two CTAs per SM of 148 (with more than 16 experts the kernel fits once: two waves).  Not the device's own SM
+    // count: the partial sums, and with them the last bits of dW_r, follow the split, and the workspace query the shape.
+    const int cap = 2 * 148 / a.col_blocks > 1 ? 2 * 148 / a.col_blocks : 1;
     a.per = (patches + cap - 1) / cap;
     a.splits = (patches + a.per - 1) / a.per;
     return a;

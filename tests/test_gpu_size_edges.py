@@ -53,7 +53,7 @@ def test_rotary_positions_of_routed_rows(name, entry):
     assert rel_inf(to_f64(y), ref) <= TOL
 
 
-# one pass over x for dW_r and dx: every column-block width, row segments (patches above 64 rows), one-row patches,
+# one pass over x for dW_r and dx: every column-block width, row segments (patches above 32 rows), one-row patches,
 # more experts than the widest register tile but one, a width that no block divides
 @pytest.mark.parametrize("kw", [dict(B=2, m=3, L=390, L_valid=301, d=200, n=20, k=5, c=2), dict(B=5, m=33, L=33, L_valid=31, d=640, n=9, k=3, c=8),
                                 dict(B=1, m=4, L=64, L_valid=64, d=72, n=3, k=1, c=1), dict(B=40, m=9, L=216, L_valid=216, d=384, n=8, k=2, c=3),
