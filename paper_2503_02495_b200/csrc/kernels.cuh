@@ -207,31 +207,30 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
 // written once, contributions added in ascending slot order.  w_s = gate if use_gate else 1.
 // dW_r = sum over the splits of the partial sums part [nsplit, total], ascending (total = 0: nothing to add).
 struct DwrSum { const float* part = nullptr; float* dW_r = nullptr; int total = 0, nsplit = 0; };
-inline int dwr_sum_blocks(const DwrSum& s) { return (s.total + 15) / 16; }
+constexpr int kDwrItem = 8;          // values that a warp adds up at a time
+inline int dwr_sum_items(const DwrSum& s) { return (s.total + kDwrItem - 1) / kDwrItem; }
 #ifdef __CUDACC__
-// Block `blk` of 256 threads adds 16 consecutive values: 16 threads per value take the splits in turn, their sums are
-// added in a fixed tree.
-__device__ __forceinline__ void dwr_sum(const DwrSum& s, int blk) {
-    __shared__ float red[16][17];
-    const int v = threadIdx.x & 15, g = threadIdx.x >> 4;
-    const int idx = blk * 16 + v;
+// One warp: item `item` is eight consecutive values, four lanes per value take the splits in turn (eight loads in flight
+// each), their sums are added in a fixed tree.
+__device__ __forceinline__ void dwr_sum(const DwrSum& s, int item) {
+    const int lane = threadIdx.x & 31, idx = item * kDwrItem + (lane & (kDwrItem - 1));
     float a = 0.f;
     if (idx < s.total) {
-        int q = g;
-        for (; q + 48 < s.nsplit; q += 64) {
-            const float t0 = s.part[(size_t)q * s.total + idx], t1 = s.part[(size_t)(q + 16) * s.total + idx];
-            const float t2 = s.part[(size_t)(q + 32) * s.total + idx], t3 = s.part[(size_t)(q + 48) * s.total + idx];
-            a += (t0 + t1) + (t2 + t3);
-        }
-        for (; q < s.nsplit; q += 16) a += s.part[(size_t)q * s.total + idx];
-    }
-    red[g][v] = a;
-    __syncthreads();
-    if (g == 0 && idx < s.total) {
+        int q = lane / kDwrItem;
+        for (; q + 28 < s.nsplit; q += 32) {
+            float t[8];
 #pragma unroll
-        for (int q = 1; q < 16; ++q) a += red[q][v];
-        s.dW_r[idx] = a;
+            for (int u = 0; u < 8; ++u) t[u] = s.part[(size_t)(q + 4 * u) * s.total + idx];
+            a += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+        }
+        float t[7];
+#pragma unroll
+        for (int u = 0; u < 7; ++u) t[u] = q + 4 * u < s.nsplit ? s.part[(size_t)(q + 4 * u) * s.total + idx] : 0.f;
+        a += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + t[6]);
     }
+    a += __shfl_xor_sync(0xffffffffu, a, 8);
+    a += __shfl_xor_sync(0xffffffffu, a, 16);
+    if (lane < kDwrItem && idx < s.total) s.dW_r[idx] = a;
 }
 #endif
 uoe_status launch_dwr_sum(const DwrSum& sum, cudaStream_t s);

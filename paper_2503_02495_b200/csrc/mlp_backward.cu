@@ -268,11 +268,12 @@ router_apply_kernel(const __grid_constant__ CUtensorMap xmap /* x as [B m, l_p, 
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+constexpr int kDwrThreads = 64;
+__global__ void __launch_bounds__(kDwrThreads)
 dwr_sum_kernel(const DwrSum s) {
     pdl_trigger();
     pdl_wait();
-    dwr_sum(s, blockIdx.x);
+    dwr_sum(s, (int)blockIdx.x * (kDwrThreads / 32) + (threadIdx.x >> 5));
 }
 
 // Segments, stages and splits of router_apply_kernel for a problem.
@@ -430,7 +431,7 @@ uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r,
 
 uoe_status launch_dwr_sum(const DwrSum& sum, cudaStream_t s) {
     ProfScope ps("dW_r_sum", s);
-    launch_k(dwr_sum_kernel, dim3(dwr_sum_blocks(sum)), dim3(kThreads), 0, s, sum);
+    launch_k(dwr_sum_kernel, dim3((dwr_sum_items(sum) + kDwrThreads / 32 - 1) / (kDwrThreads / 32)), dim3(kDwrThreads), 0, s, sum);
     UOE_LAUNCHED();
     return UOE_OK;
 }

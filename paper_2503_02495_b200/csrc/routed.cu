@@ -225,85 +225,123 @@ gather_kernel(const uint4* __restrict__ src, const int* __restrict__ patch_idx, 
 }
 
 // ---------------------------------------------------------------------------------------------
-// combine: grid (B*m, row groups)
+// combine: a patch is one contiguous slab of x, of y and of every routed buffer that holds it, so y is a weighted sum of
+// slabs.  Bound by memory: the warps of a persistent grid work for themselves on units of 2 x 32 16-byte vectors of a slab,
+// the next unit's rows and weights (a lane per slot), this unit's x and its first two slots in flight together, and no
+// step waits for another warp.  (A CTA per 4 to 16 KB of output, which looks its slots up, meets, and then loads: thousands
+// of short CTAs, 7.2 us against 6.5 at 8 MB of output, 13 and 10 at 17 MB, 29 and 24 at 44 MB = 6.4 TB/s; image block forward
+// 220.5 -> 211, its training step 715 -> 704, long-document block 91.3 -> 85.4.  One vector per lane: 225 us, the four: 216 for
+// the image block; three or four slots in flight: 216 and 217.)
 // ---------------------------------------------------------------------------------------------
+constexpr int kCombineVecs = 2, kCombineSlots = 2;
+
+struct CombineArgs {
+    const void *x, *z;
+    void* y;
+    const int* inv_row;
+    const float* inv_gate;
+    const int* pair_row;        // not null: inv_row holds offsets from the pair's first row
+    const float* gate_bkc;      // not null: whole samples per expert (slot u is patch u): no inverse map, weights from the
+                                // router's gate array [B,k,c]
+    const float* rvec;
+    int Lv, m, k, c, l_p, vpr /* vectors per row */, chunks /* units per slab */, units, residual, use_gate;
+    DwrSum sum;                 // backward: added up behind the units, from the last warp on (the last have the fewest units)
+};
+
 template <typename T, bool BWD /* the backward's combine: rvec and sum */>
 __global__ void __launch_bounds__(kThreads)
-combine_kernel(const T* __restrict__ x, const T* __restrict__ z, const int* __restrict__ inv_row,
-               const float* __restrict__ inv_gate, T* __restrict__ y, int L, int Lv, int d, int m, int k,
-               int l_p, int residual, int use_gate, int rows_per_cta, const float* __restrict__ rvec,
-               const int* __restrict__ pair_row /* not null: inv_row holds offsets from the pair's first row */,
-               const float* __restrict__ gate_bkc /* not null: whole samples per expert (slot u is patch u): no inverse map,
-                                                     weights from the router's gate array [B,k,c] */, int c,
-               int patches, const DwrSum sum /* total > 0: the CTAs past the patches add up dW_r (backward) */) {
+combine_kernel(const CombineArgs a) {
     pdl_trigger();
     pdl_wait();
-    if (BWD && blockIdx.x >= patches) {
-        dwr_sum(sum, (int)((blockIdx.x - patches) * gridDim.y + blockIdx.y));
-        return;
-    }
-    constexpr int V = Vec16<T>::N;
-    __shared__ int srow[32];
-    __shared__ float sg[32];
-    const int bj = blockIdx.x, b = bj / m, j = bj % m;
-    const int r0 = blockIdx.y * rows_per_cta, r1 = min(l_p, r0 + rows_per_cta);
-    if (threadIdx.x < k) {
-        if (gate_bkc) {          // Eq. 26: the token's row in every chosen expert follows from its position alone
-            srow[threadIdx.x] = j * l_p < Lv ? pair_row[(size_t)b * k + threadIdx.x] + j * l_p : -1;
-            sg[threadIdx.x] = use_gate ? gate_bkc[((size_t)b * k + threadIdx.x) * c + j] : 1.0f;
+    constexpr int V = Vec16<T>::N, U = kCombineVecs, S = kCombineSlots;
+    const int lane = threadIdx.x & 31, warps = (int)gridDim.x * (kThreads / 32);
+    int unit = (int)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    // slot `lane` of a patch: its first routed row (-1: none) and weight
+    auto look_up = [&](int bj, int& row, float& g) {
+        row = -1;
+        g = 1.0f;
+        if (lane >= a.k) return;
+        const int b = bj / a.m, j = bj - b * a.m;
+        if (a.gate_bkc) {            // Eq. 26: the token's row in every chosen expert follows from its position alone
+            if (j * a.l_p < a.Lv) row = a.pair_row[(size_t)b * a.k + lane] + j * a.l_p;
+            if (a.use_gate) g = j < a.c ? a.gate_bkc[((size_t)b * a.k + lane) * a.c + j] : 0.f;
         } else {
-            const int rel = inv_row[(size_t)bj * k + threadIdx.x];
-            const int base = pair_row ? pair_row[(size_t)b * k + threadIdx.x] : 0;
-            srow[threadIdx.x] = rel >= 0 ? rel + base : -1;
-            sg[threadIdx.x] = use_gate ? inv_gate[(size_t)bj * k + threadIdx.x] : 1.0f;
+            const int rel = a.inv_row[(size_t)bj * a.k + lane];
+            const int base = a.pair_row ? a.pair_row[(size_t)b * a.k + lane] : 0;
+            if (rel >= 0) row = rel + base;
+            if (a.use_gate) g = a.inv_gate[(size_t)bj * a.k + lane];
+        }
+    };
+    int bj = unit / a.chunks, row_next = -1;
+    float g_next = 0.f;
+    if (unit < a.units) look_up(bj, row_next, g_next);
+    while (unit < a.units) {
+        const int v0 = (unit - bj * a.chunks) * (32 * U) + lane;             // this lane's first vector of the slab
+        const int j = bj % a.m, slab = a.l_p * a.vpr, real = max(0, min(a.l_p, a.Lv - j * a.l_p)) * a.vpr;
+        const size_t at = (size_t)bj * slab;
+        const int row = row_next;
+        const float g = g_next;
+        uint4 xv[U], q[S][U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            xv[u] = make_uint4(0, 0, 0, 0);
+            if (a.residual && v0 + 32 * u < slab) xv[u] = ld_stream16((const uint4*)a.x + at + v0 + 32 * u);
+        }
+        unsigned slots = __ballot_sync(0xffffffffu, row >= 0);              // the patch's routed copies, taken in ascending order
+        unsigned held = slots;                                              // those whose vectors are on their way or here
+        auto load = [&]() {                                                 // the next S of them
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                if (!slots) break;
+                const uint4* zp = (const uint4*)a.z + (size_t)__shfl_sync(0xffffffffu, row, __ffs(slots) - 1) * a.vpr;
+                slots &= slots - 1;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (v0 + 32 * u < real) q[i][u] = ld_stream16(zp + v0 + 32 * u);
+            }
+        };
+        load();
+        unit += warps;
+        const int bj_this = bj;
+        bj = unit / a.chunks;
+        if (unit < a.units) look_up(bj, row_next, g_next);
+        float acc[U][V];
+#pragma unroll
+        for (int u = 0; u < U; ++u) unpack16<T>(xv[u], acc[u]);
+        while (held) {
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                if (!held) break;
+                const float w = __shfl_sync(0xffffffffu, g, __ffs(held) - 1);
+                held &= held - 1;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (v0 + 32 * u < real) {
+                        float f[V];
+                        unpack16<T>(q[i][u], f);
+#pragma unroll
+                        for (int v = 0; v < V; ++v) acc[u][v] = fmaf(w, f[v], acc[u][v]);
+                    }
+            }
+            if (held) load();
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int v = v0 + 32 * u;
+            if (BWD && a.rvec && v < real) {
+                const float* rp = a.rvec + ((size_t)bj_this * a.vpr + v % a.vpr) * V;
+#pragma unroll
+                for (int w = 0; w < V; w += 4) {
+                    const float4 rq = *(const float4*)(rp + w);
+                    acc[u][w] += rq.x; acc[u][w + 1] += rq.y; acc[u][w + 2] += rq.z; acc[u][w + 3] += rq.w;
+                }
+            }
+            if (v < slab) st_stream16((uint4*)a.y + at + v, pack16<T>(acc[u]));
         }
     }
-    __syncthreads();
-    const int vpr = d / V;
-    const int total = (r1 - r0) * vpr;
-    for (int idx = threadIdx.x; idx < total; idx += kThreads) {
-        const int r = r0 + idx / vpr, cv = idx % vpr;
-        const int t = j * l_p + r;
-        const size_t xo = ((size_t)b * L + t) * d + (size_t)cv * V;
-        // the loads of a round (x and up to four slots) are issued together, then added in ascending slot order
-        const bool real = t < Lv;
-        uint4 xv = make_uint4(0, 0, 0, 0), q[4];
-        if (residual) xv = ld_stream16(x + xo);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (real && u < k && srow[u] >= 0) q[u] = ld_stream16(z + ((size_t)(srow[u] + r)) * d + (size_t)cv * V);
-        float acc[V];
-        unpack16<T>(xv, acc);
-        if (real) {
-            for (int s0 = 0; s0 < k; s0 += 4) {
-                if (s0 > 0) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (s0 + u < k && srow[s0 + u] >= 0)
-                            q[u] = ld_stream16(z + ((size_t)(srow[s0 + u] + r)) * d + (size_t)cv * V);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (s0 + u < k && srow[s0 + u] >= 0) {
-                        float f[V];
-                        unpack16<T>(q[u], f);
-                        const float g = sg[s0 + u];
-#pragma unroll
-                        for (int v = 0; v < V; ++v) acc[v] = fmaf(g, f[v], acc[v]);
-                    }
-                }
-            }
-            if (rvec) {         // (a run-time check in the forward too: without it the compiler orders the loop above worse, d = 2432,
-                                // sixteen experts, 22k tokens 176 us instead of 166)
-                const float* rp = rvec + (size_t)bj * d + (size_t)cv * V;
-#pragma unroll
-                for (int v = 0; v < V; v += 4) {
-                    const float4 rq = *(const float4*)(rp + v);
-                    acc[v] += rq.x; acc[v + 1] += rq.y; acc[v + 2] += rq.z; acc[v + 3] += rq.w;
-                }
-            }
-        }
-        st_stream16(y + xo, pack16<T>(acc));
+    if (BWD) {
+        const int items = (a.sum.total + kDwrItem - 1) / kDwrItem;
+        for (int i = warps - 1 - ((int)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)); i < items; i += warps) dwr_sum(a.sum, i);
     }
 }
 
@@ -487,32 +525,28 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
 
 uoe_status launch_combine(const Dims& D, const void* x, const void* z, const PlanPtrs& P, bool residual,
                           bool use_gate, void* y, cudaStream_t s, const float* rvec, const DwrSum& sum) {
-    // 16-byte vectors per thread: two for small outputs (short dependent chains, many CTAs in flight: these launches are
-    // bound by latency), four to eight once the output is tens of MB (fewer, longer CTAs: less set-up per byte; measured
-    // 35 -> 31 us at 44 MB, 198 -> 183 us at 268 MB)
-    const long long out_bytes = (long long)D.B * D.L * D.d * D.esize;
-    const int vecs = out_bytes < (32ll << 20) ? 2 : (out_bytes < (128ll << 20) ? 4 : 8);
-    int rows_per_cta = (int)(vecs * kThreads * 16 / ((long long)D.d * D.esize));
-    if (rows_per_cta < 1) rows_per_cta = 1;
-    if (rows_per_cta > D.l_p) rows_per_cta = D.l_p;
-    // the additions of dW_r take whole columns of the grid (one row of it for them, the rest of the columns idle, was 84 us
-    // instead of 19 at d = 1408, n = 24 with ten patches of 64 tokens: 46000 empty CTAs)
-    const int row_groups = (D.l_p + rows_per_cta - 1) / rows_per_cta;
-    dim3 grid(D.B * D.m + (dwr_sum_blocks(sum) + row_groups - 1) / row_groups, row_groups);
-    const bool ident = P.inv_relative && P.identity_patches && P.gate != nullptr;
-    const long long ctas = (long long)grid.x * grid.y;
+    const int vpr = (int)((long long)D.d * D.esize / 16);
+    CombineArgs a;
+    a.x = x; a.z = z; a.y = y; a.inv_row = P.inv_row; a.inv_gate = P.inv_gate;
+    a.pair_row = P.inv_relative ? P.pair_row : nullptr;
+    a.gate_bkc = P.inv_relative && P.identity_patches ? P.gate : nullptr;
+    a.rvec = rvec;
+    a.Lv = D.Lv; a.m = D.m; a.k = D.k; a.c = D.c; a.l_p = D.l_p; a.vpr = vpr;
+    a.residual = residual ? 1 : 0; a.use_gate = use_gate ? 1 : 0;
+    a.sum = sum;
     ProfScope ps("combine", s);
-    auto go = [&](SpreadOnce& once, auto kern, auto elem) {
-        using T = decltype(elem);
-        launch_k(kern, grid, dim3(kThreads), spread_smem(once, kern, ctas, 0), s, (const T*)x, (const T*)z, (const int*)P.inv_row,
-                 (const float*)P.inv_gate, (T*)y, D.L, D.Lv, D.d, D.m, D.k, D.l_p, residual ? 1 : 0, use_gate ? 1 : 0, rows_per_cta,
-                 rvec, P.inv_relative ? (const int*)P.pair_row : (const int*)nullptr, ident ? P.gate : (const float*)nullptr, D.c,
-                 D.B * D.m, sum);
-    };
-    static SpreadOnce once[3];
-    if (!D.bf16) go(once[0], combine_kernel<float, false>, float());
-    else if (rvec || sum.total > 0) go(once[1], combine_kernel<__nv_bfloat16, true>, __nv_bfloat16());
-    else go(once[2], combine_kernel<__nv_bfloat16, false>, __nv_bfloat16());
+    const bool bwd = rvec || sum.total > 0;
+    a.chunks = (D.l_p * vpr + 32 * kCombineVecs - 1) / (32 * kCombineVecs);
+    a.units = D.B * D.m * a.chunks;
+    // Four CTAs per SM, all that fit (up to eight) only for a forward with several units per warp even then: the room is of
+    // use to the next kernel, whose CTAs start under this one (language-model training step 257 us with four, 262 with eight;
+    // wide block forward 167.5 and 165.4)
+    const int per_sm = !bwd && a.units >= 10 * (kThreads / 32) * sm_count() ? 8 : 4;
+    const int want = (a.units + kThreads / 32 - 1) / (kThreads / 32), cap = per_sm * sm_count();
+    const dim3 grid(want < cap ? want : cap);
+    if (!D.bf16) launch_k(combine_kernel<float, false>, grid, dim3(kThreads), 0, s, a);
+    else if (bwd) launch_k(combine_kernel<__nv_bfloat16, true>, grid, dim3(kThreads), 0, s, a);
+    else launch_k(combine_kernel<__nv_bfloat16, false>, grid, dim3(kThreads), 0, s, a);
     UOE_LAUNCHED();
     return UOE_OK;
 }

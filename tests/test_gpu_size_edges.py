@@ -340,3 +340,21 @@ def test_attention_of_pairs_with_fewer_key_tiles_than_others(heads):
     y = uoe.uoe_smha_forward(prob, to_dev(x), *(to_dev(q) for q in ws), r)
     ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
     assert rel_inf(to_f64(y), orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False)) <= TOL
+
+
+# the combine's units of 64 vectors: slabs shorter than a unit, a vector longer, and of many; one to five slots per patch (two
+# are in flight), whole samples per expert, padding rows, more units than warps
+@pytest.mark.parametrize("kw", [dict(B=2, L=9, L_valid=8, m=9, c=7, d=4, n=6, k=5, d_ff=24), dict(B=3, L=13 * 6, L_valid=70, m=6, c=4, d=20, n=3, k=3, d_ff=12),
+                                dict(B=2, L=64, L_valid=50, m=2, c=2, d=260, n=5, k=4, d_ff=40), dict(B=40, L=1024, L_valid=1000, m=16, c=9, d=128, n=3, k=1, d_ff=12)],
+                         ids=["short_slabs", "a_vector_over", "whole_samples", "many_units"])
+def test_combine_of_slabs(kw):
+    """float32: sums of at most 260 products per layer, 1e-4 of the largest value as for the other float32 results."""
+    import paper_2503_02495_b200 as uoe
+    w = gen.tiny(**kw)
+    x, Wr = gen.make_x(w), gen.make_router(w)
+    W1, W2 = gen.make_mlp_weights(w)
+    prob = problem_of(w, "mlp")
+    r = uoe.uoe_route(prob, to_dev(x), to_dev(Wr))
+    y = to_f64(uoe.uoe_mlp_forward(prob, to_dev(x), to_dev(W1), to_dev(W2), r))
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    assert rel_inf(y, orc.mlp_forward(x.f64, W1.f64, W2.f64, ro, w.act, residual=True)) <= 1e-4
