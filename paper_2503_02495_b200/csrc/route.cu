@@ -20,7 +20,7 @@ constexpr int kScoreThreads = 256;
 
 // Selection for sample b by one CTA of NT threads (all threads call).  pp: n*m floats of shared memory.
 // Written for a short dependent chain (the router is latency-bound on all but the largest inputs): a CTA barrier between
-// the first phase and the others, then the ticket.
+// the first phase and the others, the ticket under the last of them.
 //   A  a warp works 32/np2 patches at a time (np2 = n rounded up to a power of two), one lane per (patch, expert):
 //      adds the parts of the score in ascending order, softmax over the experts of the patch through segment
 //      shuffles (Eq. 14), first-stage counts of Eq. 15 when the capacity is dynamic; the raw scores are summed per
@@ -41,12 +41,13 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
     constexpr int NW = NT / 32;
     constexpr int kMaskCache = 1024;       // samples whose masks the last CTA keeps in shared memory
     __shared__ float s_raw[NW][32];        // per warp: sum over its patches of the raw scores, per expert
-    __shared__ int cnts[32];               // Eq. 16: patches each expert receives in the first routing stage; later: samples per expert
+    __shared__ int cnts[32];               // Eq. 16: patches each expert receives in the first routing stage
+    __shared__ int loads[32];              // samples per expert
     __shared__ int s_last;
     __shared__ unsigned s_masks[kMaskCache];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int use_gate = sel_flags & 1, dynamic_c = (sel_flags >> 1) & 1;
-    if (tid < 32) cnts[tid] = 0;
+    if (tid < 32) cnts[tid] = loads[tid] = 0;
     const int n_elig = (Lv + l_p - 1) / l_p;       // patches holding at least one real token (a prefix)
     // the single-mode cases: every sample uses all experts (Eq. 12-20) / a chosen expert takes the whole sample (Eq. 21-26)
     const bool all_experts = !(sel_flags & 4) && k == n;
@@ -138,7 +139,12 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
         if (warp == 0) {
             if (lane < n) p_samp[(size_t)b * n + lane] = ps;
             if (pick) expert_idx[(size_t)b * k + __popc(chosen & ((1u << lane) - 1u))] = lane;
-            if (lane == 0) masks[b] = chosen;
+        }
+        // The sample's ticket already here, by the last warp, under phase C of the others: whoever takes the last one reads the
+        // masks and nothing else of the other samples.  (Behind phase C it has to wait for that phase's stores as well.)
+        if (warp == NW - 1 && lane == 0 && !all_experts) {
+            masks[b] = chosen;
+            s_last = take_ticket(ticket) == B - 1;
         }
     }
 
@@ -213,28 +219,20 @@ __device__ void select_sample(float* pp, const float* __restrict__ partial, int 
         return;
     }
     __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = (atomicAdd(ticket, 1) == B - 1);
-        __threadfence();
-    }
-    __syncthreads();
     if (!s_last) return;
     if (tid == 0) *ticket = 0;              // left at zero for the next call
-    if (tid < 32) cnts[tid] = 0;
-    __syncthreads();
     for (int b2 = tid; b2 < B; b2 += NT) {           // samples per expert
         unsigned mk = __ldcg(masks + b2);
         if (b2 < kMaskCache) s_masks[b2] = mk;
         while (mk) {
             const int i = __ffs(mk) - 1;
             mk &= mk - 1;
-            atomicAdd(&cnts[i], 1);
+            atomicAdd(&loads[i], 1);
         }
     }
     __syncthreads();
     const int l_a = c * l_p;
-    const int rows = lane < n ? (cnts[lane] * l_a + UOE_ROW_ALIGN - 1) / UOE_ROW_ALIGN * UOE_ROW_ALIGN : 0;
+    const int rows = lane < n ? (loads[lane] * l_a + UOE_ROW_ALIGN - 1) / UOE_ROW_ALIGN * UOE_ROW_ALIGN : 0;
     int incl = rows;                        // every warp scans for itself
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -384,9 +382,7 @@ route_kernel(const T* __restrict__ x, const T* __restrict__ W_r, float* __restri
     if constexpr (TICKET) {
         __syncthreads();
         if (tid == 0) {
-            __threadfence();
-            s_mine = (atomicAdd(&sample_ticket[b], 1) == m * nparts - 1);
-            __threadfence();
+            s_mine = take_ticket(&sample_ticket[b]) == m * nparts - 1;
             if (s_mine) sample_ticket[b] = 0;         // left at zero for the next call
         }
         __syncthreads();
