@@ -26,6 +26,7 @@
 // Masks: the real keys of a pair are a prefix of its gathered order (patches ascending, pad tokens at
 // the end of the sample), so key c is kept iff c < n_valid, and with the causal flag iff also
 // c <= query row (the shared lower triangle of Fig. 4).  Only tiles that cross one of the two limits test them.
+#include "attn_out.cuh"
 #include "kernels.cuh"
 #include "tc.cuh"
 #include "tmap.cuh"
@@ -81,7 +82,7 @@ struct AttnArgs {
 template <bool FUSE_O>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmWo, const AttnArgs a) {
+                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmWo, const __grid_constant__ CUtensorMap tmZ, const AttnArgs a) {
     pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -369,6 +370,10 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
                 const float alpha = ex2_approx(m_run - m_use);
                 if (pending) { ok = take_o(); if (!ok) break; }
+                if (FUSE_O && t == 0) {              // the last unit's last piece of z has been read: P takes its place
+                    if (lane == 0) bulk_wait_read();
+                    __syncwarp();
+                }
                 // ---- second pass: p = 2^(s c - m), bf16, into shared memory (swizzled K-major, two [128 x 64] halves) ----
                 float l_add = 0.f;
                 // (the mask test is a template argument: tested per element at run time it becomes a branch per element)
@@ -440,8 +445,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
                 fence_async_smem();
                 mbar_arrive(&pc->o_ready);
-                // each warp stages a [32 rows x 64 columns] piece in the free half of P's place and writes it out with
-                // eight lanes per row, so that every store instruction covers whole 128-byte row segments
+                // each warp stages its pieces in its rows of the free half of P's place
                 uint8_t* stg = sP + TILE_BYTES + quarter * 4096;
                 const int wrow0 = q0 + quarter * 32;                  // first query row of this warp's piece
                 for (int zc = 0; zc < n_zchunk && ok; ++zc) {
@@ -459,28 +463,13 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             tc_fence_before();
                             mbar_arrive(&pc->acc_empty);
                         }
-                        __syncwarp();                                     // the previous piece has been read back
-#pragma unroll
-                        for (int ch = 0; ch < 8; ++ch) {
-                            uint4 w;
-                            w.x = pack_bf16x2(zf[ch * 8 + 0], zf[ch * 8 + 1]); w.y = pack_bf16x2(zf[ch * 8 + 2], zf[ch * 8 + 3]);
-                            w.z = pack_bf16x2(zf[ch * 8 + 4], zf[ch * 8 + 5]); w.w = pack_bf16x2(zf[ch * 8 + 6], zf[ch * 8 + 7]);
-                            *(uint4*)(stg + lane * 128 + ((ch ^ (lane & 7)) << 4)) = w;
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = i * 4 + (lane >> 3), ch = lane & 7;
-                            if (wrow0 + r < a.l_a) {
-                                const uint4 w = *(const uint4*)(stg + r * 128 + ((ch ^ (r & 7)) << 4));
-                                *(uint4*)(a.Z + (size_t)(row_base + wrow0 + r) * a.d + n0 + g64 * 64 + ch * 8) = w;
-                            }
-                        }
+                        store_z_piece(zf, stg, &tmZ, a.Z, a.d, n0 + g64 * 64, row_base + wrow0, a.l_a - wrow0, lane);
                     }
                 }
             }
         }
     }
+    if (FUSE_O && role == 0 && lane == 0) bulk_wait_all();       // this warp's tensor stores are complete
     tc_fence_before();
     __syncthreads();
     if (warp == 8) {
@@ -512,8 +501,8 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             const __grid_constant__ CUtensorMap tmV, __nv_bfloat16* __restrict__ O, float* __restrict__ lse,
             const int* __restrict__ pair_row, const int* __restrict__ patch_idx, int c, int l_p, int Lv, int l_a,
             int d_g, int heads, int causal, float scale_log2, int* status,
-            const __grid_constant__ CUtensorMap tmWo, const int* __restrict__ expert_idx, __nv_bfloat16* __restrict__ Z,
-            int d) {
+            const __grid_constant__ CUtensorMap tmWo, const __grid_constant__ CUtensorMap tmZ, const int* __restrict__ expert_idx,
+            __nv_bfloat16* __restrict__ Z, int d) {
     pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -756,9 +745,7 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         ok = mbar_wait(&ctl->bar_z, 0, abort_flag, status);
         if (__all_sync(0xffffffffu, ok && !*abort_flag)) {
             tc_fence_after();
-            // each warp stages a [32 rows x 64 columns] piece in shared memory (in place of P) and writes it out with
-            // eight lanes per row, so that every store instruction covers whole 128-byte row segments; the two warps
-            // of a lane quarter take alternate 64-column groups
+            // each warp stages its pieces in place of P; the two warps of a lane quarter take alternate 64-column groups
             uint8_t* stg = sP + warp * 4096;
             const int wrow0 = q0 + quarter * 32;                  // first query row of this warp's piece
 #pragma unroll 1
@@ -767,23 +754,7 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 tmem_ld32(t_lane + g * 64, (uint32_t*)zf);
                 tmem_ld32(t_lane + g * 64 + 32, (uint32_t*)(zf + 32));
                 tmem_ld_wait();
-                __syncwarp();                                     // the previous piece has been read back
-#pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    uint4 w;
-                    w.x = pack_bf16x2(zf[ch * 8 + 0], zf[ch * 8 + 1]); w.y = pack_bf16x2(zf[ch * 8 + 2], zf[ch * 8 + 3]);
-                    w.z = pack_bf16x2(zf[ch * 8 + 4], zf[ch * 8 + 5]); w.w = pack_bf16x2(zf[ch * 8 + 6], zf[ch * 8 + 7]);
-                    *(uint4*)(stg + lane * 128 + ((ch ^ (lane & 7)) << 4)) = w;
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = i * 4 + (lane >> 3), ch = lane & 7;
-                    if (wrow0 + r < l_a) {
-                        const uint4 w = *(const uint4*)(stg + r * 128 + ((ch ^ (r & 7)) << 4));
-                        *(uint4*)(Z + (size_t)(row_base + wrow0 + r) * d + g * 64 + ch * 8) = w;
-                    }
-                }
+                store_z_piece(zf, stg, &tmZ, Z, d, g * 64, row_base + wrow0, l_a - wrow0, lane);
             }
         }
     }
@@ -792,6 +763,7 @@ attn_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         for (int t = 0; t < 2 && t < n_kv; ++t) mbar_try_wait(&ctl->bar_kv[t], 0);
         if (FUSE_O) mbar_wait(&ctl->bar_w, 0, abort_flag, status);
     }
+    if (FUSE_O && lane == 0) bulk_wait_all();       // this warp's tensor stores are complete
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -834,7 +806,7 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
         if (st == UOE_OK) st = smem_opt_in(once_tile_fused, attn_tile_kernel<true>, TILE_SMEM_FUSED);
         if (st != UOE_OK) return st;
     }
-    CUtensorMap tm[3], tmWo;
+    CUtensorMap tm[3], tmWo, tmZ;
     const void* ptrs[3] = {q, k, v};
     for (int i = 0; i < 3; ++i) {
         const uint64_t dims[2] = {(uint64_t)D.d_g, (uint64_t)D.Rmax};
@@ -842,12 +814,16 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
         const uint32_t box[2] = {DH, 128};
         if (!make_tmap(&tm[i], ptrs[i], 2, dims, str, box)) return UOE_ERR_CUDA;
     }
-    tmWo = tm[0];
+    tmWo = tmZ = tm[0];
     if (fuse) {       // W^o [n, d_g, d]: boxes of 64 output columns x 64 contraction rows of one expert
         const uint64_t dims[3] = {(uint64_t)D.d, (uint64_t)D.d_g, (uint64_t)D.n};
         const uint64_t str[2] = {(uint64_t)D.d * 2, (uint64_t)D.d * D.d_g * 2};
         const uint32_t box[3] = {64, DH, 1};
         if (!make_tmap(&tmWo, Wo, 3, dims, str, box)) return UOE_ERR_CUDA;
+        const uint64_t zdims[2] = {(uint64_t)D.d, (uint64_t)D.Rmax};       // z in pieces of 32 rows x 64 columns
+        const uint64_t zstr[1] = {(uint64_t)D.d * 2};
+        const uint32_t zbox[2] = {64, 32};
+        if (!make_tmap(&tmZ, z, 2, zdims, zstr, zbox)) return UOE_ERR_CUDA;
     }
     const int heads = D.d_g / DH, n_qt = (D.l_a + TQ - 1) / TQ;
     const long long pairs = (long long)D.B * D.k, units = pairs * heads * n_qt;
@@ -873,18 +849,18 @@ uoe_status launch_attention(const Dims& D, const void* q, const void* k, const v
         a.status = status;
         const long long want = (units + 1) / 2;
         const int grid = (int)(want < sm_count() ? want : sm_count());
-        if (fuse) e = launch_k(attn_stream_kernel<true>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
-        else e = launch_k(attn_stream_kernel<false>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, a);
+        if (fuse) e = launch_k(attn_stream_kernel<true>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, tmZ, a);
+        else e = launch_k(attn_stream_kernel<false>, dim3(grid), dim3(kAttnThreads), ATTN_SMEM, s, tm[0], tm[1], tm[2], tmWo, tmZ, a);
     } else {
         if (pairs > 65535) return UOE_ERR_UNSUPPORTED;      // (cannot happen: fewer than two units per SM)
         dim3 grid(n_qt, heads, (unsigned)pairs);
         if (fuse)
             e = launch_k(attn_tile_kernel<true>, grid, dim3(kTileThreads), TILE_SMEM_FUSED, s, tm[0], tm[1], tm[2], (__nv_bfloat16*)o, lse,
-                         pair_row, patch_idx, D.c, D.l_p, D.Lv, D.l_a, D.d_g, heads, causal ? 1 : 0, scale_log2, status, tmWo, expert_idx,
+                         pair_row, patch_idx, D.c, D.l_p, D.Lv, D.l_a, D.d_g, heads, causal ? 1 : 0, scale_log2, status, tmWo, tmZ, expert_idx,
                          (__nv_bfloat16*)z, D.d);
         else
             e = launch_k(attn_tile_kernel<false>, grid, dim3(kTileThreads), TILE_SMEM, s, tm[0], tm[1], tm[2], (__nv_bfloat16*)o, lse,
-                         pair_row, patch_idx, D.c, D.l_p, D.Lv, D.l_a, D.d_g, heads, causal ? 1 : 0, scale_log2, status, tmWo,
+                         pair_row, patch_idx, D.c, D.l_p, D.Lv, D.l_a, D.d_g, heads, causal ? 1 : 0, scale_log2, status, tmWo, tmZ,
                          (const int*)nullptr, (__nv_bfloat16*)nullptr, D.d);
     }
     if (e != cudaSuccess) return UOE_ERR_CUDA;

@@ -362,6 +362,20 @@ uoe_status launch_mlp_fused(const Dims& D, const void* A, const void* W1, const 
                             const int* offsets, int act, const void* gather_x, const SrcMap& map, int* status,
                             cudaStream_t s, const void* b1 = nullptr, const void* b2 = nullptr);
 
+// Projections, attention and output projection in one kernel (smha_fused_tcgen05.cu) for experts of one head: whether a problem
+// takes it, and the launch.  Forward: q null, z is written (k and v are scratch of pairs with several tiles).  The backward's
+// recomputation: q, k, v, o and lse are written, z is not.
+struct SmhaFused {
+    const void* x = nullptr;
+    const void* W[3] = {nullptr, nullptr, nullptr};
+    const void* Wo = nullptr;
+    void *q = nullptr, *k = nullptr, *v = nullptr, *o = nullptr, *z = nullptr;
+    float* lse = nullptr;
+};
+bool smha_can_fuse(const Dims& D, bool recompute);
+uoe_status launch_smha_fused(const Dims& D, const SmhaFused& f, const PlanPtrs& P, const int* patch_idx, const int* expert_idx,
+                             const int* offsets, bool causal, const Rope& rope, int* status, cudaStream_t s);
+
 // ---- forward halves behind the routing plan (shared by the per-half entry points and the block entry) ----
 struct MlpFwdBufs { void* xg; void* a; void* z; };
 // Second layer + combine walked by output patch (patches of 128 tokens): whether the problem and plan allow it, the

@@ -56,15 +56,22 @@ uoe_status uoe::smha_forward_run(const Dims& D, const uoe_problem* prob, const v
         st = launch_gather(D, x, patch_idx, expert_offsets, P, xg, stream);
         if (st != UOE_OK) return st;
     }
+    const bool causal = (prob->flags & UOE_FLAG_CAUSAL) != 0;
+    const Rope rope = rope_of(D, P, patch_idx);      // Eq. 32 (nothing if d_rope = 0)
+    if (smha_can_fuse(D, false)) {
+        SmhaFused f;
+        f.x = x; f.W[0] = Wq; f.W[1] = Wk; f.W[2] = Wv; f.Wo = Wo; f.k = k; f.v = v; f.z = z; f.lse = lse;
+        st = launch_smha_fused(D, f, P, patch_idx, expert_idx, expert_offsets, causal, rope, status, stream);
+        if (st != UOE_OK) return st;
+        return launch_combine(D, x, z, P, (prob->flags & UOE_FLAG_RESIDUAL) != 0, (prob->flags & UOE_FLAG_GATE) != 0, y, stream);
+    }
     GemmArgs gq{xg, Wq, nullptr, q, nullptr, expert_offsets, D.n, D.d, D.d_g, UOE_ACT_IDENTITY, false, D.Rmax};
     if (fused) { gq.gather_x = x; gq.map = src_map_of(D, P, patch_idx); gq.l_p = D.l_p; gq.Bm = D.B * D.m; }
     gq.label = "qkv_proj";
     gq.nmat = 3; gq.W1 = Wk; gq.W2 = Wv; gq.C1 = k; gq.C2 = v;
-    const Rope rope = rope_of(D, P, patch_idx);      // Eq. 32 (nothing if d_rope = 0)
     gq.rope = &rope;
     st = launch_gemm_bf16(gq, status, stream);
     if (st != UOE_OK) return st;
-    const bool causal = (prob->flags & UOE_FLAG_CAUSAL) != 0;
     if (attention_can_fuse_out(D)) {          // Eq. 33-35 in one kernel: attention and the expert's output projection
         st = launch_attention(D, q, k, v, o, lse, P.pair_row, patch_idx, causal, status, stream, Wo, expert_idx, z);
         if (st != UOE_OK) return st;

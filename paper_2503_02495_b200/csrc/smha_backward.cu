@@ -108,16 +108,23 @@ extern "C" uoe_status uoe_smha_backward(const uoe_problem* prob, const void* x, 
     }
 
     // ---- forward recomputation (Eq. 28-34) ----
-    GemmArgs gq{xg, Wq, nullptr, q, nullptr, expert_offsets, D.n, D.d, D.d_g, UOE_ACT_IDENTITY, false, D.Rmax};
-    if (fused) { gq.gather_x = x; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m; }
-    gq.label = "qkv_proj";
-    gq.nmat = 3; gq.W1 = Wk; gq.W2 = Wv; gq.C1 = k; gq.C2 = v;
     const Rope rope = rope_of(D, P, patch_idx);      // Eq. 32 (nothing if d_rope = 0)
-    gq.rope = &rope;
-    st = launch_gemm_bf16(gq, status, stream);
-    if (st != UOE_OK) return st;
-    st = launch_attention(D, q, k, v, o, lse, P.pair_row, patch_idx, causal, status, stream);
-    if (st != UOE_OK) return st;
+    if (smha_can_fuse(D, true)) {
+        SmhaFused f;
+        f.x = x; f.W[0] = Wq; f.W[1] = Wk; f.W[2] = Wv; f.q = q; f.k = k; f.v = v; f.o = o; f.lse = lse;
+        st = launch_smha_fused(D, f, P, patch_idx, expert_idx, expert_offsets, causal, rope, status, stream);
+        if (st != UOE_OK) return st;
+    } else {
+        GemmArgs gq{xg, Wq, nullptr, q, nullptr, expert_offsets, D.n, D.d, D.d_g, UOE_ACT_IDENTITY, false, D.Rmax};
+        if (fused) { gq.gather_x = x; gq.src_patch = P.src_patch; gq.l_p = D.l_p; gq.Bm = D.B * D.m; }
+        gq.label = "qkv_proj";
+        gq.nmat = 3; gq.W1 = Wk; gq.W2 = Wv; gq.C1 = k; gq.C2 = v;
+        gq.rope = &rope;
+        st = launch_gemm_bf16(gq, status, stream);
+        if (st != UOE_OK) return st;
+        st = launch_attention(D, q, k, v, o, lse, P.pair_row, patch_idx, causal, status, stream);
+        if (st != UOE_OK) return st;
+    }
 
     // ---- out-projection backward ----
     GemmArgs gd{dyg, Wo, nullptr, dout, nullptr, expert_offsets, D.n, D.d, D.d_g, UOE_ACT_IDENTITY, true, D.Rmax};

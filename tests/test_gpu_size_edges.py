@@ -358,3 +358,41 @@ def test_combine_of_slabs(kw):
     y = to_f64(uoe.uoe_mlp_forward(prob, to_dev(x), to_dev(W1), to_dev(W2), r))
     ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
     assert rel_inf(y, orc.mlp_forward(x.f64, W1.f64, W2.f64, ro, w.act, residual=True)) <= 1e-4
+
+
+# projections and attention in one kernel: one tile (short, padded, eight-row patches, full) and clusters of two to eight tiles
+# (real keys that end before the pair's last tile, causal, rotary)
+FUSED_CASES = {
+    "short": (_att(B=3, L=96, L_valid=96, m=6, c=3, d=128, n=4, k=2, H=4), 0),
+    "causal_pad_rope": (_att(B=5, L=128, L_valid=121, m=8, c=7, d=128, n=3, k=2, H=3, causal=True), 32),
+    "patch8": (_att(B=4, L=96, L_valid=90, m=12, c=9, d=384, n=4, k=2, H=4), 0),
+    "one_full_tile": (_att(B=4, L=256, L_valid=256, m=8, c=4, d=512, n=4, k=2, H=4), 0),
+    "two_tiles_causal": (_att(B=4, L=512, L_valid=500, m=16, c=8, d=512, n=4, k=2, H=4, causal=True), 0),
+    "three_tiles_no_real_key_in_the_last": (_att(B=2, L=768, L_valid=400, m=6, c=3, d=128, n=4, k=2, H=4), 0),
+    "eight_tiles": (_att(B=2, L=2048, L_valid=2048, m=32, c=16, d=256, n=4, k=2, H=4), 0),
+    "whole_samples_causal_rope": (_att(B=1, L=1024, L_valid=1000, m=16, c=16, d=128, n=4, k=2, H=4, causal=True), 64),
+}
+
+
+@pytest.mark.parametrize("name", list(FUSED_CASES))
+def test_projection_and_attention_in_one_kernel(name):
+    import paper_2503_02495_b200 as uoe
+    w, d_rope = FUSED_CASES[name]
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w, "att").f64 * 20, w.dtype)
+    ws = gen.make_attn_weights(w)
+    prob = problem_of(w, "att", residual=False, d_rope=d_rope)
+    xd, Wrd, wd = to_dev(x), to_dev(Wr), [to_dev(q) for q in ws]
+    r = uoe.uoe_route(prob, xd, Wrd)
+    dy = gen.make_dy(w)
+    uoe.uoe_profile_enable(True)
+    y = uoe.uoe_smha_forward(prob, xd, *wd, r)
+    got = uoe.uoe_smha_backward(prob, xd, *wd, Wrd, r, to_dev(dy))
+    torch.cuda.synchronize()
+    uoe.uoe_profile_enable(False)
+    assert [n for n, _ in uoe.uoe_profile_records()].count("smha_fused") == 2
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    ref_y = orc.smha_forward(x.f64, *[q.f64 for q in ws], ro, w.d_h, w.causal, residual=False, d_rope=d_rope)
+    assert rel_inf(to_f64(y), ref_y) <= TOL
+    ref = orc.smha_backward(x.f64, *[q.f64 for q in ws], Wr.f64, ro, dy.f64, w.d_h, w.causal, residual=False, d_rope=d_rope)
+    for g, f in zip(got, ref[:6]):
+        assert rel_inf(to_f64(g), f) <= TOL
