@@ -36,14 +36,13 @@ constexpr int ZC = 128;                                  // output columns of a 
 template <bool MULTI> struct FCfg {
     static constexpr int STAGES = MULTI ? 5 : 2;
     // after the projection the ring's place holds, in units of a tile:  q, then
-    //   single: k, v, P (two halves; o in the first), a chunk of W^o from the start; later two more chunks where q and k were
-    //           and z staging in v's and the second half of P's place
+    //   single: k, v, P (two halves; o in the first), a chunk of W^o from the start; later two more where q and k were
     //   multi:  P (the same), two key stages (k | v), own k, v, two W^o chunks, z staging (two); later two more chunks where own k
     //           and v were
     static constexpr int K = MULTI ? 7 : 1, V = MULTI ? 8 : 2, P = MULTI ? 1 : 3, KV = 3;
     static constexpr int NW = MULTI ? 4 : 3;             // W^o chunks held
     __host__ __device__ static constexpr int W(int b) { return MULTI ? (b < 2 ? 9 + b : 5 + b) : (b == 0 ? 5 : b - 1); }
-    static constexpr int ZS0 = MULTI ? 11 : 2, ZS1 = MULTI ? 12 : 4, UNITS = MULTI ? 13 : 6;
+    static constexpr int UNITS = MULTI ? 13 : 6;
     static constexpr int TMEM = MULTI ? 512 : 256;       // q k v [0, 192); S [0, 128) (multi: and [128, 256)); O; z chunks [0, 256)
     static constexpr int COL_O = MULTI ? 256 : 128;
     static constexpr int SMEM = UNITS * UNIT + 1024 /*alignment*/ + 512 /*control*/;
@@ -441,7 +440,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             }
         }
         // ---- z = o W^o_i (Eq. 35), a chunk's 64-column groups dealt to the two warps of a lane quarter ----
-        uint8_t* stg = unit(warp < 4 ? Cf::ZS0 : Cf::ZS1) + quarter * 4096;
+        [[maybe_unused]] uint8_t* stg = MULTI ? unit(11 + hsel) + quarter * 4096 : nullptr;
         for (int j = 0; j < n_z && ok; ++j) {
             const int st = j & 1, col = j * ZC + hsel * 64;
             ok = __all_sync(0xffffffffu, wait(&ctl->z_full[st], (j >> 1) & 1)) != 0;
@@ -455,9 +454,12 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             }
             tc_fence_before();
             mbar_arrive(&ctl->z_free[st]);
-            if (col < a.d) store_z_piece(zf, stg, &tm.z, a.z, a.d, col, row_base + q0 + quarter * 32, left, lane);
+            if (col < a.d) {
+                if constexpr (MULTI) store_z_piece(zf, stg, &tm.z, a.z, a.d, col, row_base + q0 + quarter * 32, left, lane);
+                else store_z_direct(zf, a.z, a.d, col, row_base + q0 + quarter * 32, left, lane);
+            }
         }
-        if (lane == 0) bulk_wait_all();                  // this warp's tensor stores are complete
+        if (MULTI && lane == 0) bulk_wait_all();         // this warp's tensor stores are complete
     }
     if constexpr (MULTI) {
         if (warp != 8) cluster_wait();                   // (long complete: every thread that arrives waits)
@@ -543,10 +545,12 @@ uoe_status launch_smha_fused(const Dims& D, const SmhaFused& f, const PlanPtrs& 
         const uint64_t str[2] = {(uint64_t)D.d * 2, (uint64_t)D.d * DH * 2};
         const uint32_t box[3] = {64, DH, 1};
         if (!make_tmap(&tm.wo, f.Wo, 3, dims, str, box)) return UOE_ERR_CUDA;
-        const uint64_t zdims[2] = {(uint64_t)D.d, (uint64_t)D.Rmax};
-        const uint64_t zstr[1] = {(uint64_t)D.d * 2};
-        const uint32_t zbox[2] = {64, 32};
-        if (!make_tmap(&tm.z, f.z, 2, zdims, zstr, zbox)) return UOE_ERR_CUDA;
+        if (n_qt > 1) {
+            const uint64_t zdims[2] = {(uint64_t)D.d, (uint64_t)D.Rmax};
+            const uint64_t zstr[1] = {(uint64_t)D.d * 2};
+            const uint32_t zbox[2] = {64, 32};
+            if (!make_tmap(&tm.z, f.z, 2, zdims, zstr, zbox)) return UOE_ERR_CUDA;
+        }
     }
     FuArgs a;
     a.q = (__nv_bfloat16*)f.q; a.k = (__nv_bfloat16*)f.k; a.v = (__nv_bfloat16*)f.v; a.o = (__nv_bfloat16*)f.o; a.z = (__nv_bfloat16*)f.z;
