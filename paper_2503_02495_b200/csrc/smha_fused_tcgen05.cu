@@ -511,7 +511,19 @@ bool smha_can_fuse(const Dims& D, bool recompute) {
     if (!recompute && D.d > 512) return false;
     const int n_qt = (D.l_a + T - 1) / T;
     const long long pairs = (long long)D.B * D.k;
-    if (n_qt == 1) return pairs <= 0x7fffffffll;
+    // One tile: always while all pairs are resident at once, which leaves the launch in between as pure gain (160 pairs of 16 tokens,
+    // d = 512: forward 26.9 us, separate launches 38.7; backward 79.9 and 85.0).  Beyond that short pairs cost: a CTA projects 128 rows
+    // whatever they hold, the grouped projection packs them.  Forward, 4000 pairs, d = 256, 32 / 48 / 96 tokens: 203 / 224 / 285 us,
+    // separate 202 / 227 / 300; 600 pairs of 16 tokens 43.9 and 50.3.  The recomputation also writes q, k, v, o: backward of 4000
+    // pairs of 48 / 80 / 96 tokens, d = 512: 694 / 971 / 1120 us, separate 657 / 952 / 1133.
+    if (n_qt == 1) {
+        if (pairs <= 2ll * sm_count()) return true;
+        if (recompute) return D.l_a >= 96;
+        return D.l_a >= 48 || pairs <= 4ll * sm_count();
+    }
+    // Several tiles: while all clusters are resident at once (16 causal pairs of 256 tokens, d = 512: forward 25.2 us, separate
+    // launches 28.7; two pairs of 1024 tokens, d = 256: 29.5 and 33.8; backward 103.3 and 108.9); more units keep the tensor cores
+    // busier in the streaming kernel.
     if (D.l_a % T != 0 || n_qt > 8) return false;
     return pairs <= resident_clusters(n_qt);
 }
