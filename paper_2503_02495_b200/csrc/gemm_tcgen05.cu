@@ -51,9 +51,9 @@ template <int BN, int MT, int EPI = kForward, bool PAIR = false> struct Cfg {
     static constexpr int KSUB = PAIR ? 2 : 1;                      // 64-wide K blocks per stage (one barrier round)
     static constexpr int SUB = A_BYTES + B_BYTES;
     static constexpr int STAGE = KSUB * SUB;
-    static constexpr int STAGES = PAIR ? 3 : (MT == 2) ? 3 : ((BN == 256 || BN == 192) ? 4 : (BN == 128 ? 6 : 8));
-    static constexpr int NACC = (MT == 2) ? 1 : 2;                 // accumulator sets in TMEM
-    static constexpr int ACC_STRIDE = (BN == 192) ? 256 : BN;      // TMEM columns between the two accumulator sets
+    static constexpr int STAGES = PAIR ? 3 : (MT == 2 || BN == 384) ? 3 : ((BN == 256 || BN == 192) ? 4 : (BN == 128 ? 6 : 8));
+    static constexpr int NACC = (MT == 2 || BN == 384) ? 1 : 2;                 // accumulator sets in TMEM
+    static constexpr int ACC_STRIDE = (BN == 192 || BN == 384) ? 256 : BN;      // TMEM columns between the two accumulator sets
     static constexpr int TMEM_COLS = 2 * ACC_STRIDE;               // MT=1: two sets; MT=2: one set of two blocks
     // eight epilogue warps: with 256-row tiles one per (row block, TMEM lane quarter); with 128-row tiles two per lane
     // quarter, each draining half of the columns
@@ -111,7 +111,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         prefetch_tmap(&tmB0);
         prefetch_tmap(&tmX);
         prefetch_tmap(&tmC0);
-        if (nmat > 1 || BN == 192 || k_per_mat > 0) { prefetch_tmap(&tmB1); prefetch_tmap(&tmB2); prefetch_tmap(&tmC1); prefetch_tmap(&tmC2); }
+        if (nmat > 1 || BN == 192 || BN == 384 || k_per_mat > 0) { prefetch_tmap(&tmB1); prefetch_tmap(&tmB2); prefetch_tmap(&tmC1); prefetch_tmap(&tmC2); }
         if (EPI != kForward) prefetch_tmap(&tmC1);
     }
     if (warp == 1) {
@@ -142,10 +142,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t tmem_base = ctl->tmem_base;
 
     // tile index -> (row tile, matrix, column tile); the matrices share the A tile, so they are adjacent
-    // BN = 192 is the "three 64-wide matrices side by side" tile: the B stage holds one 64-column box of each of the
-    // three weight tensors and the three 64-column pieces of the accumulator go to the three outputs, so the A tile is
-    // loaded once for q, k and v
-    constexpr bool SIDE3 = BN == 192;
+    // BN = 192 (384) is the "three 64-wide (128-wide) matrices side by side" tile: the B stage holds a box of each of the
+    // three weight tensors and the three pieces of the accumulator go to the three outputs, so the A tile is loaded once for
+    // q, k and v.  The 384 columns leave room for one accumulator set: a tile's write-out is exposed, but its operands are 64 KB
+    // per 64 of K where three 128-column tiles take 96
+    constexpr bool SIDE3 = BN == 192 || BN == 384;
+    constexpr int SIDE_G = SIDE3 ? BN / 192 : 1;          // 64-column groups per matrix
     const int n_tiles_mat = SIDE3 ? 1 : N / BN;
     const int n_tiles = SIDE3 ? 1 : n_tiles_mat * nmat;
     const int num_kb = K / (BK * Cf::KSUB);
@@ -227,7 +229,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         else tma_load_2d(sa, &tmA, kb * BK, row0, &ctl->full[stage]);
                     }
                     if (lane < nbox_b) {
-                        if (SIDE3) tma_load_4d(sb + lane * 8192, tmB_lane, 0, kb * BK, 0, e, &ctl->full[stage]);
+                        if (SIDE3) tma_load_4d(sb + lane * (SIDE_G * 8192), tmB_lane, 0, kb * BK, 0, e, &ctl->full[stage]);
                         else if (B_KMAJOR) {
                             const int q = k_per_mat > 0 ? kb / k_per_mat : 0;
                             tma_load_3d(sb, k_per_mat > 0 ? pick(q) : tmB, (kb - q * k_per_mat) * BK, col0, e, &ctl->full[stage]);
@@ -248,7 +250,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (rank == 0) {
             // ---------------- MMA issuer (the whole warp, one elected lane issues) ----------------
             const uint32_t el = elect_one();
-            constexpr uint32_t idesc = instr_desc_bf16(PAIR ? 2 * BM : BM, BN, false, !B_KMAJOR);
+            constexpr int N_MMA = BN == 384 ? 256 : BN;             // (an instruction holds 256 columns; the other 128 are a second one)
+            constexpr uint32_t idesc = instr_desc_bf16(PAIR ? 2 * BM : BM, N_MMA, false, !B_KMAJOR);
+            [[maybe_unused]] constexpr uint32_t idesc_rest = instr_desc_bf16(BM, 128, false, !B_KMAJOR);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool stop = false;
@@ -277,6 +281,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 if (h < blocks)
                                     mma_bf16(el, d_tmem + h * BN, smem_desc(sa + h * A_BLOCK_BYTES + kq * 32, 16, 1024), bd, idesc,
                                              (kb | ks) != 0);
+                            if constexpr (BN == 384)
+                                mma_bf16(el, d_tmem + 256, smem_desc(sa + kq * 32, 16, 1024), smem_desc(sb + 4 * 8192 + kq * 2048, 8192, 1024),
+                                         idesc_rest, (kb | ks) != 0);
                         }
                     }
                     if constexpr (PAIR) mma_commit_pair(el, &ctl->empty[stage]);       // frees the stage in both CTAs
@@ -357,6 +364,20 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if constexpr (ROPE) {                            // (two dependent look-ups, under the tile's main loop)
                 int b;
                 if (half < blocks) tok = token_of(rope.map, row0 + half * BM + quarter * 32 + lane, e, ctl->offs[e], b);
+            }
+            // q, k, v side by side: a warp takes the same 32 channels of every head, so the angles are found once per row and tile,
+            // under the main loop (found per head and chunk behind it, two heads of 16384 rows, d = 1024: block forward 160.2 us, so 152.0)
+            constexpr bool BY_HALF = SIDE3 && EPI == kForward && CW == 32;
+            [[maybe_unused]] float cs[16], sn[16];
+            [[maybe_unused]] const bool rotated = [&] { if constexpr (ROPE) return wsel * 16 + 15 >= rope.pair0; else return false; }();
+            if constexpr (ROPE && BY_HALF) {
+                if (rotated)
+#pragma unroll
+                    for (int p = 0; p < 16; ++p) {
+                        cs[p] = 1.f;
+                        sn[p] = 0.f;
+                        if (wsel * 16 + p >= rope.pair0) rope_angle(rope, wsel * 16 + p, (float)max(tok, 0), cs[p], sn[p]);
+                    }
             }
             const int wrow0 = row0 + half * BM + quarter * 32;           // first row of this warp's piece
             const size_t row = (size_t)wrow0 + lane;
@@ -458,6 +479,27 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         att.delta[h] = rg != 0.f ? dot_c.x + dot_c.y : 0.f;
                         dg_part[h] = rv != 0.f ? dot.x + dot.y : 0.f;
                     }
+                } else if constexpr (BY_HALF) {
+#pragma unroll 1
+                    for (int g = 0; g < G; ++g) {
+                        uint32_t v[32];
+                        tmem_ld32(taddr + g * 64 + wsel * 32, v);
+                        tmem_ld_wait();
+                        float f[32];
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) f[q] = __uint_as_float(v[q]);
+                        if constexpr (ROPE) {
+                            if (rotated && g < 2 * SIDE_G) {     // Eq. 32 on the float32 accumulators
+#pragma unroll
+                                for (int p = 0; p < 16; ++p) {
+                                    const float a0 = f[2 * p], a1 = f[2 * p + 1];
+                                    f[2 * p] = a0 * cs[p] - a1 * sn[p];
+                                    f[2 * p + 1] = a0 * sn[p] + a1 * cs[p];
+                                }
+                            }
+                        }
+                        stage_store(f, g / SIDE_G == 0 ? &tmC0 : (g / SIDE_G == 1 ? &tmC1 : &tmC2), g % SIDE_G * 64 + wsel * 32, wrow0);
+                    }
                 } else {
 #pragma unroll 1
                     for (int g = g_lo; g < g_hi; ++g)
@@ -482,7 +524,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                         }
                         if constexpr (ROPE) {
-                            if ((SIDE3 ? g : mat) < 2) {
+                            if (mat < 2) {
                                 // Eq. 32 on the float32 accumulators: the head's last channels, two MUFU operations per pair
 #pragma unroll
                                 for (int p = 0; p < 16; ++p) {
@@ -503,7 +545,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                             for (int q = 0; q < CW; ++q) f[q] *= sc;
                         }
-                        if (SIDE3) stage_store(f, g == 0 ? &tmC0 : (g == 1 ? &tmC1 : &tmC2), c * CW, wrow0);
+                        if (SIDE3) stage_store(f, g / SIDE_G == 0 ? &tmC0 : (g / SIDE_G == 1 ? &tmC1 : &tmC2), g % SIDE_G * 64 + c * CW, wrow0);
                         else stage_store(f, tmC, col0 + col, wrow0);
                     }
                 }
@@ -574,7 +616,7 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
         } else {              // W [n, K, N] as [n][N/64 column blocks][K][64]
             const uint64_t dims[4] = {64, (uint64_t)g.K, (uint64_t)g.N / 64, (uint64_t)g.n};
             const uint64_t str[3] = {(uint64_t)g.N * 2, 128, (uint64_t)g.K * g.N * 2};
-            const uint32_t box[4] = {64, BK, (uint32_t)(BN == 192 ? 1 : (PAIR ? BN / 2 : BN) / 64), 1};
+            const uint32_t box[4] = {64, BK, (uint32_t)(BN == 192 || BN == 384 ? BN / 192 : (PAIR ? BN / 2 : BN) / 64), 1};
             if (!make_tmap(&tmB[q], Ws[q], 4, dims, str, box)) return UOE_ERR_CUDA;
         }
     }
@@ -592,7 +634,7 @@ uoe_status launch_one(const GemmArgs& g, int* status, cudaStream_t s) {
             if (!out_map(&tmC[q], Cs[q])) return UOE_ERR_CUDA;
         if (!out_map(&tmPre, g.pre ? g.pre : g.C)) return UOE_ERR_CUDA;
     }
-    long long max_tiles = ((g.rows_max / BM + Cf::UNIT - 1) / Cf::UNIT + g.n) * (BN == 192 ? 1 : (g.N / BN) * nmat);
+    long long max_tiles = ((g.rows_max / BM + Cf::UNIT - 1) / Cf::UNIT + g.n) * (BN == 192 || BN == 384 ? 1 : (g.N / BN) * nmat);
     const int walkers = PAIR ? max_pairs : sm_count();
     int grid = (int)(max_tiles < walkers ? max_tiles : walkers);
     if (grid < 1) grid = 1;
@@ -671,6 +713,10 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
         if (rope) return launch_one<192, false, kForward, 1, false, true>(g, status, s);
         return short_k ? launch_one<192, false, kForward, 1, false, false, 64>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
     }
+    // Two heads per expert: q, k, v as one 384-column tile (wide block above: forward 162.4 us with three 128-column tiles, 152.0 so,
+    // training step 527 and 504), once the row tiles alone give the SMs more than one 128-column tile each
+    if (g.nmat == 3 && g.N == 128 && !g.b_kmajor && !g.pre && !short_k && 3 * (g.rows_max / BM) > sm_count())
+        return rope ? launch_one<384, false, kForward, 1, false, true>(g, status, s) : launch_one<384, false, kForward, 1>(g, status, s);
     if (rope) return dispatch<false, kForward, true>(g, status, s);
     if (short_k) return g.b_kmajor ? dispatch<true, kForward, false, 64>(g, status, s) : dispatch<false, kForward, false, 64>(g, status, s);
     if (g.b_kmajor) return dispatch<true, kForward>(g, status, s);

@@ -309,6 +309,16 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             const int pj = u < a.c ? a.patch_idx[(size_t)pair * a.c + u] : -1;
             tok = pj >= 0 ? (pj << a.lp_log) + (qrow & (l_p - 1)) : 0;
         }
+        // a warp takes the same 32 channels of q and of k: their angles once, under the projection's products
+        [[maybe_unused]] float cs[16], sn[16];
+        if constexpr (ROPE) {
+#pragma unroll
+            for (int p = 0; p < 16; ++p) {
+                cs[p] = 1.f;
+                sn[p] = 0.f;
+                if (hsel * 16 + p >= rope.pair0) rope_angle(rope, hsel * 16 + p, (float)tok, cs[p], sn[p]);
+            }
+        }
         if (keep) {                                      // padding rows of the expert regions: zeros, as tiles may reach over them
             for (int e = blockIdx.x; e < a.n; e += gridDim.x) {
                 const int r0 = a.expert_end[e], vecs = (a.offsets[e + 1] - r0) * (DH / 8);
@@ -332,13 +342,9 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                     if (g < 2) {
 #pragma unroll
                         for (int p = 0; p < 16; ++p) {   // Eq. 32 on the float32 accumulators
-                            if (hsel * 16 + p >= rope.pair0) {
-                                float cs, sn;
-                                rope_angle(rope, hsel * 16 + p, (float)tok, cs, sn);
-                                const float x0 = f[2 * p], x1 = f[2 * p + 1];
-                                f[2 * p] = x0 * cs - x1 * sn;
-                                f[2 * p + 1] = x0 * sn + x1 * cs;
-                            }
+                            const float x0 = f[2 * p], x1 = f[2 * p + 1];
+                            f[2 * p] = x0 * cs[p] - x1 * sn[p];
+                            f[2 * p + 1] = x0 * sn[p] + x1 * cs[p];
                         }
                     }
                 }

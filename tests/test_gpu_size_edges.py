@@ -29,6 +29,8 @@ ROPE_CASES = {
     "patch20_two_heads": (_att(B=5, L=140, L_valid=133, m=7, c=4, n=3, k=2, H=6, causal=True), 32, {}),
     "whole_samples": (_att(B=4, L=160, L_valid=150, m=10, c=10, n=4, k=2, H=4), 64, {}),
     "unused_slots": (_att(B=4, L=128, L_valid=128, m=16, c=12, n=4, k=2, H=4), 16, {"dynamic_c": True}),
+    "two_heads_many_rows": (_att(B=8, L=1024, L_valid=1010, m=16, c=8, d=192, n=4, k=2, H=8, causal=True), 32, {}),
+    "two_heads_many_rows_no_rope": (_att(B=8, L=1024, L_valid=1024, m=16, c=8, d=192, n=4, k=2, H=8), 0, {}),
     "patch1": (_att(B=2, L=40, L_valid=39, m=40, c=17, n=2, k=2, H=2), 2, {}),
 }
 
