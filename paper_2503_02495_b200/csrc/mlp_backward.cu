@@ -22,13 +22,12 @@ using namespace tc;
 
 constexpr int kThreads = 256;
 
-// Gradient of the router logits of one sample from the per-row gate gradients.  grid B, 512 threads, dynamic shared
+// Gradient of the router logits of one sample from the per-row gate gradients.  grid B, 256 or 512 threads, dynamic shared
 // memory (2 n m + k c) floats.  A warp per slab adds the slab's per-row, per-column-tile partials (fixed order), then the
 // softmax Jacobians of Eq. 14 and 21:  G[b,j,i] = dlogit_patch[b,i,j]/cnt_j + dlogit_samp[b,i]/L_valid.
 // Latency-bound (a sample's partials are a few KB to a few hundred KB); one launch instead of a slab-sum kernel and a
 // Jacobian kernel whose sums over a slot list were one thread's serial loop.
-constexpr int kGradThreads = kReduceThreads;
-__global__ void __launch_bounds__(kGradThreads, 2)
+__global__ void __launch_bounds__(kReduceThreads, 2)
 router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restrict__ pair_row,
                    const int* __restrict__ expert_idx, const int* __restrict__ patch_idx,
                    const float* __restrict__ p_samp, const float* __restrict__ p_patch, int n, int k, int m, int c,
@@ -47,14 +46,14 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
     float* dpp = sm + n * m;        // [n][m] its gradient
     float* dg = sm + 2 * n * m;     // [k][c] gradient of the combine weight of every slot
     __shared__ float ps[32], dls[32], dps[32];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int idx = tid; idx < n * m; idx += kGradThreads) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, NT = blockDim.x;
+    for (int idx = tid; idx < n * m; idx += NT) { pp[idx] = p_patch[(size_t)b * n * m + idx]; dpp[idx] = 0.f; }
     if (tid < 32) { ps[tid] = tid < n ? p_samp[(size_t)b * n + tid] : 0.f; dps[tid] = 0.f; }
     // four slabs at a time, so that their look-ups and loads are in flight together (one at a time a sample of 1271 slabs of
     // four tokens took 90 us)
     const int len = l_p * nt;
     constexpr int U = 4;
-    for (int slab0 = warp * U; slab0 < k * c; slab0 += kGradThreads / 32 * U) {
+    for (int slab0 = warp * U; slab0 < k * c; slab0 += NT / 32 * U) {
         const float* src[U];
         int n_q[U];                                       // values of the slab: none of an unused slot
         float a[U];
@@ -89,7 +88,7 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
     }
     __syncthreads();
     // gate = P_samp * P_patch: a warp per chosen expert, lanes over its slots
-    for (int s = warp; s < k; s += kGradThreads / 32) {
+    for (int s = warp; s < k; s += NT / 32) {
         int i = expert_idx[(size_t)b * k + s];
         i = (unsigned)i < (unsigned)n ? i : 0;            // (the plan kernel has reported an index out of range)
         float acc = 0.f;
@@ -111,7 +110,7 @@ router_grad_kernel(const float* __restrict__ dg_part, int nt, const int* __restr
         dls[lane] = ps[lane] * (dps[lane] - dot);
     }
     __syncthreads();
-    for (int j = tid; j < m; j += kGradThreads) {         // softmax Jacobian of each patch gate (Eq. 14)
+    for (int j = tid; j < m; j += NT) {         // softmax Jacobian of each patch gate (Eq. 14)
         const int cnt = max(0, min(l_p, Lv - j * l_p));
         float dot = 0.f;
         for (int i = 0; i < n; ++i) dot += pp[i * m + j] * dpp[i * m + j];
@@ -417,7 +416,7 @@ uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r,
     const int grad_ctas = D.B + reduce.blocks;
     {
         ProfScope ps("router_grad", stream);
-        launch_k(router_grad_kernel, dim3(grad_ctas), dim3(kGradThreads), spread_smem(once, router_grad_kernel, grad_ctas, smem), stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
+        launch_k(router_grad_kernel, dim3(grad_ctas), dim3(reduce.threads), spread_smem(once, router_grad_kernel, grad_ctas, smem), stream, dgp, nt, (const int*)P.pair_row, expert_idx, patch_idx,
                  p_samp, p_patch, D.n, D.k, D.m, D.c, D.l_p, D.Lv, rs.G, D.B, reduce);
     }
     UOE_LAUNCHED();

@@ -22,9 +22,13 @@ struct WReduce {
     int per = 1;              // blocks per tile
     int part_floats = 0;      // of a part of a tile in the scratch
     int by_cut = 0;           // blocks are counted by piece boundary (more tiles than pieces), else by tile
+    int threads = 512;        // of a block
 };
 
-constexpr int kReduceThreads = 512;
+// Threads of a block: 512 where the blocks are counted by cut, which is where there are many (every block builds the line again: wide
+// block, training step 504 us, with 256 threads and twice the blocks 507), else 256, so that the blocks and the samples' CTAs beside
+// them are resident at once (language-model block 250.8 -> 248.2, image block 671 -> 670).
+constexpr int kReduceThreads = 512, kReduceThreadsFew = 256;
 
 #ifdef __CUDACC__
 struct WSched {
@@ -105,7 +109,7 @@ __device__ __forceinline__ bool wsched_next(const WSched& s, const WProblem* pro
 // last (the tile goes on).
 __device__ __forceinline__ size_t wsched_slot(const WFrag& f, int c) { return (size_t)c * 2 + (c > f.c_first ? 0 : 1); }
 
-// Adds the parts of every cut tile in ascending order.  r.per blocks of kReduceThreads threads for a tile, half a [32 x 32]
+// Adds the parts of every cut tile in ascending order.  r.per blocks of r.threads threads for a tile, half a [32 x 32]
 // piece per warp.  The blocks are counted by tile or, when there are more tiles than pieces, by the boundaries between
 // pieces: each cuts at most one tile, whose first boundary does the work.  Bound by the latency of the part loads: two
 // parts are in flight per warp (one part and a whole piece per warp: 32 us instead of 21 for the image block's MLP half).
@@ -138,7 +142,7 @@ __device__ __forceinline__ void wgrad_reduce(const WReduce& r, int blk) {
         wsched_tile(s, r.prob[p], p, tile / per_e, tile % per_e, f, begin, cost);
     }
     const WProblem& pr = r.prob[p];
-    const int piece = (blk % r.per) * (kReduceThreads / 32) + warp;
+    const int piece = (blk % r.per) * (r.threads / 32) + warp;
     const int h = piece & 1, quarter = (piece >> 1) & 3, ch = piece >> 3;
     if (f.c_first == f.c_last || ch * 32 >= f.cols) return;
     // lanes over (row, four columns) so that both the reads and the row-major writes are whole sectors; a transposed

@@ -336,8 +336,9 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     r.part_floats = a.part_floats;
     int tiles = 0;
     for (int i = 0; i < nprob; ++i) tiles += n * a.prob[i].m_tiles * a.prob[i].n_tiles;
-    r.per = (widest / 32 * 8 + kReduceThreads / 32 - 1) / (kReduceThreads / 32);
     r.by_cut = tiles > a.pieces - 1 ? 1 : 0;
+    r.threads = r.by_cut ? kReduceThreads : kReduceThreadsFew;
+    r.per = (widest / 32 * 8 + r.threads / 32 - 1) / (r.threads / 32);
     r.blocks = (r.by_cut ? a.pieces - 1 : tiles) * r.per;
     *reduce = r;
     return UOE_OK;
@@ -347,7 +348,7 @@ uoe_status launch_wgrad_reduce(const WReduce& r, cudaStream_t s) {
     if (r.blocks == 0) return UOE_OK;
     ProfScope ps("wgrad_reduce", s);
     static SpreadOnce once;
-    launch_k(wgrad_reduce_kernel, dim3(r.blocks), dim3(kReduceThreads), spread_smem(once, wgrad_reduce_kernel, r.blocks, 0), s, r);
+    launch_k(wgrad_reduce_kernel, dim3(r.blocks), dim3(r.threads), spread_smem(once, wgrad_reduce_kernel, r.blocks, 0), s, r);
     UOE_LAUNCHED();
     return UOE_OK;
 }
