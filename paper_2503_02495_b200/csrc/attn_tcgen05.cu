@@ -154,9 +154,6 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     };
     const int n_zchunk = FUSE_O ? (a.d + ZCHUNK - 1) / ZCHUNK : 0;
     auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag, status) && !*abort_flag; };
-    // the same for the one-thread roles (TMA, MMA), which sit on the critical path between the softmax warps' steps:
-    // they poll without letting the hardware suspend them first
-    auto wait1 = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_spin(bar, parity, abort_flag, status) && !*abort_flag; };
 
     if (role == 1) {
         // =========================== TMA warp ===========================
@@ -178,7 +175,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const int n_kv = kv_tiles(q0, nv);
             const bool mine = n_kv > 0;
             if (lane == 0) {
-                ok = wait1(&pc->q_empty, (q_cnt & 1) ^ 1);
+                ok = wait(&pc->q_empty, (q_cnt & 1) ^ 1);
                 if (ok) {
                     pc->row_base = row_base; pc->n_valid = nv; pc->expert = expert;
                     if (mine) {
@@ -191,7 +188,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 ++q_cnt;
                 for (int t = 0; t < n_kv && ok; ++t) {
                     const int st = kv_cnt & 1;
-                    ok = wait1(&pc->kv_empty[st], ((kv_cnt >> 1) & 1) ^ 1);
+                    ok = wait(&pc->kv_empty[st], ((kv_cnt >> 1) & 1) ^ 1);
                     if (!ok) break;
                     uint8_t* stage = sKV + st * 2 * TILE_BYTES;
                     mbar_arrive_expect_tx(&pc->kv_full[st], 2 * TILE_BYTES);
@@ -203,7 +200,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     for (int zc = 0; zc < n_zchunk && ok; ++zc) {
                         const int n0 = zc * ZCHUNK, nn = min(ZCHUNK, a.d - n0);
                         const int st = kv_cnt & 1;
-                        ok = wait1(&pc->kv_empty[st], ((kv_cnt >> 1) & 1) ^ 1);
+                        ok = wait(&pc->kv_empty[st], ((kv_cnt >> 1) & 1) ^ 1);
                         if (!ok) break;
                         uint8_t* stage = sKV + st * 2 * TILE_BYTES;
                         mbar_arrive_expect_tx(&pc->kv_full[st], (uint32_t)nn * DH * 2);
@@ -221,7 +218,7 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     } else if (role == 2) {
         // =========================== MMA warp ===========================
         const uint32_t el = elect_one();
-        auto waitw = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait1(bar, parity)) != 0; };
+        auto waitw = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait(bar, parity)) != 0; };
         constexpr uint32_t idesc_s = instr_desc_bf16(TQ, TK, false, false);
         constexpr uint32_t idesc_o = instr_desc_bf16(TQ, DH, false, true);
         uint32_t q_cnt = 0, kv_cnt = 0, acc_cnt = 0, p_cnt = 0, ready_cnt = 0;

@@ -149,7 +149,6 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
     const bool keep = a.q != nullptr;                    // the backward's recomputation
     const int n_z = keep || n_kv == 0 ? 0 : (a.d + ZC - 1) / ZC;
     auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag, status) && !*abort_flag; };
-    auto wait1 = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_spin(bar, parity, abort_flag, status) && !*abort_flag; };
 
     if (warp == 8) {
         // =========================== TMA producer ===========================
@@ -159,7 +158,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             const int st = kb % Cf::STAGES;
             int w = 1;
             if (lane == 0) {
-                w = wait1(&ctl->empty[st], ((kb / Cf::STAGES) & 1) ^ 1) ? 1 : 0;
+                w = wait(&ctl->empty[st], ((kb / Cf::STAGES) & 1) ^ 1) ? 1 : 0;
                 if (w) mbar_arrive_expect_tx(&ctl->full[st], STAGE);
             }
             ok = __shfl_sync(0xffffffffu, w, 0) != 0;
@@ -171,7 +170,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         }
         auto load_w = [&]() {                            // the next chunk of W^o
             const int j = w_issued, st = j % Cf::NW, nn = min(ZC, a.d - j * ZC);
-            if (!wait1(&ctl->w_empty[st], ((j / Cf::NW) & 1) ^ 1)) return false;
+            if (!wait(&ctl->w_empty[st], ((j / Cf::NW) & 1) ^ 1)) return false;
             mbar_arrive_expect_tx(&ctl->w_full[st], (uint32_t)nn * DH * 2);
             for (int nb = 0; nb < nn / 64; ++nb) tma_load_3d(unit(Cf::W(st)) + nb * 8192, &tm.wo, j * ZC + nb * 64, 0, expert, &ctl->w_full[st]);
             ++w_issued;
@@ -179,7 +178,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         };
         if constexpr (MULTI) {
             if (lane == 0) {                             // own k and v to memory
-                ok = ok && wait1(&ctl->qkv_ready, 0);
+                ok = ok && wait(&ctl->qkv_ready, 0);
                 if (ok && named) {
                     tma_store_2d(&tm.k, unit(Cf::K), 0, row_base + q0);
                     tma_store_2d(&tm.v, unit(Cf::V), 0, row_base + q0);
@@ -195,18 +194,18 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 fence_async_all();
                 for (int i = own ? 1 : 0; i < n_kv && ok; ++i) {
                     const int q = kv_issued, st = q & 1, t = tile_at(i);
-                    ok = wait1(&ctl->kv_empty[st], ((q >> 1) & 1) ^ 1);
+                    ok = wait(&ctl->kv_empty[st], ((q >> 1) & 1) ^ 1);
                     if (!ok) break;
                     mbar_arrive_expect_tx(&ctl->kv_full[st], 2 * UNIT);
                     tma_load_2d(unit(Cf::KV + 2 * st), &tm.k, 0, row_base + t * T, &ctl->kv_full[st]);
                     tma_load_2d(unit(Cf::KV + 2 * st + 1), &tm.v, 0, row_base + t * T, &ctl->kv_full[st]);
                     ++kv_issued;
                 }
-                if (w_issued < n_z && own) ok = ok && wait1(&ctl->own_free, 0);
+                if (w_issued < n_z && own) ok = ok && wait(&ctl->own_free, 0);
             }
         } else if (lane == 0 && ok && n_z > 0) {
             ok = load_w();
-            ok = ok && wait1(&ctl->s_full, 0);           // S is done: q and k may be overwritten
+            ok = ok && wait(&ctl->s_full, 0);           // S is done: q and k may be overwritten
         }
         if (lane == 0)
             while (ok && w_issued < n_z) ok = load_w();
@@ -219,7 +218,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
     } else if (warp == 9) {
         // =========================== MMA issuer (the whole warp, one elected lane issues) ===========================
         const uint32_t el = elect_one();
-        auto waitw = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait1(bar, parity)) != 0; };
+        auto waitw = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, wait(bar, parity)) != 0; };
         constexpr uint32_t idesc_p = instr_desc_bf16(T, 192, false, true), idesc_s = instr_desc_bf16(T, T, false, false);
         constexpr uint32_t idesc_o = instr_desc_bf16(T, DH, false, true);
         bool ok = true;
