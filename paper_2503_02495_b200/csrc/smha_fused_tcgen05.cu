@@ -51,7 +51,7 @@ static_assert(FCfg<false>::STAGES * STAGE <= FCfg<false>::W(0) * UNIT && FCfg<tr
 static_assert(2 * (FCfg<false>::SMEM + 2048 + 1024) <= 228 * 1024, "two CTAs per SM");
 
 struct FuCtl {
-    uint64_t full[5], empty[5], qkv_full, qkv_ready, kv_full[2], kv_empty[2], s_full, p_full, o_full, o_ready, own_free, w_full[4], w_empty[4],
+    uint64_t full[5], empty[5], qkv_full, qkv_ready /* multi */, kv_full[2], kv_empty[2], s_full, o_full, own_free, w_full[4], w_empty[4],
         z_full[2], z_free[2];
     uint32_t tmem_base;
     int abort_flag, n_valid, pad;
@@ -70,6 +70,11 @@ struct FuArgs {
     int* status;
 };
 
+// Hand-over from the softmax warps to the MMA warp: they arrive, it waits, on a barrier of the SM, which wakes it sooner than an mbarrier
+// does (image block forward 190.3 us through mbarriers, 187.6 so; language-model block 69.5 and 69.0).  Nobody skips one: a warp whose wait ran out arrives all the same.
+constexpr int kHandOver = 6;
+__device__ __forceinline__ void hand_over_arrive() { asm volatile("bar.arrive %0, %1;" :: "n"(kHandOver), "n"(32 * (kSoftWarps + 1)) : "memory"); }
+__device__ __forceinline__ void hand_over_wait() { asm volatile("bar.sync %0, %1;" :: "n"(kHandOver), "n"(32 * (kSoftWarps + 1)) : "memory"); }
 __device__ __forceinline__ void bar_named(int id, int threads) { asm volatile("bar.sync %0, %1;" :: "r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -104,9 +109,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         for (int s = 0; s < Cf::NW; ++s) { mbar_init(&ctl->w_full[s], 1); mbar_init(&ctl->w_empty[s], 1); }
         mbar_init(&ctl->own_free, 1);
         mbar_init(&ctl->s_full, 1);
-        mbar_init(&ctl->p_full, 32 * kSoftWarps);
         mbar_init(&ctl->o_full, 1);
-        mbar_init(&ctl->o_ready, 32 * kSoftWarps);
         ctl->abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tm.x);
@@ -235,7 +238,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         }
         if (ok) mma_commit(el, &ctl->qkv_full);
         if constexpr (MULTI) cluster_arrive();
-        ok = ok && waitw(&ctl->qkv_ready, 0);
+        hand_over_wait();                                // q, k, v are in shared memory
         const uint32_t qa = smem_u32(unit(0)), pa = smem_u32(unit(Cf::P));
         // place of the i-th tile's k and v: own, or stage q & 1 of the others
         auto stage_of = [&](int i) { return own ? i - 1 : i; };
@@ -251,9 +254,10 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             return true;
         };
         if (n_kv > 0) ok = ok && issue_s(0);
-        for (int i = 0; i < n_kv && ok; ++i) {
-            ok = waitw(&ctl->p_full, i & 1);
-            if (!ok) break;
+        for (int i = 0; i < n_kv; ++i) {
+            hand_over_wait();                            // P is
+            ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
+            if (!ok) continue;
             tc_fence_after();
             const int q = stage_of(i);
             const uint32_t va = smem_u32(MULTI && q >= 0 ? unit(Cf::KV + 2 * (q & 1) + 1) : unit(Cf::V));
@@ -265,7 +269,8 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             if (MULTI) mma_commit(el, q >= 0 ? &ctl->kv_empty[q & 1] : &ctl->own_free);
             if (i + 1 < n_kv) ok = issue_s(i + 1);       // (into the other accumulator: it runs under the O update)
         }
-        if (n_z > 0) ok = ok && waitw(&ctl->o_ready, 0);
+        if (n_kv > 0) hand_over_wait();                  // o is
+        ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
         for (int j = 0; j < n_z && ok; ++j) {
             const int st = j & 1, wb = j % Cf::NW;
             ok = waitw(&ctl->w_full[wb], (j / Cf::NW) & 1) && waitw(&ctl->z_free[st], ((j >> 1) & 1) ^ 1);
@@ -351,8 +356,9 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             }
             fence_async_smem();
             tc_fence_before();
-            mbar_arrive(&ctl->qkv_ready);
+            if (MULTI) mbar_arrive(&ctl->qkv_ready);
         }
+        hand_over_arrive();
         if constexpr (MULTI) cluster_arrive();
         if (keep) {
             bar_named(2 + quarter, 64);
@@ -411,8 +417,8 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 m_run = m_new;
                 fence_async_smem();
                 tc_fence_before();
-                mbar_arrive(&ctl->p_full);
             }
+            hand_over_arrive();
             ok = ok && __all_sync(0xffffffffu, wait(&ctl->o_full, i & 1)) != 0;
             if (ok) {
                 tc_fence_after();
@@ -437,8 +443,8 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 put(unit(Cf::P), o_acc, hsel * 4);       // o [128 x 64] where the first half of P was
                 fence_async_smem();
                 tc_fence_before();
-                mbar_arrive(&ctl->o_ready);
             }
+            hand_over_arrive();
             if (keep) {
                 bar_named(2 + quarter, 64);
                 if (ok) copy_out(unit(Cf::P), a.o);
