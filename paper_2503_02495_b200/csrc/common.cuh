@@ -294,6 +294,12 @@ __device__ __forceinline__ void st_stream16(void* p, const uint4& v) {
                  :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+// 32 bytes, one sector of L2, in one store (p a multiple of 32 bytes)
+__device__ __forceinline__ void st_sector(void* p, const uint4& a, const uint4& b) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+}
+
 // ------------------------------------------------------------------------------------------------
 // activations phi (Eq. 1) and their derivatives, float32
 // ------------------------------------------------------------------------------------------------

@@ -149,10 +149,10 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
             if (tid < n) s_end[tid] = expert_end[tid] = offs[tid] + hist[tid] * l_a;
         }
         __syncthreads();
-        for (int i = 0; i < n; ++i) {
-            for (int rb = s_end[i] / l_p + tid; rb < offs[i + 1] / l_p; rb += NT) src_patch[rb] = -1;
+        for (int i = tid >> 5; i < n; i += NT >> 5) {          // a warp per expert
+            for (int rb = s_end[i] / l_p + (tid & 31); rb < offs[i + 1] / l_p; rb += 32) src_patch[rb] = -1;
             if (row_gate)          // padding rows weigh nothing
-                for (int r = s_end[i] + tid; r < offs[i + 1]; r += NT) { row_gate[r] = 0.f; row_valid[r] = 0.f; }
+                for (int r = s_end[i] + (tid & 31); r < offs[i + 1]; r += 32) { row_gate[r] = 0.f; row_valid[r] = 0.f; }
         }
     }
     if (tails.row_bytes > 0) {
