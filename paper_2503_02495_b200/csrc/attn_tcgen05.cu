@@ -420,13 +420,11 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 if (qrow < a.l_a) {
                     __nv_bfloat16* out = a.O + (size_t)(row_base + qrow) * a.d_g + head * DH;
 #pragma unroll
-                    for (int ch = 0; ch < DH / 8; ++ch) {
-                        uint4 w;
-                        w.x = pack_bf16x2(o_acc[ch * 8 + 0] * inv, o_acc[ch * 8 + 1] * inv);
-                        w.y = pack_bf16x2(o_acc[ch * 8 + 2] * inv, o_acc[ch * 8 + 3] * inv);
-                        w.z = pack_bf16x2(o_acc[ch * 8 + 4] * inv, o_acc[ch * 8 + 5] * inv);
-                        w.w = pack_bf16x2(o_acc[ch * 8 + 6] * inv, o_acc[ch * 8 + 7] * inv);
-                        ((uint4*)out)[ch] = w;
+                    for (int ch = 0; ch < DH / 16; ++ch) {           // whole sectors
+                        uint32_t w[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) w[q] = pack_bf16x2(o_acc[ch * 16 + 2 * q] * inv, o_acc[ch * 16 + 2 * q + 1] * inv);
+                        st_sector(out + 16 * ch, make_uint4(w[0], w[1], w[2], w[3]), make_uint4(w[4], w[5], w[6], w[7]));
                     }
                 }
             } else {

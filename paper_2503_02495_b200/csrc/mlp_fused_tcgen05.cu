@@ -50,6 +50,7 @@ struct FCtl {
     int tstart[34];
 };
 
+template <bool PRE /* the pre-activation is stored too: a kernel of its own, as its code in the epilogue costs the other 0.7 % */>
 __global__ void __launch_bounds__(THREADS, 1)
 mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmX,
                  const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
@@ -268,10 +269,15 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         for (int q = 0; q < 8; ++q) f[8 * q8 + q] += bv[q];
                     }
                 }
-                if (pre) {
-                    uint4* dst = (uint4*)(pre + (size_t)(row0 + trow) * DE + g * 64);
+                if constexpr (PRE) {
+                    __nv_bfloat16* dst = pre + (size_t)(row0 + trow) * DE + g * 64;
+                    if (((uintptr_t)pre & 31) == 0) {        // (the caller's buffer) whole sectors
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) dst[c] = pack8(f + 8 * c);
+                        for (int c = 0; c < 4; ++c) st_sector(dst + 16 * c, pack8(f + 16 * c), pack8(f + 16 * c + 8));
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) ((uint4*)dst)[c] = pack8(f + 8 * c);
+                    }
                 }
                 act_apply_n<64>(f, act);
 #pragma unroll
@@ -346,9 +352,9 @@ uoe_status launch_mlp_fused(const Dims& D, const void* A, const void* W1, const 
                             cudaStream_t s, const void* b1, const void* b2) {
     if (!mlp_can_fuse(D) || D.Rmax % BM != 0) return UOE_ERR_UNSUPPORTED;
     if (gather_x && (!map.on() || D.l_p < 8 || D.l_p % 8 != 0 || BM % D.l_p != 0)) return UOE_ERR_INVALID_ARG;
-    static DeviceOnce once;
+    static DeviceOnce once[2];
     {
-        const uoe_status st = smem_opt_in(once, mlp_fused_kernel, SMEM);
+        const uoe_status st = pre ? smem_opt_in(once[1], mlp_fused_kernel<true>, SMEM) : smem_opt_in(once[0], mlp_fused_kernel<false>, SMEM);
         if (st != UOE_OK) return st;
     }
     CUtensorMap tmA, tmX, tmW1, tmW2, tmZ;
@@ -384,9 +390,12 @@ uoe_status launch_mlp_fused(const Dims& D, const void* A, const void* W1, const 
     int grid = (int)(max_tiles < sm_count() ? max_tiles : sm_count());
     if (grid < 1) grid = 1;
     ProfScope ps("mlp_fused", s);
-    launch_k(mlp_fused_kernel, dim3(grid), dim3(THREADS), (size_t)SMEM, s, tmA, tmX, tmW1, tmW2, tmZ, (__nv_bfloat16*)pre, offsets,
-             D.n, D.d, act, status, gather_x ? map : SrcMap(), D.l_p, (int)(D.B * D.m), (const __nv_bfloat16*)b1,
-             (const __nv_bfloat16*)b2);
+    auto go = [&](auto kern) {
+        launch_k(kern, dim3(grid), dim3(THREADS), (size_t)SMEM, s, tmA, tmX, tmW1, tmW2, tmZ, (__nv_bfloat16*)pre, offsets, D.n, D.d, act, status,
+                 gather_x ? map : SrcMap(), D.l_p, (int)(D.B * D.m), (const __nv_bfloat16*)b1, (const __nv_bfloat16*)b2);
+    };
+    if (pre) go(mlp_fused_kernel<true>);
+    else go(mlp_fused_kernel<false>);
     UOE_LAUNCHED();
     return UOE_OK;
 }
