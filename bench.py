@@ -91,6 +91,8 @@ def work_table(w: gen.Workload):
         t["qkv_proj"] = dict(flops=6 * R * d * dg, bytes=(R * d + 3 * R * dg + 3 * n * d * dg) * s)
         t["attention"] = dict(flops=att, bytes=4 * R * dg * s)
         t["out_proj"] = dict(flops=2 * R * dg * d, bytes=(R * dg + R * d + n * dg * d) * s)
+        # projections, attention and output projection in one kernel: q, k, v, o are neither written nor read back
+        t["smha_fused"] = dict(flops=t["qkv_proj"]["flops"] + att + t["out_proj"]["flops"], bytes=(2 * R * d + 4 * n * d * dg) * s)
     if w.H and w.backward:
         # algorithmic work of the attention backward is five l_a x l_a contractions (dV, dP, dK, dQ and the rebuilt S)
         t["attn_bwd"] = dict(flops=5 * att // 2, bytes=8 * R * dg * s)
@@ -659,7 +661,7 @@ def single_mode_of(dev, steps: int):
     return out
 
 
-TENSOR_KERNELS = ("gemm1_act", "gemm2", "mlp_fused", "qkv_proj", "out_proj", "attention", "bwd_da_dh", "bwd_dx", "wgrad_W1", "wgrad_W2",
+TENSOR_KERNELS = ("gemm1_act", "gemm2", "mlp_fused", "qkv_proj", "out_proj", "attention", "smha_fused", "bwd_da_dh", "bwd_dx", "wgrad_W1", "wgrad_W2",
                   "wgrad_mlp", "attn_bwd", "bwd_do", "bwd_dx_att", "wgrad_att")
 HBM_KERNELS = ("route", "gather", "combine", "router_apply")
 
