@@ -671,28 +671,26 @@ HBM_KERNELS = ("route", "gather", "combine", "router_apply")
 # changed since, the line reports null instead of a stale figure.  (workload, kernel label) ->
 # (bytes per launch at the benchmark's size, source file, sha1 prefix, profiles/ summary)
 NCU_TRAFFIC = {
-    ("cfg5_scale", "wgrad_W2"): (942.3e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "wgrad_W1"): (861.2e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "gemm1_act"): (943.2e6, "gemm_tcgen05.cu", "6096da824b3b", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "gemm2"): (946.7e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "bwd_da_dh"): (1128.2e6, "gemm_tcgen05.cu", "6096da824b3b", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "bwd_dx"): (937.0e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "route"): (269.4e6, "route.cu", "62d44ad6e9cd", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "route"): (8.5e6, "route.cu", "62d44ad6e9cd", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "e8274775ec74", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "attention"): (6.9e6, "attn_tcgen05.cu", "243f88391599", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "combine"): (25.2e6, "routed.cu", "6b05c28ecb78", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "qkv_proj"): (9.7e6, "gemm_tcgen05.cu", "6096da824b3b", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "route"): (16.8e6, "route.cu", "62d44ad6e9cd", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "e8274775ec74", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "attention"): (6.5e6, "attn_tcgen05.cu", "243f88391599", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "combine"): (25.2e6, "routed.cu", "6b05c28ecb78", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "qkv_proj"): (8.3e6, "gemm_tcgen05.cu", "6096da824b3b", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "route"): (38.8e6, "route.cu", "62d44ad6e9cd", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "mlp_fused"): (59.9e6, "mlp_fused_tcgen05.cu", "e8274775ec74", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "attention"): (39.0e6, "attn_tcgen05.cu", "243f88391599", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "combine"): (123.9e6, "routed.cu", "6b05c28ecb78", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "qkv_proj"): (40.1e6, "gemm_tcgen05.cu", "6096da824b3b", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "wgrad_W2"): (949.6e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "wgrad_W1"): (860.8e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "gemm1_act"): (935.3e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "gemm2"): (947.3e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "bwd_da_dh"): (1120.1e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "bwd_dx"): (931.4e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "route"): (268.9e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "route"): (8.5e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "smha_fused"): (10.3e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "route"): (16.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "attention"): (6.5e6, "attn_tcgen05.cu", "439d84d4e4fe", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "qkv_proj"): (8.3e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "route"): (38.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "mlp_fused"): (60.5e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "smha_fused"): (54.9e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "combine"): (120.6e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
 }
 
 

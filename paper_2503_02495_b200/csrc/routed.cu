@@ -53,7 +53,7 @@ plan_rows_kernel(const int* __restrict__ expert_idx, const int* __restrict__ off
 }
 
 // ---------------------------------------------------------------------------------------------
-// plan: grid B, 128 threads (512 when the backward asks for long per-row arrays), dynamic shared memory 8*k*c bytes.  Everything a sample needs from global memory
+// plan: grid B, 128 threads (512 when the backward asks for per-row arrays), dynamic shared memory 8*k*c bytes.  Everything a sample needs from global memory
 // (its routing arrays, the offsets, the expert choices of the samples before it) is fetched in one round of
 // independent loads; the rest runs out of shared memory.
 // ---------------------------------------------------------------------------------------------
@@ -73,7 +73,7 @@ plan_kernel(const int* __restrict__ expert_idx, const int* __restrict__ patch_id
     // A slot that names no expert is reported and given the last rows that hold a pair, so that whatever goes by pairs stays
     // inside the buffers (its sample's results mean nothing; no other sample reads those rows).
     __shared__ int my_e[32], prow[32], hist[33], offs[34];
-    const int b = blockIdx.x, tid = threadIdx.x, NT = blockDim.x;      // NT: 128 or 512 (long per-row arrays)
+    const int b = blockIdx.x, tid = threadIdx.x, NT = blockDim.x;      // NT: 128 or 512 (per-row arrays)
     const int l_a = c * l_p;
     if (tid < 33) hist[tid] = 0;
     __syncthreads();

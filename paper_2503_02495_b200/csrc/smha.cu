@@ -1,7 +1,8 @@
 // uoe_smha_forward: SMHA forward (Eq. 27-30, 32-36) as plan -> grouped q/k/v projections in one launch,
 // gathering x inside the TMA loads (Eq. 27-30) and rotating q and k where they leave the accumulator (RoPE, Eq. 32) -> attention over each pair's
 // gathered tokens with the expert's output projection in the same kernel (Eq. 33-35; a separate grouped GEMM
-// when an expert has several heads or d > 512) -> weighted combine (Eq. 36).
+// when an expert has several heads or d > 512) -> weighted combine (Eq. 36).  Experts of one head with few tokens per pair take
+// projections, attention and output projection in one kernel instead (smha_can_fuse, smha_fused_tcgen05.cu).
 #include "kernels.cuh"
 
 namespace uoe {
