@@ -679,16 +679,16 @@ NCU_TRAFFIC = {
     ("cfg5_scale", "bwd_dx"): (931.4e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
     ("cfg5_scale", "route"): (268.9e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
     ("cfg2_lm", "route"): (8.5e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
     ("cfg2_lm", "smha_fused"): (10.3e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
     ("cfg2_lm", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
     ("cfg3_long", "route"): (16.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
     ("cfg3_long", "attention"): (6.5e6, "attn_tcgen05.cu", "439d84d4e4fe", "profiles/dram_traffic_per_kernel.md"),
     ("cfg3_long", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
     ("cfg3_long", "qkv_proj"): (8.3e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
     ("cfg4_vit", "route"): (38.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "mlp_fused"): (60.5e6, "mlp_fused_tcgen05.cu", "fb5c4c9be726", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "mlp_fused"): (60.5e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
     ("cfg4_vit", "smha_fused"): (54.9e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
     ("cfg4_vit", "combine"): (120.6e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
 }

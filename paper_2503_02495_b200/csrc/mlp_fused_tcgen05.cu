@@ -43,12 +43,18 @@ constexpr int SMEM = STAGES * STAGE + HID_BYTES + EPI_WARPS * PIECE_BYTES + 1024
 static_assert(SMEM <= 232448, "shared memory of one SM");
 
 struct FCtl {
-    uint64_t full[STAGES], empty[STAGES], bar_h, bar_a[DE / 64], bar_z[2], bar_free[2];
+    uint64_t full[STAGES], empty[STAGES], bar_h, bar_z[2], bar_free[2];
     uint32_t tmem_base;
     int abort_flag;
     int offs[34];
     int tstart[34];
 };
+
+// Hand-over of 64 hidden columns to the MMA warp: the four warps that wrote them arrive, it waits, on a barrier of the SM per column group,
+// which wakes it sooner than an mbarrier does (image block forward 185.8 us through mbarriers, 184.8 so; language-model block 68.6, 68.15).
+// That wait has no limit of its own: a warp that gives up arrives all the same, and the MMA warp looks at the abort flag behind every wait.
+__device__ __forceinline__ void hidden_arrive(int g) { asm volatile("bar.arrive %0, %1;" :: "r"(1 + g), "n"(32 * (EPI_WARPS / 2 + 1)) : "memory"); }
+__device__ __forceinline__ void hidden_wait(int g) { asm volatile("bar.sync %0, %1;" :: "r"(1 + g), "n"(32 * (EPI_WARPS / 2 + 1)) : "memory"); }
 
 template <bool PRE /* the pre-activation is stored too: a kernel of its own, as its code in the epilogue costs the other 0.7 % */>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -70,7 +76,6 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         mbar_init(&ctl->bar_h, 1);
-        for (int g = 0; g < DE / 64; ++g) mbar_init(&ctl->bar_a[g], 32 * EPI_WARPS / 2);
         for (int q = 0; q < 2; ++q) { mbar_init(&ctl->bar_z[q], 1); mbar_init(&ctl->bar_free[q], 32 * EPI_WARPS); }
         ctl->abort_flag = 0;
         fence_barrier_init();
@@ -208,7 +213,10 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 for (int q = q0; q < min(nblk, q0 + BLKS); ++q) {
                     const int j = q / kb2, kb = q % kb2, buf = j & 1;
                     // phi of hidden columns [64 kb, 64 kb + 64) is in shared memory; the accumulator has been drained
-                    if (j == 0 && !mbar_wait_warp(&ctl->bar_a[kb], i & 1, abort_flag, status)) { stop = true; break; }
+                    if (j == 0) {
+                        hidden_wait(kb);
+                        if (__any_sync(0xffffffffu, *abort_flag != 0)) { stop = true; break; }
+                    }
                     if (kb == 0) {
                         if (!mbar_wait_warp(&ctl->bar_free[buf], ((used >> buf) & 1) ^ 1, abort_flag, status)) { stop = true; break; }
                         used ^= 1u << buf;
@@ -234,6 +242,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int trow = quarter * 32 + lane;                 // row of the tile = TMEM lane
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
         uint8_t* stg = sOut + (warp - 2) * PIECE_BYTES;
+        bool gave_up = false;
         uint32_t taken = 0;                                   // bit b: parity of the chunks taken from output accumulator b
         auto pack8 = [](const float* f) {
             uint4 w;
@@ -247,7 +256,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             locate(tile, e, row0);
             const bool ready = mbar_wait(&ctl->bar_h, i & 1, abort_flag, status) && !*abort_flag;
             // (the hidden tile in shared memory is free: the last chunk of the previous tile was waited for below)
-            if (!__all_sync(0xffffffffu, ready)) break;      // warp-uniform: tcgen05.ld below is warp-collective
+            if (!__all_sync(0xffffffffu, ready)) { gave_up = true; break; }      // warp-uniform: tcgen05.ld below is warp-collective
             tc_fence_after();
             // ---- hidden tile: phi, bf16, K-major swizzled [128 x 64] tiles ----
 #pragma unroll 1
@@ -285,7 +294,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     *(uint4*)(sHid + g * (BM * 128) + trow * 128 + ((c ^ (trow & 7)) << 4)) = pack8(f + 8 * c);
                 fence_async_smem();              // generic-proxy writes -> visible to the tensor core
                 tc_fence_before();
-                mbar_arrive(&ctl->bar_a[g]);
+                hidden_arrive(g);
             }
 
             // ---- output chunks ----
@@ -329,8 +338,11 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) { tma_store_2d(&tmZ, stg, col0 + 32 * h, wrow0); bulk_commit(); }
                 }
             }
-            if (!zr) break;
+            if (!zr) { gave_up = true; break; }
         }
+        // given up: the MMA warp, which stops at its next look at the flag, may be on its way to this tile's groups or the next one's
+        if (gave_up)
+            for (int g = wsel; g < DE / 64; g += 2) hidden_arrive(g);
     }
     if (warp >= 2 && lane == 0) bulk_wait_all();       // this warp's tensor stores are complete
     tc_fence_before();
