@@ -170,16 +170,12 @@ __device__ __forceinline__ void attn_bwd_body(const BwdMaps& m, const BwdMaps& m
                 acc[2 * i + 1] = a1 * cs - a0 * sn;
             }
         }
+        // whole sectors, two stores (in 16-byte stores, with the plan a microsecond longer: image block, training step 665.9 us, so
+        // 656.7, wide block 499.7 and 494.7, language-model block 241.9 and 238.9)
         __nv_bfloat16* o = out + (size_t)(row_base + orow) * a.ld_out + col_h + hsel * 32;
-        // whole sectors, two stores (rows and columns are multiples of 64 bytes; in 16-byte stores, with the plan a microsecond longer:
-        // image block, training step 665.9 us, so 656.7, wide block 499.7 and 494.7, language-model block 241.9 and 238.9)
+        const bool whole = sector_aligned(o);
 #pragma unroll
-        for (int ch = 0; ch < DH / 32; ++ch) {
-            uint32_t w[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w[q] = pack_bf16x2(acc[ch * 16 + 2 * q], acc[ch * 16 + 2 * q + 1]);
-            st_sector(o + 16 * ch, make_uint4(w[0], w[1], w[2], w[3]), make_uint4(w[4], w[5], w[6], w[7]));
-        }
+        for (int ch = 0; ch < DH / 32; ++ch) st_sector(o + 16 * ch, pack16<__nv_bfloat16>(acc + 16 * ch), pack16<__nv_bfloat16>(acc + 16 * ch + 8), whole);
     };
     auto stat = [&](const float* src, int q) { return q < a.l_a ? src[(size_t)(row_base + q) * a.heads + head] : 0.f; };
     constexpr float kLog2e = 1.4426950408889634f;

@@ -34,20 +34,15 @@ __device__ __forceinline__ void store_z_piece(const float* zf, uint8_t* stg, con
     }
 }
 
-// The same piece straight from registers: 32 bytes, a whole sector, per thread and store.  Where two CTAs share an SM its copy
+// The same piece straight from registers: a row's 128 bytes per thread, in whole sectors.  Where two CTAs share an SM its copy
 // engine is busy with the loads of the one while the other writes z, and tensor stores queue behind them (image block forward
 // 200.5 us with tensor stores, 192.3 so); with one CTA per SM tensor stores are the better ones (one sequence 55.4 against 56.4).
 __device__ __forceinline__ void store_z_direct(const float* zf, __nv_bfloat16* z, int d, int col, int row, int rows_left, int lane) {
     if (lane >= rows_left) return;
-    __nv_bfloat16* o = z + (size_t)(row + lane) * d + col;      // (d and col are multiples of 64, z of the workspace's 1024 bytes)
+    __nv_bfloat16* o = z + (size_t)(row + lane) * d + col;
+    const bool whole = sector_aligned(o);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint32_t w[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = pack_bf16x2(zf[16 * q + 2 * i], zf[16 * q + 2 * i + 1]);
-        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                     :: "l"(o + 16 * q), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-    }
+    for (int q = 0; q < 4; ++q) st_sector(o + 16 * q, pack16<__nv_bfloat16>(zf + 16 * q), pack16<__nv_bfloat16>(zf + 16 * q + 8), whole);
 }
 
 }  // namespace tc

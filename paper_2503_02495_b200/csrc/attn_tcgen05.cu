@@ -419,12 +419,13 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (!FUSE_O) {
                 if (qrow < a.l_a) {
                     __nv_bfloat16* out = a.O + (size_t)(row_base + qrow) * a.d_g + head * DH;
+                    const bool whole = sector_aligned(out);
 #pragma unroll
-                    for (int ch = 0; ch < DH / 16; ++ch) {           // whole sectors
-                        uint32_t w[8];
+                    for (int ch = 0; ch < DH / 16; ++ch) {
+                        float f[16];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) w[q] = pack_bf16x2(o_acc[ch * 16 + 2 * q] * inv, o_acc[ch * 16 + 2 * q + 1] * inv);
-                        st_sector(out + 16 * ch, make_uint4(w[0], w[1], w[2], w[3]), make_uint4(w[4], w[5], w[6], w[7]));
+                        for (int q = 0; q < 16; ++q) f[q] = o_acc[ch * 16 + q] * inv;
+                        st_sector(out + 16 * ch, pack16<__nv_bfloat16>(f), pack16<__nv_bfloat16>(f + 8), whole);
                     }
                 }
             } else {

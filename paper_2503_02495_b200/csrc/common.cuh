@@ -294,10 +294,17 @@ __device__ __forceinline__ void st_stream16(void* p, const uint4& v) {
                  :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// 32 bytes, one sector of L2, in one store (p a multiple of 32 bytes)
-__device__ __forceinline__ void st_sector(void* p, const uint4& a, const uint4& b) {
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 :: "l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+// 32 bytes, one sector of L2: one store where `whole` says that p is a multiple of 32 bytes, else two of 16.  Buffers (the
+// workspace, and with it every buffer carved from it, among them) are multiples of 16 bytes and no more is asked of them.
+__device__ __forceinline__ bool sector_aligned(const void* p) { return ((uintptr_t)p & 31) == 0; }
+__device__ __forceinline__ void st_sector(void* p, const uint4& a, const uint4& b, bool whole) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.u32 q, %9, 0;\n\t"
+        "@q st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n\t"
+        "@!q st.global.v4.b32 [%0], {%1,%2,%3,%4};\n\t"
+        "@!q st.global.v4.b32 [%0+16], {%5,%6,%7,%8};\n\t}"
+        :: "l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "r"((uint32_t)whole) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -280,13 +280,9 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 }
                 if constexpr (PRE) {
                     __nv_bfloat16* dst = pre + (size_t)(row0 + trow) * DE + g * 64;
-                    if (((uintptr_t)pre & 31) == 0) {        // (the caller's buffer) whole sectors
+                    const bool whole = sector_aligned(dst);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) st_sector(dst + 16 * c, pack8(f + 16 * c), pack8(f + 16 * c + 8));
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) ((uint4*)dst)[c] = pack8(f + 8 * c);
-                    }
+                    for (int c = 0; c < 4; ++c) st_sector(dst + 16 * c, pack8(f + 16 * c), pack8(f + 16 * c + 8), whole);
                 }
                 act_apply_n<64>(f, act);
 #pragma unroll
