@@ -18,6 +18,7 @@
 // of weights at d = 384, 144 KB in flight).  The chunks let the write-out of a tile run under its own GEMM2 and the next
 // GEMM1, and three W2 blocks to a stage keep the whole ring in flight; with the output in two halves drained behind the
 // last MMA the launch took 73 us, not 62, at d = 384 with five tiles per SM, and 22.9, not 21.6, at d = 512 with one.
+#include "hand_over.h"
 #include "kernels.cuh"
 #include "tc.cuh"
 #include "tmap.cuh"
@@ -50,11 +51,12 @@ struct FCtl {
     int tstart[34];
 };
 
-// Hand-over of 64 hidden columns to the MMA warp: the four warps that wrote them arrive, it waits, on a barrier of the SM per column group,
-// which wakes it sooner than an mbarrier does (image block forward 185.8 us through mbarriers, 184.8 so; language-model block 68.6, 68.15).
-// That wait has no limit of its own: a warp that gives up arrives all the same, and the MMA warp looks at the abort flag behind every wait.
-__device__ __forceinline__ void hidden_arrive(int g) { asm volatile("bar.arrive %0, %1;" :: "r"(1 + g), "n"(32 * (EPI_WARPS / 2 + 1)) : "memory"); }
-__device__ __forceinline__ void hidden_wait(int g) { asm volatile("bar.sync %0, %1;" :: "r"(1 + g), "n"(32 * (EPI_WARPS / 2 + 1)) : "memory"); }
+// Hand-over p (the CTA's p-th tile) of 64 hidden columns, group g, to the MMA warp, by the rule of hand_over.h: the four warps that wrote
+// them arrive, it waits, on two barriers of the SM per column group, which wake it sooner than an mbarrier does (image block forward
+// 185.8 us through mbarriers, 184.8 so; language-model block 68.6, 68.15).
+__device__ __forceinline__ int hidden_barrier(int p, int g) { return 1 + g + (DE / 64) * hand_over_barrier(p); }
+__device__ __forceinline__ void hidden_wait(int p, int g) { hand_over_take<32 * (EPI_WARPS / 2 + 1)>(hidden_barrier(p, g)); }
+__device__ __forceinline__ void hidden_arrive(int p, int g, bool ok) { hand_over_write<32 * (EPI_WARPS / 2 + 1)>(hidden_barrier(p, g), !ok); }
 
 template <bool PRE /* the pre-activation is stored too: a kernel of its own, as its code in the epilogue costs the other 0.7 % */>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -191,9 +193,10 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         bool stop = false;
         int i = 0;                                   // tiles done by this CTA
         uint32_t used = 0;                           // bit b: parity of the chunks put into output accumulator b so far
-        for (int tile = blockIdx.x; tile < total_tiles && !stop; tile += gridDim.x, ++i) {
+        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++i) {
+            int handed = 0;                          // column groups of this tile's hand-over
             // (the hidden accumulator is free: this thread has waited for phi of the previous tile's last columns)
-            for (int kb = 0; kb < kb1; ++kb) {
+            for (int kb = 0; kb < kb1 && !stop; ++kb) {
                 if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(smem + stage * STAGE), sb = sa + A_BYTES;
@@ -204,8 +207,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 mma_commit(el, &ctl->empty[stage]);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
-            if (stop) break;
-            mma_commit(el, &ctl->bar_h);
+            if (!stop) mma_commit(el, &ctl->bar_h);
             const uint32_t ha = smem_u32(sHid);
             for (int q0 = 0; q0 < nblk && !stop; q0 += BLKS) {
                 if (!mbar_wait_warp(&ctl->full[stage], phase, abort_flag, status)) { stop = true; break; }
@@ -214,7 +216,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     const int j = q / kb2, kb = q % kb2, buf = j & 1;
                     // phi of hidden columns [64 kb, 64 kb + 64) is in shared memory; the accumulator has been drained
                     if (j == 0) {
-                        hidden_wait(kb);
+                        hidden_wait(i, kb);
+                        handed = kb + 1;
                         if (__any_sync(0xffffffffu, *abort_flag != 0)) { stop = true; break; }
                     }
                     if (kb == 0) {
@@ -234,6 +237,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 mma_commit(el, &ctl->empty[stage]);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
+            for (; handed < kb2; ++handed) hidden_wait(i, handed);          // (only after a wait that ran out)
         }
     } else {
         // ---------------- epilogue: warps w and w + 4 drain TMEM lane quarter w % 4, alternate 64-column groups ----------------
@@ -254,9 +258,13 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++i) {
             int e, row0;
             locate(tile, e, row0);
-            const bool ready = mbar_wait(&ctl->bar_h, i & 1, abort_flag, status) && !*abort_flag;
+            const bool ready = !gave_up && mbar_wait(&ctl->bar_h, i & 1, abort_flag, status) && !*abort_flag;
             // (the hidden tile in shared memory is free: the last chunk of the previous tile was waited for below)
-            if (!__all_sync(0xffffffffu, ready)) { gave_up = true; break; }      // warp-uniform: tcgen05.ld below is warp-collective
+            if (!__all_sync(0xffffffffu, ready)) {           // warp-uniform: tcgen05.ld below is warp-collective
+                gave_up = true;
+                for (int g = wsel; g < DE / 64; g += 2) hidden_arrive(i, g, false);
+                continue;
+            }
             tc_fence_after();
             // ---- hidden tile: phi, bf16, K-major swizzled [128 x 64] tiles ----
 #pragma unroll 1
@@ -290,7 +298,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     *(uint4*)(sHid + g * (BM * 128) + trow * 128 + ((c ^ (trow & 7)) << 4)) = pack8(f + 8 * c);
                 fence_async_smem();              // generic-proxy writes -> visible to the tensor core
                 tc_fence_before();
-                hidden_arrive(g);
+                hidden_arrive(i, g, true);
             }
 
             // ---- output chunks ----
@@ -334,11 +342,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) { tma_store_2d(&tmZ, stg, col0 + 32 * h, wrow0); bulk_commit(); }
                 }
             }
-            if (!zr) { gave_up = true; break; }
+            gave_up = !zr;
         }
-        // given up: the MMA warp, which stops at its next look at the flag, may be on its way to this tile's groups or the next one's
-        if (gave_up)
-            for (int g = wsel; g < DE / 64; g += 2) hidden_arrive(g);
     }
     if (warp >= 2 && lane == 0) bulk_wait_all();       // this warp's tensor stores are complete
     tc_fence_before();

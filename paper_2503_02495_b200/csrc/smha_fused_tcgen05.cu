@@ -16,6 +16,7 @@
 //
 // With `q` set the kernel is the backward's recomputation instead: q, k, v, o and the log-sum-exp are written, z is not.
 #include "attn_out.cuh"
+#include "hand_over.h"
 #include "kernels.cuh"
 #include "tc.cuh"
 #include "tmap.cuh"
@@ -70,11 +71,11 @@ struct FuArgs {
     int* status;
 };
 
-// Hand-over from the softmax warps to the MMA warp: they arrive, it waits, on a barrier of the SM, which wakes it sooner than an mbarrier
-// does (image block forward 190.3 us through mbarriers, 187.6 so; language-model block 69.5 and 69.0).  Nobody skips one: a warp whose wait ran out arrives all the same.
-constexpr int kHandOver = 6;
-__device__ __forceinline__ void hand_over_arrive() { asm volatile("bar.arrive %0, %1;" :: "n"(kHandOver), "n"(32 * (kSoftWarps + 1)) : "memory"); }
-__device__ __forceinline__ void hand_over_wait() { asm volatile("bar.sync %0, %1;" :: "n"(kHandOver), "n"(32 * (kSoftWarps + 1)) : "memory"); }
+// Hand-over p from the softmax warps to the MMA warp, by the rule of hand_over.h: they arrive, it waits, on a barrier of the SM, which
+// wakes it sooner than an mbarrier does (image block forward 190.3 us through mbarriers, 187.6 so; language-model block 69.5 and 69.0).
+constexpr int kHandOver = 6;              // and 7
+__device__ __forceinline__ void hand_over_wait(int p) { hand_over_take<32 * (kSoftWarps + 1)>(kHandOver + hand_over_barrier(p)); }
+__device__ __forceinline__ void hand_over_arrive(int p, bool ok) { hand_over_write<32 * (kSoftWarps + 1)>(kHandOver + hand_over_barrier(p), !ok); }
 __device__ __forceinline__ void bar_named(int id, int threads) { asm volatile("bar.sync %0, %1;" :: "r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -238,7 +239,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         }
         if (ok) mma_commit(el, &ctl->qkv_full);
         if constexpr (MULTI) cluster_arrive();
-        hand_over_wait();                                // q, k, v are in shared memory
+        hand_over_wait(0);                               // q, k, v are in shared memory
         const uint32_t qa = smem_u32(unit(0)), pa = smem_u32(unit(Cf::P));
         // place of the i-th tile's k and v: own, or stage q & 1 of the others
         auto stage_of = [&](int i) { return own ? i - 1 : i; };
@@ -255,7 +256,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         };
         if (n_kv > 0) ok = ok && issue_s(0);
         for (int i = 0; i < n_kv; ++i) {
-            hand_over_wait();                            // P is
+            hand_over_wait(MULTI ? 1 + i : 1);           // P is
             ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
             if (!ok) continue;
             tc_fence_after();
@@ -269,7 +270,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             if (MULTI) mma_commit(el, q >= 0 ? &ctl->kv_empty[q & 1] : &ctl->own_free);
             if (i + 1 < n_kv) ok = issue_s(i + 1);       // (into the other accumulator: it runs under the O update)
         }
-        if (n_kv > 0) hand_over_wait();                  // o is
+        if (n_kv > 0) hand_over_wait(MULTI ? 1 + n_kv : 2);      // o is
         ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
         for (int j = 0; j < n_z && ok; ++j) {
             const int st = j & 1, wb = j % Cf::NW;
@@ -285,7 +286,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
         }
     } else {
         // =========================== softmax warps ===========================
-        // (a wait that runs out leaves ok false: the work is skipped, the CTA's and the cluster's barriers are not)
+        // (a wait that runs out leaves ok false: the work is skipped, the hand-overs and the barriers of CTA and cluster are not)
         const int quarter = warp & 3, hsel = warp >> 2;  // TMEM lane quarter; half of the columns
         const int trow = quarter * 32 + lane, qrow = q0 + trow, sw = trow & 7;
         const uint32_t t_lane = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -358,7 +359,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
             tc_fence_before();
             if (MULTI) mbar_arrive(&ctl->qkv_ready);
         }
-        hand_over_arrive();
+        hand_over_arrive(0, ok);
         if constexpr (MULTI) cluster_arrive();
         if (keep) {
             bar_named(2 + quarter, 64);
@@ -418,7 +419,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 fence_async_smem();
                 tc_fence_before();
             }
-            hand_over_arrive();
+            hand_over_arrive(MULTI ? 1 + i : 1, ok);
             ok = ok && __all_sync(0xffffffffu, wait(&ctl->o_full, i & 1)) != 0;
             if (ok) {
                 tc_fence_after();
@@ -444,7 +445,7 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 fence_async_smem();
                 tc_fence_before();
             }
-            hand_over_arrive();
+            hand_over_arrive(MULTI ? 1 + n_kv : 2, ok);
             if (keep) {
                 bar_named(2 + quarter, 64);
                 if (ok) copy_out(unit(Cf::P), a.o);

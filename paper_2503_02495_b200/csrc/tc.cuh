@@ -1,6 +1,7 @@
 // PTX wrappers for the Blackwell (sm_100a) data path: mbarrier, TMA tensor loads, tcgen05 MMA with
-// TMEM accumulators.  Every wait is bounded: when a wait runs out it raises the CTA's abort flag and
-// records UOE_ERR_TIMEOUT in the device status word, and the kernel winds down without trapping.
+// TMEM accumulators.  Every wait for an mbarrier is bounded: when a wait runs out it raises the CTA's abort flag and
+// records UOE_ERR_TIMEOUT in the device status word, and the kernel winds down without trapping.  Barriers of the SM and of a cluster
+// have no limit of their own: every warp takes part in every one of them, also after a wait that ran out (hand_over.h).
 #pragma once
 #include "common.cuh"
 
