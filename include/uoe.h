@@ -219,7 +219,8 @@ uoe_status uoe_mlp_backward(const uoe_problem* prob, const void* x, const void* 
  * keys and, with UOE_FLAG_CAUSAL, key position > query position in gathered order is masked.  The
  * projected result is added back as in uoe_mlp_forward:  y = x + sum gate * (o Wo[i]).
  * lse, if not NULL, receives the log-sum-exp of every (routed row, head of the expert):
- * [uoe_max_routed_rows, H/n] float32.  All pointers except prob are device pointers.
+ * [uoe_max_routed_rows, H/n] float32; -infinity on the rows of a pair whose slots are all unused.  Padding rows between
+ * the experts' regions are not written.  All pointers except prob are device pointers.
  */
 uoe_status uoe_smha_forward(const uoe_problem* prob, const void* x, const void* Wq, const void* Wk,
                             const void* Wv, const void* Wo,

@@ -312,7 +312,10 @@ attn_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (lane == 0) mbar_arrive(&pc->q_empty);
             const int q0 = qt * TQ, qrow = q0 + trow;
             const int n_kv = kv_tiles(q0, n_valid);
-            if (n_kv == 0) continue;
+            if (n_kv == 0) {                                   // a pair without a key
+                if (a.lse && qrow < a.l_a) a.lse[(size_t)(row_base + qrow) * a.heads + head] = -INFINITY;
+                continue;
+            }
             const int kv_lim = min(n_valid, a.l_a);
 
             float o_acc[DH];

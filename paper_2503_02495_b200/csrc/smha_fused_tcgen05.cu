@@ -450,6 +450,8 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
                 bar_named(2 + quarter, 64);
                 if (ok) copy_out(unit(Cf::P), a.o);
             }
+        } else if (a.lse && named && hsel == 0 && qrow < a.l_a) {
+            a.lse[row_base + qrow] = -INFINITY;          // a pair without a key
         }
         // ---- z = o W^o_i (Eq. 35), a chunk's 64-column groups dealt to the two warps of a lane quarter ----
         [[maybe_unused]] uint8_t* stg = MULTI ? unit(11 + hsel) + quarter * 4096 : nullptr;

@@ -114,3 +114,70 @@ def test_pairs_without_a_patch(B, heads):
     ref = orc.smha_backward(layer.x.f64, *[q.f64 for q in layer.ws], layer.Wr.f64, ro, dy.f64, w.d_h, w.causal, False)
     for g, r in zip(layer.backward(dy), ref):
         assert rel_inf(to_f64(g), r) <= 2e-2
+
+
+# one routed row per (row, head): every kernel that produces lse -- one tile per pair and clusters in one kernel with the
+# projections, a CTA per unit and two pipelines per CTA, each with the output projection inside and without
+LSE = {
+    "one_tile": dict(B=12, L=48, L_valid=45, m=3, c=2, n=2, H=2),
+    "cluster": dict(B=4, L=512, L_valid=500, m=16, c=8, n=2, H=2, causal=True),
+    "cta_per_unit_out": dict(B=6, L=320, L_valid=311, m=10, c=5, n=2, H=2),
+    "cta_per_unit": dict(B=12, L=48, L_valid=45, m=3, c=2, n=2, H=4),
+    "pipelines_out": dict(B=120, L=320, L_valid=311, m=10, c=5, n=2, H=2),
+    "pipelines": dict(B=240, L=48, L_valid=45, m=3, c=2, n=2, H=4),
+}
+
+
+@pytest.mark.parametrize("name", list(LSE))
+def test_log_sum_exp_of_every_routed_row(name):
+    """Every third pair has only unused slots (-inf), every fifth one an unused last slot.  Scores of a few units, q and k rounded
+    to bfloat16 (2^-9 each): 2e-2 of the largest log-sum-exp, as for the other bfloat16 results."""
+    w = _att(**LSE[name])
+    layer = Layer(w, "att")
+    patch = layer.r.patch_idx.cpu().numpy().copy()
+    flat = patch.reshape(w.B * w.k, w.c)
+    flat[::5, -1] = -1
+    flat[::3] = -1
+    ro = layer.use(layer.r.expert_idx.cpu().numpy(), patch)
+    heads = w.d_g // w.d_h
+    lse = torch.full((layer.uoe.uoe_max_routed_rows(layer.prob), heads), 77.0, device="cuda")
+    y = layer.uoe.uoe_smha_forward(layer.prob, layer.xd, *layer.wd, layer.r, lse=lse)
+    ref_y, ref = orc.smha_forward(layer.x.f64, *[q.f64 for q in layer.ws], ro, w.d_h, w.causal, residual=False, return_lse=True)
+    assert rel_inf(to_f64(y), ref_y) <= 2e-2
+    got, top = to_f64(lse), max(np.abs(v).max() for v in ref.values())
+    l_a = w.c * (w.L // w.m)
+    for b in range(w.B):
+        for s in range(w.k):
+            row = orc.buffer_row(ro, b, s)
+            for hd in range(heads):
+                have = got[row:row + l_a, hd]
+                if (b, s, hd) not in ref:
+                    assert np.all(have == -np.inf)
+                else:
+                    want = ref[b, s, hd]
+                    assert np.abs(have[:len(want)] - want).max() <= 2e-2 * top
+
+
+@pytest.mark.parametrize("causal", [False, True])
+def test_clusters_with_unused_slots_and_a_pair_without_a_patch(causal):
+    """Pairs of two 128-row tiles in one kernel: fewer keys than tiles, none at all, an expert out of range."""
+    w = _att(B=5, L=512, L_valid=500, m=16, c=8, n=3, k=2, H=3, causal=causal)
+    layer = Layer(w, "att", d_rope=32)
+    patch = layer.r.patch_idx.cpu().numpy().copy()
+    flat = patch.reshape(w.B * w.k, w.c)
+    flat[1, 1:] = -1
+    flat[4, 4:] = -1
+    flat[7] = -1
+    ro = layer.use(layer.r.expert_idx.cpu().numpy(), patch)
+    good = layer.forward()
+    assert rel_inf(to_f64(good), layer.reference(ro)) <= 2e-2
+    dy = gen.make_dy(w)
+    ref = orc.smha_backward(layer.x.f64, *[q.f64 for q in layer.ws], layer.Wr.f64, ro, dy.f64, w.d_h, w.causal, False, d_rope=32)
+    for g, r in zip(layer.backward(dy), ref):
+        assert rel_inf(to_f64(g), r) <= 2e-2
+    layer.r.expert_idx[-1, 0] = 1 << 20
+    y = torch.zeros_like(good)
+    with pytest.raises(layer.uoe.UoeError) as ei:
+        layer.uoe.uoe_smha_forward(layer.prob, layer.xd, *layer.wd, layer.r, y=y)
+    assert ei.value.status == 6
+    assert torch.equal(y[:-1], good[:-1])
