@@ -27,6 +27,7 @@
 // The A operand is either a routed buffer (2-D tensor map) or gathered on the fly from x, one TMA box per
 // source patch (Eq. 18 inside the GEMM).
 #include "kernels.cuh"
+#include "launch_rules.h"
 #include "tc.cuh"
 #include "tmap.cuh"
 
@@ -714,8 +715,8 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
         return short_k ? launch_one<192, false, kForward, 1, false, false, 64>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
     }
     // Two heads per expert: q, k, v as one 384-column tile (wide block above: forward 162.4 us with three 128-column tiles, 152.0 so,
-    // training step 527 and 504), once the row tiles alone give the SMs more than one 128-column tile each
-    if (g.nmat == 3 && g.N == 128 && !g.b_kmajor && !g.pre && !short_k && 3 * (g.rows_max / BM) > sm_count())
+    // training step 527 and 504)
+    if (g.nmat == 3 && g.N == 128 && !g.b_kmajor && !g.pre && !short_k && qkv_as_one_tile(g.rows_max, g.n, sm_count()))
         return rope ? launch_one<384, false, kForward, 1, false, true>(g, status, s) : launch_one<384, false, kForward, 1>(g, status, s);
     if (rope) return dispatch<false, kForward, true>(g, status, s);
     if (short_k) return g.b_kmajor ? dispatch<true, kForward, false, 64>(g, status, s) : dispatch<false, kForward, false, 64>(g, status, s);

@@ -43,3 +43,13 @@ def test_hand_over_between_warps_ends_in_every_order(tmp_path):
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     assert r.stdout.strip().endswith("ok")
+
+
+def test_rules_of_launches(tmp_path):
+    exe = str(tmp_path / "launch_rules_check")
+    src = os.path.join(ROOT, "tests", "host", "launch_rules_check.cpp")
+    inc = os.path.join(ROOT, "paper_2503_02495_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", inc, src, "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout.strip() == "ok"
