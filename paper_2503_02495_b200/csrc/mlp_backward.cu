@@ -12,6 +12,7 @@
 // feeds dW_r (through the pooled token sums) and one more term of dx.
 #include "balance.cuh"
 #include "kernels.cuh"
+#include "launch_rules.h"
 #include "tc.cuh"
 #include "tmap.cuh"
 
@@ -406,8 +407,10 @@ BwdWs bwd_ws(const Dims& D) {
 uoe_status launch_router_backward(const Dims& D, const void* x, const void* W_r, const int* expert_idx,
                                   const int* patch_idx, const float* p_samp, const float* p_patch, const PlanPtrs& P,
                                   const float* dgp, int nt, const RouterBwdScratch& rs, float* dW_r, DwrSum* sum,
-                                  int* status, cudaStream_t stream, const WReduce& reduce) {
+                                  int* status, cudaStream_t stream, const WReduce& cut) {
     if (!D.bf16) return UOE_ERR_UNSUPPORTED;
+    WReduce reduce = cut;
+    if (reduce.blocks > 0) reduce.use_threads(router_grad_threads(reduce.by_cut != 0, D.B, (long long)D.k * D.c));
     const size_t smem = ((size_t)2 * D.n * D.m + (size_t)D.k * D.c) * sizeof(float);
     if ((size_t)2 * D.n * D.m * sizeof(float) > 40 * 1024) return UOE_ERR_UNSUPPORTED;
     static SpreadOnce once;

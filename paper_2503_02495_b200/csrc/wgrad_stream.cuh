@@ -23,12 +23,12 @@ struct WReduce {
     int part_floats = 0;      // of a part of a tile in the scratch
     int by_cut = 0;           // blocks are counted by piece boundary (more tiles than pieces), else by tile
     int threads = 512;        // of a block
+    int halves = 0, places = 0;      // half pieces of the widest tile; boundaries or tiles that blocks are counted by
+    // the blocks for `t` threads each, a warp per half piece
+    void use_threads(int t) { threads = t; per = (halves + t / 32 - 1) / (t / 32); blocks = places * per; }
 };
 
-// Threads of a block: 512 where the blocks are counted by cut, which is where there are many (every block builds the line again: wide
-// block, training step 504 us, with 256 threads and twice the blocks 507), else 256, so that the blocks and the samples' CTAs beside
-// them are resident at once (language-model block 250.8 -> 248.2, image block 671 -> 670).
-constexpr int kReduceThreads = 512, kReduceThreadsFew = 256;
+constexpr int kReduceThreads = 512;      // of a block, at most
 
 #ifdef __CUDACC__
 struct WSched {

@@ -19,6 +19,7 @@
 //   warp 1      MMA issuer: tcgen05.mma 128 x BN x 16, two accumulator sets (the write-out of a tile runs under the next)
 //   warps 2-9   write-out, two per TMEM lane quarter, 32-column chunks in turn
 #include "kernels.cuh"
+#include "launch_rules.h"
 #include "tc.cuh"
 #include "tmap.cuh"
 #include "wgrad_stream.cuh"
@@ -337,9 +338,9 @@ uoe_status launch_wgrad_stream(const WStreamProblem* probs, int nprob, const int
     int tiles = 0;
     for (int i = 0; i < nprob; ++i) tiles += n * a.prob[i].m_tiles * a.prob[i].n_tiles;
     r.by_cut = tiles > a.pieces - 1 ? 1 : 0;
-    r.threads = r.by_cut ? kReduceThreads : kReduceThreadsFew;
-    r.per = (widest / 32 * 8 + r.threads / 32 - 1) / (r.threads / 32);
-    r.blocks = (r.by_cut ? a.pieces - 1 : tiles) * r.per;
+    r.halves = widest / 32 * 8;
+    r.places = r.by_cut ? a.pieces - 1 : tiles;
+    r.use_threads(router_grad_threads(r.by_cut != 0, 0, 0));
     *reduce = r;
     return UOE_OK;
 }

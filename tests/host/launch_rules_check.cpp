@@ -26,6 +26,9 @@ int main() {
     const long long pad = 8 * (kRowTile - 1);
     auto bound = [&](long long rows) { return (rows + pad) / kRowTile * kRowTile; };
     if (qkv_as_one_tile(bound(49 * 128), 8, 148) || !qkv_as_one_tile(bound(50 * 128), 8, 148)) return 4;
+    // a sample of many slabs gets all warps, whatever the number of weight-gradient tiles
+    if (router_grad_threads(false, 4, 1280) != 512 || router_grad_threads(false, 300, 1280) != 512 || router_grad_threads(false, 8, 240) != 512) return 5;
+    if (router_grad_threads(false, 24, 240) != 256 || router_grad_threads(false, 8, 32) != 256 || router_grad_threads(true, 8, 32) != 512) return 6;
     std::printf("ok\n");
     return 0;
 }
