@@ -526,6 +526,8 @@ uoe_status launch_gather(const Dims& D, const void* src, const int* patch_idx, c
 uoe_status launch_combine(const Dims& D, const void* x, const void* z, const PlanPtrs& P, bool residual,
                           bool use_gate, void* y, cudaStream_t s, const float* rvec, const DwrSum& sum) {
     const int vpr = (int)((long long)D.d * D.esize / 16);
+    const long long chunks = ((long long)D.l_p * vpr + 32 * kCombineVecs - 1) / (32 * kCombineVecs), units = (long long)D.B * D.m * chunks;
+    if ((long long)D.l_p * vpr > (1ll << 31) - 16384 || units > (1ll << 31) - 16384) return UOE_ERR_UNSUPPORTED;      // the kernel counts both in 32 bits
     CombineArgs a;
     a.x = x; a.z = z; a.y = y; a.inv_row = P.inv_row; a.inv_gate = P.inv_gate;
     a.pair_row = P.inv_relative ? P.pair_row : nullptr;
@@ -536,17 +538,24 @@ uoe_status launch_combine(const Dims& D, const void* x, const void* z, const Pla
     a.sum = sum;
     ProfScope ps("combine", s);
     const bool bwd = rvec || sum.total > 0;
-    a.chunks = (D.l_p * vpr + 32 * kCombineVecs - 1) / (32 * kCombineVecs);
-    a.units = D.B * D.m * a.chunks;
+    a.chunks = (int)chunks;
+    a.units = (int)units;
     // Four CTAs per SM, all that fit (up to eight) only for a forward with several units per warp even then: the room is of
     // use to the next kernel, whose CTAs start under this one (language-model training step 257 us with four, 262 with eight;
     // wide block forward 167.5 and 165.4)
     const int per_sm = !bwd && a.units >= 10 * (kThreads / 32) * sm_count() ? 8 : 4;
     const int want = (a.units + kThreads / 32 - 1) / (kThreads / 32), cap = per_sm * sm_count();
     const dim3 grid(want < cap ? want : cap);
-    if (!D.bf16) launch_k(combine_kernel<float, false>, grid, dim3(kThreads), 0, s, a);
-    else if (bwd) launch_k(combine_kernel<__nv_bfloat16, true>, grid, dim3(kThreads), 0, s, a);
-    else launch_k(combine_kernel<__nv_bfloat16, false>, grid, dim3(kThreads), 0, s, a);
+    // A unit per warp: CTAs kept apart (block forwards, without and with: 304 CTAs 76.8 and 69.5 us, 112 CTAs 76.7 and 72.4, 498 CTAs 65.2
+    // and 61.8).  Not where warps go on to further units, there the room is the next kernel's (training steps, 592 CTAs: 172.4 and 173.9,
+    // 251.2 and 253.5).
+    auto go = [&](SpreadOnce& once, auto kern) {
+        launch_k(kern, grid, dim3(kThreads), want < cap ? spread_smem(once, kern, grid.x, 0) : 0, s, a);
+    };
+    static SpreadOnce once[3];
+    if (!D.bf16) go(once[0], combine_kernel<float, false>);
+    else if (bwd) go(once[1], combine_kernel<__nv_bfloat16, true>);
+    else go(once[2], combine_kernel<__nv_bfloat16, false>);
     UOE_LAUNCHED();
     return UOE_OK;
 }
