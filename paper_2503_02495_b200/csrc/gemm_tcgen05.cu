@@ -710,13 +710,15 @@ uoe_status launch_gemm_bf16(const GemmArgs& g, int* status, cudaStream_t s) {
     // head, 25600 rows x 1024 columns: 21 us in 32-column chunks, 19 so; K = 128, N = 1408, 67k rows, with the pre-activation: 82
     // and 68; on CTA pairs 131k rows, N = 1024: K = 256 115 and 99, K = 384 117 and 107, K = 512 equal, K = 1024 213 and 224.
     const bool short_k = g.K <= 128;
-    if (g.nmat == 3 && g.N == 64 && !g.b_kmajor && !g.pre) {
+    // (the epilogue of three matrices side by side stores the products as they are: no activation, like no bias and no factor above)
+    const bool side_by_side = g.nmat == 3 && !g.b_kmajor && g.act == UOE_ACT_IDENTITY;
+    if (side_by_side && g.N == 64) {
         if (rope) return launch_one<192, false, kForward, 1, false, true>(g, status, s);
         return short_k ? launch_one<192, false, kForward, 1, false, false, 64>(g, status, s) : launch_one<192, false, kForward, 1>(g, status, s);
     }
     // Two heads per expert: q, k, v as one 384-column tile (wide block above: forward 162.4 us with three 128-column tiles, 152.0 so,
     // training step 527 and 504)
-    if (g.nmat == 3 && g.N == 128 && !g.b_kmajor && !g.pre && !short_k && qkv_as_one_tile(g.rows_max, g.n, sm_count()))
+    if (side_by_side && g.N == 128 && !short_k && qkv_as_one_tile(g.rows_max, g.n, sm_count()))
         return rope ? launch_one<384, false, kForward, 1, false, true>(g, status, s) : launch_one<384, false, kForward, 1>(g, status, s);
     if (rope) return dispatch<false, kForward, true>(g, status, s);
     if (short_k) return g.b_kmajor ? dispatch<true, kForward, false, 64>(g, status, s) : dispatch<false, kForward, false, 64>(g, status, s);
