@@ -398,3 +398,66 @@ def test_projection_and_attention_in_one_kernel(name):
     ref = orc.smha_backward(x.f64, *[q.f64 for q in ws], Wr.f64, ro, dy.f64, w.d_h, w.causal, residual=False, d_rope=d_rope)
     for g, f in zip(got, ref[:6]):
         assert rel_inf(to_f64(g), f) <= TOL
+
+
+# which calls take that kernel, on both sides of each line (pairs against SMs, tokens per pair, whole tiles, resident clusters, width), and
+# widths whose last chunk of output columns is half a chunk; a width that 128 does not divide has no backward.  Pairs are counted in
+# SMs: (twice the SMs, + 2) and so on, two experts per sample.
+def _pairs(times, more=0):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+    return (times * sms + more) // 2
+
+
+def _short(pairs, l_a, **kw):
+    return _att(**{**dict(B=pairs, L=2 * l_a, L_valid=2 * l_a, m=4, c=2, d=128, n=4, k=2, H=4), **kw})
+
+
+DISPATCH = {
+    "d192_one_tile": (lambda: _att(B=3, L=192, L_valid=185, m=6, c=3, d=192, n=4, k=2, H=4), True, None),
+    "d448_one_tile": (lambda: _att(B=3, L=192, L_valid=185, m=6, c=3, d=448, n=4, k=2, H=4, causal=True), True, None),
+    "d192_cluster": (lambda: _att(B=3, L=512, L_valid=500, m=16, c=8, d=192, n=4, k=2, H=4, causal=True), True, None),
+    "d448_cluster": (lambda: _att(B=2, L=768, L_valid=700, m=12, c=6, d=448, n=4, k=2, H=4), True, None),
+    "d512": (lambda: _short(4, 64, d=512), True, True),
+    "d640": (lambda: _short(4, 64, d=640), False, True),
+    "two_pairs_per_sm": (lambda: _short(_pairs(2), 16), True, True),
+    "more_pairs_short": (lambda: _short(_pairs(2, 2), 16), True, False),
+    "four_pairs_per_sm": (lambda: _short(_pairs(4), 32), True, False),
+    "many_pairs_32": (lambda: _short(_pairs(4, 2), 32), False, False),
+    "many_pairs_48": (lambda: _short(_pairs(4, 2), 48, L=96, m=6, c=3), True, False),
+    "many_pairs_96": (lambda: _short(_pairs(5, 2), 96, L=192, L_valid=180, m=12, c=6), True, True),
+    "many_pairs_128": (lambda: _short(_pairs(5, 2), 128, causal=True), True, True),
+    "ragged_tiles": (lambda: _att(B=4, L=320, L_valid=320, m=10, c=5, d=128, n=4, k=2, H=4), False, False),
+    "nine_tiles": (lambda: _att(B=1, L=2304, L_valid=2300, m=18, c=9, d=128, n=2, k=1, H=2), False, False),
+    "clusters_beyond_a_wave": (lambda: _short(_pairs(1), 256, m=16, c=8), False, False),
+}
+
+
+@pytest.mark.parametrize("name", list(DISPATCH))
+def test_which_calls_take_the_one_kernel(name):
+    import paper_2503_02495_b200 as uoe
+    make, forward, backward = DISPATCH[name]
+    w = make()
+    x, Wr = gen.make_x(w), gen.store(gen.make_router(w, "att").f64 * 20, w.dtype)
+    ws, dy = gen.make_attn_weights(w), gen.make_dy(w)
+    prob = problem_of(w, "att", residual=False)
+    xd, Wrd, wd = to_dev(x), to_dev(Wr), [to_dev(q) for q in ws]
+    r = uoe.uoe_route(prob, xd, Wrd)
+    ro = orc.with_selection(x.f64, Wr.f64, r.expert_idx.cpu().numpy(), r.patch_idx.cpu().numpy(), w.m, w.L_valid)
+    fs = [q.f64 for q in ws]
+
+    def launched(call):
+        uoe.uoe_profile_enable(True)
+        out = call()
+        torch.cuda.synchronize()
+        uoe.uoe_profile_enable(False)
+        return out, "smha_fused" in [n for n, _ in uoe.uoe_profile_records()]
+
+    y, fused = launched(lambda: uoe.uoe_smha_forward(prob, xd, *wd, r))
+    assert fused == forward
+    assert rel_inf(to_f64(y), orc.smha_forward(x.f64, *fs, ro, w.d_h, w.causal, residual=False)) <= TOL
+    if backward is None:
+        return
+    got, fused = launched(lambda: uoe.uoe_smha_backward(prob, xd, *wd, Wrd, r, to_dev(dy)))
+    assert fused == backward
+    for g, f in zip(got, orc.smha_backward(x.f64, *fs, Wr.f64, ro, dy.f64, w.d_h, w.causal, residual=False)[:6]):
+        assert rel_inf(to_f64(g), f) <= TOL
