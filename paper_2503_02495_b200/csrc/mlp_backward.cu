@@ -21,8 +21,6 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 256;
-
 // Gradient of the router logits of one sample from the per-row gate gradients.  grid B, 256 or 512 threads, dynamic shared
 // memory (2 n m + k c) floats.  A warp per slab adds the slab's per-row, per-column-tile partials (fixed order), then the
 // softmax Jacobians of Eq. 14 and 21:  G[b,j,i] = dlogit_patch[b,i,j]/cnt_j + dlogit_samp[b,i]/L_valid.

@@ -231,7 +231,8 @@ gather_kernel(const uint4* __restrict__ src, const int* __restrict__ patch_idx, 
 // step waits for another warp.  (A CTA per 4 to 16 KB of output, which looks its slots up, meets, and then loads: thousands
 // of short CTAs, 7.2 us against 6.5 at 8 MB of output, 13 and 10 at 17 MB, 29 and 24 at 44 MB = 6.4 TB/s; image block forward
 // 220.5 -> 211, its training step 715 -> 704, long-document block 91.3 -> 85.4.  One vector per lane: 225 us, the four: 216 for
-// the image block; three or four slots in flight: 216 and 217.)
+// the image block; three or four slots in flight: 216 and 217.  With up to sixteen slots per patch, two / four in flight: 16 samples of 1024
+// tokens, d = 512, 495.6 / 499.5 us, 4 of them 165.5 / 171.2; one sample 87.0 / 82.9, d = 256 74.3 / 72.3, where the rounds are a chain.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kCombineVecs = 2, kCombineSlots = 2;
 

@@ -146,7 +146,11 @@ smha_fused_kernel(const __grid_constant__ FuMaps tm, const FuArgs a,
     int kv_end = min(ctl->n_valid, a.l_a);
     if (a.causal) kv_end = min(kv_end, q0 + T);
     const int n_kv = (kv_end + T - 1) / T;               // key tiles of this CTA's queries; 0 for a pair without a patch
-    // multi: the CTA's own tile first (it is in shared memory, the others are on their way), then the others in order
+    // multi: the CTA's own tile first (it is in shared memory, the others are on their way), then the others in order.  (In
+    // ascending order, as in the separate kernels, the own tile waits for the others': one sequence 54.6 us, so 52.9, language-model block
+    // 66.7 and 64.4, its training step 227.8 and 223.6.  The sums round in another order: gradients move by up to 8e-4 of their norm,
+    // the distance of dW_q, dW_k, dW_v, dW_o from float64, 2.8e-3 to 3.7e-3, by less than 0.1 %, that of dW_r, 2.6e-3 to 2.8e-3, by
+    // -2.3 to +0.5 %.)
     const bool own = !MULTI || qt < n_kv;
     auto tile_at = [&](int i) { return !MULTI ? 0 : (!own ? i : (i == 0 ? qt : (i - 1 < qt ? i - 1 : i))); };
     const int num_kb = a.d / BK;
@@ -522,14 +526,20 @@ int resident_clusters(int size) {
 
 bool smha_can_fuse(const Dims& D, bool recompute) {
     if (!can_fuse_gather(D) || D.d_h != DH || D.d_g != DH || D.n > 31) return false;
+    // Forward: widths up to 512, where the kernel was made.  Beyond, block forward, one kernel / separate: d = 576 71.1 / 74.2 us (64 pairs
+    // of 128 tokens), 286 / 318 (600), 80.4 / 90.2 (64 causal pairs of 256); d = 640 73.1 / 76.8, 276 / 296, 80.5 / 88.0; d = 1024 89.2 / 85.9,
+    // 398 / 409, 93.8 / 101.3: the line could lie higher except for few pairs of one tile, whose CTAs have a long projection to themselves.
     if (!recompute && D.d > 512) return false;
     const int n_qt = (D.l_a + T - 1) / T;
     const long long pairs = (long long)D.B * D.k;
-    // One tile: always while all pairs are resident at once, which leaves the launch in between as pure gain (160 pairs of 16 tokens,
-    // d = 512: forward 26.9 us, separate launches 38.7; backward 79.9 and 85.0).  Beyond that short pairs cost: a CTA projects 128 rows
-    // whatever they hold, the grouped projection packs them.  Forward, 4000 pairs, d = 256, 32 / 48 / 96 tokens: 203 / 224 / 285 us,
-    // separate 202 / 227 / 300; 600 pairs of 16 tokens 43.9 and 50.3.  The recomputation also writes q, k, v, o: backward of 4000
-    // pairs of 48 / 80 / 96 tokens, d = 512: 694 / 971 / 1120 us, separate 657 / 952 / 1133.
+    // One tile: always while all pairs are resident at once, which leaves the launch in between as pure gain (400 pairs of 16 / 48 tokens,
+    // d = 512: block forward 82.0 / 97.6 us, separate launches 88.1 / 110.5).  Beyond that short pairs cost: a CTA projects 128 rows
+    // whatever they hold, the grouped projection packs them.  Block forward, d = 512, one kernel / separate: pairs of 48 tokens 122 / 132 us
+    // (600 of them), 312 / 334 (2000); of 32 tokens 117 / 124.5 (600), 184 / 193 (1200), 269 / 279 (2000); of 16 tokens 97.5 / 102.6 (600),
+    // 158 / 164 (1200), 211 / 210 (2000); d = 256, 4000 pairs of 32 tokens 203 / 202.  So the lines at 48 tokens and at four pairs per SM
+    // are on the safe side: up to 2000 pairs of 16 tokens and more of 32 the one kernel would still gain 2 to 6 %.
+    // The recomputation also writes q, k, v, o.  Training step, d = 512, one kernel / separate: 1600 pairs of 16 / 48 / 80 tokens 548 / 522,
+    // 788 / 776, 1019 / 1014 us, 300 pairs 238 / 236, 259 / 255, 309 / 311; backward of 4000 pairs of 80 / 96 tokens 971 / 952, 1120 / 1133.
     if (n_qt == 1) {
         if (pairs <= 2ll * sm_count()) return true;
         if (recompute) return D.l_a >= 96;
