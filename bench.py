@@ -671,26 +671,26 @@ HBM_KERNELS = ("route", "gather", "combine", "router_apply")
 # changed since, the line reports null instead of a stale figure.  (workload, kernel label) ->
 # (bytes per launch at the benchmark's size, source file, sha1 prefix, profiles/ summary)
 NCU_TRAFFIC = {
-    ("cfg5_scale", "wgrad_W2"): (949.6e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "wgrad_W1"): (860.8e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "gemm1_act"): (935.3e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "gemm2"): (947.3e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "bwd_da_dh"): (1120.1e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "bwd_dx"): (931.4e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg5_scale", "route"): (268.9e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "wgrad_W2"): (943.9e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "wgrad_W1"): (862.7e6, "wgrad_tcgen05.cu", "7a029204e417", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "gemm1_act"): (934.9e6, "gemm_tcgen05.cu", "6e1197b3efc4", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "gemm2"): (948.3e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "bwd_da_dh"): (1117.9e6, "gemm_tcgen05.cu", "6e1197b3efc4", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "bwd_dx"): (937.3e6, "gemm2_patch_tcgen05.cu", "9b1f0f0d537d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg5_scale", "route"): (269.0e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
     ("cfg2_lm", "route"): (8.5e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "smha_fused"): (10.3e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg2_lm", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "mlp_fused"): (12.3e6, "mlp_fused_tcgen05.cu", "6456cbf86c3d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "smha_fused"): (10.3e6, "smha_fused_tcgen05.cu", "0802d76376a3", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg2_lm", "combine"): (25.2e6, "routed.cu", "dc63ec10246c", "profiles/dram_traffic_per_kernel.md"),
     ("cfg3_long", "route"): (16.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "attention"): (6.5e6, "attn_tcgen05.cu", "439d84d4e4fe", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "combine"): (25.2e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg3_long", "qkv_proj"): (8.3e6, "gemm_tcgen05.cu", "114bcd0660a9", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "mlp_fused"): (9.0e6, "mlp_fused_tcgen05.cu", "6456cbf86c3d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "attention"): (6.5e6, "attn_tcgen05.cu", "4cdb5440a2c7", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "combine"): (25.2e6, "routed.cu", "dc63ec10246c", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg3_long", "qkv_proj"): (8.3e6, "gemm_tcgen05.cu", "6e1197b3efc4", "profiles/dram_traffic_per_kernel.md"),
     ("cfg4_vit", "route"): (38.8e6, "route.cu", "dd411372f114", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "mlp_fused"): (60.5e6, "mlp_fused_tcgen05.cu", "30bdd2ad96af", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "smha_fused"): (54.9e6, "smha_fused_tcgen05.cu", "3777cb784ed7", "profiles/dram_traffic_per_kernel.md"),
-    ("cfg4_vit", "combine"): (120.6e6, "routed.cu", "b8e6bf03b44c", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "mlp_fused"): (59.7e6, "mlp_fused_tcgen05.cu", "6456cbf86c3d", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "smha_fused"): (53.9e6, "smha_fused_tcgen05.cu", "0802d76376a3", "profiles/dram_traffic_per_kernel.md"),
+    ("cfg4_vit", "combine"): (120.7e6, "routed.cu", "dc63ec10246c", "profiles/dram_traffic_per_kernel.md"),
 }
 
 
